@@ -131,49 +131,50 @@ __device__ __forceinline__ void tc_fence_after() {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
 
-// D[tmem] (+)= A[smem] * B[smem]^T, one thread issues
-__device__ __forceinline__ void umma_f16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
-                                         uint32_t idesc, uint32_t accumulate) {
+// One lane of a converged warp, the same one each time (1 there, 0 elsewhere).
+__device__ __forceinline__ uint32_t elect_one() {
+  uint32_t l;
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate));
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(l));
+  return l;
 }
 
-// The same with a usage hint for the A operand's collector buffer: U = 1
-// reads A from shared memory and keeps it (fill), U = 2 reuses the kept A
-// (use), U = 3 reuses it for the last time (lastuse), U = 0 reads A and does
-// not keep it (discard, the default).  A run fill, use..., lastuse must pass
-// the same A descriptor and be consecutive MMAs of this thread.
+// D[tmem] (+)= A[smem] * B[smem]^T, issued by the lane whose `lead` is 1 of a
+// converged warp: with the whole warp at the instruction the compiler keeps
+// the descriptors in uniform registers, which tcgen05.mma reads.  Issued from
+// under a single-thread branch the same instruction took ~80 clocks instead
+// of ~49 (128 x 96 x 16, the time of the product itself).
+// U is a usage hint for the A operand's collector buffer: U = 1 reads A from
+// shared memory and keeps it (fill), U = 2 reuses the kept A (use), U = 3
+// reuses it for the last time (lastuse), U = 0 reads A and does not keep it
+// (discard, the default).  A run fill, use..., lastuse must pass the same A
+// descriptor and be consecutive MMAs of this thread.
+#define CC3_UMMA(HINT)                                                             \
+  asm volatile(                                                                    \
+      "{\n\t.reg .pred p, l;\n\t"                                                  \
+      "setp.ne.b32 p, %4, 0;\n\t"                                                  \
+      "setp.ne.b32 l, %5, 0;\n\t"                                                  \
+      "@l tcgen05.mma.cta_group::1.kind::f16" HINT " [%0], %1, %2, %3, p;\n\t}" ::"r"( \
+          d_tmem),                                                                 \
+      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(lead))
 template <int U>
-__device__ __forceinline__ void umma_f16_a(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
-                                           uint32_t idesc, uint32_t accumulate) {
+__device__ __forceinline__ void umma_f16_a(uint32_t lead, uint32_t d_tmem, uint64_t a_desc,
+                                           uint64_t b_desc, uint32_t idesc,
+                                           uint32_t accumulate) {
   if constexpr (U == 1) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16.collector::a::fill [%0], %1, %2, %3, p;\n\t}" ::"r"(
-            d_tmem),
-        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate));
+    CC3_UMMA(".collector::a::fill");
   } else if constexpr (U == 2) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16.collector::a::use [%0], %1, %2, %3, p;\n\t}" ::"r"(
-            d_tmem),
-        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate));
+    CC3_UMMA(".collector::a::use");
   } else if constexpr (U == 3) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16.collector::a::lastuse [%0], %1, %2, %3, p;\n\t}" ::"r"(
-            d_tmem),
-        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate));
+    CC3_UMMA(".collector::a::lastuse");
   } else {
-    umma_f16(d_tmem, a_desc, b_desc, idesc, accumulate);
+    CC3_UMMA("");
   }
 }
+#undef CC3_UMMA
 
 // arrive on `bar` when every previously issued tcgen05.mma of this thread completes
 __device__ __forceinline__ void umma_commit(uint64_t *bar) {

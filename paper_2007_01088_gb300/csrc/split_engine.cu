@@ -55,35 +55,41 @@ __device__ __forceinline__ long long s_rowoff(int m, int m_in, long long s1, lon
   return (long long)(m / m_in) * s1 + (long long)(m % m_in) * s0;
 }
 
+// Whether the first product into an accumulator adds to what it holds (1) or
+// overwrites it (0): low for accumulators 0..3, high for the shared one.
+struct AccMode {
+  uint32_t low, high;
+};
+
 // One slice product p x q into accumulator min(p + q, 4), as element `i` of
 // a run of `n` products that share A slice p (the run keeps A in the
 // collector buffer instead of reading it from shared memory again).
 template <int S>
-__device__ __forceinline__ void issue_one(uint32_t tmem, uint64_t dA, uint64_t dB, uint32_t a16,
-                                          uint32_t b16, uint32_t Nt, uint32_t idesc,
-                                          uint32_t &fresh, int p, int q, int i, int n) {
+__device__ __forceinline__ void issue_one(uint32_t lead, uint32_t tmem, uint64_t dA, uint64_t dB,
+                                          uint32_t Nt, uint32_t idesc, uint32_t en, int p, int q,
+                                          int i, int n) {
   const int lv = p + q;
-  const int acc = lv < 4 ? lv : 4;
-  const uint32_t d = tmem + (uint32_t)acc * Nt, en = ((fresh >> acc) & 1u) ^ 1u;
-  const uint64_t a = dA + (uint64_t)(p * a16), b = dB + (uint64_t)(q * b16);
+  const uint32_t d = tmem + (uint32_t)(lv < 4 ? lv : 4) * Nt;
+  // slices are 256 bytes (16 descriptor units) apart
+  const uint64_t a = dA + (uint64_t)(p * 16), b = dB + (uint64_t)(q * 16);
   if (n == 1)
-    umma_f16_a<0>(d, a, b, idesc, en);
+    umma_f16_a<0>(lead, d, a, b, idesc, en);
   else if (i == 0)
-    umma_f16_a<1>(d, a, b, idesc, en);
+    umma_f16_a<1>(lead, d, a, b, idesc, en);
   else if (i == n - 1)
-    umma_f16_a<3>(d, a, b, idesc, en);
+    umma_f16_a<3>(lead, d, a, b, idesc, en);
   else
-    umma_f16_a<2>(d, a, b, idesc, en);
-  fresh &= ~(1u << acc);
+    umma_f16_a<2>(lead, d, a, b, idesc, en);
 }
 
 // Issues the slice products of one K step whose level is >= 4 (HIGH) or
-// <= 3 (!HIGH), fully unrolled; bit L of `fresh` marks accumulator L as not
-// yet written since its last reset (its first product overwrites it).
+// <= 3 (!HIGH), fully unrolled; `en` is the mode of each accumulator's first
+// product here.  That product is (0, level) for levels <= 3; the shared
+// accumulator's is (0, 4).
 template <int S, bool HIGH>
-__device__ __forceinline__ void issue_products(uint32_t tmem, uint64_t dA, uint64_t dB,
-                                               uint32_t a16, uint32_t b16, uint32_t Nt,
-                                               uint32_t idesc, uint32_t &fresh) {
+__device__ __forceinline__ void issue_products(uint32_t lead, uint32_t tmem, uint64_t dA,
+                                               uint64_t dB, uint32_t Nt, uint32_t idesc,
+                                               uint32_t en) {
 #pragma unroll
   for (int p = 0; p < S; ++p) {
     // q range of this group for slice p
@@ -91,7 +97,8 @@ __device__ __forceinline__ void issue_products(uint32_t tmem, uint64_t dA, uint6
     const int qhi = HIGH ? S - 1 - p : (3 - p < S - 1 - p ? 3 - p : S - 1 - p);
 #pragma unroll
     for (int q = qlo; q <= qhi; ++q)
-      issue_one<S>(tmem, dA, dB, a16, b16, Nt, idesc, fresh, p, q, q - qlo, qhi - qlo + 1);
+      issue_one<S>(lead, tmem, dA, dB, Nt, idesc, p == 0 && q <= 4 ? en : 1u, p, q, q - qlo,
+                   qhi - qlo + 1);
   }
 }
 
@@ -99,14 +106,15 @@ __device__ __forceinline__ void issue_products(uint32_t tmem, uint64_t dA, uint6
 // that does not wait for a drain): A is read from shared memory S times
 // instead of once per product.
 template <int S>
-__device__ __forceinline__ void issue_products_all(uint32_t tmem, uint64_t dA, uint64_t dB,
-                                                   uint32_t a16, uint32_t b16, uint32_t Nt,
-                                                   uint32_t idesc, uint32_t &fresh) {
+__device__ __forceinline__ void issue_products_all(uint32_t lead, uint32_t tmem, uint64_t dA,
+                                                   uint64_t dB, uint32_t Nt, uint32_t idesc,
+                                                   AccMode en) {
 #pragma unroll
   for (int p = 0; p < S; ++p)
 #pragma unroll
     for (int q = 0; q < S - p; ++q)
-      issue_one<S>(tmem, dA, dB, a16, b16, Nt, idesc, fresh, p, q, q, S - p);
+      issue_one<S>(lead, tmem, dA, dB, Nt, idesc,
+                   p == 0 && q <= 4 ? (q < 4 ? en.low : en.high) : 1u, p, q, q, S - p);
 }
 
 // The slice products of two consecutive K steps with their A-slice runs
@@ -115,17 +123,19 @@ __device__ __forceinline__ void issue_products_all(uint32_t tmem, uint64_t dA, u
 // step's products instead of waiting alone.  Each run keeps its A slice in
 // the collector buffer, as in issue_products_all.
 template <int S>
-__device__ __forceinline__ void issue_products_pair(uint32_t tmem, uint64_t dA0, uint64_t dB0,
-                                                    uint32_t id0, uint64_t dA1, uint64_t dB1,
-                                                    uint32_t id1, uint32_t Nt, uint32_t &fresh) {
+__device__ __forceinline__ void issue_products_pair(uint32_t lead, uint32_t tmem, uint64_t dA0,
+                                                    uint64_t dB0, uint32_t id0, uint64_t dA1,
+                                                    uint64_t dB1, uint32_t id1, uint32_t Nt,
+                                                    AccMode en) {
 #pragma unroll
   for (int p = 0; p < S; ++p) {
 #pragma unroll
     for (int q = 0; q < S - p; ++q)
-      issue_one<S>(tmem, dA0, dB0, 16u, 16u, Nt, id0, fresh, p, q, q, S - p);
+      issue_one<S>(lead, tmem, dA0, dB0, Nt, id0,
+                   p == 0 && q <= 4 ? (q < 4 ? en.low : en.high) : 1u, p, q, q, S - p);
 #pragma unroll
     for (int q = 0; q < S - p; ++q)
-      issue_one<S>(tmem, dA1, dB1, 16u, 16u, Nt, id1, fresh, p, q, q, S - p);
+      issue_one<S>(lead, tmem, dA1, dB1, Nt, id1, 1u, p, q, q, S - p);
   }
 }
 
@@ -417,36 +427,39 @@ split_engine_kernel(const SJob *__restrict__ jobs, int njobs, const STerm *__res
         mbar_wait_quiet(&full[i % S_STAGES], (i / S_STAGES) & 1, 500000000ull);
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      // MMA issuer
+    {
+      // MMA issuer: the warp stays converged (every lane waits and steps, the
+      // elected one issues), see umma_f16_a
+      const uint32_t lead = elect_one();
       int it = 0, nd = 0;
       bool ok = true;
       for (int i = 0; ok; ++i) {
         const int q = i % TQ;
-        if (!mbar_wait(&tfull[q], (i / TQ) & 1, &err)) break;
+        if (!__all_sync(0xffffffffu, mbar_wait(&tfull[q], (i / TQ) & 1, &err))) break;
         const long long tile = tq[q];
-        const TileInfo ti = tinfo[q];  // read before the slot is handed back
-        mbar_arrive(&tempty[q]);
+        const int Nt = tinfo[q].Nt, g0 = tinfo[q].g0, g1 = tinfo[q].g1;
+        __syncwarp();  // every lane has read the slot before it is handed back
+        if (lead) mbar_arrive(&tempty[q]);
         if (tile < 0) break;
-        const int Nt = ti.Nt;
         const uint32_t id_pos = idesc_bf16(S_BM, Nt, 0), id_neg = idesc_bf16(S_BM, Nt, 1);
         // the epilogue has read the previous tile's accumulators
         if (i > 0) {
-          if (!mbar_wait(&accempty, (i - 1) & 1, &err)) break;
+          if (!__all_sync(0xffffffffu, mbar_wait(&accempty, (i - 1) & 1, &err))) break;
           tc_fence_after();
         }
-        uint32_t fresh = (1u << S_NACC) - 1;
+        AccMode en = {0u, 0u};
         int since = 0;
         bool pending = false;
         // K steps two at a time (drains come every kdrain_steps, an even
         // number, so a pair never straddles one); a lone last step of a tile
         // goes alone
-        for (int g = ti.g0; g < ti.g1;) {
-          const bool two = g + 1 < ti.g1;
+        for (int g = g0; g < g1;) {
+          const bool two = g + 1 < g1;
           const int st0 = it % S_STAGES, ph0 = (it / S_STAGES) & 1;
           const int st1 = (it + 1) % S_STAGES, ph1 = ((it + 1) / S_STAGES) & 1;
-          if (!mbar_wait(&full[st0], ph0, &err)) { ok = false; break; }
-          if (two && !mbar_wait(&full[st1], ph1, &err)) { ok = false; break; }
+          bool here = mbar_wait(&full[st0], ph0, &err);
+          if (two) here = here && mbar_wait(&full[st1], ph1, &err);
+          if (!__all_sync(0xffffffffu, here)) { ok = false; break; }
           tc_fence_after();
           const uint32_t id0 = sneg[st0] ? id_neg : id_pos, id1 = sneg[st1] ? id_neg : id_pos;
           const size_t stage_bytes = (size_t)s * (a_bytes + S_NT_MAX * 32);
@@ -459,38 +472,47 @@ split_engine_kernel(const SJob *__restrict__ jobs, int njobs, const STerm *__res
                          dB1 = smem_desc_kmajor(sa1 + (uint32_t)s * a_bytes, 256u * s);
           if (pending) {
             // levels >= 4 first (they never wait for a drain), then levels 0..3
-            issue_products<S, true>(tmem, dA0, dB0, 16u, 16u, (uint32_t)Nt, id0, fresh);
-            if (two) issue_products<S, true>(tmem, dA1, dB1, 16u, 16u, (uint32_t)Nt, id1, fresh);
-            if (!mbar_wait(&drainempty, nd & 1, &err)) { ok = false; break; }
+            issue_products<S, true>(lead, tmem, dA0, dB0, (uint32_t)Nt, id0, 1u);
+            if (two) issue_products<S, true>(lead, tmem, dA1, dB1, (uint32_t)Nt, id1, 1u);
+            if (!__all_sync(0xffffffffu, mbar_wait(&drainempty, nd & 1, &err))) {
+              ok = false;
+              break;
+            }
             tc_fence_after();
             ++nd;
             pending = false;
-            fresh |= 0xFu;
-            issue_products<S, false>(tmem, dA0, dB0, 16u, 16u, (uint32_t)Nt, id0, fresh);
-            if (two) issue_products<S, false>(tmem, dA1, dB1, 16u, 16u, (uint32_t)Nt, id1, fresh);
+            issue_products<S, false>(lead, tmem, dA0, dB0, (uint32_t)Nt, id0, 0u);
+            if (two) issue_products<S, false>(lead, tmem, dA1, dB1, (uint32_t)Nt, id1, 1u);
           } else if (two) {
-            issue_products_pair<S>(tmem, dA0, dB0, id0, dA1, dB1, id1, (uint32_t)Nt, fresh);
+            issue_products_pair<S>(lead, tmem, dA0, dB0, id0, dA1, dB1, id1, (uint32_t)Nt, en);
           } else {
-            issue_products_all<S>(tmem, dA0, dB0, 16u, 16u, (uint32_t)Nt, id0, fresh);
+            issue_products_all<S>(lead, tmem, dA0, dB0, (uint32_t)Nt, id0, en);
           }
-          umma_commit(&empty[st0]);
-          if (two) umma_commit(&empty[st1]);
+          en = {1u, 1u};
           const int n = two ? 2 : 1;
           g += n;
           it += n;
           since += n;
-          if (since >= kdrain_steps && g < ti.g1) {
-            umma_commit(&drainfull);
+          const bool drain = since >= kdrain_steps && g < g1;
+          if (lead) {
+            umma_commit(&empty[st0]);
+            if (two) umma_commit(&empty[st1]);
+            if (drain) umma_commit(&drainfull);
+          }
+          __syncwarp();
+          if (drain) {
             pending = true;
             since = 0;
           }
         }
         if (!ok) break;
-        umma_commit(&accfull);
+        if (lead) umma_commit(&accfull);
+        __syncwarp();
       }
       // every product this thread issued has landed in tensor memory before
       // the CTA frees it, also after a give-up (bounded)
-      umma_commit(&mmafin);
+      __syncwarp();
+      if (lead) umma_commit(&mmafin);
       mbar_wait_quiet(&mmafin, 0, 500000000ull);
     }
   } else {
