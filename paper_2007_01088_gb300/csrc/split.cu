@@ -366,7 +366,6 @@ int new_sjob(SPlan &P, int M, int N, int Ntile, int batch, int ksplit, int mode,
   j.expo = expo;
   j.expo_slot = -1;
   j.expo_slot2 = -1;
-  j.mult = 1.0f;
   j.tiles_m = (M + S_BM - 1) / S_BM;
   j.tiles_n = (N + Ntile - 1) / Ntile;
   j.term0 = (int)P.terms.size();
@@ -419,9 +418,11 @@ const WMaps kStdMaps = {MA_T2S, MB_T2S, MA_T2C, MB_T2C, MA_T2R, MB_T2R,
 // (x, 0..nv-1)); it is the A operand, its nv slabs read as one array of
 // nv * rows flattened rows (rows: the slab's row count, nv padded to 8), so
 // the tiles cover the nv^2 x nv block of W without M padding.
-//   phase 1: rows (c, a), columns b -> W_1[c][a][b]
+//   phase 1: rows (c, a), columns b -> W_1[c][b][a]
 //   phase 2: rows (c, b), columns a -> W_2[c][a][b]
 //   phase 3: rows (a, b), columns c -> W_3[c][a][b]
+// The fastest index of each output is the fastest one of its tile's rows, so
+// that the 32 rows of a warp store 256 contiguous bytes per column.
 // The three phases write separate buffers (W_2 in the tau~ workspace), so one
 // launch runs them all; the element-wise step forms tau = (W_1 + W_2 + W_3) /
 // (w - eps) and tau~ from the three.
@@ -432,7 +433,7 @@ int w_job(SPlan &P, int nv, int rows, int Nt, int phase, int slot, int E, double
   OutD C = outd(phase == 1 ? B_WS_W : (phase == 2 ? B_WS_TT : B_WS_W3), slot * nv3, 0, 0);
   C.m_in = rows;
   if (phase == 1) {
-    C.sm1 = nv2, C.sm0 = nv, C.sn0 = 1;
+    C.sm1 = nv2, C.sm0 = 1, C.sn0 = nv;
   } else if (phase == 2) {
     C.sm1 = nv2, C.sm0 = 1, C.sn0 = nv;
   } else {
@@ -1868,7 +1869,7 @@ int split_left_jacobian(cc3_ctx *c, int nvec, const double *w, const double *L1d
     TRY(run(pQ.v[b], aq, P, TR_SPLIT_OMEGA));
     TRY(run(pAB.v[b], jr, PR, TR_SPLIT_W));
     trace_begin(c, TR_SPLIT_ELEM, st);
-    TRY(launch_left_outer_dd(Wj, tri_all + 3 * t0, bj, ns, nslot, l1dd, ltdd, ovdd, fdd, no, nv,
+    TRY(launch_left_outer_dd(W3j, tri_all + 3 * t0, bj, ns, nslot, l1dd, ltdd, ovdd, fdd, no, nv,
                              st));
     trace_end(c, TR_SPLIT_ELEM, st, 0.0, 0.0);
     *L += 1;
@@ -2256,7 +2257,7 @@ int split_density(cc3_ctx *c, double w, const double *L1d, const double *L2d, do
     // exponent for the batch) with its slices, kept resident
     TRY(run(ab, jr, PR, TR_SPLIT_W));
     trace_begin(c, TR_SPLIT_ELEM, st);
-    TRY(launch_left_outer_dd(Wj, tri_ext + 3 * t0, bj, ns, ns, l1dd, ltdd, ovdd, fdd, no, nv, st));
+    TRY(launch_left_outer_dd(W3j, tri_ext + 3 * t0, bj, ns, ns, l1dd, ltdd, ovdd, fdd, no, nv, st));
     CU(cudaMemsetAsync(maxj, 0, sizeof(unsigned int) * bj, st));
     TRY(launch_tau_contravariant_dd(Wj, TTj, W3j, TTj, S->evdd, eol + t0, 0.f, 0.f, nv, ns, maxj,
                                     st));

@@ -9,23 +9,34 @@
 // does not round to nearest when addends of very different size meet, so
 // each level L = p + q <= 3 gets its own tensor-memory accumulator, whose
 // values stay exactly representable (multiples of 2^-8L below 2^(24-8L))
-// because it is drained into double-float registers every 256 K (at most
-// 4 products of |d d'| <= 2^14 per K); the levels >= 4 share a fifth,
-// rounded accumulator (its error stays below 2^-50 of the result).
+// because it is drained into 64-bit fixed-point registers every 256 or 512 K;
+// the levels >= 4 share a fifth, rounded accumulator (its error stays below
+// 2^-50 of the result).
 //
 // Warp roles (576 threads): warp 0 issues one bulk copy per operand tile (all
 // s slices of a 128 x 16 A tile, resp. an Ntile x 16 B tile, pre-tiled in
 // global memory in the canonical no-swizzle order with the slices interleaved
 // per row group; one copy per slab when the A rows are flattened over slabs)
-// into a ring of stages; one thread of warp 1 issues tcgen05.mma (M = 128,
-// N = Ntile <= 96, K = 16, FP32 accumulate, A kept in the collector buffer
-// across the products of one A slice) and owns the tensor-memory allocation
-// (5 x Ntile columns); warps 2-17 drain and finish the accumulators (each
-// quadrant of 32 TMEM lanes is read by four warps, one per column quarter, 4
-// columns per load) and write the outputs (double-float stores, FP64 atomics
-// or 128-bit fixed-point atomics) through up to four output descriptors.  At
-// a drain point the issuer queues the next step's level >= 4 products before
-// it waits for the drain, so the drain overlaps tensor work.  Every wait is
+// into a ring of stages; warp 1 issues tcgen05.mma (M = 128, N = Ntile <= 96,
+// K = 16, FP32 accumulate, A kept in the collector buffer across the products
+// of one A slice) and owns the tensor-memory allocation (5 x 96 columns);
+// warps 2-17 drain and finish the accumulators (each quadrant of 32 TMEM lanes
+// is read by four warps, one per column quarter, 4 columns per load) and write
+// the outputs (double-float stores, FP64 atomics or 128-bit fixed-point
+// atomics) through up to four output descriptors.  At a drain point the issuer
+// queues the next steps' products into the other accumulators before it waits
+// for the drain; at a tile's end it issues levels 0..3 first, so that they are
+// read while the shared accumulator's products run, and the next tile starts
+// with levels 0..3 while that one is read.
+//
+// What bounds it: a 128 x 96 x 16 product takes 53 clocks here (48 at the
+// nominal rate; 21 of them per K step, 1118 clocks, next to 43 KB of operands
+// arriving).  Measured in the engine on 96 triples of the no=22 nv=250
+// residual, per K step: 1902 clocks with the sums in double-float arithmetic
+// (a tile's read-back 7600 clocks, its outputs 23,700: FP64 conversions, one
+// 8-byte store per 32-byte sector in the W build's first phase), 1570 with the
+// fixed-point sums (read-back 3600, of which ~1000 stall the tensor cores;
+// outputs 11,100).  Every wait is
 // bounded: on timeout the CTA sets an error word that the host turns into
 // CC3_ERR_TIMEOUT; before it exits, the CTA waits (bounded again) for its own
 // bulk copies and tensor-core products in flight, then frees its tensor
@@ -55,21 +66,16 @@ __device__ __forceinline__ long long s_rowoff(int m, int m_in, long long s1, lon
   return (long long)(m / m_in) * s1 + (long long)(m % m_in) * s0;
 }
 
-// Whether the first product into an accumulator adds to what it holds (1) or
-// overwrites it (0): low for accumulators 0..3, high for the shared one.
-struct AccMode {
-  uint32_t low, high;
-};
-
-// One slice product p x q into accumulator min(p + q, 4), as element `i` of
+// One slice product p x q into accumulator min(p + q, 4) (at a fixed column,
+// so that tiles of different N keep out of each other's), as element `i` of
 // a run of `n` products that share A slice p (the run keeps A in the
 // collector buffer instead of reading it from shared memory again).
 template <int S>
 __device__ __forceinline__ void issue_one(uint32_t lead, uint32_t tmem, uint64_t dA, uint64_t dB,
-                                          uint32_t Nt, uint32_t idesc, uint32_t en, int p, int q,
-                                          int i, int n) {
+                                          uint32_t idesc, uint32_t en, int p, int q, int i,
+                                          int n) {
   const int lv = p + q;
-  const uint32_t d = tmem + (uint32_t)(lv < 4 ? lv : 4) * Nt;
+  const uint32_t d = tmem + (uint32_t)((lv < 4 ? lv : 4) * S_NT_MAX);
   // slices are 256 bytes (16 descriptor units) apart
   const uint64_t a = dA + (uint64_t)(p * 16), b = dB + (uint64_t)(q * 16);
   if (n == 1)
@@ -82,61 +88,132 @@ __device__ __forceinline__ void issue_one(uint32_t lead, uint32_t tmem, uint64_t
     umma_f16_a<2>(lead, d, a, b, idesc, en);
 }
 
-// Issues the slice products of one K step whose level is >= 4 (HIGH) or
-// <= 3 (!HIGH), fully unrolled; `en` is the mode of each accumulator's first
-// product here.  That product is (0, level) for levels <= 3; the shared
-// accumulator's is (0, 4).
-template <int S, bool HIGH>
+// The accumulators that drain d of a tile (counted from 0) empties: levels 0,
+// 2 and 3 at every drain, level 1 too at every second one.  With a drain every
+// 256 K (or fewer) that keeps them exact: per K at most 1, 2, 3, 4 products of
+// |d d'| <= 2^14 reach level 0, 1, 2, 3, so the sums stay within 2^22, 2^24
+// (512 K), 3 2^22 and 2^24 of their unit 2^-8L.
+__device__ __forceinline__ bool drains_all(int d) { return (d & 1) != 0; }
+constexpr uint32_t DRAIN_SOME = 0xDu, DRAIN_ALL = 0xFu, ACC_HIGH = 0x10u;
+
+// K steps between drains of a tile of `steps` steps: equal parts of at most
+// kdrain_steps, an even number (the issuer takes steps in pairs).
+__device__ __forceinline__ int drain_interval(int steps, int kdrain_steps) {
+  const int parts = (steps + kdrain_steps - 1) / kdrain_steps;
+  return parts > 1 ? 2 * ((steps + 2 * parts - 1) / (2 * parts)) : kdrain_steps;
+}
+
+// Issues the slice products of one K step into the accumulators of MASK (bit
+// L: accumulator L), A slice by A slice, fully unrolled; `en` is the mode of
+// each accumulator's first product here, which is its product with A slice 0.
+template <int S, uint32_t MASK>
 __device__ __forceinline__ void issue_products(uint32_t lead, uint32_t tmem, uint64_t dA,
-                                               uint64_t dB, uint32_t Nt, uint32_t idesc,
-                                               uint32_t en) {
+                                               uint64_t dB, uint32_t idesc, uint32_t en) {
 #pragma unroll
   for (int p = 0; p < S; ++p) {
-    // q range of this group for slice p
-    const int qlo = HIGH ? (4 - p > 0 ? 4 - p : 0) : 0;
-    const int qhi = HIGH ? S - 1 - p : (3 - p < S - 1 - p ? 3 - p : S - 1 - p);
+    int n = 0;
 #pragma unroll
-    for (int q = qlo; q <= qhi; ++q)
-      issue_one<S>(lead, tmem, dA, dB, Nt, idesc, p == 0 && q <= 4 ? en : 1u, p, q, q - qlo,
-                   qhi - qlo + 1);
+    for (int q = 0; q < S - p; ++q) n += (MASK >> (p + q < 4 ? p + q : 4)) & 1u;
+    int i = 0;
+#pragma unroll
+    for (int q = 0; q < S - p; ++q)
+      if ((MASK >> (p + q < 4 ? p + q : 4)) & 1u) {
+        issue_one<S>(lead, tmem, dA, dB, idesc, p == 0 && q <= 4 ? en : 1u, p, q, i, n);
+        ++i;
+      }
   }
 }
 
-// All slice products of one K step, A slice by A slice (the order of a step
-// that does not wait for a drain): A is read from shared memory S times
-// instead of once per product.
-template <int S>
-__device__ __forceinline__ void issue_products_all(uint32_t lead, uint32_t tmem, uint64_t dA,
-                                                   uint64_t dB, uint32_t Nt, uint32_t idesc,
-                                                   AccMode en) {
-#pragma unroll
-  for (int p = 0; p < S; ++p)
-#pragma unroll
-    for (int q = 0; q < S - p; ++q)
-      issue_one<S>(lead, tmem, dA, dB, Nt, idesc,
-                   p == 0 && q <= 4 ? (q < 4 ? en.low : en.high) : 1u, p, q, q, S - p);
+// The K steps right after a drain point: first the products into the
+// accumulators that are not being emptied (MASK: those that are), then, once
+// the epilogue has read them, the others, which start anew.
+template <int S, uint32_t MASK>
+__device__ __forceinline__ bool issue_after_drain(uint32_t lead, uint32_t tmem, uint64_t dA0,
+                                                  uint64_t dB0, uint32_t id0, uint64_t dA1,
+                                                  uint64_t dB1, uint32_t id1, bool two,
+                                                  uint64_t *empty, int parity,
+                                                  volatile int *err) {
+  constexpr uint32_t KEEP = 0x1Fu & ~MASK;
+  issue_products<S, KEEP>(lead, tmem, dA0, dB0, id0, 1u);
+  if (two) issue_products<S, KEEP>(lead, tmem, dA1, dB1, id1, 1u);
+  if (!__all_sync(0xffffffffu, mbar_wait(empty, parity, err))) return false;
+  tc_fence_after();
+  issue_products<S, MASK>(lead, tmem, dA0, dB0, id0, 0u);
+  if (two) issue_products<S, MASK>(lead, tmem, dA1, dB1, id1, 1u);
+  return true;
 }
 
 // The slice products of two consecutive K steps with their A-slice runs
 // interleaved (run p of step 0, run p of step 1, run p + 1 of step 0, ...):
 // the first products that read a newly landed stage then overlap the other
 // step's products instead of waiting alone.  Each run keeps its A slice in
-// the collector buffer, as in issue_products_all.
+// the collector buffer: A is read from shared memory S times per step instead
+// of once per product.
 template <int S>
 __device__ __forceinline__ void issue_products_pair(uint32_t lead, uint32_t tmem, uint64_t dA0,
                                                     uint64_t dB0, uint32_t id0, uint64_t dA1,
-                                                    uint64_t dB1, uint32_t id1, uint32_t Nt,
-                                                    AccMode en) {
+                                                    uint64_t dB1, uint32_t id1) {
 #pragma unroll
   for (int p = 0; p < S; ++p) {
 #pragma unroll
     for (int q = 0; q < S - p; ++q)
-      issue_one<S>(lead, tmem, dA0, dB0, Nt, id0,
-                   p == 0 && q <= 4 ? (q < 4 ? en.low : en.high) : 1u, p, q, q, S - p);
+      issue_one<S>(lead, tmem, dA0, dB0, id0, 1u, p, q, q, S - p);
 #pragma unroll
     for (int q = 0; q < S - p; ++q)
-      issue_one<S>(lead, tmem, dA1, dB1, Nt, id1, 1u, p, q, q, S - p);
+      issue_one<S>(lead, tmem, dA1, dB1, id1, 1u, p, q, q, S - p);
   }
+}
+
+// The epilogue's sum of one output element: a fixed-point integer with
+// S_ACC_FRAC fraction bits.  The accumulators of levels 0..3 hold integers
+// times 2^-8L below 2^(24-8L), so they convert to int exactly and the sum is
+// exact; the shared one is rounded at 2^-33, far below the slice products that
+// the expansion leaves out (~2^-28 of the same unit for K = 500).
+// |sum| < 2^31 while a tile has at most S_MAX_TILE_STEPS K steps, and the
+// shared accumulator's conversion stays below 2^31 as well.
+//
+// Conversions to int run at a quarter of the FP32 rate, so two of the four
+// levels take none: adding FX_R0 = 1.5 2^23 to an integer |v0| <= 2^22 leaves
+// v0 in the low bits of the sum's pattern (above those of FX_R0 itself), and
+// adding FX_R2 = 1.5 2^9 to |v2| <= 192 leaves v2 in units of 2^-14; what that
+// rounds off, at most 2^-15, joins level 3.
+constexpr float FX_R0 = 12582912.f, FX_R2 = 768.f;
+constexpr unsigned long long FX_W2 = 1ull << (S_ACC_FRAC - 14);
+__device__ __forceinline__ long long fx_levels(long long a, float v0, float v2, float v3) {
+  const float t0 = __fadd_rn(v0, FX_R0), t2 = __fadd_rn(v2, FX_R2);
+  const float r = __fsub_rn(v2, __fsub_rn(t2, FX_R2));
+  const int i3 = __float2int_rn(__fadd_rn(r, v3) * 0x1p24f);
+  unsigned long long u = (unsigned long long)a + ((unsigned long long)__float_as_uint(t0) << 32);
+  u += (unsigned long long)__float_as_uint(t2) * FX_W2;
+  return (long long)u + (long long)i3 * 256;
+}
+
+// a 2^e2 as a double, rounded once, from integer operations: the FP64 pipe of
+// this part takes ~16 clocks per warp instruction and SM, and the conversions
+// through it were most of the output time.
+__device__ __forceinline__ double fixed_to_double(long long a, int e2) {
+  const unsigned long long sign = (unsigned long long)a & 0x8000000000000000ull;
+  const unsigned long long u = sign ? 0ull - (unsigned long long)a : (unsigned long long)a;
+  const int lz = __clzll((long long)u);
+  const int e = 63 - lz + e2 + 1022;  // biased exponent less one: the mantissa carries it
+  if (u == 0ull || e < 0) return 0.0;
+  const unsigned long long m = u << lz;
+  const unsigned long long r = (m >> 11) + ((m >> 10) & 1ull);
+  const unsigned long long b = ((unsigned long long)min(e, 2045) << 52) + r;
+  return __longlong_as_double((long long)(b | sign));
+}
+// a 2^e2 as a double-float pair: the leading 24 bits, rounded, and 24 more.
+__device__ __forceinline__ float2 fixed_to_dd(long long a, int e2) {
+  const unsigned int sign = a < 0 ? 0x80000000u : 0u;
+  const unsigned long long u = a < 0 ? 0ull - (unsigned long long)a : (unsigned long long)a;
+  const int lz = __clzll((long long)u);
+  const int e = 64 - lz + e2 + 127;  // u << lz is 2^64 times a value in [1/2, 1)
+  if (u == 0ull || e < 1) return make_float2(0.f, 0.f);
+  const unsigned long long m = u << lz;
+  const unsigned int h = (unsigned int)(m >> 40) + ((unsigned int)(m >> 39) & 1u);
+  const int rest = (int)((long long)(m - ((unsigned long long)h << 40)) >> 9);  // |.| <= 2^30
+  const float f = __int_as_float((int)(((unsigned int)min(e, 254) << 23) | sign));
+  return make_float2(__uint2float_rn(h) * 0x1p-24f * f, __int2float_rn(rest) * 0x1p-55f * f);
 }
 
 // Kept out of line: inlined into the unrolled output loop it would make the
@@ -195,15 +272,18 @@ split_engine_kernel(const SJob *__restrict__ jobs, int njobs, const STerm *__res
   constexpr int s = S;
   constexpr int S_STAGES = s_stages(S);
   constexpr int TQ = 4;  // depth of the tile hand-off ring
-  // accumulators that receive products: level L <= 3 exists iff L <= S-1,
-  // the shared one (levels >= 4) iff S >= 5
+  // accumulators that receive products: level L <= 3 exists iff L <= S-1
+  // (S >= 3), the shared one (levels >= 4) iff S >= 5
   constexpr int NLOW = S < 4 ? S : 4;
   constexpr bool HAS_HIGH = S >= 5;
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   __shared__ __align__(8) uint64_t full[S_STAGES], empty[S_STAGES];
-  __shared__ __align__(8) uint64_t accfull, accempty, drainfull, drainempty, mmafin;
+  // lowfull / lowempty: accumulators 0..3 at a tile's end; accfull / accempty:
+  // the shared one (and the tile)
+  __shared__ __align__(8) uint64_t lowfull, lowempty, accfull, accempty, drainfull, drainempty,
+      mmafin;
   __shared__ __align__(8) uint64_t tfull[TQ], tempty[TQ];
   __shared__ long long tq[TQ];
   // the producer decodes each tile once for everyone (tinfo, with tq) and
@@ -228,6 +308,8 @@ split_engine_kernel(const SJob *__restrict__ jobs, int njobs, const STerm *__res
       mbar_init(&tfull[i], 1);
       mbar_init(&tempty[i], 1 + S_EPI_WARPS);
     }
+    mbar_init(&lowfull, 1);
+    mbar_init(&lowempty, S_EPI_WARPS);
     mbar_init(&accfull, 1);
     mbar_init(&accempty, S_EPI_WARPS);
     mbar_init(&drainfull, 1);
@@ -442,19 +524,28 @@ split_engine_kernel(const SJob *__restrict__ jobs, int njobs, const STerm *__res
         if (lead) mbar_arrive(&tempty[q]);
         if (tile < 0) break;
         const uint32_t id_pos = idesc_bf16(S_BM, Nt, 0), id_neg = idesc_bf16(S_BM, Nt, 1);
-        // the epilogue has read the previous tile's accumulators
-        if (i > 0) {
-          if (!__all_sync(0xffffffffu, mbar_wait(&accempty, (i - 1) & 1, &err))) break;
+        // the epilogue has read the previous tile's accumulators: levels 0..3
+        // and, later, the shared one
+        auto low_free = [&]() {
+          if (i > 0 && !__all_sync(0xffffffffu, mbar_wait(&lowempty, (i - 1) & 1, &err)))
+            return false;
           tc_fence_after();
-        }
-        AccMode en = {0u, 0u};
-        int since = 0;
+          return true;
+        };
+        auto high_free = [&]() {
+          if (i > 0 && !__all_sync(0xffffffffu, mbar_wait(&accempty, (i - 1) & 1, &err)))
+            return false;
+          tc_fence_after();
+          return true;
+        };
+        const int kdrain = drain_interval(g1 - g0, kdrain_steps);
+        int since = 0, ndt = 0;  // K steps since the last drain, drains of this tile
         bool pending = false;
-        // K steps two at a time (drains come every kdrain_steps, an even
-        // number, so a pair never straddles one); a lone last step of a tile
-        // goes alone
+        // K steps two at a time (drains come after an even number of steps, so
+        // a pair never straddles one); a lone last step of a tile goes alone
         for (int g = g0; g < g1;) {
           const bool two = g + 1 < g1;
+          const int n = two ? 2 : 1;
           const int st0 = it % S_STAGES, ph0 = (it / S_STAGES) & 1;
           const int st1 = (it + 1) % S_STAGES, ph1 = ((it + 1) / S_STAGES) & 1;
           bool here = mbar_wait(&full[st0], ph0, &err);
@@ -470,30 +561,36 @@ split_engine_kernel(const SJob *__restrict__ jobs, int njobs, const STerm *__res
                          dB0 = smem_desc_kmajor(sa0 + (uint32_t)s * a_bytes, 256u * s),
                          dA1 = smem_desc_kmajor(sa1, 256u * s),
                          dB1 = smem_desc_kmajor(sa1 + (uint32_t)s * a_bytes, 256u * s);
+          const bool first = g == g0, last = g + n >= g1;
           if (pending) {
-            // levels >= 4 first (they never wait for a drain), then levels 0..3
-            issue_products<S, true>(lead, tmem, dA0, dB0, (uint32_t)Nt, id0, 1u);
-            if (two) issue_products<S, true>(lead, tmem, dA1, dB1, (uint32_t)Nt, id1, 1u);
-            if (!__all_sync(0xffffffffu, mbar_wait(&drainempty, nd & 1, &err))) {
-              ok = false;
-              break;
-            }
-            tc_fence_after();
+            ok = drains_all(ndt - 1)
+                     ? issue_after_drain<S, DRAIN_ALL>(lead, tmem, dA0, dB0, id0, dA1, dB1, id1,
+                                                       two, &drainempty, nd & 1, &err)
+                     : issue_after_drain<S, DRAIN_SOME>(lead, tmem, dA0, dB0, id0, dA1, dB1, id1,
+                                                        two, &drainempty, nd & 1, &err);
+            if (!ok) break;
             ++nd;
             pending = false;
-            issue_products<S, false>(lead, tmem, dA0, dB0, (uint32_t)Nt, id0, 0u);
-            if (two) issue_products<S, false>(lead, tmem, dA1, dB1, (uint32_t)Nt, id1, 1u);
-          } else if (two) {
-            issue_products_pair<S>(lead, tmem, dA0, dB0, id0, dA1, dB1, id1, (uint32_t)Nt, en);
+            if (last && lead) umma_commit(&lowfull);
+          } else if (first || last) {
+            // a tile's ends: levels 0..3 and the shared accumulator apart, so
+            // that the epilogue reads the ones while products go to the other
+            const uint32_t en = first ? 0u : 1u;
+            if (first && !low_free()) { ok = false; break; }
+            issue_products<S, DRAIN_ALL>(lead, tmem, dA0, dB0, id0, en);
+            if (two) issue_products<S, DRAIN_ALL>(lead, tmem, dA1, dB1, id1, 1u);
+            if (last && lead) umma_commit(&lowfull);
+            __syncwarp();
+            if (first && !high_free()) { ok = false; break; }
+            issue_products<S, ACC_HIGH>(lead, tmem, dA0, dB0, id0, en);
+            if (two) issue_products<S, ACC_HIGH>(lead, tmem, dA1, dB1, id1, 1u);
           } else {
-            issue_products_all<S>(lead, tmem, dA0, dB0, (uint32_t)Nt, id0, en);
+            issue_products_pair<S>(lead, tmem, dA0, dB0, id0, dA1, dB1, id1);
           }
-          en = {1u, 1u};
-          const int n = two ? 2 : 1;
           g += n;
           it += n;
           since += n;
-          const bool drain = since >= kdrain_steps && g < g1;
+          const bool drain = since >= kdrain && g < g1;
           if (lead) {
             umma_commit(&empty[st0]);
             if (two) umma_commit(&empty[st1]);
@@ -503,9 +600,14 @@ split_engine_kernel(const SJob *__restrict__ jobs, int njobs, const STerm *__res
           if (drain) {
             pending = true;
             since = 0;
+            ++ndt;
           }
         }
         if (!ok) break;
+        if (g0 == g1) {  // no K steps: nothing to wait for but the protocol
+          if (!low_free() || !high_free()) break;
+          if (lead) umma_commit(&lowfull);
+        }
         if (lead) umma_commit(&accfull);
         __syncwarp();
       }
@@ -522,7 +624,7 @@ split_engine_kernel(const SJob *__restrict__ jobs, int njobs, const STerm *__res
     int nd = 0, jh = 0;
     for (int i = 0;; ++i) {
       const int q = i % TQ;
-      if (!mbar_wait_sleep(&tfull[q], (i / TQ) & 1, &err)) break;
+      if (!__all_sync(0xffffffffu, mbar_wait_sleep(&tfull[q], (i / TQ) & 1, &err))) break;
       const long long tile = tq[q];
       __syncwarp();
       if (lane == 0) mbar_arrive(&tempty[q]);
@@ -540,84 +642,81 @@ split_engine_kernel(const SJob *__restrict__ jobs, int njobs, const STerm *__res
       const SJob &J = ejob[ew];
       const int Nt = ti.Nt;
       const int nsteps = ti.g1 - ti.g0;
-      const int ndrains = nsteps > 0 ? (nsteps - 1) / kdrain_steps : 0;
+      const int ndrains =
+          nsteps > 0 ? (nsteps - 1) / drain_interval(nsteps, kdrain_steps) : 0;
       const int qc = Nt >> 2;   // columns per quarter (multiple of 4, <= 24)
       const int nch = qc >> 2;  // 4-column chunks (<= 6)
       const uint32_t tb = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(part * qc);
-      dd::df acc[6][4];
+      long long acc[6][4];
+      {  // less what every read below adds with the bits of its two rounding constants
+        const unsigned long long z =
+            0ull - (unsigned long long)(ndrains + 1) *
+                       (((unsigned long long)__float_as_uint(FX_R0) << 32) +
+                        (unsigned long long)__float_as_uint(FX_R2) * FX_W2);
 #pragma unroll
-      for (int c = 0; c < 6; ++c)
+        for (int c = 0; c < 6; ++c)
 #pragma unroll
-        for (int k = 0; k < 4; ++k) acc[c][k] = {0.f, 0.f};
+          for (int k = 0; k < 4; ++k) acc[c][k] = nsteps > 0 ? (long long)z : 0ll;
+      }
+      // the drains, then (d == ndrains) levels 0..3 at the tile's end
       bool ok = true;
-      for (int d = 0; d < ndrains && ok; ++d, ++nd) {
-        ok = mbar_wait_sleep(&drainfull, nd & 1, &err);
+      for (int d = 0; d <= ndrains; ++d) {
+        const bool last = d == ndrains;
+        ok = __all_sync(0xffffffffu,
+                        mbar_wait(last ? &lowfull : &drainfull, (last ? i : nd) & 1, &err));
         if (!ok) break;
         tc_fence_after();
+        if (nsteps > 0) {
+          const bool with1 = last || drains_all(d);
 #pragma unroll
-        for (int c = 0; c < 6; ++c) {
-          if (c < nch) {
+          for (int c = 0; c < 6; ++c) {
+            if (c >= nch) break;
             float v[4][4];
 #pragma unroll
-            for (int L = 0; L < 4; ++L) {
-              if (L < NLOW) {
-                tmem_ld4(tb + L * Nt + c * 4, v[L]);
-              } else {
-#pragma unroll
-                for (int k = 0; k < 4; ++k) v[L][k] = 0.f;
-              }
-            }
+            for (int k = 0; k < 4; ++k) v[1][k] = v[3][k] = 0.f;
+            tmem_ld4(tb + c * 4, v[0]);
+            tmem_ld4(tb + 2 * S_NT_MAX + c * 4, v[2]);
+            if (NLOW > 3) tmem_ld4(tb + 3 * S_NT_MAX + c * 4, v[3]);
+            if (with1) tmem_ld4(tb + S_NT_MAX + c * 4, v[1]);
             tmem_wait_ld();
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              dd::df x = dd::two_sum(v[0][k], v[1][k]);
-              x = dd::add_f(x, v[2][k]);
-              x = dd::add_f(x, v[3][k]);
-              acc[c][k] = dd::add(acc[c][k], x);
+            for (int k = 0; k < 4; ++k) acc[c][k] = fx_levels(acc[c][k], v[0][k], v[2][k], v[3][k]);
+            if (with1) {
+#pragma unroll
+              for (int k = 0; k < 4; ++k)
+                acc[c][k] += (long long)__float2int_rn(v[1][k] * 0x1p8f) * (1ll << 24);
             }
           }
         }
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(&drainempty);
+        if (lane == 0) mbar_arrive(last ? &lowempty : &drainempty);
+        if (!last) ++nd;
       }
       if (!ok) break;
-      if (!mbar_wait_sleep(&accfull, i & 1, &err)) break;
-      tc_fence_after();
-      // fold the final partial sums into acc, then hand the accumulators back
+      // the shared accumulator
+      if (!__all_sync(0xffffffffu, mbar_wait(&accfull, i & 1, &err))) break;
+      if (HAS_HIGH && nsteps > 0) {
+        tc_fence_after();
 #pragma unroll
-      for (int c = 0; c < 6; ++c) {
-        if (c < nch && nsteps > 0) {
-          float v[5][4];
-#pragma unroll
-          for (int L = 0; L < 5; ++L) {
-            if (L < NLOW || (L == 4 && HAS_HIGH)) {
-              tmem_ld4(tb + L * Nt + c * 4, v[L]);
-            } else {
-#pragma unroll
-              for (int k = 0; k < 4; ++k) v[L][k] = 0.f;
-            }
-          }
+        for (int c = 0; c < 6; ++c) {
+          if (c >= nch) break;
+          float v[4];
+          tmem_ld4(tb + 4 * S_NT_MAX + c * 4, v);
           tmem_wait_ld();
 #pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            dd::df x = dd::two_sum(v[0][k], v[1][k]);
-            x = dd::add_f(x, v[2][k]);
-            x = dd::add_f(x, v[3][k]);
-            x = dd::add(acc[c][k], x);
-            acc[c][k] = dd::add_f(x, v[4][k]);
-          }
+          for (int k = 0; k < 4; ++k) acc[c][k] += (long long)__float2int_rn(v[k] * 0x1p32f);
         }
+        tc_fence_before();
       }
-      tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&accempty);
-      const int bi = ti.bi, n0 = ti.n0, m = ti.m0 + row;
+      const int bi = ti.bi, n0 = ti.n0 + part * qc, m = ti.m0 + row;
       const int *slot_ex = reinterpret_cast<const int *>(P.p[B_SLOTEXP]);
       const bool seg2 = J.msplit > 0 && m >= J.msplit;  // second row segment
       // the per-triple exponent table is read only by jobs that name a slot
       const int es = seg2 ? J.expo_slot2 : J.expo_slot;
-      const float sc = ldexpf(J.mult, J.expo + (es >= 0 ? slot_ex[es] : 0));
+      const int e2 = J.expo + (es >= 0 ? slot_ex[es] : 0) - S_ACC_FRAC;
       const int mo = seg2 ? m - J.msplit : m;  // row within its output
       const bool row_ok = m < J.M && !(J.m_pad > 0 && (m % J.m_pad) >= J.m_valid);
       // the thread's row is fixed for the tile: its output row offsets once.
@@ -627,46 +726,57 @@ split_engine_kernel(const SJob *__restrict__ jobs, int njobs, const STerm *__res
       const OutD &Cm = seg2 ? J.C2 : J.C;
       const long long rowM =
           row_ok ? Cm.off + (long long)bi * Cm.sb + s_rowoff(mo, Cm.m_in, Cm.sm1, Cm.sm0) : 0;
+      if (J.mode == SEPI_DD_STORE) {  // main columns only (checked at upload)
+        float2 *out = reinterpret_cast<float2 *>(P.p[Cm.buf]) + rowM + (long long)n0 * Cm.sn0;
+        const long long sn = Cm.sn0;
+        const int ncol = row_ok ? J.n_valid - n0 : 0;
+#pragma unroll
+        for (int c = 0; c < 6; ++c) {
+          if (c >= nch) break;
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            if (c * 4 + k < ncol) *out = fixed_to_dd(acc[c][k], e2);
+            out += sn;
+          }
+        }
+        continue;
+      }
+      if (!row_ok) continue;
       const int mq = mo / Cm.m_in, mr = mo % Cm.m_in;  // route 1: shared by its outputs
 #pragma unroll
       for (int c = 0; c < 6; ++c) {
-        if (c < nch) {
+        if (c >= nch) break;
 #pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const dd::df x = dd::scale(acc[c][k], sc);
-            const int n = n0 + part * qc + c * 4 + k;
-            if (!row_ok || n >= J.N) continue;
-            long long off;
-            int buf;
-            if (J.route == 1) {  // two column segments (see SJob)
-              const bool sg = n >= J.Nm2;
-              const int jc = sg ? n - J.Nm2 : n;
-              if (jc >= J.Nm + J.tw) continue;
-              const OutD &O = jc < J.Nm ? (sg ? J.C2 : J.C) : (sg ? J.Ct2 : J.Ct);
-              off = O.off + (long long)bi * O.sb + (long long)mq * O.sm1 + (long long)mr * O.sm0 +
-                    (long long)(jc < J.Nm ? jc : jc - J.Nm) * O.sn0;
-              buf = O.buf;
-            } else if (n < J.Nm) {
-              if (n >= J.n_valid) continue;
-              off = rowM + (long long)n * Cm.sn0;
-              buf = Cm.buf;
-            } else {  // tail columns are few: their offsets on the fly
-              const OutD &Ctl = seg2 ? J.Ct2 : J.Ct;
-              const int tlo = seg2 ? (J.Nm2 > 0 ? J.Nm2 : J.N) : J.Nm;
-              const int thi = seg2 ? J.N : (J.Nm2 > 0 ? J.Nm2 : J.N);
-              if (n < tlo || n >= thi) continue;
-              off = Ctl.off + (long long)bi * Ctl.sb + s_rowoff(mo, Ctl.m_in, Ctl.sm1, Ctl.sm0) +
-                    (long long)(n - tlo) * Ctl.sn0;
-              buf = Ctl.buf;
-            }
-            if (J.mode == SEPI_DD_STORE) {
-              reinterpret_cast<float2 *>(P.p[buf])[off] = make_float2(x.hi, x.lo);
-            } else if (P.fx[buf]) {
-              fx_add_call(P.fx[buf] + 2 * off, dd::to_double(x));
-            } else {
-              atomicAdd(reinterpret_cast<double *>(P.p[buf]) + off, dd::to_double(x));
-            }
+        for (int k = 0; k < 4; ++k) {
+          const int n = n0 + c * 4 + k;
+          long long off;
+          int buf;
+          if (J.route == 1) {  // two column segments (see SJob)
+            const bool sg = n >= J.Nm2;
+            const int jc = sg ? n - J.Nm2 : n;
+            if (n >= J.N || jc >= J.Nm + J.tw) continue;
+            const OutD &O = jc < J.Nm ? (sg ? J.C2 : J.C) : (sg ? J.Ct2 : J.Ct);
+            off = O.off + (long long)bi * O.sb + (long long)mq * O.sm1 + (long long)mr * O.sm0 +
+                  (long long)(jc < J.Nm ? jc : jc - J.Nm) * O.sn0;
+            buf = O.buf;
+          } else if (n < J.Nm) {
+            if (n >= J.n_valid) continue;
+            off = rowM + (long long)n * Cm.sn0;
+            buf = Cm.buf;
+          } else {  // tail columns are few: their offsets on the fly
+            const OutD &Ctl = seg2 ? J.Ct2 : J.Ct;
+            const int tlo = seg2 ? (J.Nm2 > 0 ? J.Nm2 : J.N) : J.Nm;
+            const int thi = seg2 ? J.N : (J.Nm2 > 0 ? J.Nm2 : J.N);
+            if (n < tlo || n >= thi) continue;
+            off = Ctl.off + (long long)bi * Ctl.sb + s_rowoff(mo, Ctl.m_in, Ctl.sm1, Ctl.sm0) +
+                  (long long)(n - tlo) * Ctl.sn0;
+            buf = Ctl.buf;
           }
+          const double x = fixed_to_double(acc[c][k], e2);
+          if (P.fx[buf])
+            fx_add_call(P.fx[buf] + 2 * off, x);
+          else
+            atomicAdd(reinterpret_cast<double *>(P.p[buf]) + off, x);
         }
       }
     }
@@ -690,17 +800,34 @@ int s_upload_plan(const SPlan &p, SDevPlan *d, cudaStream_t s) {
     for (const OutD *o : outs)
       if (o && (o->n_in < j.N || (r1 && o->m_in != j.C.m_in))) return CC3_ERR_ARG;
     if (r1 && (two || j.Nm2 <= 0 || j.Nm + j.tw > j.Nm2)) return CC3_ERR_ARG;
+    // stores take the main columns of one row segment
+    if (j.mode == SEPI_DD_STORE && (two || r1 || j.Nm < j.N || j.ksplit != 1)) return CC3_ERR_ARG;
+  }
+  // tiles of more than S_MAX_TILE_STEPS K steps are split over K (their
+  // partial sums add in the output)
+  std::vector<SJob> jobs = p.jobs;
+  long long tiles = 0;
+  for (SJob &j : jobs) {
+    long long steps = 0;
+    for (int t = 0; t < j.nterm; ++t) steps += p.terms[j.term0 + t].ksteps;
+    const long long need = (steps + S_MAX_TILE_STEPS - 1) / S_MAX_TILE_STEPS;
+    if (need > j.ksplit) {
+      if (j.mode == SEPI_DD_STORE) return CC3_ERR_ARG;
+      j.ksplit = (int)need;
+    }
+    j.tile_base = tiles;
+    tiles += (long long)j.batch * j.tiles_m * j.tiles_n * j.ksplit;
   }
   if (cudaMalloc(&d->counter, sizeof(unsigned long long)) != cudaSuccess) return CC3_ERR_OOM;
-  d->njobs = (int)p.jobs.size();
-  d->tiles = p.tiles;
+  d->njobs = (int)jobs.size();
+  d->tiles = tiles;
   d->flop = p.flop;
   d->slice_flop = p.slice_flop;
   if (d->njobs == 0) return CC3_OK;
-  if (cudaMalloc(&d->jobs, sizeof(SJob) * p.jobs.size()) != cudaSuccess) return CC3_ERR_OOM;
+  if (cudaMalloc(&d->jobs, sizeof(SJob) * jobs.size()) != cudaSuccess) return CC3_ERR_OOM;
   if (cudaMalloc(&d->terms, sizeof(STerm) * (p.terms.size() + 1)) != cudaSuccess)
     return CC3_ERR_OOM;
-  if (cudaMemcpyAsync(d->jobs, p.jobs.data(), sizeof(SJob) * p.jobs.size(),
+  if (cudaMemcpyAsync(d->jobs, jobs.data(), sizeof(SJob) * jobs.size(),
                       cudaMemcpyHostToDevice, s) != cudaSuccess)
     return CC3_ERR_CUDA;
   if (!p.terms.empty() &&

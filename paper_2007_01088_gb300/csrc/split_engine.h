@@ -7,7 +7,11 @@
 namespace cc3 {
 
 enum { SMAX_MAPS = 48, S_BM = 128, S_BK = 16, S_STAGES_MAX = 6, S_MAX_SLICES = 7,
-       S_NT_MAX = 96, S_NACC = 5, S_DRAIN_STEPS = 16, S_EPI_WARPS = 16, S_THREADS = 64 + 32 * S_EPI_WARPS };
+       S_NT_MAX = 96, S_DRAIN_STEPS = 16, S_EPI_WARPS = 16, S_THREADS = 64 + 32 * S_EPI_WARPS,
+       // fraction bits of the epilogue's fixed-point sums, and the K steps of a
+       // tile that keep them in 64 bits (and the shared accumulator's terms in 32:
+       // 5 2^14 (1 + 2^-6) 16 S_MAX_TILE_STEPS < 2^31)
+       S_ACC_FRAC = 32, S_MAX_TILE_STEPS = 1600 };
 
 // A BF16 slice array in the tensor cores' canonical no-swizzle K-major order
 // with the slices interleaved per core-matrix row group:
@@ -72,7 +76,6 @@ struct SJob {
   int expo_slot;  // >= 0: add the per-triple exponent ex[expo_slot]
   int m_pad, m_valid;  // m_pad > 0: rows with m % m_pad >= m_valid are padding
   int n_valid;         // columns n in [n_valid, Nm) are padding
-  float mult;  // +-1 or 2 (exact)
   OutD C, Ct;  // output element (b, m, n) for n < Nm, resp. (b, m, n - Nm);
                // buffer of float2 (dd) or double
   // rows m >= msplit (msplit > 0) belong to a second output: main columns to

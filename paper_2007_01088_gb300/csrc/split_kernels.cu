@@ -135,8 +135,8 @@ __global__ void maxabs_kernel(const double *__restrict__ x, long long n,
 // tau = (W_1 + W_2 + W_3) / (w - e_a - e_b - e_c + e_ijk) from the three
 // partial sums of the W build, then
 // tau~ = 4 tau^{abc} - 2 tau^{acb} - 2 tau^{cba} - 2 tau^{bac} + tau^{bca} + tau^{cab},
-// all in double-float.  The partial sums are stored as W[slot][c][a][b]; tau~
-// is written as TT[slot][a][b][c], together with the max |tau~| of each slot
+// all in double-float.  The partial sums are stored as W_2, W_3[slot][c][a][b]
+// and W_1[slot][c][b][a]; tau~ is written as TT[slot][a][b][c], together with the max |tau~| of each slot
 // (float bits, atomic max).  TT may be the buffer of W_2 (see below).
 //
 // The six values tau^{pi(a,b,c)} over the permutations pi are the same set
@@ -206,7 +206,7 @@ tau_contravariant_dd_kernel(const float2 *__restrict__ W1, const float2 *W2,
         const int gx = cx[q] * 8 + x, gy = cy[q] * 8 + y, gz = cz[q] * 8 + z;
         if (slot[q] == q && gx < nv && gy < nv && gz < nv) {
           const long long i = sbase + (long long)gz * nv2 + (long long)gx * nv + gy;
-          la[k][h][0] = W1[i];
+          la[k][h][0] = W1[sbase + (long long)gz * nv2 + (long long)gy * nv + gx];
           la[k][h][1] = W2[i];
           la[k][h][2] = W3[i];
         }
@@ -512,7 +512,7 @@ __global__ void to_dd_kernel(const double *__restrict__ x, float2 *__restrict__ 
 }
 
 // The outer products of the left transformation's L3 numerator, added to the
-// W build's first partial sum W1[u][c][a][b] (double-float) of slot u = v * bj
+// W build's third partial sum W3[u][c][a][b] (double-float) of slot u = v * bj
 // + t (vector v, triple t of the batch; slots with t >= ns are idle):
 //   sum over the six terms of P of L1[o0][x] (o1 y|o2 z) + Lt2[o0][o1][x][y] F[o2][z],
 // (o0,o1,o2) = (ijk[s0], ijk[s1], ijk[s2]), (x,y,z) = (v[s0], v[s1], v[s2]),
@@ -522,7 +522,7 @@ __global__ void to_dd_kernel(const double *__restrict__ x, float2 *__restrict__ 
 // and Lt2's pair symmetry), so that every factor that varies along b is read
 // contiguously.
 __global__ void __launch_bounds__(256)
-left_outer_dd_kernel(float2 *__restrict__ W1, const int *__restrict__ tri, int bj, int ns,
+left_outer_dd_kernel(float2 *__restrict__ W3, const int *__restrict__ tri, int bj, int ns,
                      const float2 *__restrict__ L1, const float2 *__restrict__ Lt,
                      const float2 *__restrict__ ovov, const float2 *__restrict__ F, int no,
                      int nv) {
@@ -533,7 +533,7 @@ left_outer_dd_kernel(float2 *__restrict__ W1, const int *__restrict__ tri, int b
   const long long nv2 = (long long)nv * nv, nv3 = nv2 * nv;
   const long long n1 = (long long)no * nv, nt2 = n1 * no * nv;
   const float2 *l1 = L1 + vec * n1, *lt = Lt + vec * nt2;
-  float2 *W = W1 + (long long)u * nv3;
+  float2 *W = W3 + (long long)u * nv3;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < nv3;
        e += (long long)gridDim.x * blockDim.x) {
     const int b = (int)(e % nv), a = (int)((e / nv) % nv), c = (int)(e / nv2);
@@ -592,14 +592,14 @@ int launch_to_dd(const double *x, float2 *y, long long n, cudaStream_t st) {
   to_dd_kernel<<<grid_for(n), 256, 0, st>>>(x, y, n);
   return cudaGetLastError() == cudaSuccess ? CC3_OK : CC3_FAIL(CC3_ERR_CUDA, "to_dd launch");
 }
-int launch_left_outer_dd(float2 *W1, const int *tri, int bj, int ns, int nslot, const float2 *L1,
+int launch_left_outer_dd(float2 *W3, const int *tri, int bj, int ns, int nslot, const float2 *L1,
                          const float2 *Lt, const float2 *ovov, const float2 *F, int no, int nv,
                          cudaStream_t st) {
   if (nslot <= 0) return CC3_OK;
   if (nslot > 65535) return CC3_FAIL(CC3_ERR_ARG, "left outer products: slots");
   const long long nv3 = (long long)nv * nv * nv;
   const int blocks = (int)std::min<long long>((nv3 + 255) / 256, 2048);
-  left_outer_dd_kernel<<<dim3(blocks, nslot), 256, 0, st>>>(W1, tri, bj, ns, L1, Lt, ovov, F, no,
+  left_outer_dd_kernel<<<dim3(blocks, nslot), 256, 0, st>>>(W3, tri, bj, ns, L1, Lt, ovov, F, no,
                                                             nv);
   return cudaGetLastError() == cudaSuccess ? CC3_OK
                                            : CC3_FAIL(CC3_ERR_CUDA, "left outer products launch");

@@ -27,7 +27,7 @@ struct Gather {
 int launch_slice_gather(const double *src, __nv_bfloat16 *dst, int s, int e, const Gather &g,
                         long long nrows, int Kp, int rps, cudaStream_t st);
 int launch_maxabs(const double *x, long long n, unsigned long long *out, cudaStream_t st);
-// tau from the W build's three partial sums W1 + W2 + W3 (dd, [slot][c][a][b])
+// tau from the W build's three partial sums W1 + W2 + W3 (dd, W2 and W3 [slot][c][a][b], W1 [slot][c][b][a])
 // over (w - eps), and tau~ (dd, [slot][a][b][c]) into tt, which may be W2;
 // ev: dd virtual orbital energies, eo: dd e_i + e_j + e_k of each slot
 // tau_out (optional): tau itself, [slot][a][b][c] (dd), written as well
@@ -47,10 +47,10 @@ int launch_common_exponent(const unsigned int *maxbits, int *ex, int nslot, int 
 // y[e] = x[e] as a double-float pair
 int launch_to_dd(const double *x, float2 *y, long long n, cudaStream_t st);
 // the left transformation's outer products L1 (x) g_ovov + Lt2 (x) F of the L3
-// numerator (six terms of P) added to W1[u][c][a][b] (dd) of the nslot slots
+// numerator (six terms of P) added to W3[u][c][a][b] (dd) of the nslot slots
 // u = v * bj + t of a batch of ns triples (tri: 3 ints per triple); all
 // factors as dd pairs (L1[v][i][a], Lt[v][i][j][a][b], ovov, F_ov)
-int launch_left_outer_dd(float2 *W1, const int *tri, int bj, int ns, int nslot, const float2 *L1,
+int launch_left_outer_dd(float2 *W3, const int *tri, int bj, int ns, int nslot, const float2 *L1,
                          const float2 *Lt, const float2 *ovov, const float2 *F, int no, int nv,
                          cudaStream_t st);
 // v: device array of 3 pointers (one per cyclic layout)
