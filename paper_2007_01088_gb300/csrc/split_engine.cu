@@ -13,7 +13,8 @@
 // the levels >= 4 share a fifth, rounded accumulator (its error stays below
 // 2^-50 of the result).
 //
-// Warp roles (576 threads): warp 0 issues one bulk copy per operand tile (all
+// Warp roles (608 threads): warp 18 decodes tiles and their terms ahead of the
+// others; warp 0 issues one bulk copy per operand tile (all
 // s slices of a 128 x 16 A tile, resp. an Ntile x 16 B tile, pre-tiled in
 // global memory in the canonical no-swizzle order with the slices interleaved
 // per row group; one copy per slab when the A rows are flattened over slabs)
@@ -223,46 +224,51 @@ __device__ __noinline__ void fx_add_call(unsigned long long *slot, double v) { f
 // Position of one tile within its job: batch index, K-split part, M/N tile
 // and its K-step range [g0, g1) over the concatenated terms.
 struct TileInfo {
-  int j, bi, m0, n0, Nt, g0, g1;
+  int bi, m0, n0, Nt, g0, g1;
 };
-
-// jhint: the job of this CTA's previous tile (tiles are taken in increasing
-// order, so the search only moves forward).
-__device__ __forceinline__ TileInfo decode_tile(const SJob *__restrict__ jobs, int njobs,
-                                                const STerm *__restrict__ terms, long long tile,
-                                                int &jhint) {
-  int j = jhint;
-  if (j >= njobs || jobs[j].tile_base > tile) j = 0;
-  while (j + 1 < njobs && jobs[j + 1].tile_base <= tile) ++j;
-  jhint = j;
-  const SJob &J = jobs[j];
+__device__ __forceinline__ TileInfo decode_tile(const SJob &J, long long tile) {
   TileInfo t;
-  t.j = j;
-  const long long local = tile - J.tile_base;
+  const int local = (int)(tile - J.tile_base);
   const int per_batch = J.tiles_m * J.tiles_n * J.ksplit;
-  t.bi = (int)(local / per_batch);
-  int r = (int)(local % per_batch);
+  t.bi = local / per_batch;
+  int r = local % per_batch;
   const int ks = r % J.ksplit;
   r /= J.ksplit;
-  const int tn = r % J.tiles_n, tm = r / J.tiles_n;
-  t.m0 = tm * S_BM;
+  t.m0 = r / J.tiles_n * S_BM;
   t.Nt = J.Ntile;
-  t.n0 = tn * J.Ntile;
-  int total = 0;
-  for (int q = 0; q < J.nterm; ++q) total += terms[J.term0 + q].ksteps;
-  const int per = (total + J.ksplit - 1) / J.ksplit;
-  t.g0 = min(total, ks * per);
-  t.g1 = min(total, t.g0 + per);
+  t.n0 = r % J.tiles_n * J.Ntile;
+  const int per = (J.ksteps + J.ksplit - 1) / J.ksplit;
+  t.g0 = min(J.ksteps, ks * per);
+  t.g1 = min(J.ksteps, t.g0 + per);
   return t;
 }
 
+// A term of a tile as bulk copies, from its first K step in the tile: copy c
+// takes bytes[c] from src[c] (kbs[c] elements further each K step) to dst[c]
+// in the stage; total bytes per K step; steps = 0: no more terms.
+struct TermSlot {
+  static constexpr int LANES = 28;
+  const __nv_bfloat16 *src[LANES];
+  long long kbs[LANES];
+  uint32_t bytes[LANES], dst[LANES];
+  uint32_t total;
+  int steps, neg;
+};
+
+// One entry of the tile hand-off ring (tile < 0: no more tiles).
+struct TileSlot {
+  long long tile;
+  TileInfo ti;
+  SJob job;
+};
+
 // Persistent: one CTA per SM takes tiles from a launch-wide counter (the plan
 // lists long tiles first) and keeps the stage ring, the TMEM allocation and
-// the barriers across tiles.  The producer fetches each tile index and hands
-// it to the MMA thread and the epilogue warps through a small ring in shared
-// memory; the epilogue releases the accumulators as soon as it has read them,
+// the barriers across tiles.  The decoder fetches each tile index and hands
+// it, decoded, to the MMA warp and the epilogue warps through a small ring in
+// shared memory; the epilogue releases the accumulators as soon as it has read them,
 // so the next tile's products start while it finishes the previous outputs.
-// 96 registers: the 18 warps sit 5 to a sub-partition of 16,384 registers.
+// 96 registers: the 19 warps sit 5 to a sub-partition of 16,384 registers.
 template <int S>
 __global__ void __maxnreg__(96)
 split_engine_kernel(const SJob *__restrict__ jobs, int njobs, const STerm *__restrict__ terms,
@@ -271,7 +277,7 @@ split_engine_kernel(const SJob *__restrict__ jobs, int njobs, const STerm *__res
                     long long ntiles) {
   constexpr int s = S;
   constexpr int S_STAGES = s_stages(S);
-  constexpr int TQ = 4;  // depth of the tile hand-off ring
+  constexpr int TQ = 4, KQ = 4;  // depths of the tile and the term hand-off rings
   // accumulators that receive products: level L <= 3 exists iff L <= S-1
   // (S >= 3), the shared one (levels >= 4) iff S >= 5
   constexpr int NLOW = S < 4 ? S : 4;
@@ -285,18 +291,16 @@ split_engine_kernel(const SJob *__restrict__ jobs, int njobs, const STerm *__res
   __shared__ __align__(8) uint64_t lowfull, lowempty, accfull, accempty, drainfull, drainempty,
       mmafin;
   __shared__ __align__(8) uint64_t tfull[TQ], tempty[TQ];
-  __shared__ long long tq[TQ];
-  // the producer decodes each tile once for everyone (tinfo, with tq) and
-  // marks each stage with the sign of its term, so that the MMA thread and
-  // the epilogue read no job or term tables
-  __shared__ TileInfo tinfo[TQ];
+  // the decoder decodes each tile once for everyone, with a copy of its job
+  // (the output loop reads its fields for every element), and marks each stage
+  // with the sign of its term, so that no other warp reads the tables
+  __shared__ TileSlot tslot[TQ];
+  __shared__ STerm sterm[S_TERM_CHUNK];  // the decoder's terms of the current tile
+  __shared__ TermSlot termslot[KQ];
+  __shared__ __align__(8) uint64_t termfull[KQ], termempty[KQ];
   __shared__ int sneg[S_STAGES];
   __shared__ uint32_t tmem_base_sh;
   __shared__ volatile int err;
-  // each epilogue warp's copy of its current tile's job: the output loop reads
-  // its fields for every element, and global reads of them (L1 is small next
-  // to 216 KB of shared memory) put an L2 round trip on each element's path
-  __shared__ SJob ejob[S_EPI_WARPS];
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
@@ -307,6 +311,10 @@ split_engine_kernel(const SJob *__restrict__ jobs, int njobs, const STerm *__res
     for (int i = 0; i < TQ; ++i) {
       mbar_init(&tfull[i], 1);
       mbar_init(&tempty[i], 1 + S_EPI_WARPS);
+    }
+    for (int i = 0; i < KQ; ++i) {
+      mbar_init(&termfull[i], 1);
+      mbar_init(&termempty[i], 1);
     }
     mbar_init(&lowfull, 1);
     mbar_init(&lowempty, S_EPI_WARPS);
@@ -326,187 +334,216 @@ split_engine_kernel(const SJob *__restrict__ jobs, int njobs, const STerm *__res
   const uint32_t a_bytes = S_BM * 32;
 
   if (warp == 0) {
-    if (lane == 0) {
-      // producer: tile indices, then the operand tiles of every K step
-      int issued = 0, jh = 0;
-      for (int i = 0;; ++i) {
-        const int q = i % TQ;
-        if (!mbar_wait(&tempty[q], ((i / TQ) & 1) ^ 1, &err)) break;
-        const long long tile = (long long)atomicAdd(tile_ctr, 1ull);
-        TileInfo ti;
-        if (tile < ntiles) {
-          ti = decode_tile(jobs, njobs, terms, tile, jh);
-          tinfo[q] = ti;
+    // producer: the bulk copies of every K step, one lane each (see the decoder)
+    int issued = 0;
+    bool ok = true;
+    for (int k = 0; ok; ++k) {
+      TermSlot &ts = termslot[k % KQ];
+      if (!__all_sync(0xffffffffu, mbar_wait(&termfull[k % KQ], (k / KQ) & 1, &err))) break;
+      const int steps = ts.steps, neg = ts.neg;
+      if (steps == 0) break;
+      const uint32_t total = ts.total;
+      const int own = min(lane, TermSlot::LANES - 1);
+      const __nv_bfloat16 *src = ts.src[own];
+      const long long kbs = ts.kbs[own];
+      const uint32_t bytes = lane < TermSlot::LANES ? ts.bytes[own] : 0u, dst = ts.dst[own];
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&termempty[k % KQ]);
+      for (int g = 0; g < steps; ++g) {
+        const int st = issued % S_STAGES, ph = (issued / S_STAGES) & 1;
+        if (!__all_sync(0xffffffffu, mbar_wait(&empty[st], ph ^ 1, &err))) {
+          ok = false;
+          break;
         }
-        tq[q] = tile < ntiles ? tile : -1;
-        mbar_arrive(&tfull[q]);
-        if (tile >= ntiles) break;
-        const int Nt = ti.Nt, bi = ti.bi, m0 = ti.m0, n0 = ti.n0;
-        const int term0 = jobs[ti.j].term0, nterm = jobs[ti.j].nterm;
-        // term cursor; per-term operand addresses live in registers (the
-        // barrier asm below would otherwise force the term and array
-        // descriptors to be reloaded from memory every K step)
-        int t = 0, kbase = 0;
-        while (t < nterm && kbase + terms[term0 + t].ksteps <= ti.g0) {
-          kbase += terms[term0 + t].ksteps;
-          ++t;
-        }
-        int kend = -1, neg = 0;
-        const __nv_bfloat16 *ga0 = nullptr, *gb0 = nullptr, *gt0 = nullptr, *ga20 = nullptr,
-                            *gt20 = nullptr;
-        long long kbsA = 0, kbsB = 0, kbsT = 0, kbsA2 = 0, kbsT2 = 0;
-        int kmax = 0;
-        uint32_t abytes = 0, mbytes = 0, tbytes = 0, toff = 0, a2bytes = 0, a2off = 0,
-                 t2bytes = 0, t2off = 0;
-        // flattened A rows: rows to load (0: not flattened), rows in the first
-        // slab, rows per slab, slab stride and row 0 of the first slab
-        int fra = 0, fseg = 0, frows = 0;
-        long long fstride = 0;
-        const __nv_bfloat16 *gaf = nullptr;
-        bool bad = false;
-        for (int g = ti.g0; g < ti.g1; ++g) {
-          if (g >= kend) {
-            if (kend >= 0) {
-              kbase = kend;
-              ++t;
-            }
-            const STerm T = terms[term0 + t];
-            neg = T.negA;
-            kend = kbase + T.ksteps;
-            const SArr XA = arrs.a[T.A.map], XB = arrs.a[T.B.map], XT = arrs.a[T.Bt.map];
-            const int ar = T.A.row0 + bi * T.A.row_b + m0, as = T.A.slab0 + bi * T.A.slab_b;
-            const int bs = T.B.slab0 + bi * T.B.slab_b, ts = T.Bt.slab0 + bi * T.Bt.slab_b;
-            // B tile rows [n0, n0 + Nt): main rows from B, rows in [nbm, nbm2) from
-            // the tail Bt, rows >= nbm2 from the second tail Bt2
-            const int nbm = T.nbm > 0 ? T.nbm : (1 << 30);
-            const int nbm2 = T.nbm2 > 0 ? T.nbm2 : (1 << 30);
-            const int br = T.B.row0 + bi * T.B.row_b + n0;
-            const int nmain = max(0, min(min(Nt, nbm - n0), XB.rows - br));
-            const int tfirst = max(n0, nbm);                  // first tail row of the tile
-            const int tr = T.Bt.row0 + tfirst - nbm;          // its row in Bt
-            const int ntail =
-                T.nbm > 0 ? max(0, min(min(n0 + Nt, nbm2) - tfirst, XT.rows - tr)) : 0;
-            kmax = XA.kblocks;
-            if (nmain > 0) kmax = min(kmax, XB.kblocks);
-            if (ntail > 0) kmax = min(kmax, XT.kblocks);
-            // A rows: [ar, ar + ra) of slab as, or flattened over slabs as, as + 1, ...
-            int ra = 0, fs = as, fr = ar;
-            bool abad = as < 0 || ar < 0;
-            if (!abad && T.aflat > 0) {
-              ra = min(S_BM, T.aflat - ar);
-              fs = as + ar / XA.rows;
-              fr = ar % XA.rows;
-              abad = ra <= 0 || as + (ar + ra - 1) / XA.rows >= XA.slabs || T.asplit > 0;
-            } else if (!abad) {
-              abad = as >= XA.slabs || ar >= XA.rows;
-              ra = min(S_BM, XA.rows - ar);
-              if (T.asplit > 0) ra = min(ra, T.asplit);
-            }
-            if (abad || (nmain > 0 && (bs < 0 || bs >= XB.slabs || br < 0)) ||
-                (ntail > 0 && (ts < 0 || ts >= XT.slabs || tr < 0 || ((tfirst - n0) & 7) != 0))) {
-              err = 2;  // a plan addressed outside its slice array: stop, report
-              bad = true;
-              break;
-            }
-            abytes = (uint32_t)ra * 32u;
-            fra = T.aflat > 0 ? ra : 0;
-            fseg = min(ra, XA.rows - fr);
-            frows = XA.rows;
-            fstride = XA.slab_stride;
-            gaf = reinterpret_cast<const __nv_bfloat16 *>(XA.base) + (long long)fs * XA.slab_stride;
-            mbytes = (uint32_t)nmain * 32u;
-            tbytes = (uint32_t)ntail * 32u;
-            toff = (uint32_t)(tfirst - n0) * 32u * s;
-            a2bytes = 0;
-            t2bytes = 0;
-            if (T.asplit > 0) {  // second A segment
-              const SArr XA2 = arrs.a[T.A2.map];
-              const int ar2 = T.A2.row0 + bi * T.A2.row_b, as2 = T.A2.slab0 + bi * T.A2.slab_b;
-              const int ra2 = min(S_BM - T.asplit, XA2.rows - ar2);
-              if (as2 < 0 || as2 >= XA2.slabs || ar2 < 0 || ra2 <= 0 || (T.asplit & 7) != 0) {
-                err = 2;
-                bad = true;
-                break;
-              }
-              kmax = min(kmax, XA2.kblocks);
-              a2bytes = (uint32_t)ra2 * 32u;
-              a2off = (uint32_t)T.asplit * 32u * s;
-              ga20 = reinterpret_cast<const __nv_bfloat16 *>(XA2.base) +
-                     (long long)as2 * XA2.slab_stride + (long long)ar2 * 16 * s;
-              kbsA2 = XA2.kb_stride;
-            }
-            if (T.nbm2 > 0) {  // second tail
-              const SArr XT2 = arrs.a[T.Bt2.map];
-              const int t2first = max(n0, nbm2), ts2 = T.Bt2.slab0 + bi * T.Bt2.slab_b;
-              const int tr2 = T.Bt2.row0 + t2first - nbm2;
-              const int ntail2 = max(0, min(n0 + Nt - t2first, XT2.rows - tr2));
-              if (ntail2 > 0) {
-                if (ts2 < 0 || ts2 >= XT2.slabs || tr2 < 0 || ((t2first - n0) & 7) != 0) {
-                  err = 2;
-                  bad = true;
-                  break;
-                }
-                kmax = min(kmax, XT2.kblocks);
-                t2bytes = (uint32_t)ntail2 * 32u;
-                t2off = (uint32_t)(t2first - n0) * 32u * s;
-                gt20 = reinterpret_cast<const __nv_bfloat16 *>(XT2.base) +
-                       (long long)ts2 * XT2.slab_stride + (long long)tr2 * 16 * s;
-                kbsT2 = XT2.kb_stride;
-              }
-            }
-            // one bulk copy per operand tile: its s slices are contiguous
-            ga0 = gaf + (long long)fr * 16 * s;
-            gb0 = reinterpret_cast<const __nv_bfloat16 *>(XB.base) + (long long)bs * XB.slab_stride +
-                  (long long)br * 16 * s;
-            gt0 = reinterpret_cast<const __nv_bfloat16 *>(XT.base) + (long long)ts * XT.slab_stride +
-                  (long long)tr * 16 * s;
-            kbsA = XA.kb_stride;
-            kbsB = XB.kb_stride;
-            kbsT = XT.kb_stride;
-          }
-          const int kb = g - kbase;
-          if (kb >= kmax) {
-            err = 2;
-            bad = true;
-            break;
-          }
-          const int st = issued % S_STAGES, ph = (issued / S_STAGES) & 1;
-          if (!mbar_wait(&empty[st], ph ^ 1, &err)) { bad = true; break; }
+        if (lane == 0) {
           sneg[st] = neg;
-          mbar_arrive_expect_tx(&full[st],
-                                (uint32_t)s * (abytes + a2bytes + mbytes + tbytes + t2bytes));
-          // stage layout: s A slices (128 rows) then s B slices (S_NT_MAX rows)
-          uint8_t *sa = smem + (size_t)st * ((size_t)s * (a_bytes + S_NT_MAX * 32));
-          uint8_t *sb = sa + (size_t)s * a_bytes;
-          if (fra > 0) {  // one copy per slab the tile's rows touch
-            const __nv_bfloat16 *src = ga0 + (long long)kb * kbsA, *sp = gaf + (long long)kb * kbsA;
-            int r = 0, cnt = fseg;
-            for (;;) {
-              bulk_load(sa + (uint32_t)r * 32u * s, src, (uint32_t)cnt * 32u * s, &full[st]);
-              r += cnt;
-              if (r >= fra) break;
-              sp += fstride;
-              src = sp;
-              cnt = min(fra - r, frows);
-            }
-          } else {
-            bulk_load(sa, ga0 + (long long)kb * kbsA, (uint32_t)s * abytes, &full[st]);
-          }
-          if (a2bytes)
-            bulk_load(sa + a2off, ga20 + (long long)kb * kbsA2, (uint32_t)s * a2bytes, &full[st]);
-          if (mbytes) bulk_load(sb, gb0 + (long long)kb * kbsB, (uint32_t)s * mbytes, &full[st]);
-          if (tbytes)
-            bulk_load(sb + toff, gt0 + (long long)kb * kbsT, (uint32_t)s * tbytes, &full[st]);
-          if (t2bytes)
-            bulk_load(sb + t2off, gt20 + (long long)kb * kbsT2, (uint32_t)s * t2bytes, &full[st]);
-          ++issued;
+          mbar_arrive_expect_tx(&full[st], total);
         }
-        if (bad) break;
+        __syncwarp();
+        // stage layout: s A slices (128 rows) then s B slices (S_NT_MAX rows)
+        if (bytes)
+          bulk_load(smem + (size_t)st * ((size_t)s * (a_bytes + S_NT_MAX * 32)) + dst, src, bytes,
+                    &full[st]);
+        __syncwarp();
+        src += kbs;
+        ++issued;
       }
-      // let every issued copy land before the CTA may exit, also after a
-      // give-up (bounded; the wait ignores the error word)
-      for (int i = (issued > S_STAGES ? issued - S_STAGES : 0); i < issued; ++i)
-        mbar_wait_quiet(&full[i % S_STAGES], (i / S_STAGES) & 1, 500000000ull);
+    }
+    // let every issued copy land before the CTA may exit, also after a
+    // give-up (bounded; the wait ignores the error word)
+    for (int i = (issued > S_STAGES ? issued - S_STAGES : 0); i < issued; ++i)
+      mbar_wait_quiet(&full[i % S_STAGES], (i / S_STAGES) & 1, 500000000ull);
+  } else if (warp == 18) {
+    // decoder: takes tiles, hands each with its job to the issuer and the
+    // epilogue, and resolves its terms into bulk copies a few terms ahead of
+    // the producer (resolving one takes ~2000 clocks, a W build tile has two
+    // terms of two K steps each).  Each lane owns one of a K step's copies
+    // (source, stride, destination and size are fixed for a term): lanes 0..23
+    // the A segments (one per slab the tile's rows touch), lane 24 A2, 25 B,
+    // 26 Bt, 27 Bt2.
+    int j = 0, k = 0;
+    bool fail = false;
+    long long next = 0;
+    if (lane == 0) next = (long long)atomicAdd(tile_ctr, 1ull);
+    for (int i = 0; !fail; ++i) {
+      const int q = i % TQ;
+      if (!__all_sync(0xffffffffu, mbar_wait_sleep(&tempty[q], ((i / TQ) & 1) ^ 1, &err))) break;
+      const long long tile = __shfl_sync(0xffffffffu, next, 0);
+      TileSlot &slot = tslot[q];
+      if (tile >= ntiles) {
+        if (lane == 0) {
+          slot.tile = -1;
+          mbar_arrive(&tfull[q]);
+        }
+        if (!__all_sync(0xffffffffu,
+                        mbar_wait_sleep(&termempty[k % KQ], ((k / KQ) & 1) ^ 1, &err)))
+          break;
+        if (lane == 0) {
+          termslot[k % KQ].steps = 0;  // no more copies
+          mbar_arrive(&termfull[k % KQ]);
+        }
+        break;
+      }
+      if (lane == 0) next = (long long)atomicAdd(tile_ctr, 1ull);  // back by the next tile
+      // its job: the last one with tile_base <= tile (tiles come in increasing
+      // order, so the search moves forward only), 32 jobs at a time
+      for (;;) {
+        const int c = j + 1 + lane;
+        const bool before = c < njobs && jobs[c].tile_base <= tile;
+        const int n = __popc(__ballot_sync(0xffffffffu, before));
+        j += n;
+        if (n < 32) break;
+      }
+      {
+        const uint32_t *src = reinterpret_cast<const uint32_t *>(jobs + j);
+        uint32_t *dst = reinterpret_cast<uint32_t *>(&slot.job);
+        for (int w = lane; w < (int)(sizeof(SJob) / 4); w += 32) dst[w] = src[w];
+      }
+      __syncwarp();
+      const TileInfo ti = decode_tile(slot.job, tile);
+      const int term0 = slot.job.term0, nterm = slot.job.nterm;
+      if (lane == 0) {
+        slot.tile = tile;
+        slot.ti = ti;
+        mbar_arrive(&tfull[q]);
+      }
+      const int Nt = ti.Nt, bi = ti.bi, m0 = ti.m0, n0 = ti.n0;
+      int kend = 0;
+      for (int t = 0; t < nterm && kend < ti.g1; ++t) {
+        if (t % S_TERM_CHUNK == 0) {
+          __syncwarp();
+          const int n = min((int)S_TERM_CHUNK, nterm - t) * (int)(sizeof(STerm) / 4);
+          const uint32_t *from = reinterpret_cast<const uint32_t *>(terms + term0 + t);
+          uint32_t *to = reinterpret_cast<uint32_t *>(sterm);
+          for (int w = lane; w < n; w += 32) to[w] = from[w];
+          __syncwarp();
+        }
+        const STerm &T = sterm[t % S_TERM_CHUNK];
+        const int kbase = kend;
+        kend += T.ksteps;
+        if (kend <= ti.g0) continue;
+        const SArr &XA = arrs.a[T.A.map], &XB = arrs.a[T.B.map], &XT = arrs.a[T.Bt.map];
+        const int ar = T.A.row0 + bi * T.A.row_b + m0, as = T.A.slab0 + bi * T.A.slab_b;
+        const int bs = T.B.slab0 + bi * T.B.slab_b, ts = T.Bt.slab0 + bi * T.Bt.slab_b;
+        // B tile rows [n0, n0 + Nt): main rows from B, rows in [nbm, nbm2) from
+        // the tail Bt, rows >= nbm2 from the second tail Bt2
+        const int nbm = T.nbm > 0 ? T.nbm : (1 << 30);
+        const int nbm2 = T.nbm2 > 0 ? T.nbm2 : (1 << 30);
+        const int br = T.B.row0 + bi * T.B.row_b + n0;
+        const int nmain = max(0, min(min(Nt, nbm - n0), XB.rows - br));
+        const int tfirst = max(n0, nbm);           // first tail row of the tile
+        const int tr = T.Bt.row0 + tfirst - nbm;   // its row in Bt
+        const int ntail = T.nbm > 0 ? max(0, min(min(n0 + Nt, nbm2) - tfirst, XT.rows - tr)) : 0;
+        int kmax = XA.kblocks;
+        if (nmain > 0) kmax = min(kmax, XB.kblocks);
+        if (ntail > 0) kmax = min(kmax, XT.kblocks);
+        // A rows: [ar, ar + ra) of slab as, or flattened over slabs as, as + 1, ...
+        int ra = 0, fs = as, fr = ar;
+        bool abad = as < 0 || ar < 0;
+        if (!abad && T.aflat > 0) {
+          ra = min(S_BM, T.aflat - ar);
+          fs = as + ar / XA.rows;
+          fr = ar % XA.rows;
+          abad = ra <= 0 || as + (ar + ra - 1) / XA.rows >= XA.slabs || T.asplit > 0;
+        } else if (!abad) {
+          abad = as >= XA.slabs || ar >= XA.rows;
+          ra = min(S_BM, XA.rows - ar);
+          if (T.asplit > 0) ra = min(ra, T.asplit);
+        }
+        bool bad = abad || (nmain > 0 && (bs < 0 || bs >= XB.slabs || br < 0)) ||
+              (ntail > 0 && (ts < 0 || ts >= XT.slabs || tr < 0 || ((tfirst - n0) & 7) != 0));
+        // second A segment
+        const SArr &XA2 = arrs.a[T.A2.map];
+        const int ar2 = T.A2.row0 + bi * T.A2.row_b, as2 = T.A2.slab0 + bi * T.A2.slab_b;
+        int ra2 = 0;
+        if (!bad && T.asplit > 0) {
+          ra2 = min(S_BM - T.asplit, XA2.rows - ar2);
+          bad = as2 < 0 || as2 >= XA2.slabs || ar2 < 0 || ra2 <= 0 || (T.asplit & 7) != 0;
+          kmax = min(kmax, XA2.kblocks);
+        }
+        // second tail
+        const SArr &XT2 = arrs.a[T.Bt2.map];
+        const int t2first = max(n0, nbm2), ts2 = T.Bt2.slab0 + bi * T.Bt2.slab_b;
+        const int tr2 = T.Bt2.row0 + t2first - nbm2;
+        int ntail2 = 0;
+        if (!bad && T.nbm2 > 0) {
+          ntail2 = max(0, min(n0 + Nt - t2first, XT2.rows - tr2));
+          if (ntail2 > 0) {
+            bad = ts2 < 0 || ts2 >= XT2.slabs || tr2 < 0 || ((t2first - n0) & 7) != 0;
+            kmax = min(kmax, XT2.kblocks);
+          }
+        }
+        if (bad || kend - kbase > kmax) {
+          fail = true;  // a plan addressed outside its slice array
+          break;
+        }
+        // this lane's copy: rows [row, row + n) of a slab to rows at d of A or B
+        const SArr *X = &XA;
+        int slab = fs, row = fr, n = 0, d = 0;
+        uint32_t side = 0;
+        if (lane < 24) {
+          // segment `lane` of the A rows: the first slab's rest, then whole slabs
+          const int first = T.aflat > 0 ? min(ra, XA.rows - fr) : ra;
+          d = lane == 0 ? 0 : first + (lane - 1) * XA.rows;
+          n = lane == 0 ? first : min(ra - d, XA.rows);
+          slab = fs + lane;
+          row = lane == 0 ? fr : 0;
+        } else if (lane == 24) {
+          X = &XA2, slab = as2, row = ar2, n = ra2, d = T.asplit;
+        } else {
+          side = (uint32_t)s * a_bytes;
+          if (lane == 25) X = &XB, slab = bs, row = br, n = nmain;
+          if (lane == 26) X = &XT, slab = ts, row = tr, n = ntail, d = tfirst - n0;
+          if (lane == 27) X = &XT2, slab = ts2, row = tr2, n = ntail2, d = t2first - n0;
+        }
+        const uint32_t bytes = n > 0 ? (uint32_t)n * 32u * s : 0u;
+        const uint32_t dst = side + (uint32_t)d * 32u * s;
+        const __nv_bfloat16 *src = reinterpret_cast<const __nv_bfloat16 *>(X->base) +
+              (long long)slab * X->slab_stride + (long long)row * 16 * s;
+        const uint32_t total = __reduce_add_sync(0xffffffffu, bytes);
+        const int ks = max(ti.g0, kbase), ke = min(ti.g1, kend);
+        TermSlot &out = termslot[k % KQ];
+        if (!__all_sync(0xffffffffu,
+                        mbar_wait_sleep(&termempty[k % KQ], ((k / KQ) & 1) ^ 1, &err))) {
+          fail = true;
+          break;
+        }
+        if (lane < TermSlot::LANES) {
+          out.src[lane] = src + (long long)(ks - kbase) * X->kb_stride;
+          out.kbs[lane] = X->kb_stride;
+          out.bytes[lane] = bytes;
+          out.dst[lane] = dst;
+        }
+        __syncwarp();
+        if (lane == 0) {
+          out.steps = ke - ks;
+          out.neg = T.negA;
+          out.total = total;
+          mbar_arrive(&termfull[k % KQ]);
+        }
+        ++k;
+      }
+      if (fail && lane == 0 && !err) err = 2;
     }
   } else if (warp == 1) {
     {
@@ -518,8 +555,8 @@ split_engine_kernel(const SJob *__restrict__ jobs, int njobs, const STerm *__res
       for (int i = 0; ok; ++i) {
         const int q = i % TQ;
         if (!__all_sync(0xffffffffu, mbar_wait(&tfull[q], (i / TQ) & 1, &err))) break;
-        const long long tile = tq[q];
-        const int Nt = tinfo[q].Nt, g0 = tinfo[q].g0, g1 = tinfo[q].g1;
+        const long long tile = tslot[q].tile;
+        const int Nt = tslot[q].ti.Nt, g0 = tslot[q].ti.g0, g1 = tslot[q].ti.g1;
         __syncwarp();  // every lane has read the slot before it is handed back
         if (lead) mbar_arrive(&tempty[q]);
         if (tile < 0) break;
@@ -621,25 +658,17 @@ split_engine_kernel(const SJob *__restrict__ jobs, int njobs, const STerm *__res
     // epilogue: warps 2..17
     const int ew = warp - 2, quad = warp & 3, part = ew >> 2;
     const int row = quad * 32 + lane;
-    int nd = 0, jh = 0;
+    int nd = 0;
     for (int i = 0;; ++i) {
       const int q = i % TQ;
-      if (!__all_sync(0xffffffffu, mbar_wait_sleep(&tfull[q], (i / TQ) & 1, &err))) break;
-      const long long tile = tq[q];
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&tempty[q]);
-      if (tile < 0) break;
-      // decoded again from the (read-only) tables: the compiler may reload
-      // these values instead of holding them in registers across the asm
-      const TileInfo ti = decode_tile(jobs, njobs, terms, tile, jh);
-      __syncwarp();  // every lane is done with the previous tile's job
-      {
-        const uint32_t *src = reinterpret_cast<const uint32_t *>(jobs + ti.j);
-        uint32_t *dst = reinterpret_cast<uint32_t *>(&ejob[ew]);
-        for (int w = lane; w < (int)(sizeof(SJob) / 4); w += 32) dst[w] = src[w];
+      if (i > 0) {  // done with the previous tile's slot
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&tempty[(i - 1) % TQ]);
       }
-      __syncwarp();
-      const SJob &J = ejob[ew];
+      if (!__all_sync(0xffffffffu, mbar_wait_sleep(&tfull[q], (i / TQ) & 1, &err))) break;
+      if (tslot[q].tile < 0) break;
+      const SJob &J = tslot[q].job;
+      const TileInfo &ti = tslot[q].ti;
       const int Nt = ti.Nt;
       const int nsteps = ti.g1 - ti.g0;
       const int ndrains =
@@ -810,6 +839,9 @@ int s_upload_plan(const SPlan &p, SDevPlan *d, cudaStream_t s) {
   for (SJob &j : jobs) {
     long long steps = 0;
     for (int t = 0; t < j.nterm; ++t) steps += p.terms[j.term0 + t].ksteps;
+    if (steps > 0x7fffffffLL || (long long)j.batch * j.tiles_m * j.tiles_n * j.ksplit > 0x7fffffffLL)
+      return CC3_ERR_ARG;
+    j.ksteps = (int)steps;
     const long long need = (steps + S_MAX_TILE_STEPS - 1) / S_MAX_TILE_STEPS;
     if (need > j.ksplit) {
       if (j.mode == SEPI_DD_STORE) return CC3_ERR_ARG;
