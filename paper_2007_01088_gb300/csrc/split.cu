@@ -847,11 +847,10 @@ int omega_sequence(cc3_ctx *c, SplitState *S, cudaStream_t st) {
   VPtrTable P;
   fill_vptrs(c, S, &P);
   const int nv = c->nv;
-  const int kdrain = S_DRAIN_STEPS;
   for (size_t b = 0, t0 = 0; b < S->ab.size(); t0 += S->nslot[b], ++b) {
     const int ns = S->nslot[b];
     trace_begin(c, TR_SPLIT_W, st);
-    TRY(s_launch_plan(S->ab[b], S->arrs, P, s, kdrain, S->status, st, &c->counters.launches));
+    TRY(s_launch_plan(S->ab[b], S->arrs, P, s, S->status, st, &c->counters.launches));
     trace_end(c, TR_SPLIT_W, st, S->ab[b].flop, S->ab[b].slice_flop);
     trace_begin(c, TR_SPLIT_ELEM, st);
     CU(cudaMemsetAsync(S->maxbits, 0, sizeof(unsigned int) * ns, st));
@@ -862,7 +861,7 @@ int omega_sequence(cc3_ctx *c, SplitState *S, cudaStream_t st) {
     trace_end(c, TR_SPLIT_ELEM, st, 0.0, 0.0);
     c->counters.launches += 3;
     trace_begin(c, TR_SPLIT_OMEGA, st);
-    TRY(s_launch_plan(S->om[b], S->arrs, P, s, kdrain, S->status, st, &c->counters.launches));
+    TRY(s_launch_plan(S->om[b], S->arrs, P, s, S->status, st, &c->counters.launches));
     trace_end(c, TR_SPLIT_OMEGA, st, S->om[b].flop, S->om[b].slice_flop);
   }
   return CC3_OK;
@@ -1256,7 +1255,7 @@ int split_jacobian(cc3_ctx *c, int nvec, const double *w, const double *R1d, con
       std::memset(&vp2, 0, sizeof(vp2));
       vp2.p[0] = hv + v * nvvvo;
       trace_begin(c, TR_SPLIT_W, st);
-      const int lrc = s_launch_plan(D, la, vp2, s, S_DRAIN_STEPS, S->status, st,
+      const int lrc = s_launch_plan(D, la, vp2, s, S->status, st,
                                     &c->counters.launches);
       trace_end(c, TR_SPLIT_W, st, D.flop, D.slice_flop);
       CU(cudaStreamSynchronize(st));
@@ -1458,11 +1457,10 @@ int split_jacobian(cc3_ctx *c, int nvec, const double *w, const double *R1d, con
   PR.p[B_WS_TT] = TTj;
   PR.p[B_WS_W3] = W3j;
   PR.p[B_SLOTEXP] = exj;
-  const int kd = S_DRAIN_STEPS;
   long long *L = &c->counters.launches;
   auto run = [&](const SDevPlan &d, const SArrTable &a, const VPtrTable &pt, int cls) -> int {
     trace_begin(c, cls, st);
-    TRY(s_launch_plan(d, a, pt, s, kd, S->status, st, L));
+    TRY(s_launch_plan(d, a, pt, s, S->status, st, L));
     trace_end(c, cls, st, d.flop, d.slice_flop);
     return CC3_OK;
   };
@@ -1841,11 +1839,10 @@ int split_left_jacobian(cc3_ctx *c, int nvec, const double *w, const double *L1d
   PR.p[B_OMT] = s2raw;
   PR.p[B_G] = G;
   PR.p[B_H] = H;
-  const int kd = S_DRAIN_STEPS;
   long long *L = &c->counters.launches;
   auto run = [&](const SDevPlan &d, const SArrTable &a, const VPtrTable &pt, int cls) -> int {
     trace_begin(c, cls, st);
-    TRY(s_launch_plan(d, a, pt, s, kd, S->status, st, L));
+    TRY(s_launch_plan(d, a, pt, s, S->status, st, L));
     trace_end(c, cls, st, d.flop, d.slice_flop);
     return CC3_OK;
   };
@@ -2205,7 +2202,6 @@ int split_density(cc3_ctx *c, double w, const double *L1d, const double *L2d, do
   VPtrTable PV = PR;
   PV.p[B_SLOTEXP] = exs;
   PV.p[B_DVV] = Dvv;
-  const int kd = S_DRAIN_STEPS;
   long long *Lc = &c->counters.launches;
   double ex = 0.0;
   auto run = [&](const SPlan &p, const SArrTable &a, const VPtrTable &pt, int cls) -> int {
@@ -2213,7 +2209,7 @@ int split_density(cc3_ctx *c, double w, const double *L1d, const double *L2d, do
     SDevPlan d;
     TRY(s_upload_plan(p, &d, st));
     trace_begin(c, cls, st);
-    const int rc = s_launch_plan(d, a, pt, s, kd, S->status, st, Lc);
+    const int rc = s_launch_plan(d, a, pt, s, S->status, st, Lc);
     trace_end(c, cls, st, d.flop, d.slice_flop);
     CU(cudaStreamSynchronize(st));  // the tables are freed next
     s_free_plan(&d);
@@ -2378,7 +2374,7 @@ int debug_split_gemm(int M, int N, int K, const double *A, const double *B, doub
     add_sterm(P, jb, opd(0, 0), opd(1, 0), Kp, 0, ex, s);
     CK(s_upload_plan(P, &D, st));
     ptr.p[0] = dC;
-    CK(s_launch_plan(D, arrs, ptr, s, S_DRAIN_STEPS, status, st, nullptr));
+    CK(s_launch_plan(D, arrs, ptr, s, status, st, nullptr));
     int hs = 0;
     CKC(cudaMemcpyAsync(&hs, status, sizeof(int), cudaMemcpyDeviceToHost, st));
     CKC(cudaMemcpyAsync(C, dC, sizeof(double) * M * N, cudaMemcpyDeviceToHost, st));

@@ -9,7 +9,7 @@
 // does not round to nearest when addends of very different size meet, so
 // each level L = p + q <= 3 gets its own tensor-memory accumulator, whose
 // values stay exactly representable (multiples of 2^-8L below 2^(24-8L))
-// because it is drained into 64-bit fixed-point registers every 256 or 512 K;
+// because it is drained into 64-bit fixed-point registers every 256 to 900 K;
 // the levels >= 4 share a fifth, rounded accumulator (its error stays below
 // 2^-50 of the result).
 //
@@ -32,12 +32,15 @@
 //
 // What bounds it: a 128 x 96 x 16 product takes 53 clocks here (48 at the
 // nominal rate; 21 of them per K step, 1118 clocks, next to 43 KB of operands
-// arriving).  Measured in the engine on 96 triples of the no=22 nv=250
-// residual, per K step: 1902 clocks with the sums in double-float arithmetic
-// (a tile's read-back 7600 clocks, its outputs 23,700: FP64 conversions, one
-// 8-byte store per 32-byte sector in the W build's first phase), 1570 with the
-// fixed-point sums (read-back 3600, of which ~1000 stall the tensor cores;
-// outputs 11,100).  Every wait is
+// arriving), so the issuer must add little to that.  Measured in the engine on
+// 96 triples of the no=22 nv=250 residual, clocks per K step: 1902 with the
+// sums in double-float arithmetic (a tile's read-back 7600 clocks, its outputs
+// 23,700: FP64 conversions, one 8-byte store per 32-byte sector in the W
+// build's first phase); 1570 with fixed-point sums and overlapped tile ends;
+// 1525 with the decoder warp; 1361 with the issuer's operands known to be
+// uniform (4 instructions per product instead of 11; the kernel's code
+// 178 -> 88 KB, it had outgrown the instruction cache), one level drained at a
+// time and the last column tile trimmed.  Every wait is
 // bounded: on timeout the CTA sets an error word that the host turns into
 // CC3_ERR_TIMEOUT; before it exits, the CTA waits (bounded again) for its own
 // bulk copies and tensor-core products in flight, then frees its tensor
@@ -67,126 +70,160 @@ __device__ __forceinline__ long long s_rowoff(int m, int m_in, long long s1, lon
   return (long long)(m / m_in) * s1 + (long long)(m % m_in) * s0;
 }
 
-// One slice product p x q into accumulator min(p + q, 4) (at a fixed column,
-// so that tiles of different N keep out of each other's), as element `i` of
-// a run of `n` products that share A slice p (the run keeps A in the
-// collector buffer instead of reading it from shared memory again).
+// A value that all lanes of the warp hold, as one the compiler knows to be
+// uniform: tcgen05.mma takes its operands from uniform registers.
+__device__ __forceinline__ int uniform(int x) { return __shfl_sync(0xffffffffu, x, 0); }
+__device__ __forceinline__ uint32_t uniform(uint32_t x) { return __shfl_sync(0xffffffffu, x, 0); }
+
+// The next group of (one or two) K steps: whether its stages have landed.
+// The issuer looks while it still has products to queue, so that a landed
+// stage costs no round trip between two groups.
+struct Ahead {
+  uint64_t *b0, *b1;  // full barriers of the next two stages
+  uint32_t p0, p1;    // their parities
+  bool r0, r1;
+  __device__ __forceinline__ void look() {
+    r0 = __all_sync(0xffffffffu, mbar_test(b0, p0));
+    r1 = __all_sync(0xffffffffu, mbar_test(b1, p1));
+  }
+};
+
+// All slice products of one or two K steps, the A-slice runs of two steps
+// interleaved (run p of step 0, run p of step 1, run p + 1 of step 0, ...).
+// Product p x q goes into accumulator min(p + q, 4), each at a fixed column so
+// that tiles of different N keep out of each other's.  Each run keeps its A
+// slice in the collector buffer: A is read from shared memory S times per step
+// instead of once per product (53 clocks per 128 x 96 x 16 product, 57
+// without).  Slices are 256 bytes (16 descriptor units) apart.
 template <int S>
-__device__ __forceinline__ void issue_one(uint32_t lead, uint32_t tmem, uint64_t dA, uint64_t dB,
-                                          uint32_t idesc, uint32_t en, int p, int q, int i,
-                                          int n) {
-  const int lv = p + q;
-  const uint32_t d = tmem + (uint32_t)((lv < 4 ? lv : 4) * S_NT_MAX);
-  // slices are 256 bytes (16 descriptor units) apart
-  const uint64_t a = dA + (uint64_t)(p * 16), b = dB + (uint64_t)(q * 16);
-  if (n == 1)
-    umma_f16_a<0>(lead, d, a, b, idesc, en);
-  else if (i == 0)
-    umma_f16_a<1>(lead, d, a, b, idesc, en);
-  else if (i == n - 1)
-    umma_f16_a<3>(lead, d, a, b, idesc, en);
-  else
-    umma_f16_a<2>(lead, d, a, b, idesc, en);
-}
-
-// The accumulators that drain d of a tile (counted from 0) empties: levels 0,
-// 2 and 3 at every drain, level 1 too at every second one.  With a drain every
-// 256 K (or fewer) that keeps them exact: per K at most 1, 2, 3, 4 products of
-// |d d'| <= 2^14 reach level 0, 1, 2, 3, so the sums stay within 2^22, 2^24
-// (512 K), 3 2^22 and 2^24 of their unit 2^-8L.
-__device__ __forceinline__ bool drains_all(int d) { return (d & 1) != 0; }
-constexpr uint32_t DRAIN_SOME = 0xDu, DRAIN_ALL = 0xFu, ACC_HIGH = 0x10u;
-
-// K steps between drains of a tile of `steps` steps: equal parts of at most
-// kdrain_steps, an even number (the issuer takes steps in pairs).
-__device__ __forceinline__ int drain_interval(int steps, int kdrain_steps) {
-  const int parts = (steps + kdrain_steps - 1) / kdrain_steps;
-  return parts > 1 ? 2 * ((steps + 2 * parts - 1) / (2 * parts)) : kdrain_steps;
-}
-
-// Issues the slice products of one K step into the accumulators of MASK (bit
-// L: accumulator L), A slice by A slice, fully unrolled; `en` is the mode of
-// each accumulator's first product here, which is its product with A slice 0.
-template <int S, uint32_t MASK>
-__device__ __forceinline__ void issue_products(uint32_t lead, uint32_t tmem, uint64_t dA,
-                                               uint64_t dB, uint32_t idesc, uint32_t en) {
+__device__ __forceinline__ void issue_all(uint32_t lead, uint32_t tmem, uint64_t dA0, uint64_t dB0,
+                                          uint32_t id0, uint64_t dA1, uint64_t dB1, uint32_t id1,
+                                          bool two, Ahead &next) {
 #pragma unroll
   for (int p = 0; p < S; ++p) {
-    int n = 0;
+    if (p == S - 3) next.look();  // 6 products of each step to go
 #pragma unroll
-    for (int q = 0; q < S - p; ++q) n += (MASK >> (p + q < 4 ? p + q : 4)) & 1u;
-    int i = 0;
+    for (int j = 0; j < 2; ++j) {
+      if (j == 1 && !two) break;
+      const uint64_t a = (j ? dA1 : dA0) + (uint64_t)(p * 16), dB = j ? dB1 : dB0;
+      const uint32_t id = j ? id1 : id0;
 #pragma unroll
-    for (int q = 0; q < S - p; ++q)
-      if ((MASK >> (p + q < 4 ? p + q : 4)) & 1u) {
-        issue_one<S>(lead, tmem, dA, dB, idesc, p == 0 && q <= 4 ? en : 1u, p, q, i, n);
+      for (int q = 0; q < S - p; ++q) {
+        const uint32_t d = tmem + (uint32_t)((p + q < 4 ? p + q : 4) * S_NT_MAX);
+        const uint64_t b = dB + (uint64_t)(q * 16);
+        if (S - p == 1)
+          umma_f16_a<0>(lead, d, a, b, id, 1u);
+        else if (q == 0)
+          umma_f16_a<1>(lead, d, a, b, id, 1u);
+        else if (q == S - p - 1)
+          umma_f16_a<3>(lead, d, a, b, id, 1u);
+        else
+          umma_f16_a<2>(lead, d, a, b, id, 1u);
+      }
+    }
+  }
+}
+
+// The slice products of one or two K steps that go into the accumulators of
+// MASK (bit L: accumulator L), A slice by A slice; with FRESH they start anew.
+template <int S, uint32_t MASK, bool FRESH>
+__device__ __forceinline__ void issue_some(uint32_t lead, uint32_t tmem, uint64_t dA0,
+                                           uint64_t dB0, uint32_t id0, uint64_t dA1, uint64_t dB1,
+                                           uint32_t id1, bool two) {
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    if (j == 1 && !two) break;
+    const uint64_t dA = j ? dA1 : dA0, dB = j ? dB1 : dB0;
+    const uint32_t id = j ? id1 : id0;
+#pragma unroll
+    for (int p = 0; p < S; ++p) {
+      int n = 0, i = 0;
+#pragma unroll
+      for (int q = 0; q < S - p; ++q) n += (MASK >> (p + q < 4 ? p + q : 4)) & 1u;
+#pragma unroll
+      for (int q = 0; q < S - p; ++q) {
+        const int L = p + q < 4 ? p + q : 4;
+        if (!((MASK >> L) & 1u)) continue;
+        const uint32_t d = tmem + (uint32_t)(L * S_NT_MAX);
+        const uint64_t a = dA + (uint64_t)(p * 16), b = dB + (uint64_t)(q * 16);
+        // an accumulator's first product is its one with A slice 0
+        const uint32_t en = FRESH && j == 0 && p == 0 && q <= 4 ? 0u : 1u;
+        if (n == 1)
+          umma_f16_a<0>(lead, d, a, b, id, en);
+        else if (i == 0)
+          umma_f16_a<1>(lead, d, a, b, id, en);
+        else if (i == n - 1)
+          umma_f16_a<3>(lead, d, a, b, id, en);
+        else
+          umma_f16_a<2>(lead, d, a, b, id, en);
         ++i;
       }
+    }
   }
 }
 
-// The K steps right after a drain point: first the products into the
-// accumulators that are not being emptied (MASK: those that are), then, once
-// the epilogue has read them, the others, which start anew.
-template <int S, uint32_t MASK>
-__device__ __forceinline__ bool issue_after_drain(uint32_t lead, uint32_t tmem, uint64_t dA0,
-                                                  uint64_t dB0, uint32_t id0, uint64_t dA1,
-                                                  uint64_t dB1, uint32_t id1, bool two,
-                                                  uint64_t *empty, int parity,
-                                                  volatile int *err) {
-  constexpr uint32_t KEEP = 0x1Fu & ~MASK;
-  issue_products<S, KEEP>(lead, tmem, dA0, dB0, id0, 1u);
-  if (two) issue_products<S, KEEP>(lead, tmem, dA1, dB1, id1, 1u);
-  if (!__all_sync(0xffffffffu, mbar_wait(empty, parity, err))) return false;
-  tc_fence_after();
-  issue_products<S, MASK>(lead, tmem, dA0, dB0, id0, 0u);
-  if (two) issue_products<S, MASK>(lead, tmem, dA1, dB1, id1, 1u);
-  return true;
+// Drains keep the exact accumulators exact: per K at most 1, 2, 3, 4 products
+// of |d d'| <= 2^14 reach level 0, 1, 2, 3, so level 3 is emptied after at most
+// 16 K steps of 16, level 2 after 20, level 1 after 28 and level 0 after 56
+// (sums within 2^24, 0.94 2^24, 0.88 2^24 and 0.88 2^24 of their unit 2^-8L).
+// One level is emptied at a time, between two K steps, so that the products
+// into the other four accumulators (17 to 20 of the 21 of each step) cover the
+// read-back: drained four levels at a time, a drain took 2900 clocks, 1800 of
+// them stalls.  A level is due once it holds drain_at(L) steps, unless the
+// tile ends within its limit; level 3 goes first.  Since a drain is followed
+// by two K steps before the next, the limits hold: 12 + 2, 16 + 2 + 2,
+// 24 + 3 and 48 + 6.
+__device__ __forceinline__ constexpr int drain_at(int L) {
+  return L == 3 ? 12 : (L == 2 ? 16 : (L == 1 ? 24 : 48));
 }
-
-// The slice products of two consecutive K steps with their A-slice runs
-// interleaved (run p of step 0, run p of step 1, run p + 1 of step 0, ...):
-// the first products that read a newly landed stage then overlap the other
-// step's products instead of waiting alone.  Each run keeps its A slice in
-// the collector buffer: A is read from shared memory S times per step instead
-// of once per product.
-template <int S>
-__device__ __forceinline__ void issue_products_pair(uint32_t lead, uint32_t tmem, uint64_t dA0,
-                                                    uint64_t dB0, uint32_t id0, uint64_t dA1,
-                                                    uint64_t dB1, uint32_t id1) {
-#pragma unroll
-  for (int p = 0; p < S; ++p) {
-#pragma unroll
-    for (int q = 0; q < S - p; ++q)
-      issue_one<S>(lead, tmem, dA0, dB0, id0, 1u, p, q, q, S - p);
-#pragma unroll
-    for (int q = 0; q < S - p; ++q)
-      issue_one<S>(lead, tmem, dA1, dB1, id1, 1u, p, q, q, S - p);
-  }
+__device__ __forceinline__ constexpr int drain_limit(int L) {
+  return L == 3 ? 16 : (L == 2 ? 20 : (L == 1 ? 28 : 56));
 }
+constexpr int EV_END = 4;  // epilogue event: 0..3 = drain that level, 4 = the tile's end
 
-// The epilogue's sum of one output element: a fixed-point integer with
-// S_ACC_FRAC fraction bits.  The accumulators of levels 0..3 hold integers
-// times 2^-8L below 2^(24-8L), so they convert to int exactly and the sum is
-// exact; the shared one is rounded at 2^-33, far below the slice products that
-// the expansion leaves out (~2^-28 of the same unit for K = 500).
-// |sum| < 2^31 while a tile has at most S_MAX_TILE_STEPS K steps, and the
-// shared accumulator's conversion stays below 2^31 as well.
-//
-// Conversions to int run at a quarter of the FP32 rate, so two of the four
-// levels take none: adding FX_R0 = 1.5 2^23 to an integer |v0| <= 2^22 leaves
-// v0 in the low bits of the sum's pattern (above those of FX_R0 itself), and
-// adding FX_R2 = 1.5 2^9 to |v2| <= 192 leaves v2 in units of 2^-14; what that
-// rounds off, at most 2^-15, joins level 3.
-constexpr float FX_R0 = 12582912.f, FX_R2 = 768.f;
+// Conversions to int run at a quarter of the FP32 rate, so at a tile's end two
+// of the four levels take none: adding FX_R0 = 1.5 2^25 to an integer |v0| <
+// 2^24 leaves v0 in units of 4 in the low bits of the sum's pattern (above
+// those of FX_R0 itself), and adding FX_R2 = 1.5 2^9 to |v2| <= 240 leaves v2
+// in units of 2^-14; what the two round off, at most 2 and 2^-15, joins levels
+// 1 and 3 exactly.  FX_BIAS: what the patterns of the constants add.
+constexpr float FX_R0 = 50331648.f, FX_R2 = 768.f;
 constexpr unsigned long long FX_W2 = 1ull << (S_ACC_FRAC - 14);
-__device__ __forceinline__ long long fx_levels(long long a, float v0, float v2, float v3) {
+constexpr unsigned long long FX_BIAS = (0x4C400000ull << 34) + 0x44400000ull * FX_W2;
+__device__ __forceinline__ long long fx_levels(long long a, float v0, float v1, float v2,
+                                               float v3) {
   const float t0 = __fadd_rn(v0, FX_R0), t2 = __fadd_rn(v2, FX_R2);
-  const float r = __fsub_rn(v2, __fsub_rn(t2, FX_R2));
-  const int i3 = __float2int_rn(__fadd_rn(r, v3) * 0x1p24f);
-  unsigned long long u = (unsigned long long)a + ((unsigned long long)__float_as_uint(t0) << 32);
-  u += (unsigned long long)__float_as_uint(t2) * FX_W2;
-  return (long long)u + (long long)i3 * 256;
+  const float r0 = __fsub_rn(v0, __fsub_rn(t0, FX_R0)), r2 = __fsub_rn(v2, __fsub_rn(t2, FX_R2));
+  const int i1 = __float2int_rn(__fadd_rn(r0, v1) * 0x1p8f),
+            i3 = __float2int_rn(__fadd_rn(r2, v3) * 0x1p24f);
+  unsigned long long u = (unsigned long long)a + ((unsigned long long)__float_as_uint(t0) << 34);
+  u += (unsigned long long)__float_as_uint(t2) * FX_W2 - FX_BIAS;
+  return (long long)u + (long long)i1 * (1ll << 24) + (long long)i3 * 256;
+}
+// Reads one level of this warp's columns (nch chunks of 4 from TMEM address tb,
+// which is that level's) into the sums: v 2^(8L) as an integer, times 2^(32 - 8L).
+__device__ __forceinline__ void drain_level(uint32_t tb, int L, int nch, long long (&acc)[6][4]) {
+  const float up = __int_as_float((127 + 8 * L) << 23);
+  const long long w = 1ll << (S_ACC_FRAC - 8 * L);
+#pragma unroll
+  for (int c = 0; c < 6; ++c) {
+    if (c >= nch) break;
+    float v[4];
+    tmem_ld4(tb + c * 4, v);
+    tmem_wait_ld();
+#pragma unroll
+    for (int k = 0; k < 4; ++k) acc[c][k] += (long long)__float2int_rn(v[k] * up) * w;
+  }
+}
+
+// Moves chunk 1 to 0, 2 to 1, ...: the output loops take chunk 0 of a rolled
+// loop, which costs 40 moves per chunk but keeps their code a sixth of the
+// unrolled size (it was 98 KB, more than half of the kernel).
+__device__ __forceinline__ void next_chunk(long long (&acc)[6][4]) {
+#pragma unroll
+  for (int c = 0; c < 5; ++c)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) acc[c][k] = acc[c + 1][k];
 }
 
 // a 2^e2 as a double, rounded once, from integer operations: the FP64 pipe of
@@ -235,8 +272,8 @@ __device__ __forceinline__ TileInfo decode_tile(const SJob &J, long long tile) {
   const int ks = r % J.ksplit;
   r /= J.ksplit;
   t.m0 = r / J.tiles_n * S_BM;
-  t.Nt = J.Ntile;
   t.n0 = r % J.tiles_n * J.Ntile;
+  t.Nt = min(J.Ntile, (J.N - t.n0 + 15) / 16 * 16);  // the last column tile is trimmed
   const int per = (J.ksteps + J.ksplit - 1) / J.ksplit;
   t.g0 = min(J.ksteps, ks * per);
   t.g1 = min(J.ksteps, t.g0 + per);
@@ -273,7 +310,7 @@ template <int S>
 __global__ void __maxnreg__(96)
 split_engine_kernel(const SJob *__restrict__ jobs, int njobs, const STerm *__restrict__ terms,
                     const __grid_constant__ SArrTable arrs, VPtrTable P,
-                    int kdrain_steps, int *status, unsigned long long *tile_ctr,
+                    int *status, unsigned long long *tile_ctr,
                     long long ntiles) {
   constexpr int s = S;
   constexpr int S_STAGES = s_stages(S);
@@ -286,10 +323,11 @@ split_engine_kernel(const SJob *__restrict__ jobs, int njobs, const STerm *__res
   uint8_t *smem = reinterpret_cast<uint8_t *>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   __shared__ __align__(8) uint64_t full[S_STAGES], empty[S_STAGES];
-  // lowfull / lowempty: accumulators 0..3 at a tile's end; accfull / accempty:
-  // the shared one (and the tile)
-  __shared__ __align__(8) uint64_t lowfull, lowempty, accfull, accempty, drainfull, drainempty,
-      mmafin;
+  // evfull: an event for the epilogue (drain a level, or the tile's end), which
+  // answers on drainempty or lowempty; accfull / accempty: the shared accumulator
+  // at the tile's end.  One event is outstanding at a time.
+  __shared__ __align__(8) uint64_t evfull, drainempty, lowempty, accfull, accempty, mmafin;
+  __shared__ volatile int event;
   __shared__ __align__(8) uint64_t tfull[TQ], tempty[TQ];
   // the decoder decodes each tile once for everyone, with a copy of its job
   // (the output loop reads its fields for every element), and marks each stage
@@ -302,7 +340,8 @@ split_engine_kernel(const SJob *__restrict__ jobs, int njobs, const STerm *__res
   __shared__ uint32_t tmem_base_sh;
   __shared__ volatile int err;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // broadcast, so that the compiler knows the roles' branches to be uniform
+  const int warp = uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int i = 0; i < S_STAGES; ++i) {
       mbar_init(&full[i], 1);
@@ -316,11 +355,10 @@ split_engine_kernel(const SJob *__restrict__ jobs, int njobs, const STerm *__res
       mbar_init(&termfull[i], 1);
       mbar_init(&termempty[i], 1);
     }
-    mbar_init(&lowfull, 1);
+    mbar_init(&evfull, 2);  // the event's word and the products before it
     mbar_init(&lowempty, S_EPI_WARPS);
     mbar_init(&accfull, 1);
     mbar_init(&accempty, S_EPI_WARPS);
-    mbar_init(&drainfull, 1);
     mbar_init(&drainempty, S_EPI_WARPS);
     mbar_init(&mmafin, 1);
     err = 0;
@@ -330,7 +368,7 @@ split_engine_kernel(const SJob *__restrict__ jobs, int njobs, const STerm *__res
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = tmem_base_sh;
+  const uint32_t tmem = uniform(tmem_base_sh);
   const uint32_t a_bytes = S_BM * 32;
 
   if (warp == 0) {
@@ -550,16 +588,19 @@ split_engine_kernel(const SJob *__restrict__ jobs, int njobs, const STerm *__res
       // MMA issuer: the warp stays converged (every lane waits and steps, the
       // elected one issues), see umma_f16_a
       const uint32_t lead = elect_one();
-      int it = 0, nd = 0;
+      int nd = 0, st0 = 0;  // drains so far, the next stage and its parity
+      uint32_t ph0 = 0;
+      Ahead next = {&full[0], &full[0], 0u, 0u, false, false};
       bool ok = true;
       for (int i = 0; ok; ++i) {
         const int q = i % TQ;
         if (!__all_sync(0xffffffffu, mbar_wait(&tfull[q], (i / TQ) & 1, &err))) break;
-        const long long tile = tslot[q].tile;
-        const int Nt = tslot[q].ti.Nt, g0 = tslot[q].ti.g0, g1 = tslot[q].ti.g1;
+        const int more = uniform(tslot[q].tile >= 0);
+        const int Nt = uniform(tslot[q].ti.Nt), g0 = uniform(tslot[q].ti.g0),
+                  g1 = uniform(tslot[q].ti.g1);
         __syncwarp();  // every lane has read the slot before it is handed back
         if (lead) mbar_arrive(&tempty[q]);
-        if (tile < 0) break;
+        if (!more) break;
         const uint32_t id_pos = idesc_bf16(S_BM, Nt, 0), id_neg = idesc_bf16(S_BM, Nt, 1);
         // the epilogue has read the previous tile's accumulators: levels 0..3
         // and, later, the shared one
@@ -569,27 +610,41 @@ split_engine_kernel(const SJob *__restrict__ jobs, int njobs, const STerm *__res
           tc_fence_after();
           return true;
         };
+        // an event for the epilogue, due when the products issued so far are done
+        auto signal = [&](int ev) {
+          if (lead) {
+            event = ev;
+            mbar_arrive(&evfull);
+            umma_commit(&evfull);
+          }
+          __syncwarp();
+        };
         auto high_free = [&]() {
           if (i > 0 && !__all_sync(0xffffffffu, mbar_wait(&accempty, (i - 1) & 1, &err)))
             return false;
           tc_fence_after();
           return true;
         };
-        const int kdrain = drain_interval(g1 - g0, kdrain_steps);
-        int since = 0, ndt = 0;  // K steps since the last drain, drains of this tile
-        bool pending = false;
-        // K steps two at a time (drains come after an even number of steps, so
-        // a pair never straddles one); a lone last step of a tile goes alone
+        int held[4] = {0, 0, 0, 0};  // K steps that each level holds
+        int pending = -1;            // the level being drained
+        // K steps two at a time; a lone last step of a tile goes alone
         for (int g = g0; g < g1;) {
+          const bool first = g == g0, last = g + 2 >= g1;
           const bool two = g + 1 < g1;
           const int n = two ? 2 : 1;
-          const int st0 = it % S_STAGES, ph0 = (it / S_STAGES) & 1;
-          const int st1 = (it + 1) % S_STAGES, ph1 = ((it + 1) / S_STAGES) & 1;
-          bool here = mbar_wait(&full[st0], ph0, &err);
-          if (two) here = here && mbar_wait(&full[st1], ph1, &err);
+          const int st1 = st0 + 1 == S_STAGES ? 0 : st0 + 1;
+          const uint32_t ph1 = st1 == 0 ? ph0 ^ 1 : ph0;
+          bool here = next.r0 || mbar_wait(&full[st0], ph0, &err);
+          if (two) here = here && (next.r1 || mbar_wait(&full[st1], ph1, &err));
           if (!__all_sync(0xffffffffu, here)) { ok = false; break; }
           tc_fence_after();
-          const uint32_t id0 = sneg[st0] ? id_neg : id_pos, id1 = sneg[st1] ? id_neg : id_pos;
+          // the stages after this group's
+          const int sn = two ? (st1 + 1 == S_STAGES ? 0 : st1 + 1) : st1;
+          const uint32_t pn = two ? (sn == 0 ? ph1 ^ 1 : ph1) : ph1;
+          const int sm = sn + 1 == S_STAGES ? 0 : sn + 1;
+          next = Ahead{&full[sn], &full[sm], pn, sm == 0 ? pn ^ 1 : pn, false, false};
+          const uint32_t id0 = uniform(sneg[st0]) ? id_neg : id_pos,
+                         id1 = uniform(sneg[st1]) ? id_neg : id_pos;
           const size_t stage_bytes = (size_t)s * (a_bytes + S_NT_MAX * 32);
           const uint32_t sa0 = smem_u32(smem + (size_t)st0 * stage_bytes),
                          sa1 = smem_u32(smem + (size_t)st1 * stage_bytes);
@@ -598,52 +653,77 @@ split_engine_kernel(const SJob *__restrict__ jobs, int njobs, const STerm *__res
                          dB0 = smem_desc_kmajor(sa0 + (uint32_t)s * a_bytes, 256u * s),
                          dA1 = smem_desc_kmajor(sa1, 256u * s),
                          dB1 = smem_desc_kmajor(sa1 + (uint32_t)s * a_bytes, 256u * s);
-          const bool first = g == g0, last = g + n >= g1;
-          if (pending) {
-            ok = drains_all(ndt - 1)
-                     ? issue_after_drain<S, DRAIN_ALL>(lead, tmem, dA0, dB0, id0, dA1, dB1, id1,
-                                                       two, &drainempty, nd & 1, &err)
-                     : issue_after_drain<S, DRAIN_SOME>(lead, tmem, dA0, dB0, id0, dA1, dB1, id1,
-                                                        two, &drainempty, nd & 1, &err);
-            if (!ok) break;
-            ++nd;
-            pending = false;
-            if (last && lead) umma_commit(&lowfull);
-          } else if (first || last) {
-            // a tile's ends: levels 0..3 and the shared accumulator apart, so
-            // that the epilogue reads the ones while products go to the other
-            const uint32_t en = first ? 0u : 1u;
-            if (first && !low_free()) { ok = false; break; }
-            issue_products<S, DRAIN_ALL>(lead, tmem, dA0, dB0, id0, en);
-            if (two) issue_products<S, DRAIN_ALL>(lead, tmem, dA1, dB1, id1, 1u);
-            if (last && lead) umma_commit(&lowfull);
-            __syncwarp();
-            if (first && !high_free()) { ok = false; break; }
-            issue_products<S, ACC_HIGH>(lead, tmem, dA0, dB0, id0, en);
-            if (two) issue_products<S, ACC_HIGH>(lead, tmem, dA1, dB1, id1, 1u);
+          if (pending >= 0 || first || last) {
+            // in two parts.  After a drain point: the products into the
+            // accumulators that are not being emptied, then, once the epilogue
+            // has read it, the one that is, which starts anew.  At a tile's
+            // ends: levels 0..3, then the shared accumulator, so that the
+            // epilogue reads the ones while products go to the other.
+#define CC3_SOME(MASK, FRESH) \
+  issue_some<S, MASK, FRESH>(lead, tmem, dA0, dB0, id0, dA1, dB1, id1, two)
+            if (pending >= 0) {
+              switch (pending) {
+                case 0: CC3_SOME(0x1Eu, false); break;
+                case 1: CC3_SOME(0x1Du, false); break;
+                case 2: CC3_SOME(0x1Bu, false); break;
+                default: CC3_SOME(0x17u, false); break;
+              }
+              next.look();
+              ok = __all_sync(0xffffffffu, mbar_wait(&drainempty, nd & 1, &err));
+              if (!ok) break;
+              tc_fence_after();
+              ++nd;
+              switch (pending) {
+                case 0: CC3_SOME(0x1u, true); break;
+                case 1: CC3_SOME(0x2u, true); break;
+                case 2: CC3_SOME(0x4u, true); break;
+                default: CC3_SOME(0x8u, true); break;
+              }
+              pending = -1;
+            } else if (first) {
+              ok = low_free();
+              if (!ok) break;
+              CC3_SOME(0xFu, true);
+              if (last) signal(EV_END);
+              next.look();
+              ok = high_free();
+              if (!ok) break;
+              CC3_SOME(0x10u, true);
+            } else {
+              CC3_SOME(0xFu, false);
+              signal(EV_END);
+              next.look();
+              CC3_SOME(0x10u, false);
+            }
+#undef CC3_SOME
           } else {
-            issue_products_pair<S>(lead, tmem, dA0, dB0, id0, dA1, dB1, id1);
+            issue_all<S>(lead, tmem, dA0, dB0, id0, dA1, dB1, id1, two, next);
           }
           g += n;
-          it += n;
-          since += n;
-          const bool drain = since >= kdrain && g < g1;
           if (lead) {
             umma_commit(&empty[st0]);
             if (two) umma_commit(&empty[st1]);
-            if (drain) umma_commit(&drainfull);
           }
           __syncwarp();
-          if (drain) {
-            pending = true;
-            since = 0;
-            ++ndt;
+          st0 = sn;
+          ph0 = pn;
+          const int left = g1 - g;
+#pragma unroll
+          for (int L = 0; L < 4; ++L) held[L] += n;
+          if (left > 2) {  // never right before the tile's last steps
+#pragma unroll
+            for (int L = NLOW - 1; L >= 0; --L)
+              if (pending < 0 && held[L] >= drain_at(L) && held[L] + left > drain_limit(L)) {
+                pending = L;
+                held[L] = 0;
+              }
+            if (pending >= 0) signal(pending);
           }
         }
         if (!ok) break;
         if (g0 == g1) {  // no K steps: nothing to wait for but the protocol
           if (!low_free() || !high_free()) break;
-          if (lead) umma_commit(&lowfull);
+          signal(EV_END);
         }
         if (lead) umma_commit(&accfull);
         __syncwarp();
@@ -658,7 +738,7 @@ split_engine_kernel(const SJob *__restrict__ jobs, int njobs, const STerm *__res
     // epilogue: warps 2..17
     const int ew = warp - 2, quad = warp & 3, part = ew >> 2;
     const int row = quad * 32 + lane;
-    int nd = 0;
+    int nev = 0;
     for (int i = 0;; ++i) {
       const int q = i % TQ;
       if (i > 0) {  // done with the previous tile's slot
@@ -671,58 +751,47 @@ split_engine_kernel(const SJob *__restrict__ jobs, int njobs, const STerm *__res
       const TileInfo &ti = tslot[q].ti;
       const int Nt = ti.Nt;
       const int nsteps = ti.g1 - ti.g0;
-      const int ndrains =
-          nsteps > 0 ? (nsteps - 1) / drain_interval(nsteps, kdrain_steps) : 0;
       const int qc = Nt >> 2;   // columns per quarter (multiple of 4, <= 24)
       const int nch = qc >> 2;  // 4-column chunks (<= 6)
       const uint32_t tb = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(part * qc);
       long long acc[6][4];
-      {  // less what every read below adds with the bits of its two rounding constants
-        const unsigned long long z =
-            0ull - (unsigned long long)(ndrains + 1) *
-                       (((unsigned long long)__float_as_uint(FX_R0) << 32) +
-                        (unsigned long long)__float_as_uint(FX_R2) * FX_W2);
 #pragma unroll
-        for (int c = 0; c < 6; ++c)
+      for (int c = 0; c < 6; ++c)
 #pragma unroll
-          for (int k = 0; k < 4; ++k) acc[c][k] = nsteps > 0 ? (long long)z : 0ll;
-      }
-      // the drains, then (d == ndrains) levels 0..3 at the tile's end
+        for (int k = 0; k < 4; ++k) acc[c][k] = 0ll;
+      // the drains, then levels 0..3 at the tile's end
       bool ok = true;
-      for (int d = 0; d <= ndrains; ++d) {
-        const bool last = d == ndrains;
-        ok = __all_sync(0xffffffffu,
-                        mbar_wait(last ? &lowfull : &drainfull, (last ? i : nd) & 1, &err));
+      for (;;) {
+        ok = __all_sync(0xffffffffu, mbar_wait(&evfull, nev & 1, &err));
         if (!ok) break;
+        ++nev;
+        const int ev = event;
         tc_fence_after();
-        if (nsteps > 0) {
-          const bool with1 = last || drains_all(d);
-#pragma unroll
-          for (int c = 0; c < 6; ++c) {
-            if (c >= nch) break;
-            float v[4][4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) v[1][k] = v[3][k] = 0.f;
-            tmem_ld4(tb + c * 4, v[0]);
-            tmem_ld4(tb + 2 * S_NT_MAX + c * 4, v[2]);
-            if (NLOW > 3) tmem_ld4(tb + 3 * S_NT_MAX + c * 4, v[3]);
-            if (with1) tmem_ld4(tb + S_NT_MAX + c * 4, v[1]);
-            tmem_wait_ld();
-#pragma unroll
-            for (int k = 0; k < 4; ++k) acc[c][k] = fx_levels(acc[c][k], v[0][k], v[2][k], v[3][k]);
-            if (with1) {
-#pragma unroll
-              for (int k = 0; k < 4; ++k)
-                acc[c][k] += (long long)__float2int_rn(v[1][k] * 0x1p8f) * (1ll << 24);
-            }
-          }
-        }
+        if (ev == EV_END) break;
+        drain_level(tb + (uint32_t)(ev * S_NT_MAX), ev, nch, acc);
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(last ? &lowempty : &drainempty);
-        if (!last) ++nd;
+        if (lane == 0) mbar_arrive(&drainempty);
       }
       if (!ok) break;
+      if (nsteps > 0) {
+#pragma unroll
+        for (int c = 0; c < 6; ++c) {
+          if (c >= nch) break;
+          float v[4][4];
+#pragma unroll
+          for (int k = 0; k < 4; ++k) v[3][k] = 0.f;
+#pragma unroll
+          for (int L = 0; L < NLOW; ++L) tmem_ld4(tb + L * S_NT_MAX + c * 4, v[L]);
+          tmem_wait_ld();
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+            acc[c][k] = fx_levels(acc[c][k], v[0][k], v[1][k], v[2][k], v[3][k]);
+        }
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&lowempty);
       // the shared accumulator
       if (!__all_sync(0xffffffffu, mbar_wait(&accfull, i & 1, &err))) break;
       if (HAS_HIGH && nsteps > 0) {
@@ -759,22 +828,21 @@ split_engine_kernel(const SJob *__restrict__ jobs, int njobs, const STerm *__res
         float2 *out = reinterpret_cast<float2 *>(P.p[Cm.buf]) + rowM + (long long)n0 * Cm.sn0;
         const long long sn = Cm.sn0;
         const int ncol = row_ok ? J.n_valid - n0 : 0;
-#pragma unroll
-        for (int c = 0; c < 6; ++c) {
-          if (c >= nch) break;
+#pragma unroll 1
+        for (int c = 0; c < nch; ++c) {
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
-            if (c * 4 + k < ncol) *out = fixed_to_dd(acc[c][k], e2);
+            if (c * 4 + k < ncol) *out = fixed_to_dd(acc[0][k], e2);
             out += sn;
           }
+          next_chunk(acc);
         }
         continue;
       }
       if (!row_ok) continue;
       const int mq = mo / Cm.m_in, mr = mo % Cm.m_in;  // route 1: shared by its outputs
-#pragma unroll
-      for (int c = 0; c < 6; ++c) {
-        if (c >= nch) break;
+#pragma unroll 1
+      for (int c = 0; c < nch; ++c, next_chunk(acc)) {
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
           const int n = n0 + c * 4 + k;
@@ -801,7 +869,7 @@ split_engine_kernel(const SJob *__restrict__ jobs, int njobs, const STerm *__res
                   (long long)(n - tlo) * Ctl.sn0;
             buf = Ctl.buf;
           }
-          const double x = fixed_to_double(acc[c][k], e2);
+          const double x = fixed_to_double(acc[0][k], e2);
           if (P.fx[buf])
             fx_add_call(P.fx[buf] + 2 * off, x);
           else
@@ -882,16 +950,11 @@ void s_free_plan(SDevPlan *d) {
 }
 
 int s_launch_plan(const SDevPlan &d, const SArrTable &arrs, const VPtrTable &ptrs,
-                  int slices, int kdrain_steps, int *status, cudaStream_t s,
+                  int slices, int *status, cudaStream_t s,
                   long long *launches) {
   if (d.njobs == 0 || d.tiles == 0) return CC3_OK;
   if (d.tiles > 0x7fffffffLL) return CC3_ERR_ARG;
   if (slices < 3 || slices > S_MAX_SLICES) return CC3_ERR_ARG;
-  // the issuer takes K steps in pairs, so the exact accumulators are drained
-  // after an even number of steps: the interval must be even (and at most 16,
-  // the bound that keeps them exact)
-  if (kdrain_steps < 2 || kdrain_steps > 16 || (kdrain_steps & 1))
-    return CC3_FAIL(CC3_ERR_ARG, "drain interval");
   // at least 120 KB so that one CTA (and one 512-column TMEM allocation) per SM
   const size_t smem = std::max<size_t>(s_smem_bytes(slices, S_NT_MAX), 120 * 1024);
   // per device, once; several host threads (serving slots) may get here at once
@@ -926,7 +989,7 @@ int s_launch_plan(const SDevPlan &d, const SArrTable &arrs, const VPtrTable &ptr
 #define CC3_SPLIT_LAUNCH(S_)                                                              \
   case S_:                                                                                \
     split_engine_kernel<S_><<<grid, S_THREADS, smem, s>>>(                                \
-        d.jobs, d.njobs, d.terms, arrs, ptrs, kdrain_steps, status, d.counter, d.tiles);  \
+        d.jobs, d.njobs, d.terms, arrs, ptrs, status, d.counter, d.tiles);                \
     break;
     CC3_SPLIT_LAUNCH(3)
     CC3_SPLIT_LAUNCH(4)

@@ -7,7 +7,7 @@
 namespace cc3 {
 
 enum { SMAX_MAPS = 48, S_BM = 128, S_BK = 16, S_STAGES_MAX = 6, S_MAX_SLICES = 7,
-       S_NT_MAX = 96, S_DRAIN_STEPS = 16, S_EPI_WARPS = 16, S_THREADS = 96 + 32 * S_EPI_WARPS,
+       S_NT_MAX = 96, S_EPI_WARPS = 16, S_THREADS = 96 + 32 * S_EPI_WARPS,
        // fraction bits of the epilogue's fixed-point sums, and the K steps of a
        // tile that keep them in 64 bits (and the shared accumulator's terms in 32:
        // 5 2^14 (1 + 2^-6) 16 S_MAX_TILE_STEPS < 2^31)
@@ -119,7 +119,7 @@ struct SDevPlan {
 int s_upload_plan(const SPlan &p, SDevPlan *d, cudaStream_t s);
 void s_free_plan(SDevPlan *d);
 int s_launch_plan(const SDevPlan &d, const SArrTable &arrs, const VPtrTable &ptrs,
-                  int slices, int kdrain_steps, int *status, cudaStream_t s,
+                  int slices, int *status, cudaStream_t s,
                   long long *launches);
 size_t s_smem_bytes(int slices, int ntile);
 
