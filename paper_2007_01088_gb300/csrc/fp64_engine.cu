@@ -9,8 +9,15 @@
 // On this GPU the FP64 pipe retires ~2 DFMA per clock per SM (about 1 TFLOP/s
 // for the chip), so an FP64 contraction is compute bound at any practical
 // tile size; the tile is sized for DFMA latency hiding (16 independent
-// accumulators per thread), not for bandwidth.
+// accumulators per thread), not for bandwidth.  What is left to lose is work on
+// padding and idle SMs: a tile skips the row and column groups of 16 (64 in
+// the thin tile) that lie outside its job (nv = 48 fills 9 of the 16 groups of
+// a 64 x 64 tile, a job of 16 columns a quarter of them), and launches of few
+// tiles are split over K when their jobs accumulate (upload_plan).
 #include <cuda_runtime.h>
+
+#include <algorithm>
+#include <vector>
 
 #include "cc3_internal.h"
 #include "fx128.cuh"
@@ -27,8 +34,9 @@ __global__ void __launch_bounds__(256)
 fp64_engine_kernel(const Job *__restrict__ jobs, int njobs,
                    const Term *__restrict__ terms, PtrTable P) {
   static_assert((BM / TM) * (BN / TN) == 256, "256 threads");
-  __shared__ double sA[BK][BM];
-  __shared__ double sB[BK][BN];
+  // one double of padding per row: the loads below store along kk
+  __shared__ double sA[BK][BM + 1];
+  __shared__ double sB[BK][BN + 1];
   const long long cta = blockIdx.x;
   int lo = 0, hi = njobs - 1;
   while (lo < hi) {
@@ -49,6 +57,11 @@ fp64_engine_kernel(const Job *__restrict__ jobs, int njobs,
   constexpr int NTX = BN / TN;
   const int tid = threadIdx.x;
   const int tx = tid % NTX, ty = tid / NTX;
+  // groups of rows / columns of this tile that its job reaches, and the rows
+  // and columns to load for them
+  constexpr int GM = BM / TM, GN = NTX;
+  const int im = min(TM, (M - m0 + GM - 1) / GM), jn = min(TN, (N - n0 + GN - 1) / GN);
+  const int lm = im * GM, ln = jn * GN;
   double acc[TM][TN];
 #pragma unroll
   for (int i = 0; i < TM; ++i)
@@ -67,7 +80,7 @@ fp64_engine_kernel(const Job *__restrict__ jobs, int njobs,
     const double *Bb = P.p[T.B.buf] + T.B.off + (long long)bi * T.B.sb;
     const double *Btb = P.p[T.Bt.buf] + T.Bt.off + (long long)bi * T.Bt.sb;
     for (int k0 = kbeg; k0 < kend; k0 += BK) {
-      for (int e = tid; e < BM * BK; e += 256) {
+      for (int e = tid; e < lm * BK; e += 256) {
         const int mm = e / BK, kk = e % BK;
         const int m = m0 + mm, k = k0 + kk;
         double v = 0.0;
@@ -76,7 +89,7 @@ fp64_engine_kernel(const Job *__restrict__ jobs, int njobs,
                  rowoff(k, T.A.k_in, T.A.sk1, T.A.sk0)];
         sA[kk][mm] = T.A.neg ? -v : v;
       }
-      for (int e = tid; e < BN * BK; e += 256) {
+      for (int e = tid; e < ln * BK; e += 256) {
         const int nn = e / BK, kk = e % BK;
         const int n = n0 + nn, k = k0 + kk;
         double v = 0.0;
@@ -95,17 +108,22 @@ fp64_engine_kernel(const Job *__restrict__ jobs, int njobs,
         sB[kk][nn] = v;
       }
       __syncthreads();
+      const int kn = min(BK, kend - k0);  // the occupied sums are short
 #pragma unroll
       for (int kk = 0; kk < BK; ++kk) {
+        if (kk >= kn) break;
         double a[TM], b[TN];
 #pragma unroll
-        for (int i = 0; i < TM; ++i) a[i] = sA[kk][ty + i * (BM / TM)];
+        for (int i = 0; i < TM; ++i) a[i] = i < im ? sA[kk][ty + i * GM] : 0.0;
 #pragma unroll
-        for (int j = 0; j < TN; ++j) b[j] = sB[kk][tx + j * NTX];
+        for (int j = 0; j < TN; ++j) b[j] = j < jn ? sB[kk][tx + j * GN] : 0.0;
 #pragma unroll
-        for (int i = 0; i < TM; ++i)
+        for (int i = 0; i < TM; ++i) {
+          if (i >= im) break;
 #pragma unroll
-          for (int j = 0; j < TN; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+          for (int j = 0; j < TN; ++j)
+            if (j < jn) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+        }
       }
       __syncthreads();
     }
@@ -144,16 +162,45 @@ fp64_engine_kernel(const Job *__restrict__ jobs, int njobs,
   }
 }
 
+// Splits the accumulating jobs of a launch over K so that its work spreads
+// over FILL tiles (four per SM): a chunk of K is the launch's total K x tiles
+// over FILL, at least 64.  Launches of many tiles keep their jobs whole.
+// sigma1's Cholesky contraction at no=9 nv=81 (an 81 x 9 output over K =
+// 21,870: 3 tiles) took 9 ms on 3 SMs.
+static long long split_small_launch(std::vector<Job> &jobs, const std::vector<Term> &terms) {
+  constexpr double FILL = 608.0;
+  double work = 0.0;
+  auto longest = [&](const Job &j) {
+    int k = 0;
+    for (int t = 0; t < j.nterm; ++t) k = std::max(k, terms[j.term0 + t].K);
+    return k;
+  };
+  for (const Job &j : jobs) {
+    double k = 0.0;
+    for (int t = 0; t < j.nterm; ++t) k += terms[j.term0 + t].K;
+    work += k * j.tiles_m * j.tiles_n * j.batch;
+  }
+  const int chunk = (int)std::min(1e9, std::max(64.0, work / FILL));
+  long long tiles = 0;
+  for (Job &j : jobs) {
+    if (j.mode == EPI_ATOMIC) j.ksplit = std::max(j.ksplit, (longest(j) + chunk - 1) / chunk);
+    j.tile_base = tiles;
+    tiles += (long long)j.batch * j.tiles_m * j.tiles_n * j.ksplit;
+  }
+  return tiles;
+}
+
 int upload_plan(const Plan &p, DevPlan *d, cudaStream_t s) {
   free_plan(d);
-  d->njobs = (int)p.jobs.size();
-  d->tiles = p.tiles;
+  std::vector<Job> jobs = p.jobs;
+  d->njobs = (int)jobs.size();
+  d->tiles = split_small_launch(jobs, p.terms);
   if (d->njobs == 0) return CC3_OK;
-  if (cudaMalloc(&d->jobs, sizeof(Job) * p.jobs.size()) != cudaSuccess)
+  if (cudaMalloc(&d->jobs, sizeof(Job) * jobs.size()) != cudaSuccess)
     return CC3_ERR_OOM;
   if (cudaMalloc(&d->terms, sizeof(Term) * (p.terms.size() + 1)) != cudaSuccess)
     return CC3_ERR_OOM;
-  if (cudaMemcpyAsync(d->jobs, p.jobs.data(), sizeof(Job) * p.jobs.size(),
+  if (cudaMemcpyAsync(d->jobs, jobs.data(), sizeof(Job) * jobs.size(),
                       cudaMemcpyHostToDevice, s) != cudaSuccess)
     return CC3_ERR_CUDA;
   if (!p.terms.empty() &&

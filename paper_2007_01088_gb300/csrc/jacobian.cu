@@ -248,7 +248,9 @@ int dress(cc3_ctx *c, const PtrTable &pt, cudaStream_t s, bool chol = true) {
   p0.jobs[jb].C = o;
   p0.jobs[jb].Ct = o;
   // F^_kc = sum_ld [2 (kc|ld) - (kd|lc)] R^d_l   (one tail column, thin tiles)
-  jb = new_job(pf, 1, no * nv, 1, 0, 1, 1, EPI_STORE);
+  // accumulated from zero, so that its long sum is split over K
+  TRY(launch_zero(pt.p[B_HF], (size_t)nvo, s));
+  jb = new_job(pf, 1, no * nv, 1, 0, 1, 1, EPI_ATOMIC);
   {
     const Opnd Bt = with_k2(op(B_R1, 0, 0, 1), nv, nv);
     const Opnd Aa = with_k2(with_m2(op(B_OVOV, 0, nvo, 1), nv, ovovl), nv, nv);
