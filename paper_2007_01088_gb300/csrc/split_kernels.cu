@@ -516,45 +516,51 @@ __global__ void to_dd_kernel(const double *__restrict__ x, float2 *__restrict__ 
 // + t (vector v, triple t of the batch; slots with t >= ns are idle):
 //   sum over the six terms of P of L1[o0][x] (o1 y|o2 z) + Lt2[o0][o1][x][y] F[o2][z],
 // (o0,o1,o2) = (ijk[s0], ijk[s1], ijk[s2]), (x,y,z) = (v[s0], v[s1], v[s2]),
-// v = (a, b, c).  All factors come as double-float pairs.  Consecutive threads
-// take consecutive b; where b is y, the ovov factor is read as (o2 z|o1 y) and
-// where b is x, the Lt2 factor as Lt2[o1][o0][y][x] (the integrals' pair symmetry
-// and Lt2's pair symmetry), so that every factor that varies along b is read
-// contiguously.
+// v = (a, b, c).  By the pair symmetry of the integrals and of Lt2 the terms
+// are equal in twos (s1 and s2, resp. s0 and s1, swapped), so three of each are
+// formed and doubled.  Bound by the double-float arithmetic (~190 operations
+// per element): a warp takes a row (c, a), so that no element divides its
+// index, with b along the lanes, and every factor that varies along b is read
+// contiguously.  At no=12 nv=120 the six terms of each element, with their
+// 64-bit index divisions, took 11.0 ms per density.
 __global__ void __launch_bounds__(256)
 left_outer_dd_kernel(float2 *__restrict__ W3, const int *__restrict__ tri, int bj, int ns,
                      const float2 *__restrict__ L1, const float2 *__restrict__ Lt,
                      const float2 *__restrict__ ovov, const float2 *__restrict__ F, int no,
                      int nv) {
-  constexpr int P6[6][3] = {{0, 1, 2}, {1, 0, 2}, {2, 1, 0}, {0, 2, 1}, {1, 2, 0}, {2, 0, 1}};
   const int u = blockIdx.y, vec = u / bj, t = u % bj;
   if (t >= ns) return;
-  const int ijk[3] = {tri[3 * t], tri[3 * t + 1], tri[3 * t + 2]};
+  const int i = tri[3 * t], j = tri[3 * t + 1], k = tri[3 * t + 2];
   const long long nv2 = (long long)nv * nv, nv3 = nv2 * nv;
   const long long n1 = (long long)no * nv, nt2 = n1 * no * nv;
   const float2 *l1 = L1 + vec * n1, *lt = Lt + vec * nt2;
   float2 *W = W3 + (long long)u * nv3;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < nv3;
-       e += (long long)gridDim.x * blockDim.x) {
-    const int b = (int)(e % nv), a = (int)((e / nv) % nv), c = (int)(e / nv2);
-    const int v[3] = {a, b, c};
-    dd::df sum = {0.f, 0.f};
-#pragma unroll
-    for (int q = 0; q < 6; ++q) {
-      const int o0 = ijk[P6[q][0]], o1 = ijk[P6[q][1]], o2 = ijk[P6[q][2]];
-      const int x = v[P6[q][0]], y = v[P6[q][1]], z = v[P6[q][2]];
-      const float2 f1 = l1[(long long)o0 * nv + x];
-      const float2 g1 = P6[q][1] == 1 ? ovov[(((long long)o2 * nv + z) * no + o1) * nv + y]
-                                      : ovov[(((long long)o1 * nv + y) * no + o2) * nv + z];
-      const float2 f2 = P6[q][0] == 1 ? lt[(((long long)o1 * no + o0) * nv + y) * nv + x]
-                                      : lt[(((long long)o0 * no + o1) * nv + x) * nv + y];
-      const float2 g2 = F[(long long)o2 * nv + z];
-      sum = dd::add(sum, dd::add(dd::mul(dd::df{f1.x, f1.y}, dd::df{g1.x, g1.y}),
-                                 dd::mul(dd::df{f2.x, f2.y}, dd::df{g2.x, g2.y})));
+  auto val = [](const float2 *p) {
+    const float2 x = *p;
+    return dd::df{x.x, x.y};
+  };
+  const int lane = threadIdx.x & 31, warps = (int)gridDim.x * 8;
+  for (int r = blockIdx.x * 8 + (threadIdx.x >> 5); r < nv * nv; r += warps) {
+    const int c = r / nv, a = r % nv;
+    const dd::df l_ia = val(l1 + (long long)i * nv + a), l_kc = val(l1 + (long long)k * nv + c),
+                 f_ia = val(F + (long long)i * nv + a), f_kc = val(F + (long long)k * nv + c),
+                 g_iakc = val(ovov + (((long long)i * nv + a) * no + k) * nv + c),
+                 t_ikac = val(lt + (((long long)i * no + k) * nv + a) * nv + c);
+    const float2 *l_j = l1 + (long long)j * nv, *f_j = F + (long long)j * nv,
+                 *g_kcj = ovov + (((long long)k * nv + c) * no + j) * nv,
+                 *g_iaj = ovov + (((long long)i * nv + a) * no + j) * nv,
+                 *t_kjc = lt + (((long long)k * no + j) * nv + c) * nv,
+                 *t_ija = lt + (((long long)i * no + j) * nv + a) * nv;
+    float2 *w = W + (long long)r * nv;
+    for (int b = lane; b < nv; b += 32) {
+      dd::df sum = dd::add(dd::mul(l_ia, val(g_kcj + b)), dd::mul(val(l_j + b), g_iakc));
+      sum = dd::add(sum, dd::mul(l_kc, val(g_iaj + b)));
+      sum = dd::add(sum, dd::mul(val(t_kjc + b), f_ia));
+      sum = dd::add(sum, dd::mul(t_ikac, val(f_j + b)));
+      sum = dd::add(sum, dd::mul(val(t_ija + b), f_kc));
+      const dd::df x = dd::add(val(w + b), dd::scale(sum, 2.f));
+      w[b] = make_float2(x.hi, x.lo);
     }
-    const float2 w0 = W[e];
-    const dd::df r = dd::add(dd::df{w0.x, w0.y}, sum);
-    W[e] = make_float2(r.hi, r.lo);
   }
 }
 
@@ -597,8 +603,7 @@ int launch_left_outer_dd(float2 *W3, const int *tri, int bj, int ns, int nslot, 
                          cudaStream_t st) {
   if (nslot <= 0) return CC3_OK;
   if (nslot > 65535) return CC3_FAIL(CC3_ERR_ARG, "left outer products: slots");
-  const long long nv3 = (long long)nv * nv * nv;
-  const int blocks = (int)std::min<long long>((nv3 + 255) / 256, 2048);
+  const int blocks = std::min((nv * nv + 7) / 8, 2048);
   left_outer_dd_kernel<<<dim3(blocks, nslot), 256, 0, st>>>(W3, tri, bj, ns, L1, Lt, ovov, F, no,
                                                             nv);
   return cudaGetLastError() == cudaSuccess ? CC3_OK
