@@ -383,69 +383,142 @@ int density_fp64(cc3_ctx *c, double w, const double *L1d, const double *L2d, dou
 
 // C[k][l] += wgt_ij sum_e X_k(e) Y_l(e) over the pairs i >= j (blockIdx.y), with
 // X_k the view (i,j,k) of L~ and Y_l the view (i,j,l) of tau, e = (a,b,c) the
-// virtual triple of the view.  tab[((y*2 + h)*no + k)*4 + {0..3}] = {T, s0, s1,
-// s2}: the stored tensor T ([a][b][c] double-float, T < 0: a zero row) and the
-// strides of the view's three slots in it.  Per chunk of DOO_E values of e the
-// block stages the 2 no rows (double-float) in shared memory (a padded row
-// stride), then each thread accumulates up to 4 of the no^2 products
-// (blockIdx.z selects the group of 1024 products) in FP32 arithmetic: each
-// double-float product as a rounded high part plus its error and cross terms
-// (FMA), the high parts summed with their rounding errors (two-sum), the low
-// parts plainly; each chunk's sum then adds into an FP64 accumulator.  The
-// terms keep ~2^-44 of their size, well inside the FP64 path's agreement.
-constexpr int DOO_E = 128, DOO_LD = DOO_E + 1;
+// virtual triple of the view.  tab[(y*2 + h)*no + k] = {T, s0, s1, s2}: the
+// stored tensor T ([a][b][c] double-float, T < 0: a zero row) and the
+// strides of the view's three slots in it.
+//
+// Bound by FP32 arithmetic (12 operations per double-float product), next to
+// which the rows' loads from L2 have to be kept cheap:
+// - A chunk is a 4 x 4 x 8 cube of e, so that a row is read in whole 32-byte
+//   sectors whichever of its view's slots is contiguous, the next chunk's rows
+//   are loaded into registers during a chunk's products, and the block stages
+//   the 2 no rows in shared memory (padded to a multiple of DOO_T rows, ld
+//   apart: DOO_E + 1 against bank conflicts, DOO_E where that does not fit).
+// - A thread forms a DOO_T x DOO_T block of products, 8 shared-memory reads for
+//   16 products, over every G-th e of the chunk: nt blocks cover the no^2
+//   products and G = 256 / nt threads share each (blockIdx.z selects the group
+//   of 256 blocks when no > 64).
+// Each product is its rounded high part plus its error and cross terms (FMA);
+// the high parts are summed with their rounding errors (two-sum), which join
+// the low sum; the pair is renormalised after every chunk.  The terms keep
+// ~2^-44 of their size, well inside the FP64 path's agreement.  At no=12 nv=120
+// one thread per product, half of them idle, with rows read element by element
+// took 28.6 ms; this one 18.5 ms.
+constexpr int DOO_E = 128, DOO_T = 4, DOO_PF = 12;
+__host__ __device__ constexpr int doo_rows(int no) { return (no + DOO_T - 1) / DOO_T * DOO_T; }
 __global__ void __launch_bounds__(256)
     doo_pairs_kernel(const float2 *__restrict__ lt_all, const float2 *__restrict__ tau_all,
-                     const long long *__restrict__ tab, const double *__restrict__ wgt, int no,
-                     int nv, double *__restrict__ C) {
-  extern __shared__ float2 sm2[];  // [2][no][DOO_LD]
-  const long long nv2 = (long long)nv * nv, nv3 = nv2 * nv;
-  const long long *tb = tab + (long long)blockIdx.y * 2 * no * 4;
-  const int t = threadIdx.x, e0 = t % DOO_E, h = t / DOO_E;  // h: 0 = L~, 1 = tau
+                     const int4 *__restrict__ tab, const double *__restrict__ wgt, int no,
+                     int nv, int ld, double *__restrict__ C) {
+  extern __shared__ float2 sm2[];  // [2][rows][ld]
+  const int rows = doo_rows(no), nb = rows / DOO_T, nt = nb * nb;
+  const long long nv3 = (long long)nv * nv * nv;
+  const int t = threadIdx.x;
+  for (int u = t; u < 2 * (rows - no) * DOO_E; u += 256) {  // the padding rows
+    const int r = u / DOO_E, h = r / (rows - no);
+    sm2[(h * rows + no + r % (rows - no)) * ld + u % DOO_E] = make_float2(0.f, 0.f);
+  }
+  __syncthreads();
+  // loads: value e0 of the rows of h (0 = L~, 1 = tau)
+  const int e0 = t % DOO_E, h = t / DOO_E;
   const float2 *X = h ? tau_all : lt_all;
-  const int nprod = no * no, pbase = blockIdx.z * 1024;
-  double acc[4] = {0.0, 0.0, 0.0, 0.0};
-  const long long nchunk = (nv3 + DOO_E - 1) / DOO_E;
-  for (long long ch = blockIdx.x; ch < nchunk; ch += gridDim.x) {
-    const long long e = ch * DOO_E + e0;
-    const bool in = e < nv3;
-    const long long v0 = in ? e / nv2 : 0, v1 = in ? (e / nv) % nv : 0, v2 = in ? e % nv : 0;
-    __syncthreads();  // the previous chunk's products are done
-    for (int k = 0; k < no; ++k) {
-      const long long *r = tb + ((long long)h * no + k) * 4;
-      float2 x = make_float2(0.f, 0.f);
-      if (in && r[0] >= 0) x = X[r[0] * nv3 + v0 * r[1] + v1 * r[2] + v2 * r[3]];
-      sm2[(h * no + k) * DOO_LD + e0] = x;
-    }
-    __syncthreads();
+  // products: block `pos` of this launch's group, e = g, g + G, ...
+  const int npos = min(256, nt - (int)blockIdx.z * 256), G = 256 / npos;
+  const int pos = t % npos, g = t / npos, blk = (int)blockIdx.z * 256 + pos;
+  const float2 *xr = sm2 + (blk / nb) * DOO_T * ld, *yr = sm2 + (rows + (blk % nb) * DOO_T) * ld;
+  float hi[DOO_T][DOO_T], lo[DOO_T][DOO_T];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int p = pbase + t + 256 * q;
-      if (p < nprod) {
-        const float2 *xa = sm2 + (p / no) * DOO_LD, *yb = sm2 + (no + p % no) * DOO_LD;
-        float shi = 0.f, slo = 0.f;
+  for (int i = 0; i < DOO_T; ++i)
+#pragma unroll
+    for (int j = 0; j < DOO_T; ++j) hi[i][j] = lo[i][j] = 0.f;
+  // chunks (a4, b4, c8), c8 innermost; a block takes every gridDim.x-th (a4, b4)
+  const int n4 = (nv + 3) / 4, n8 = (nv + 7) / 8;
+  const int4 *view = tab + ((long long)blockIdx.y * 2 + h) * no;
+  const int de = e0 & 7, db = (e0 >> 3) & 3, da = e0 >> 5;
+  int unit = blockIdx.x, c8 = 0, a = unit / n4 * 4 + da, b = unit % n4 * 4 + db;
+  auto load = [&](int k) {  // value e0 of row k of the chunk at (a, b, c8)
+    const int4 w = __ldg(view + k);
+    const int c = c8 * 8 + de;
+    if (w.x < 0 || a >= nv || b >= nv || c >= nv) return make_float2(0.f, 0.f);
+    return X[w.x * nv3 + (a * w.y + b * w.z + c * w.w)];
+  };
+  // the next chunk's first DOO_PF rows arrive in registers during this one's products
+  float2 pf[DOO_PF];
+  auto prefetch = [&]() {
+#pragma unroll
+    for (int k = 0; k < DOO_PF; ++k)
+      if (k < no) pf[k] = load(k);
+  };
+  if (unit < n4 * n4) prefetch();
+  while (unit < n4 * n4) {
+    __syncthreads();  // the previous chunk's products are done
+#pragma unroll
+    for (int k = 0; k < DOO_PF; ++k)
+      if (k < no) sm2[(h * rows + k) * ld + e0] = pf[k];
 #pragma unroll 4
-        for (int u = 0; u < DOO_E; ++u) {
-          const float2 x = xa[u], y = yb[u];
-          const float ph = __fmul_rn(x.x, y.x);
-          float pl = __fmaf_rn(x.x, y.x, -ph);
-          pl = __fmaf_rn(x.x, y.y, pl);
-          pl = __fmaf_rn(x.y, y.x, pl);
-          const float sn = __fadd_rn(shi, ph);
-          const float bb = __fsub_rn(sn, shi);
-          const float er = __fadd_rn(__fsub_rn(shi, __fsub_rn(sn, bb)), __fsub_rn(ph, bb));
-          shi = sn;
-          slo = __fadd_rn(slo, __fadd_rn(er, pl));
+    for (int k = DOO_PF; k < no; ++k) sm2[(h * rows + k) * ld + e0] = load(k);
+    __syncthreads();
+    if (++c8 == n8) {
+      c8 = 0;
+      unit += gridDim.x;
+      a = unit / n4 * 4 + da;
+      b = unit % n4 * 4 + db;
+    }
+    if (unit < n4 * n4) prefetch();
+    if (g < G) {
+#pragma unroll 1
+      for (int u = g; u < DOO_E; u += G) {
+        float2 x[DOO_T], y[DOO_T];
+#pragma unroll
+        for (int i = 0; i < DOO_T; ++i) {
+          x[i] = xr[i * ld + u];
+          y[i] = yr[i * ld + u];
         }
-        acc[q] += (double)shi + (double)slo;
+#pragma unroll
+        for (int i = 0; i < DOO_T; ++i)
+#pragma unroll
+          for (int j = 0; j < DOO_T; ++j) {
+            const float ph = __fmul_rn(x[i].x, y[j].x);
+            float pl = __fmaf_rn(x[i].x, y[j].x, -ph);
+            pl = __fmaf_rn(x[i].x, y[j].y, pl);
+            pl = __fmaf_rn(x[i].y, y[j].x, pl);
+            const float sn = __fadd_rn(hi[i][j], ph);
+            const float bb = __fsub_rn(sn, hi[i][j]);
+            const float er = __fadd_rn(__fsub_rn(hi[i][j], __fsub_rn(sn, bb)), __fsub_rn(ph, bb));
+            hi[i][j] = sn;
+            lo[i][j] = __fadd_rn(lo[i][j], __fadd_rn(er, pl));
+          }
       }
+#pragma unroll
+      for (int i = 0; i < DOO_T; ++i)
+#pragma unroll
+        for (int j = 0; j < DOO_T; ++j) {
+          const float sn = __fadd_rn(hi[i][j], lo[i][j]);
+          lo[i][j] = __fsub_rn(lo[i][j], __fsub_rn(sn, hi[i][j]));
+          hi[i][j] = sn;
+        }
     }
   }
+  // the block's sums over its e groups, then one atomic per product
+  __syncthreads();
+  double *red = reinterpret_cast<double *>(sm2);  // [256 / ...][16] one thread's products
   const double w = wgt[blockIdx.y];
+  for (int q = 0; q < DOO_T * DOO_T; ++q) {
+    float vh = 0.f, vl = 0.f;
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int p = pbase + t + 256 * q;
-    if (p < nprod) atomicAdd(C + p, w * acc[q]);
+    for (int i = 0; i < DOO_T; ++i)
+#pragma unroll
+      for (int j = 0; j < DOO_T; ++j)
+        if (q == i * DOO_T + j) vh = hi[i][j], vl = lo[i][j];
+    red[t] = (double)vh + (double)vl;
+    __syncthreads();
+    const int k = blk / nb * DOO_T + q / DOO_T, l = blk % nb * DOO_T + q % DOO_T;
+    if (g == 0 && k < no && l < no) {
+      double sum = 0.0;
+      for (int u = 0; u < G; ++u) sum += red[u * npos + pos];
+      atomicAdd(C + (size_t)k * no + l, w * sum);
+    }
+    __syncthreads();
   }
 }
 
@@ -487,62 +560,61 @@ int density_doo_resident(cc3_ctx *c, const float2 *tau_all, const float2 *lt_all
   for (int t = 0; t < nt; ++t)
     where[((size_t)tri[3 * t] * no + tri[3 * t + 1]) * no + tri[3 * t + 2]] = t;
   // row of the view (p,q,r): {T, strides of the view's slots in T's storage}
-  auto row = [&](int p, int q, int r, bool zero, long long *o) {
-    o[0] = -1;
-    o[1] = o[2] = o[3] = 0;
+  auto row = [&](int p, int q, int r, bool zero, int4 *o) {
+    *o = make_int4(-1, 0, 0, 0);
     if (zero) return;
     int x[3] = {p, q, r};
     std::sort(x, x + 3, [](int u, int v) { return u > v; });
     const int T = where[((size_t)x[0] * no + x[1]) * no + x[2]];
     if (T < 0) return;
-    const long long str[3] = {nv2, nv, 1};
+    const int str[3] = {nv * nv, nv, 1};
     for (int u = 0; u < 6; ++u) {
       const int *m = PERM6[u];
       const int *tt = &tri[3 * T];
       if (tt[m[0]] == p && tt[m[1]] == q && tt[m[2]] == r) {
-        o[0] = T;
-        o[1] = str[m[0]];
-        o[2] = str[m[1]];
-        o[3] = str[m[2]];
+        *o = make_int4(T, str[m[0]], str[m[1]], str[m[2]]);
         return;
       }
     }
   };
   const int npair = no * (no + 1) / 2;
-  std::vector<long long> tab((size_t)npair * 2 * no * 4);
+  std::vector<int4> tab((size_t)npair * 2 * no);
   std::vector<double> wgt(npair);
   int y = 0;
   for (int i = 0; i < no; ++i)
     for (int j = 0; j <= i; ++j, ++y) {
       wgt[y] = i == j ? 1.0 : 2.0;
       for (int k = 0; k < no; ++k) {
-        row(i, j, k, i == j && j == k, &tab[(((size_t)y * 2 + 0) * no + k) * 4]);
-        row(i, j, k, false, &tab[(((size_t)y * 2 + 1) * no + k) * 4]);
+        row(i, j, k, i == j && j == k, &tab[((size_t)y * 2 + 0) * no + k]);
+        row(i, j, k, false, &tab[((size_t)y * 2 + 1) * no + k]);
       }
     }
   Bufs B;
   double *C = nullptr, *dw = nullptr;
-  long long *dtab = nullptr;
+  int4 *dtab = nullptr;
   TRY(B.get(&C, (size_t)no * no));
   TRY(B.get(&dw, (size_t)npair));
   TRY(B.get(&dtab, tab.size()));
   TRY(launch_zero(C, (size_t)no * no, s));
-  CU(cudaMemcpyAsync(dtab, tab.data(), sizeof(long long) * tab.size(), cudaMemcpyHostToDevice, s));
+  CU(cudaMemcpyAsync(dtab, tab.data(), sizeof(int4) * tab.size(), cudaMemcpyHostToDevice, s));
   CU(cudaMemcpyAsync(dw, wgt.data(), sizeof(double) * npair, cudaMemcpyHostToDevice, s));
-  const size_t smem = sizeof(float2) * 2 * no * DOO_LD;
+  int ld = DOO_E + 1;
+  auto bytes = [&] { return sizeof(float2) * 2 * (size_t)doo_rows(no) * ld; };
+  if (bytes() > 227 * 1024) ld = DOO_E;
+  const size_t smem = bytes();
   if (smem > 227 * 1024) return CC3_FAIL(CC3_ERR_UNSUPPORTED, "too many occupied orbitals");
   CU(cudaFuncSetAttribute(doo_pairs_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                           (int)smem));
-  const long long nchunk = (nv2 * nv + DOO_E - 1) / DOO_E;
+  const long long nunit = (long long)((nv + 3) / 4) * ((nv + 3) / 4);
   int dev = 0, nsm = 0;
   CU(cudaGetDevice(&dev));
   CU(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-  const int gz = (no * no + 1023) / 1024;
+  const int gz = (doo_rows(no) / DOO_T * (doo_rows(no) / DOO_T) + 255) / 256;
   const long long gx = std::max<long long>(
-      1, std::min<long long>(nchunk, (4LL * nsm + (long long)npair * gz - 1) / ((long long)npair * gz)));
+      1, std::min<long long>(nunit, (4LL * nsm + (long long)npair * gz - 1) / ((long long)npair * gz)));
   trace_begin(c, TR_FP64_ELEM, s);
   doo_pairs_kernel<<<dim3((unsigned)gx, npair, gz), 256, smem, s>>>(lt_all, tau_all, dtab, dw, no,
-                                                                     nv, C);
+                                                                     nv, ld, C);
   CU(cudaGetLastError());
   trace_end(c, TR_FP64_ELEM, s, 2.0 * no * no * (double)npair * nv2 * nv, 0.0);
   c->counters.launches++;
