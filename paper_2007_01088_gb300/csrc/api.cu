@@ -55,7 +55,7 @@ cudaMemcpyKind out_kind(const cc3_ctx *c) {
 int dalloc(double **p, size_t n) {
   *p = nullptr;
   if (n == 0) n = 1;
-  if (cudaMalloc(p, n * sizeof(double)) != cudaSuccess) {
+  if (dev_malloc(p, n * sizeof(double)) != cudaSuccess) {
     cudaGetLastError();
     return CC3_ERR_OOM;
   }
@@ -170,8 +170,8 @@ int choose_batch(cc3_ctx *c) { return batch_for(c->nv, c->ntri); }
 
 int alloc_workspace(cc3_ctx *c) {
   const size_t nv3 = (size_t)c->nv * c->nv * c->nv;
-  if (c->ws_w) cudaFree(c->ws_w);
-  if (c->ws_tt) cudaFree(c->ws_tt);
+  if (c->ws_w) dev_free(c->ws_w);
+  if (c->ws_tt) dev_free(c->ws_tt);
   c->ws_w = c->ws_tt = nullptr;
   TRY(dalloc(&c->ws_w, nv3 * c->batch));
   TRY(dalloc(&c->ws_tt, nv3 * c->batch));
@@ -336,11 +336,21 @@ const char *cc3_strerror(int status) {
 
 void cc3_ctx_destroy(cc3_ctx *c) {
   if (!c) return;
+  cudaDeviceSynchronize();  // the context's last call may still run, on any stream
+  cudaGetLastError();
+  ctx_release(c, nullptr);
+}
+
+}  // extern "C"
+
+namespace cc3 {
+void ctx_release(cc3_ctx *c, cudaStream_t s) {
+  StreamScope scope(s);
   CtxExtra *X = extra(c);
   if (X) {
     free_omega_plans(X->omega);
-    if (X->escr) cudaFree(X->escr);
-    if (X->om2tmp) cudaFree(X->om2tmp);
+    if (X->escr) dev_free(X->escr);
+    if (X->om2tmp) dev_free(X->om2tmp);
     delete X;
   }
   split_destroy(c);
@@ -352,14 +362,14 @@ void cc3_ctx_destroy(cc3_ctx *c) {
                     c->ws_tt, c->ws_tt2, c->omt, c->om1, c->Zv, c->Zo, c->R2,
                     c->hvvvo, c->hoovo, c->hF, c->rhot, c->rho1};
   for (double *p : bufs)
-    if (p) cudaFree(p);
-  if (c->status) cudaFree(c->status);
-  if (c->omt_fx) cudaFree(c->omt_fx);
-  if (c->om1_fx) cudaFree(c->om1_fx);
+    if (p) dev_free(p);
+  if (c->status) dev_free(c->status);
+  if (c->omt_fx) dev_free(c->omt_fx);
+  if (c->om1_fx) dev_free(c->om1_fx);
   delete c;
+  dev_ctx_gone();
 }
-
-}  // extern "C"
+}  // namespace cc3
 
 // Context creation shared by the symmetric and the general entry points:
 // g_oovo and g_vvov are null for symmetric integrals (oovo is then the
@@ -382,6 +392,8 @@ static int ctx_create_impl(cc3_ctx **out, int no, int nv, const double *eps_o,
   if (!c) return CC3_ERR_OOM;
   c->ext = new (std::nothrow) CtxExtra();
   if (!c->ext) { delete c; return CC3_ERR_OOM; }
+  StreamScope scope(s);
+  dev_ctx_born();
   c->no = no;
   c->nv = nv;
   c->naux = chol_L ? naux : 0;
@@ -422,14 +434,14 @@ static int ctx_create_impl(cc3_ctx **out, int no, int nv, const double *eps_o,
   if ((rc = dalloc(&c->omt, nt2)) != CC3_OK) goto fail;
   if ((rc = dalloc(&c->om1, (size_t)no * nv)) != CC3_OK) goto fail;
   if (flags & CC3_DETERMINISTIC) {
-    if (cudaMalloc(&c->omt_fx, sizeof(unsigned long long) * 2 * nt2) != cudaSuccess ||
-        cudaMalloc(&c->om1_fx, sizeof(unsigned long long) * 2 * (size_t)no * nv) != cudaSuccess) {
+    if (dev_malloc(&c->omt_fx, sizeof(unsigned long long) * 2 * nt2) != cudaSuccess ||
+        dev_malloc(&c->om1_fx, sizeof(unsigned long long) * 2 * (size_t)no * nv) != cudaSuccess) {
       rc = CC3_ERR_OOM;
       goto fail;
     }
   }
   if ((rc = dalloc(&extra(c)->escr, 257)) != CC3_OK) goto fail;
-  if (cudaMalloc(&c->status, sizeof(int) * 4) != cudaSuccess) { rc = CC3_ERR_OOM; goto fail; }
+  if (dev_malloc(&c->status, sizeof(int) * 4) != cudaSuccess) { rc = CC3_ERR_OOM; goto fail; }
   if (cudaMemsetAsync(c->status, 0, sizeof(int) * 4, s) != cudaSuccess) { rc = CC3_ERR_CUDA; goto fail; }
   default_triples(c);
   c->batch = choose_batch(c);
@@ -450,8 +462,9 @@ static int ctx_create_impl(cc3_ctx **out, int no, int nv, const double *eps_o,
   *out = c;
   return CC3_OK;
 fail:
+  cudaStreamSynchronize(s);
   cudaGetLastError();
-  cc3_ctx_destroy(c);
+  ctx_release(c, s);
   return rc;
 }
 
@@ -490,10 +503,15 @@ int cc3_ctx_set_triples(cc3_ctx *c, int ntri, const int *ijk) {
     c->tri_host = v;
     c->ntri = ntri;
   }
+  // the buffers freed below may be in use by an earlier call, on any stream
+  cudaDeviceSynchronize();
+  cudaGetLastError();
+  StreamScope scope(nullptr);
   const int nb = choose_batch(c);
   if (nb != c->batch) {
     c->batch = nb;
     TRY(alloc_workspace(c));
+    CU(cudaStreamSynchronize(nullptr));  // usable on every stream
   }
   extra(c)->omega.valid = false;
   split_invalidate(c);
@@ -553,6 +571,7 @@ int cc3_ctx_autotune(cc3_ctx *c, void *cuda_stream, int *ksteps_per_tile, int *n
   if (!c) return CC3_ERR_ARG;
   std::lock_guard<std::mutex> lk(c->mu);
   if (c->ntri == 0) return CC3_OK;
+  StreamScope scope((cudaStream_t)cuda_stream);
   return split_autotune(c, (cudaStream_t)cuda_stream, ksteps_per_tile, ntile_w);
 }
 
@@ -564,6 +583,9 @@ int cc3_ctx_get_tuning(cc3_ctx *c, int *ksteps_per_tile, int *ntile_w) {
 
 int cc3_ctx_set_slices(cc3_ctx *c, int slices) {
   if (!c || slices < 3 || slices > 7) return CC3_ERR_ARG;
+  cudaDeviceSynchronize();  // as above: the split state is freed
+  cudaGetLastError();
+  StreamScope scope(nullptr);
   c->slices = slices;
   split_invalidate(c);
   return CC3_OK;
@@ -640,6 +662,7 @@ int cc3_omega_triples(cc3_ctx *c, cc3_prec prec, double *Omega1,
   if (prec == CC3_SPLIT_INT8) return CC3_ERR_UNSUPPORTED;
   std::lock_guard<std::mutex> lk(c->mu);
   cudaStream_t s = (cudaStream_t)cuda_stream;
+  StreamScope scope(s);
   const int no = c->no, nv = c->nv;
   const size_t nt2 = (size_t)no * no * nv * nv;
   c->counters = cc3_counters{};

@@ -160,6 +160,33 @@ int record_error(int status, const char *file, int line, const char *what);
 #define CC3_FAIL(status, what) ::cc3::record_error((status), __FILE__, __LINE__, (what))
 
 // engine (fp64_engine.cu)
+// ---- device memory (memory.cu) ----
+// The stream that this thread's allocations and frees are ordered on, for the
+// lifetime of the object: every entry point that takes a stream sets it.
+struct StreamScope {
+  explicit StreamScope(cudaStream_t s);
+  ~StreamScope();
+  StreamScope(const StreamScope &) = delete;
+  StreamScope &operator=(const StreamScope &) = delete;
+
+ private:
+  cudaStream_t prev;
+};
+cudaError_t dev_malloc_bytes(void **p, size_t n);
+template <class T>
+cudaError_t dev_malloc(T **p, size_t n) {
+  return dev_malloc_bytes(reinterpret_cast<void **>(p), n);
+}
+void dev_free(void *p);  // p may be null; its last use must precede on the stream
+size_t dev_mem_free();   // free device bytes, with what the pool holds unused
+void dev_ctx_born();
+void dev_ctx_gone();
+void dev_give_back();  // returns the pool's unused memory if no context is left
+// Copies a host table to the device, ordered on s; src may be reused on return.
+int dev_upload(void *dst, const void *src, size_t n, cudaStream_t s);
+// Frees a context whose work is complete, or ordered before on s.
+void ctx_release(cc3_ctx *c, cudaStream_t s);
+
 int upload_plan(const Plan &p, DevPlan *d, cudaStream_t s);
 void free_plan(DevPlan *d);
 int launch_plan(const DevPlan &d, const PtrTable &ptrs, cudaStream_t s,

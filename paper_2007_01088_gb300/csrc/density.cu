@@ -174,12 +174,12 @@ struct Bufs {
   std::vector<void *> p;
   ~Bufs() {
     for (void *x : p)
-      if (x) cudaFree(x);
+      if (x) dev_free(x);
   }
   template <class T>
   int get(T **out, size_t n) {
     *out = nullptr;
-    if (cudaMalloc(out, sizeof(T) * (n ? n : 1)) != cudaSuccess) {
+    if (dev_malloc(out, sizeof(T) * (n ? n : 1)) != cudaSuccess) {
       cudaGetLastError();
       return CC3_FAIL(CC3_ERR_OOM, "density workspace");
     }
@@ -667,6 +667,7 @@ extern "C" int cc3_density_triples(cc3_ctx *c, cc3_prec prec, double omega, cons
                       "the frequency lies within CC3_DENOM_MIN of a triples denominator");
   }
   cudaStream_t s = (cudaStream_t)cuda_stream;
+  StreamScope scope(s);
   const size_t n1 = (size_t)no * nv, nt2 = n1 * no * nv, noo = (size_t)no * no,
                nvv = (size_t)nv * nv;
   c->counters = cc3_counters{};
@@ -681,7 +682,7 @@ extern "C" int cc3_density_triples(cc3_ctx *c, cc3_prec prec, double omega, cons
          *dov = D_ov, *dvv = D_vv;
   std::vector<double *> tmp;
   auto mk = [&](double **p, size_t n) {
-    if (cudaMalloc(p, sizeof(double) * (n ? n : 1)) != cudaSuccess) {
+    if (dev_malloc(p, sizeof(double) * (n ? n : 1)) != cudaSuccess) {
       cudaGetLastError();
       return false;
     }
@@ -708,7 +709,7 @@ extern "C" int cc3_density_triples(cc3_ctx *c, cc3_prec prec, double omega, cons
       rc = CC3_FAIL(CC3_ERR_CUDA, "density download");
   }
   cudaStreamSynchronize(s);
-  for (double *p : tmp) cudaFree(p);
+  for (double *p : tmp) dev_free(p);
   if (rc == CC3_OK) rc = trace_collect(c, s);
   return rc;
 }

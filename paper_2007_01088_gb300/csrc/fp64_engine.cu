@@ -17,6 +17,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cstring>
 #include <vector>
 
 #include "cc3_internal.h"
@@ -196,25 +197,23 @@ int upload_plan(const Plan &p, DevPlan *d, cudaStream_t s) {
   d->njobs = (int)jobs.size();
   d->tiles = split_small_launch(jobs, p.terms);
   if (d->njobs == 0) return CC3_OK;
-  if (cudaMalloc(&d->jobs, sizeof(Job) * jobs.size()) != cudaSuccess)
+  // one allocation: the jobs, then the terms
+  const size_t jb = (sizeof(Job) * jobs.size() + 15) / 16 * 16, tb = sizeof(Term) * p.terms.size();
+  std::vector<char> host(jb + tb);
+  std::memcpy(host.data(), jobs.data(), sizeof(Job) * jobs.size());
+  if (tb) std::memcpy(host.data() + jb, p.terms.data(), tb);
+  char *base = nullptr;
+  if (dev_malloc(&base, jb + tb + sizeof(Term)) != cudaSuccess) {
+    cudaGetLastError();
     return CC3_ERR_OOM;
-  if (cudaMalloc(&d->terms, sizeof(Term) * (p.terms.size() + 1)) != cudaSuccess)
-    return CC3_ERR_OOM;
-  if (cudaMemcpyAsync(d->jobs, jobs.data(), sizeof(Job) * jobs.size(),
-                      cudaMemcpyHostToDevice, s) != cudaSuccess)
-    return CC3_ERR_CUDA;
-  if (!p.terms.empty() &&
-      cudaMemcpyAsync(d->terms, p.terms.data(), sizeof(Term) * p.terms.size(),
-                      cudaMemcpyHostToDevice, s) != cudaSuccess)
-    return CC3_ERR_CUDA;
-  // the host vectors may die after return: make the copies complete
-  if (cudaStreamSynchronize(s) != cudaSuccess) return CC3_ERR_CUDA;
-  return CC3_OK;
+  }
+  d->jobs = reinterpret_cast<Job *>(base);
+  d->terms = reinterpret_cast<Term *>(base + jb);
+  return dev_upload(base, host.data(), host.size(), s);
 }
 
 void free_plan(DevPlan *d) {
-  if (d->jobs) cudaFree(d->jobs);
-  if (d->terms) cudaFree(d->terms);
+  if (d->jobs) dev_free(d->jobs);
   d->jobs = nullptr;
   d->terms = nullptr;
   d->njobs = 0;

@@ -56,7 +56,7 @@ JacState *jst(cc3_ctx *c) {
 
 int dalloc(double **p, size_t n) {
   *p = nullptr;
-  if (cudaMalloc(p, sizeof(double) * (n ? n : 1)) != cudaSuccess) {
+  if (dev_malloc(p, sizeof(double) * (n ? n : 1)) != cudaSuccess) {
     cudaGetLastError();
     return CC3_FAIL(CC3_ERR_OOM, "Jacobian workspace");
   }
@@ -77,7 +77,6 @@ int run_plan(cc3_ctx *c, const Plan &p, int kind, const PtrTable &pt, cudaStream
   const int rc = launch_plan(d, pt, s, &c->counters.launches);
   trace_end(c, TR_FP64_ENGINE, s, f, 0.0);
   c->counters.executed_flop += f;
-  cudaStreamSynchronize(s);  // the tables are freed next
   free_plan(&d);
   return rc;
 }
@@ -459,8 +458,8 @@ int jacobian_fp64(cc3_ctx *c, int nvec, const double *w, const double *R1d, cons
   const int bj = std::max(1, std::min(c->batch, c->batch / nvec));
   const int nslot = bj * nvec;
   if (J->wsb != nslot) {
-    if (J->wsWR) cudaFree(J->wsWR);
-    if (J->wsTTR) cudaFree(J->wsTTR);
+    if (J->wsWR) dev_free(J->wsWR);
+    if (J->wsTTR) dev_free(J->wsTTR);
     J->wsWR = J->wsTTR = nullptr;
     J->wsb = 0;
     TRY(dalloc(&J->wsWR, (size_t)nv3 * nslot));
@@ -475,7 +474,7 @@ int jacobian_fp64(cc3_ctx *c, int nvec, const double *w, const double *R1d, cons
     double **p[6];
     ~Guard() {
       for (double **q : p)
-        if (*q) cudaFree(*q);
+        if (*q) dev_free(*q);
     }
   } guard{{&hv, &ho, &hf, &mj, &rt, &r1a}};
   TRY(dalloc(&hv, (size_t)nvvvo * nvec));
@@ -593,7 +592,7 @@ void jacobian_destroy(cc3_ctx *c) {
   if (!J) return;
   double *b[] = {J->oooo, J->oovv, J->Zv, J->Zo, J->wsWR, J->wsTTR};
   for (double *p : b)
-    if (p) cudaFree(p);
+    if (p) dev_free(p);
   delete J;
   c->jac = nullptr;
 }
@@ -629,6 +628,7 @@ extern "C" int cc3_jacobian_triples(cc3_ctx *c, cc3_prec prec, int nvec, const d
                                      "denominator");
   }
   cudaStream_t s = (cudaStream_t)cuda_stream;
+  StreamScope scope(s);
   const int no = c->no, nv = c->nv;
   const size_t n1 = (size_t)no * nv, nt2 = (size_t)no * no * nv * nv;
   long long wsum = 0;
@@ -644,7 +644,7 @@ extern "C" int cc3_jacobian_triples(cc3_ctx *c, cc3_prec prec, int nvec, const d
          *dr2 = rho2;
   std::vector<double *> tmp;
   auto mk = [&](double **p, size_t n) {
-    if (cudaMalloc(p, sizeof(double) * n) != cudaSuccess) {
+    if (dev_malloc(p, sizeof(double) * n) != cudaSuccess) {
       cudaGetLastError();
       return false;
     }
@@ -678,7 +678,7 @@ extern "C" int cc3_jacobian_triples(cc3_ctx *c, cc3_prec prec, int nvec, const d
       rc = CC3_FAIL(CC3_ERR_CUDA, "Jacobian download");
   }
   cudaStreamSynchronize(s);
-  for (double *p : tmp) cudaFree(p);
+  for (double *p : tmp) dev_free(p);
   if (rc == CC3_OK) rc = trace_collect(c, s);
   return rc;
 }

@@ -99,12 +99,12 @@ struct Bufs {
   std::vector<void *> p;
   ~Bufs() {
     for (void *x : p)
-      if (x) cudaFree(x);
+      if (x) dev_free(x);
   }
   template <class T>
   int get(T **out, size_t n) {
     *out = nullptr;
-    if (cudaMalloc(out, sizeof(T) * (n ? n : 1)) != cudaSuccess) {
+    if (dev_malloc(out, sizeof(T) * (n ? n : 1)) != cudaSuccess) {
       cudaGetLastError();
       return CC3_FAIL(CC3_ERR_OOM, "left Jacobian workspace");
     }
@@ -424,6 +424,7 @@ extern "C" int cc3_left_jacobian_triples(cc3_ctx *c, cc3_prec prec, int nvec,
                                      "denominator");
   }
   cudaStream_t s = (cudaStream_t)cuda_stream;
+  StreamScope scope(s);
   const int no = c->no, nv = c->nv;
   const size_t n1 = (size_t)no * nv, nt2 = n1 * no * nv;
   long long wsum = 0;
@@ -439,7 +440,7 @@ extern "C" int cc3_left_jacobian_triples(cc3_ctx *c, cc3_prec prec, int nvec,
          *ds2 = sigma2;
   std::vector<double *> tmp;
   auto mk = [&](double **p, size_t n) {
-    if (cudaMalloc(p, sizeof(double) * n) != cudaSuccess) {
+    if (dev_malloc(p, sizeof(double) * n) != cudaSuccess) {
       cudaGetLastError();
       return false;
     }
@@ -477,7 +478,7 @@ extern "C" int cc3_left_jacobian_triples(cc3_ctx *c, cc3_prec prec, int nvec,
       rc = CC3_FAIL(CC3_ERR_CUDA, "left Jacobian download");
   }
   cudaStreamSynchronize(s);
-  for (double *p : tmp) cudaFree(p);
+  for (double *p : tmp) dev_free(p);
   if (rc == CC3_OK) rc = trace_collect(c, s);
   return rc;
 }

@@ -1,0 +1,192 @@
+// Device memory of the library: stream-ordered allocations from a private pool
+// of the device, and host-to-device copies of small tables.
+//
+// A Jacobian, left transformation or density call allocates a few dozen
+// temporaries and a few tables per batch of triples, and a serving slot builds
+// a context per request.  cudaMalloc and cudaFree cost 10-40 us each, and
+// cudaFree waits for the whole device, which made the serving slots take turns
+// (a burst of six small requests on four slots: 1630 calls, 59 ms, of which the
+// device worked 26 ms).  From the pool both cost 1-2 us and order themselves on
+// the calling stream.
+//
+// The pool keeps at most 1/16 of the device's memory while a context exists and
+// at most KEEP bytes after the last one is gone; cc3_serve_stop gives back the
+// rest as well when no context is left.  A failed allocation first returns all
+// that is unused and tries again.  dev_mem_free counts what the pool holds
+// unused as free.
+#include <cuda_runtime.h>
+
+#include <atomic>
+#include <cstring>
+#include <mutex>
+#include <vector>
+
+#include "cc3_internal.h"
+
+namespace cc3 {
+namespace {
+constexpr size_t KEEP = 1ull << 30;
+constexpr int MAX_DEV = 64;
+
+std::mutex g_mu;
+cudaMemPool_t g_pool[MAX_DEV] = {nullptr};
+bool g_tried[MAX_DEV] = {false};
+std::atomic<int> g_live{0};
+thread_local cudaStream_t t_stream = nullptr;
+
+// The device's pool; null where pools are not supported (then cudaMalloc serves).
+cudaMemPool_t pool_of(int dev) {
+  if (dev < 0 || dev >= MAX_DEV) return nullptr;
+  std::lock_guard<std::mutex> lk(g_mu);
+  if (!g_tried[dev]) {
+    g_tried[dev] = true;
+    int ok = 0;
+    cudaDeviceGetAttribute(&ok, cudaDevAttrMemoryPoolsSupported, dev);
+    cudaMemPoolProps p;
+    std::memset(&p, 0, sizeof(p));
+    p.allocType = cudaMemAllocationTypePinned;
+    p.handleTypes = cudaMemHandleTypeNone;
+    p.location.type = cudaMemLocationTypeDevice;
+    p.location.id = dev;
+    cudaMemPool_t pool = nullptr;
+    size_t fr = 0, tot = 0;
+    if (ok && cudaMemPoolCreate(&pool, &p) == cudaSuccess) {
+      cudaMemGetInfo(&fr, &tot);
+      unsigned long long keep = tot / 16;
+      if (cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) == cudaSuccess)
+        g_pool[dev] = pool;
+      else
+        cudaMemPoolDestroy(pool);
+    }
+    cudaGetLastError();
+  }
+  return g_pool[dev];
+}
+
+int device() {
+  int dev = -1;
+  cudaGetDevice(&dev);
+  return dev;
+}
+
+// Pinned buffers for table uploads: taken when the copy out of them is done.
+struct HostBuf {
+  char *p;
+  cudaEvent_t done;
+  int dev;
+};
+constexpr size_t HOST_BYTES = 256 << 10;
+constexpr int HOST_MAX = 64;
+std::mutex g_host_mu;
+std::vector<HostBuf> g_host;  // idle or with a copy in flight (see done)
+int g_host_made = 0;
+
+bool host_take(HostBuf *out, int dev) {
+  std::lock_guard<std::mutex> lk(g_host_mu);
+  for (size_t i = 0; i < g_host.size(); ++i)
+    if (g_host[i].dev == dev && cudaEventQuery(g_host[i].done) == cudaSuccess) {
+      *out = g_host[i];
+      g_host[i] = g_host.back();
+      g_host.pop_back();
+      return true;
+    }
+  cudaGetLastError();  // cudaErrorNotReady of the queries
+  if (g_host_made >= HOST_MAX) return false;
+  HostBuf b{nullptr, nullptr, dev};
+  if (cudaMallocHost(&b.p, HOST_BYTES) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  if (cudaEventCreateWithFlags(&b.done, cudaEventDisableTiming) != cudaSuccess) {
+    cudaGetLastError();
+    cudaFreeHost(b.p);
+    return false;
+  }
+  ++g_host_made;
+  *out = b;
+  return true;
+}
+}  // namespace
+
+StreamScope::StreamScope(cudaStream_t s) : prev(t_stream) { t_stream = s; }
+StreamScope::~StreamScope() { t_stream = prev; }
+
+cudaError_t dev_malloc_bytes(void **p, size_t n) {
+  *p = nullptr;
+  cudaMemPool_t pool = pool_of(device());
+  if (!pool) return cudaMalloc(p, n);
+  // no allocation becomes part of a caller's graph
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  cudaError_t e = cudaStreamIsCapturing(t_stream, &cap);
+  if (e != cudaSuccess) return e;
+  if (cap != cudaStreamCaptureStatusNone) return cudaErrorStreamCaptureUnsupported;
+  e = cudaMallocFromPoolAsync(p, n, pool, t_stream);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    cudaDeviceSynchronize();
+    cudaMemPoolTrimTo(pool, 0);
+    e = cudaMallocFromPoolAsync(p, n, pool, t_stream);
+  }
+  if (e != cudaSuccess) *p = nullptr;
+  return e;
+}
+
+void dev_free(void *p) {
+  if (!p) return;
+  if (!pool_of(device())) {
+    cudaFree(p);
+  } else if (cudaFreeAsync(p, t_stream) != cudaSuccess) {
+    cudaGetLastError();
+    cudaFree(p);
+  }
+}
+
+size_t dev_mem_free() {
+  size_t fr = 0, tot = 0;
+  if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  if (cudaMemPool_t pool = pool_of(device())) {
+    unsigned long long held = 0, used = 0;
+    if (cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &held) == cudaSuccess &&
+        cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess &&
+        held > used)
+      fr += (size_t)(held - used);
+  }
+  return fr;
+}
+
+void dev_ctx_born() { ++g_live; }
+void dev_ctx_gone() {
+  if (--g_live > 0) return;
+  if (cudaMemPool_t pool = pool_of(device())) cudaMemPoolTrimTo(pool, KEEP);
+  cudaGetLastError();
+}
+void dev_give_back() {
+  if (g_live > 0) return;
+  if (cudaMemPool_t pool = pool_of(device())) cudaMemPoolTrimTo(pool, 0);
+  cudaGetLastError();
+}
+
+int dev_upload(void *dst, const void *src, size_t n, cudaStream_t s) {
+  if (n == 0) return CC3_OK;
+  HostBuf b;
+  if (n <= HOST_BYTES && host_take(&b, device())) {
+    std::memcpy(b.p, src, n);
+    cudaError_t e = cudaMemcpyAsync(dst, b.p, n, cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaEventRecord(b.done, s);
+    if (e != cudaSuccess) cudaStreamSynchronize(s);  // no copy out of the buffer is left
+    {
+      std::lock_guard<std::mutex> lk(g_host_mu);
+      g_host.push_back(b);
+    }
+    return e == cudaSuccess ? CC3_OK : CC3_FAIL(CC3_ERR_CUDA, cudaGetErrorString(e));
+  }
+  // large tables: the copy is complete on return
+  cudaError_t e = cudaMemcpyAsync(dst, src, n, cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  return e == cudaSuccess ? CC3_OK : CC3_FAIL(CC3_ERR_CUDA, cudaGetErrorString(e));
+}
+
+}  // namespace cc3

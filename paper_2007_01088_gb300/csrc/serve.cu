@@ -151,8 +151,8 @@ int execute(Req *r, cudaStream_t st) {
   cc3_counters cnt{};
   cc3_ctx_counters(ctx, &cnt);
   r->nominal = cnt.nominal_flop;
-  cc3_ctx_destroy(ctx);
   cudaStreamSynchronize(st);
+  cc3::ctx_release(ctx, st);  // without waiting for the other slots' streams
   return rc;
 }
 
@@ -235,9 +235,8 @@ int cc3_serve_start(cc3_server **out, size_t hbm_budget_bytes, int max_slots) {
   if (!S) return CC3_ERR_OOM;
   cudaGetDevice(&S->device);
   if (hbm_budget_bytes == 0) {
-    size_t fr = 0, tot = 0;
-    if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) {
-      cudaGetLastError();
+    const size_t fr = cc3::dev_mem_free();
+    if (fr == 0) {
       delete S;
       return CC3_FAIL(CC3_ERR_CUDA, "cudaMemGetInfo");
     }
@@ -410,6 +409,7 @@ int cc3_serve_stop(cc3_server *S) {
   S->cv_done.notify_all();
   for (auto &t : S->workers) t.join();
   delete S;
+  cc3::dev_give_back();
   return CC3_OK;
 }
 

@@ -140,7 +140,7 @@ SplitState *state(cc3_ctx *c) { return reinterpret_cast<SplitState *>(c->split);
 template <class T>
 int alloc(T **p, size_t n) {
   *p = nullptr;
-  if (cudaMalloc(p, sizeof(T) * (n ? n : 1)) != cudaSuccess) {
+  if (dev_malloc(p, sizeof(T) * (n ? n : 1)) != cudaSuccess) {
     cudaGetLastError();
     return CC3_ERR_OOM;
   }
@@ -159,7 +159,7 @@ void free_state_buffers(SplitState *S) {
                   S->OVD, S->OVZA, S->OVZB, S->LVV, S->evdd, S->Wdd, S->TTdd, S->W3dd, S->eo_tri, S->V[0], S->V[1], S->V[2], S->vptr, S->maxbits,
                   S->slot_ex, S->status};
   for (void *p : bufs)
-    if (p) cudaFree(p);
+    if (p) dev_free(p);
   for (auto *v : {&S->ab, &S->om})
     for (auto &d : *v) s_free_plan(&d);
 }
@@ -200,7 +200,7 @@ int stage(cc3_ctx *c, SplitState *S, cudaStream_t st) {
   unsigned long long h[8];
   CU(cudaMemcpyAsync(h, mx, sizeof(h), cudaMemcpyDeviceToHost, st));
   CU(cudaStreamSynchronize(st));
-  cudaFree(mx);
+  dev_free(mx);
   double hv[5];
   for (int i = 0; i < 5; ++i) std::memcpy(&hv[i], &h[i], 8);
   S->Et = exponent_of(hv[0]);
@@ -259,7 +259,7 @@ int stage(cc3_ctx *c, SplitState *S, cudaStream_t st) {
     g = {0, 0, 0, nv, 0, 1, 1, 1 << 30, vp, nv, 1};
     TRY(slab(&S->OO, oo, (long long)no * no * (no + 1), vp, S->Eg, g, no + 1));
     CU(cudaStreamSynchronize(st));
-    cudaFree(oo);
+    dev_free(oo);
   }
   // OV[(q,r)][0][(u,w)] = ovov[q][u][r][w]
   g = {0, 0, (long long)nv * no * nv, nv, (long long)no * nv, 1, no, no, nv, nv, nv, 1};
@@ -741,7 +741,7 @@ int build_plans(cc3_ctx *c, SplitState *S, cudaStream_t st) {
       const dd::df ed = dd::from_double_host(eo[ijk[0]] + eo[ijk[1]] + eo[ijk[2]]);
       eot[t] = make_float2(ed.hi, ed.lo);
     }
-    if (S->eo_tri) cudaFree(S->eo_tri);
+    if (S->eo_tri) dev_free(S->eo_tri);
     S->eo_tri = nullptr;
     TRY(alloc(&S->eo_tri, eot.size()));
     CU(cudaMemcpyAsync(S->eo_tri, eot.data(), sizeof(float2) * eot.size(),
@@ -1161,7 +1161,7 @@ struct JacBufs {
   std::vector<void *> p;
   ~JacBufs() {
     for (void *x : p)
-      if (x) cudaFree(x);
+      if (x) dev_free(x);
   }
   template <class T>
   int get(T **out, size_t n) {
@@ -1258,7 +1258,6 @@ int split_jacobian(cc3_ctx *c, int nvec, const double *w, const double *R1d, con
       const int lrc = s_launch_plan(D, la, vp2, s, S->status, st,
                                     &c->counters.launches);
       trace_end(c, TR_SPLIT_W, st, D.flop, D.slice_flop);
-      CU(cudaStreamSynchronize(st));
       s_free_plan(&D);
       TRY(lrc);
     }
@@ -1737,8 +1736,7 @@ int split_left_jacobian(cc3_ctx *c, int nvec, const double *w, const double *L1d
   // batches than the right transformation's (up to 120 GB, at most 40 % of the free
   // memory) give the grouped G jobs more terms
   const double per_slot = (double)nv2 * nv * 24.0 + 3.0 * s * nv2 * vp * 2.0;
-  size_t free_b = 0, total_b = 0;
-  cudaMemGetInfo(&free_b, &total_b);
+  const size_t free_b = dev_mem_free();
   const double slot_budget = std::min(120.0e9, 0.4 * (double)free_b);
   const int bj = std::max(1, std::min(S->batch, (int)(slot_budget / (per_slot * nvec))));
   const int nslot = nvec * bj;
@@ -1954,7 +1952,6 @@ int split_left_jacobian(cc3_ctx *c, int nvec, const double *w, const double *L1d
       SDevPlan d;
       TRY(s_upload_plan(pc, &d, st));
       const int rc = run(d, ac, PC, TR_SPLIT_OMEGA);
-      CU(cudaStreamSynchronize(st));  // the plan's tables are freed next
       s_free_plan(&d);
       TRY(rc);
     }
@@ -2053,8 +2050,7 @@ int split_density(cc3_ctx *c, double w, const double *L1d, const double *L2d, do
   float2 *tau_all = nullptr, *lt_all = nullptr;
   {
     const size_t need = 2 * (size_t)next * (size_t)nv3 * sizeof(float2);
-    size_t free_b = 0, total_b = 0;
-    cudaMemGetInfo(&free_b, &total_b);
+    const size_t free_b = dev_mem_free();
     if (need > free_b / 2)
       return CC3_FAIL(CC3_ERR_OOM, "split densities: tau and L3 of every triple do not fit");
   }
@@ -2211,7 +2207,6 @@ int split_density(cc3_ctx *c, double w, const double *L1d, const double *L2d, do
     trace_begin(c, cls, st);
     const int rc = s_launch_plan(d, a, pt, s, S->status, st, Lc);
     trace_end(c, cls, st, d.flop, d.slice_flop);
-    CU(cudaStreamSynchronize(st));  // the tables are freed next
     s_free_plan(&d);
     return rc;
   };
@@ -2385,7 +2380,7 @@ done:
   s_free_plan(&D);
   void *bufs[] = {dA, dB, dC, sA, sB, mx, status};
   for (void *p : bufs)
-    if (p) cudaFree(p);
+    if (p) dev_free(p);
   cudaGetLastError();
   return rc;
 #undef CK
@@ -2396,5 +2391,6 @@ done:
 
 extern "C" int cc3_debug_split_gemm(int M, int N, int K, const double *A, const double *B,
                                     double *C, int slices) {
+  cc3::StreamScope scope(nullptr);
   return cc3::debug_split_gemm(M, N, K, A, B, C, slices, nullptr);
 }

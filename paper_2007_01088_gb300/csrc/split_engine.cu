@@ -51,6 +51,8 @@
 #include <mutex>
 
 #include <algorithm>
+#include <cstring>
+#include <vector>
 
 #include <cuda_bf16.h>
 
@@ -918,31 +920,30 @@ int s_upload_plan(const SPlan &p, SDevPlan *d, cudaStream_t s) {
     j.tile_base = tiles;
     tiles += (long long)j.batch * j.tiles_m * j.tiles_n * j.ksplit;
   }
-  if (cudaMalloc(&d->counter, sizeof(unsigned long long)) != cudaSuccess) return CC3_ERR_OOM;
   d->njobs = (int)jobs.size();
   d->tiles = tiles;
   d->flop = p.flop;
   d->slice_flop = p.slice_flop;
-  if (d->njobs == 0) return CC3_OK;
-  if (cudaMalloc(&d->jobs, sizeof(SJob) * jobs.size()) != cudaSuccess) return CC3_ERR_OOM;
-  if (cudaMalloc(&d->terms, sizeof(STerm) * (p.terms.size() + 1)) != cudaSuccess)
+  // one allocation: the tile counter, the jobs, the terms
+  const size_t jb = (sizeof(SJob) * jobs.size() + 15) / 16 * 16,
+               tb = sizeof(STerm) * p.terms.size();
+  std::vector<char> host(16 + jb + tb, 0);
+  if (!jobs.empty()) std::memcpy(host.data() + 16, jobs.data(), sizeof(SJob) * jobs.size());
+  if (tb) std::memcpy(host.data() + 16 + jb, p.terms.data(), tb);
+  char *base = nullptr;
+  if (dev_malloc(&base, host.size() + sizeof(STerm)) != cudaSuccess) {
+    cudaGetLastError();
     return CC3_ERR_OOM;
-  if (cudaMemcpyAsync(d->jobs, jobs.data(), sizeof(SJob) * jobs.size(),
-                      cudaMemcpyHostToDevice, s) != cudaSuccess)
-    return CC3_ERR_CUDA;
-  if (!p.terms.empty() &&
-      cudaMemcpyAsync(d->terms, p.terms.data(), sizeof(STerm) * p.terms.size(),
-                      cudaMemcpyHostToDevice, s) != cudaSuccess)
-    return CC3_ERR_CUDA;
-  if (cudaStreamSynchronize(s) != cudaSuccess) return CC3_ERR_CUDA;
-  return CC3_OK;
+  }
+  d->counter = reinterpret_cast<unsigned long long *>(base);
+  d->jobs = reinterpret_cast<SJob *>(base + 16);
+  d->terms = reinterpret_cast<STerm *>(base + 16 + jb);
+  return dev_upload(base, host.data(), host.size(), s);
 }
 
 void s_free_plan(SDevPlan *d) {
-  if (d->counter) cudaFree(d->counter);
+  if (d->counter) dev_free(d->counter);
   d->counter = nullptr;
-  if (d->jobs) cudaFree(d->jobs);
-  if (d->terms) cudaFree(d->terms);
   d->jobs = nullptr;
   d->terms = nullptr;
   d->njobs = 0;
