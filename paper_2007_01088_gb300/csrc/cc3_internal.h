@@ -107,6 +107,7 @@ struct Tracer {
 }  // namespace cc3
 
 struct cc3_ctx {
+  bool small_batch = false;  // the split path's batches within the serving footprint
   int no = 0, nv = 0, naux = 0;
   unsigned flags = 0;
   int device = 0;

@@ -136,6 +136,7 @@ int execute(Req *r, cudaStream_t st) {
                           r->vvvo.data(), r->ooov.data(), r->ovov.data(), r->F.data(),
                           q.naux > 0 ? r->chol.data() : nullptr, q.naux, q.flags, st);
   if (rc != CC3_OK) return rc;
+  ctx->small_batch = true;
   const size_t n1 = (size_t)q.no * q.nv, nt2 = n1 * q.no * q.nv;
   if (q.kind == 0) {
     r->o1.resize(n1);

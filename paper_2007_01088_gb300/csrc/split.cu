@@ -164,6 +164,22 @@ void free_state_buffers(SplitState *S) {
     for (auto &d : *v) s_free_plan(&d);
 }
 
+// Triples in flight: up to 16 within 6 GB of workspace and, where they are
+// small, up to 48 within 1 GB, in batches of about equal size: a batch costs
+// four launches and two tails of the engine's tiles, which at nv = 30 is most
+// of its time.  Contexts of the serving loop keep to 16, the figure its
+// footprints are computed with.  Measured (with the launches per batch going
+// from nine to four): no=5 nv=30 307 -> 240 us, no=8 nv=72 4.20 -> 3.47 ms, no=11
+// nv=87 14.1 -> 12.9 ms; at nv = 160 the rule keeps 16.
+int slots_of(int nv, int s, int ntri, bool small) {
+  const double nv2 = (double)nv * nv, per_slot = nv2 * nv * 24.0 + 6.0 * s * nv2 * rup(nv, 16);
+  double most = std::min(16.0, 6.0e9 / per_slot);
+  if (!small) most = std::max(most, std::min(48.0, 1.0e9 / per_slot));
+  const int n = (int)std::max(1.0, most), t = std::max(1, ntri);
+  const int batches = (t + n - 1) / n;
+  return (t + batches - 1) / batches;
+}
+
 // oo[(q,r)][l'][z] = ooov[q][l'][r][z] (l' < no), -F[r][z] (l' = no)
 __global__ void build_oo_kernel(const double *__restrict__ ooov, const double *__restrict__ F,
                                 double *__restrict__ oo, int no, int nv) {
@@ -278,9 +294,7 @@ int stage(cc3_ctx *c, SplitState *S, cudaStream_t st) {
     CU(cudaMemcpyAsync(S->evdd, evd.data(), sizeof(float2) * nv, cudaMemcpyHostToDevice, st));
   }
   // per-batch workspace
-  const double per_slot = (double)nv2 * nv * 24.0 + 3.0 * s * nv2 * vp * 2.0;
-  S->batch = (int)std::max(1.0, std::min(16.0, 6.0e9 / per_slot));
-  S->batch = std::min(S->batch, std::max(1, c->ntri));
+  S->batch = slots_of(nv, s, c->ntri, c->small_batch);
   const size_t nb = (size_t)S->batch;
   TRY(alloc(&S->Wdd, nb * nv2 * nv));
   TRY(alloc(&S->TTdd, nb * nv2 * nv));
@@ -295,7 +309,7 @@ int stage(cc3_ctx *c, SplitState *S, cudaStream_t st) {
     TRY(alloc(&S->vptr, 3));
     CU(cudaMemcpyAsync(S->vptr, h, sizeof(h), cudaMemcpyHostToDevice, st));
   }
-  TRY(alloc(&S->maxbits, nb));
+  TRY(alloc(&S->maxbits, (size_t)c->ntri + no));  // of every triple (densities: and i = j = k)
   TRY(alloc(&S->slot_ex, nb));
   TRY(alloc(&S->status, 4));
   CU(cudaMemsetAsync(S->status, 0, 4 * sizeof(int), st));
@@ -847,19 +861,18 @@ int omega_sequence(cc3_ctx *c, SplitState *S, cudaStream_t st) {
   VPtrTable P;
   fill_vptrs(c, S, &P);
   const int nv = c->nv;
+  CU(cudaMemsetAsync(S->maxbits, 0, sizeof(unsigned int) * c->ntri, st));
   for (size_t b = 0, t0 = 0; b < S->ab.size(); t0 += S->nslot[b], ++b) {
     const int ns = S->nslot[b];
     trace_begin(c, TR_SPLIT_W, st);
     TRY(s_launch_plan(S->ab[b], S->arrs, P, s, S->status, st, &c->counters.launches));
     trace_end(c, TR_SPLIT_W, st, S->ab[b].flop, S->ab[b].slice_flop);
     trace_begin(c, TR_SPLIT_ELEM, st);
-    CU(cudaMemsetAsync(S->maxbits, 0, sizeof(unsigned int) * ns, st));
     TRY(launch_tau_contravariant_dd(S->Wdd, S->TTdd, S->W3dd, S->TTdd, S->evdd, S->eo_tri + t0,
-                                    0.f, 0.f, nv, ns, S->maxbits, st));
-    TRY(launch_slot_exponent(S->maxbits, S->slot_ex, ns, st));
-    TRY(launch_slice_tt(S->TTdd, S->vptr, nv, S->vp, s, S->slot_ex, ns, S->batch, st));
+                                    0.f, 0.f, nv, ns, S->maxbits + t0, st));
+    TRY(launch_slice_tt(S->TTdd, S->vptr, nv, S->vp, s, S->slot_ex, S->maxbits + t0, ns, st));
     trace_end(c, TR_SPLIT_ELEM, st, 0.0, 0.0);
-    c->counters.launches += 3;
+    c->counters.launches += 2;
     trace_begin(c, TR_SPLIT_OMEGA, st);
     TRY(s_launch_plan(S->om[b], S->arrs, P, s, S->status, st, &c->counters.launches));
     trace_end(c, TR_SPLIT_OMEGA, st, S->om[b].flop, S->om[b].slice_flop);
@@ -909,6 +922,7 @@ int split_omega(cc3_ctx *c, cudaStream_t st) {
   CU(cudaStreamSynchronize(st));
   if (hs != 0) {
     cudaMemsetAsync(S->status, 0, sizeof(int), st);
+    S->planned = false;  // the plans' tile counters did not return to 0
     return hs == 2 ? CC3_FAIL(CC3_ERR_ARG, "a contraction plan addressed outside a slice array")
                    : CC3_FAIL(CC3_ERR_TIMEOUT, "split engine wait gave up");
   }
@@ -1028,11 +1042,9 @@ size_t split_footprint(int no, int nv, int s, int ntri) {
   b += sl((long long)no * no * (no + 1), vp, no + 1);  // OO
   b += (size_t)no * no * (no + 1) * nv * sizeof(double);  // its FP64 staging copy
   b += sl((long long)no * no, (long long)nv * vp, 1);  // OV
-  const double per_slot = (double)nv2 * nv * 24.0 + 3.0 * s * nv2 * vp * 2.0;
-  int batch = (int)std::max(1.0, std::min(16.0, 6.0e9 / per_slot));
-  batch = std::min(batch, std::max(1, ntri));
+  const int batch = slots_of(nv, s, ntri, true);
   b += 3 * (size_t)batch * nv2 * nv * sizeof(float2);  // Wdd, TTdd, W3dd
-  b += (size_t)std::max(1, ntri) * sizeof(float2);       // eo_tri
+  b += (size_t)std::max(1, ntri) * (sizeof(float2) + sizeof(int));  // eo_tri, maxbits
   b += 3 * arr_elems((long long)nv * vp, nv, batch, s) * sizeof(__nv_bfloat16);  // V[3]
   b += (size_t)nv * sizeof(float2) + 4096;
   return b;
@@ -1348,7 +1360,10 @@ int split_jacobian(cc3_ctx *c, int nvec, const double *w, const double *R1d, con
   TRY(B.get(&TTj, (size_t)nslot * nv2 * nv));
   TRY(B.get(&W3j, (size_t)nslot * nv2 * nv));
   TRY(B.get(&eoj, (size_t)nslot));
-  TRY(B.get(&maxj, (size_t)nslot));
+  const int nb = (c->ntri + bj - 1) / bj;
+  TRY(B.get(&maxj, (size_t)nslot * nb));
+  CU(cudaMemsetAsync(maxj, 0, sizeof(unsigned int) * nslot * nb, st));
+  CU(cudaMemsetAsync(S->maxbits, 0, sizeof(unsigned int) * c->ntri, st));
   TRY(B.get(&exj, (size_t)nslot));
   TRY(B.get(&vptrj, 3));
   const long long nv8 = (nv + 7) / 8 * 8;
@@ -1369,7 +1384,6 @@ int split_jacobian(cc3_ctx *c, int nvec, const double *w, const double *R1d, con
   const int rows = (nv + 7) / 8 * 8;
   const int ks4 = S->ks4;
   const bool stack = S->stack_vvov && nv >= S_BM && nv % 8 == 0 && nv % S_BM != 0;
-  const int nb = (c->ntri + bj - 1) / bj;
   JacPlans pT, pAB, pF, pZ, pO;
   pT.v.resize(nb);
   pAB.v.resize(nb);
@@ -1466,25 +1480,22 @@ int split_jacobian(cc3_ctx *c, int nvec, const double *w, const double *R1d, con
   // tau (or R3) and tau~ from the W build's partial sums, slot exponents and
   // the slices of the contravariant amplitudes
   auto elem = [&](float2 *W1, float2 *W2, float2 *W3, const float2 *eo, int ns,
-                  unsigned int *mb, int *exs, __nv_bfloat16 **vp_dev, int nalloc) -> int {
+                  unsigned int *mb, int *exs, __nv_bfloat16 **vp_dev) -> int {
     trace_begin(c, TR_SPLIT_ELEM, st);
-    CU(cudaMemsetAsync(mb, 0, sizeof(unsigned int) * ns, st));
     TRY(launch_tau_contravariant_dd(W1, W2, W3, W2, S->evdd, eo, 0.f, 0.f, nv, ns, mb, st));
-    TRY(launch_slot_exponent(mb, exs, ns, st));
-    TRY(launch_slice_tt(W2, vp_dev, nv, vp, s, exs, ns, nalloc, st));
+    TRY(launch_slice_tt(W2, vp_dev, nv, vp, s, exs, mb, ns, st));
     trace_end(c, TR_SPLIT_ELEM, st, 0.0, 0.0);
-    *L += 3;
+    *L += 2;
     return CC3_OK;
   };
   for (int b = 0; b < nb; ++b) {
     const int t0 = b * bj, ns = std::min(c->ntri, t0 + bj) - t0;
     TRY(run(pT.v[b], S->arrs, P, TR_SPLIT_W));
-    TRY(elem(S->Wdd, S->TTdd, S->W3dd, S->eo_tri + t0, ns, S->maxbits, S->slot_ex, S->vptr,
-             S->batch));
+    TRY(elem(S->Wdd, S->TTdd, S->W3dd, S->eo_tri + t0, ns, S->maxbits + t0, S->slot_ex, S->vptr));
     if (prep) TRY(run(pZ.v[b], S->arrs, P, TR_SPLIT_OMEGA));
     TRY(run(pF.v[b], S->arrs, P, TR_SPLIT_OMEGA));
     TRY(run(pAB.v[b], jr, PR, TR_SPLIT_W));
-    TRY(elem(Wj, TTj, W3j, eoj_all + (size_t)b * nslot, nslot, maxj, exj, vptrj, nslot));
+    TRY(elem(Wj, TTj, W3j, eoj_all + (size_t)b * nslot, nslot, maxj + (size_t)b * nslot, exj, vptrj));
     TRY(run(pO.v[b], jr, PR, TR_SPLIT_OMEGA));
   }
   int hs = 0;
@@ -1748,7 +1759,10 @@ int split_left_jacobian(cc3_ctx *c, int nvec, const double *w, const double *L1d
   TRY(B.get(&Wj, (size_t)nslot * nv2 * nv));
   TRY(B.get(&TTj, (size_t)nslot * nv2 * nv));
   TRY(B.get(&W3j, (size_t)nslot * nv2 * nv));
-  TRY(B.get(&maxj, (size_t)nslot));
+  const int nb = (c->ntri + bj - 1) / bj;
+  TRY(B.get(&maxj, (size_t)nslot * nb));
+  CU(cudaMemsetAsync(maxj, 0, sizeof(unsigned int) * nslot * nb, st));
+  CU(cudaMemsetAsync(S->maxbits, 0, sizeof(unsigned int) * c->ntri, st));
   TRY(B.get(&exj, (size_t)nslot));
   TRY(B.get(&vptrj, 3));
   const long long nv8 = (nv + 7) / 8 * 8;
@@ -1766,7 +1780,6 @@ int split_left_jacobian(cc3_ctx *c, int nvec, const double *w, const double *L1d
   const int rows = (nv + 7) / 8 * 8;
   const int ks4 = S->ks4;
   const int Ec = ELt + S->Eg;
-  const int nb = (c->ntri + bj - 1) / bj;
   JacPlans pT, pZ, pQ, pAB, pO;
   pT.v.resize(nb);
   pZ.v.resize(nb);
@@ -1845,21 +1858,18 @@ int split_left_jacobian(cc3_ctx *c, int nvec, const double *w, const double *L1d
     return CC3_OK;
   };
   auto elem = [&](float2 *W1, float2 *W2, float2 *W3, const float2 *eo, int ns, unsigned int *mb,
-                  int *exs, __nv_bfloat16 **vp_dev, int nalloc) -> int {
+                  int *exs, __nv_bfloat16 **vp_dev) -> int {
     trace_begin(c, TR_SPLIT_ELEM, st);
-    CU(cudaMemsetAsync(mb, 0, sizeof(unsigned int) * ns, st));
     TRY(launch_tau_contravariant_dd(W1, W2, W3, W2, S->evdd, eo, 0.f, 0.f, nv, ns, mb, st));
-    TRY(launch_slot_exponent(mb, exs, ns, st));
-    TRY(launch_slice_tt(W2, vp_dev, nv, vp, s, exs, ns, nalloc, st));
+    TRY(launch_slice_tt(W2, vp_dev, nv, vp, s, exs, mb, ns, st));
     trace_end(c, TR_SPLIT_ELEM, st, 0.0, 0.0);
-    *L += 3;
+    *L += 2;
     return CC3_OK;
   };
   for (int b = 0; b < nb; ++b) {
     const int t0 = b * bj, ns = std::min(c->ntri, t0 + bj) - t0;
     TRY(run(pT.v[b], S->arrs, P, TR_SPLIT_W));
-    TRY(elem(S->Wdd, S->TTdd, S->W3dd, S->eo_tri + t0, ns, S->maxbits, S->slot_ex, S->vptr,
-             S->batch));
+    TRY(elem(S->Wdd, S->TTdd, S->W3dd, S->eo_tri + t0, ns, S->maxbits + t0, S->slot_ex, S->vptr));
     if (prep) TRY(run(pZ.v[b], S->arrs, P, TR_SPLIT_OMEGA));
     TRY(run(pQ.v[b], aq, P, TR_SPLIT_OMEGA));
     TRY(run(pAB.v[b], jr, PR, TR_SPLIT_W));
@@ -1870,11 +1880,10 @@ int split_left_jacobian(cc3_ctx *c, int nvec, const double *w, const double *L1d
     *L += 1;
     // L3 of the batch: one exponent for all its slots (the grouped G jobs)
     trace_begin(c, TR_SPLIT_ELEM, st);
-    CU(cudaMemsetAsync(maxj, 0, sizeof(unsigned int) * nslot, st));
     TRY(launch_tau_contravariant_dd(Wj, TTj, W3j, TTj, S->evdd, eoj_all + (size_t)b * nslot, 0.f,
-                                    0.f, nv, nslot, maxj, st));
-    TRY(launch_common_exponent(maxj, exj, nslot, bj, ns, st));
-    TRY(launch_slice_tt(TTj, vptrj, nv, vp, s, exj, nslot, nslot, st));
+                                    0.f, nv, nslot, maxj + (size_t)b * nslot, st));
+    TRY(launch_common_exponent(maxj + (size_t)b * nslot, exj, nslot, bj, ns, st));
+    TRY(launch_slice_tt(TTj, vptrj, nv, vp, s, exj, nullptr, nslot, st));
     trace_end(c, TR_SPLIT_ELEM, st, 0.0, 0.0);
     *L += 3;
     TRY(run(pO.v[b], jr, PR, TR_SPLIT_OMEGA));
@@ -2154,8 +2163,11 @@ int split_density(cc3_ctx *c, double w, const double *L1d, const double *L2d, do
   TRY(B.get(&TTj, (size_t)bj * nv3));
   TRY(B.get(&W3j, (size_t)bj * nv3));
   TRY(B.get(&eol, (size_t)next));
-  TRY(B.get(&maxj, (size_t)bj));
-  TRY(B.get(&maxt, (size_t)bj));
+  TRY(B.get(&maxj, (size_t)next));
+  TRY(B.get(&maxt, (size_t)next));
+  CU(cudaMemsetAsync(maxj, 0, sizeof(unsigned int) * next, st));
+  CU(cudaMemsetAsync(maxt, 0, sizeof(unsigned int) * next, st));
+  CU(cudaMemsetAsync(S->maxbits, 0, sizeof(unsigned int) * next, st));
   TRY(B.get(&exj, (size_t)bj));
   TRY(B.get(&ext_, (size_t)bj));
   TRY(B.get(&exs, (size_t)bj));
@@ -2231,34 +2243,29 @@ int split_density(cc3_ctx *c, double w, const double *L1d, const double *L2d, do
     // tau: W build, then tau (resident) and tau~ with its slices
     TRY(run(tb, S->arrs, P, TR_SPLIT_W));
     trace_begin(c, TR_SPLIT_ELEM, st);
-    CU(cudaMemsetAsync(S->maxbits, 0, sizeof(unsigned int) * ns, st));
     TRY(launch_tau_contravariant_dd(S->Wdd, S->TTdd, S->W3dd, S->TTdd, S->evdd, eo_ext + t0, 0.f,
-                                    0.f, nv, ns, S->maxbits, st, tau_all + (size_t)t0 * nv3));
-    TRY(launch_slot_exponent(S->maxbits, S->slot_ex, ns, st));
-    TRY(launch_slice_tt(S->TTdd, S->vptr, nv, vp, s, S->slot_ex, ns, S->batch, st));
+                                    0.f, nv, ns, S->maxbits + t0, st,
+                                    tau_all + (size_t)t0 * nv3, maxt + t0));
+    TRY(launch_slice_tt(S->TTdd, S->vptr, nv, vp, s, S->slot_ex, S->maxbits + t0, ns, st));
     // the slices of tau itself, one exponent for the batch
-    CU(cudaMemsetAsync(maxt, 0, sizeof(unsigned int) * bj, st));
-    TRY(launch_slot_maxabs_dd(tau_all + (size_t)t0 * nv3, nv3, ns, maxt, st));
-    TRY(launch_common_exponent(maxt, ext_, bj, bj, ns, st));
-    TRY(launch_slice_tt(tau_all + (size_t)t0 * nv3, vptrt, nv, vp, s, ext_, ns, bj, st));
+    TRY(launch_common_exponent(maxt + t0, ext_, bj, bj, ns, st));
+    TRY(launch_slice_tt(tau_all + (size_t)t0 * nv3, vptrt, nv, vp, s, ext_, nullptr, ns, st));
     trace_end(c, TR_SPLIT_ELEM, st, 0.0, 0.0);
-    *Lc += 7;
+    *Lc += 4;
     TRY(run(qp, aq, P, TR_SPLIT_OMEGA));
     // L3 of the left state: W-build bracket, outer products, (w - eps), L~ (one
     // exponent for the batch) with its slices, kept resident
     TRY(run(ab, jr, PR, TR_SPLIT_W));
     trace_begin(c, TR_SPLIT_ELEM, st);
     TRY(launch_left_outer_dd(W3j, tri_ext + 3 * t0, bj, ns, ns, l1dd, ltdd, ovdd, fdd, no, nv, st));
-    CU(cudaMemsetAsync(maxj, 0, sizeof(unsigned int) * bj, st));
-    TRY(launch_tau_contravariant_dd(Wj, TTj, W3j, TTj, S->evdd, eol + t0, 0.f, 0.f, nv, ns, maxj,
-                                    st));
-    TRY(launch_common_exponent(maxj, exj, bj, bj, ns, st));
-    TRY(launch_slice_tt(TTj, vptrj, nv, vp, s, exj, ns, bj, st));
-    CU(cudaMemcpyAsync(lt_all + (size_t)t0 * nv3, TTj, sizeof(float2) * (size_t)ns * nv3,
-                       cudaMemcpyDeviceToDevice, st));
+    float2 *lt_t0 = lt_all + (size_t)t0 * nv3;
+    TRY(launch_tau_contravariant_dd(Wj, TTj, W3j, lt_t0, S->evdd, eol + t0, 0.f, 0.f, nv, ns,
+                                    maxj + t0, st));
+    TRY(launch_common_exponent(maxj + t0, exj, bj, bj, ns, st));
+    TRY(launch_slice_tt(lt_t0, vptrj, nv, vp, s, exj, nullptr, ns, st));
     TRY(launch_add_int(exj, ext_, exs, bj, st));
     trace_end(c, TR_SPLIT_ELEM, st, 0.0, 0.0);
-    *Lc += 6;
+    *Lc += 5;
     TRY(run(py, jr, PR, TR_SPLIT_OMEGA));
     TRY(run(pv, jr, PV, TR_SPLIT_OMEGA));
   }

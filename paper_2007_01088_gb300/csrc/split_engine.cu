@@ -312,7 +312,7 @@ template <int S>
 __global__ void __maxnreg__(96)
 split_engine_kernel(const SJob *__restrict__ jobs, int njobs, const STerm *__restrict__ terms,
                     const __grid_constant__ SArrTable arrs, VPtrTable P,
-                    int *status, unsigned long long *tile_ctr,
+                    int *status, unsigned int *tile_ctr,
                     long long ntiles) {
   constexpr int s = S;
   constexpr int S_STAGES = s_stages(S);
@@ -421,10 +421,13 @@ split_engine_kernel(const SJob *__restrict__ jobs, int njobs, const STerm *__res
     // (source, stride, destination and size are fixed for a term): lanes 0..23
     // the A segments (one per slab the tile's rows touch), lane 24 A2, 25 B,
     // 26 Bt, 27 Bt2.
+    // The counter returns to 0 by itself: a launch takes each tile once and one
+    // index past the end per CTA, after which the increment wraps.
+    const unsigned int wrap = (unsigned int)ntiles + gridDim.x - 1u;
     int j = 0, k = 0;
     bool fail = false;
     long long next = 0;
-    if (lane == 0) next = (long long)atomicAdd(tile_ctr, 1ull);
+    if (lane == 0) next = (long long)atomicInc(tile_ctr, wrap);
     for (int i = 0; !fail; ++i) {
       const int q = i % TQ;
       if (!__all_sync(0xffffffffu, mbar_wait_sleep(&tempty[q], ((i / TQ) & 1) ^ 1, &err))) break;
@@ -444,7 +447,7 @@ split_engine_kernel(const SJob *__restrict__ jobs, int njobs, const STerm *__res
         }
         break;
       }
-      if (lane == 0) next = (long long)atomicAdd(tile_ctr, 1ull);  // back by the next tile
+      if (lane == 0) next = (long long)atomicInc(tile_ctr, wrap);  // back by the next tile
       // its job: the last one with tile_base <= tile (tiles come in increasing
       // order, so the search moves forward only), 32 jobs at a time
       for (;;) {
@@ -935,7 +938,7 @@ int s_upload_plan(const SPlan &p, SDevPlan *d, cudaStream_t s) {
     cudaGetLastError();
     return CC3_ERR_OOM;
   }
-  d->counter = reinterpret_cast<unsigned long long *>(base);
+  d->counter = reinterpret_cast<unsigned int *>(base);
   d->jobs = reinterpret_cast<SJob *>(base + 16);
   d->terms = reinterpret_cast<STerm *>(base + 16 + jb);
   return dev_upload(base, host.data(), host.size(), s);
@@ -984,8 +987,6 @@ int s_launch_plan(const SDevPlan &d, const SArrTable &arrs, const VPtrTable &ptr
   static int sms[64] = {0};
   if (!sms[dev]) cudaDeviceGetAttribute(&sms[dev], cudaDevAttrMultiProcessorCount, dev);
   const unsigned grid = (unsigned)std::min<long long>(d.tiles, std::max(1, sms[dev]));
-  const cudaError_t me = cudaMemsetAsync(d.counter, 0, sizeof(unsigned long long), s);
-  if (me != cudaSuccess) return CC3_FAIL(CC3_ERR_CUDA, cudaGetErrorString(me));
   switch (slices) {
 #define CC3_SPLIT_LAUNCH(S_)                                                              \
   case S_:                                                                                \

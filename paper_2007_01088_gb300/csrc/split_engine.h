@@ -108,7 +108,9 @@ struct SPlan {
 };
 
 struct SDevPlan {
-  unsigned long long *counter = nullptr;  // tiles handed out in the current launch
+  // tiles handed out in the current launch; 0 between launches (after a launch
+  // that gave up the plan must be uploaded again)
+  unsigned int *counter = nullptr;
   SJob *jobs = nullptr;
   STerm *terms = nullptr;
   int njobs = 0;

@@ -161,7 +161,7 @@ tau_contravariant_dd_kernel(const float2 *__restrict__ W1, const float2 *W2,
                             const float2 *__restrict__ W3, float2 *tt,
                             const float2 *__restrict__ ev, const float2 *__restrict__ eo,
                             float w_hi, float w_lo, int nv, unsigned int *__restrict__ maxbits,
-                            float2 *__restrict__ tau_out) {
+                            float2 *__restrict__ tau_out, unsigned int *__restrict__ maxtau) {
   __shared__ float2 sm[6][CV_SLOT];
   const long long nv2 = (long long)nv * nv, nv3 = nv2 * nv;
   const long long sbase = blockIdx.y * nv3;
@@ -264,6 +264,7 @@ tau_contravariant_dd_kernel(const float2 *__restrict__ W1, const float2 *W2,
   stage(4);
   __syncthreads();
   if (tau_out) {  // tau itself, [slot][a][b][c] like tau~ (the densities' D_vv and D_oo)
+    float mt = 0.f;
 #pragma unroll
     for (int q = 0; q < 6; ++q) {
       if (slot[q] != q) continue;
@@ -271,11 +272,15 @@ tau_contravariant_dd_kernel(const float2 *__restrict__ W1, const float2 *W2,
       for (int h = 0; h < 2; ++h) {
         const int e = t + 256 * h, z = e & 7, y = (e >> 3) & 7, x = e >> 6;
         const int gx = cx[q] * 8 + x, gy = cy[q] * 8 + y, gz = cz[q] * 8 + z;
-        if (gx < nv && gy < nv && gz < nv)
-          tau_out[sbase + (long long)gx * nv2 + (long long)gy * nv + gz] =
-              sm[q][z * CV_SZ + x * CV_SX + y];
+        if (gx < nv && gy < nv && gz < nv) {
+          const float2 v = sm[q][z * CV_SZ + x * CV_SX + y];
+          tau_out[sbase + (long long)gx * nv2 + (long long)gy * nv + gz] = v;
+          mt = fmaxf(mt, fabsf(v.x));
+        }
       }
     }
+    for (int o = 16; o > 0; o >>= 1) mt = fmaxf(mt, __shfl_xor_sync(0xffffffffu, mt, o));
+    if ((t & 31) == 0) atomicMax(maxtau + blockIdx.y, __float_as_uint(mt));
   }
   dd::df v[2][6];
   bool own[2];
@@ -333,16 +338,11 @@ tau_contravariant_dd_kernel(const float2 *__restrict__ W1, const float2 *W2,
 }
 
 // exponent e with max < 2^e (max slightly enlarged to cover the dd low part)
-__global__ void slot_exponent_kernel(const unsigned int *__restrict__ maxbits, int *__restrict__ ex,
-                                     int nslot) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= nslot) return;
-  const float m = __uint_as_float(maxbits[i]) * (1.0f + 1e-6f);
+__device__ __forceinline__ int exponent_of_max(unsigned int maxbits) {
+  const float m = __uint_as_float(maxbits) * (1.0f + 1e-6f);
   int e = 0;
-  if (m > 0.f) {
-    frexpf(m, &e);  // m = f 2^e, f in [0.5, 1)
-  }
-  ex[i] = e;
+  if (m > 0.f) frexpf(m, &e);  // m = f 2^e, f in [0.5, 1)
+  return e;
 }
 
 // One exponent for every active slot of a batch (slot u active when u % bj <
@@ -360,9 +360,7 @@ __global__ void common_exponent_kernel(const unsigned int *__restrict__ maxbits,
     if ((int)threadIdx.x < w) red[threadIdx.x] = max(red[threadIdx.x], red[threadIdx.x + w]);
     __syncthreads();
   }
-  const float mf = __uint_as_float(red[0]) * (1.0f + 1e-6f);
-  int e = 0;
-  if (mf > 0.f) frexpf(mf, &e);
+  const int e = exponent_of_max(red[0]);
   for (int i = threadIdx.x; i < nslot; i += blockDim.x) ex[i] = e;
 }
 
@@ -383,9 +381,8 @@ __global__ void common_exponent_kernel(const unsigned int *__restrict__ maxbits,
 constexpr int TT_PAD = 18, TT_APLANE = 16 * TT_PAD + 2, TT_PLANE = 16 * TT_APLANE;
 __global__ void __launch_bounds__(256)
 slice_tt_kernel(const float2 *__restrict__ tt, __nv_bfloat16 *const *__restrict__ v, int nv,
-                int vp, int s, const int *__restrict__ ex, int nslot_alloc) {
+                int vp, int s, int *__restrict__ ex, const unsigned int *__restrict__ maxbits) {
   extern __shared__ __nv_bfloat16 dig[];  // [p][a][b][c] (c padded to TT_PAD)
-  (void)nslot_alloc;
   const int nx = (nv + 15) / 16, nzb = vp / 16;
   int blk = blockIdx.x;
   const int cb = blk % nx;
@@ -395,7 +392,10 @@ slice_tt_kernel(const float2 *__restrict__ tt, __nv_bfloat16 *const *__restrict_
   const int slot = blockIdx.y;
   const long long nv2 = (long long)nv * nv;
   const float2 *T = tt + (long long)slot * nv2 * nv;
-  const int sh = 7 + 8 * (s - 1) - ex[slot];
+  // the slot's exponent: from its maximum, recorded in ex, or as given there
+  const int e = maxbits ? exponent_of_max(maxbits[slot]) : ex[slot];
+  if (maxbits && blockIdx.x == 0 && threadIdx.x == 0) ex[slot] = e;
+  const int sh = 7 + 8 * (s - 1) - e;
   const int plane = TT_PLANE;
   // 2^sh and 2^(sh-24) as floats (the 32-bit digit path of s = 6)
   const float s0 = ldexpf(1.f, sh), s24 = ldexpf(1.f, sh - 24);
@@ -584,13 +584,13 @@ int launch_maxabs(const double *x, long long n, unsigned long long *out, cudaStr
 int launch_tau_contravariant_dd(const float2 *W1, const float2 *W2, const float2 *W3,
                                 float2 *tt, const float2 *ev, const float2 *eo, float w_hi,
                                 float w_lo, int nv, int nslot, unsigned int *maxbits,
-                                cudaStream_t st, float2 *tau_out) {
+                                cudaStream_t st, float2 *tau_out, unsigned int *maxtau) {
   if (nslot <= 0) return CC3_OK;
   const long long nx = (nv + 7) / 8, ncube = nx * (nx + 1) * (nx + 2) / 6;  // A >= B >= C
   if (ncube > 0x7fffffffLL || nslot > 65535)
     return CC3_FAIL(CC3_ERR_ARG, "tau_contravariant_dd grid");
   tau_contravariant_dd_kernel<<<dim3((unsigned)ncube, nslot), 256, 0, st>>>(
-      W1, W2, W3, tt, ev, eo, w_hi, w_lo, nv, maxbits, tau_out);
+      W1, W2, W3, tt, ev, eo, w_hi, w_lo, nv, maxbits, tau_out, maxtau);
   return cudaGetLastError() == cudaSuccess ? CC3_OK : CC3_FAIL(CC3_ERR_CUDA, "split element-wise kernel launch");
 }
 int launch_to_dd(const double *x, float2 *y, long long n, cudaStream_t st) {
@@ -609,33 +609,10 @@ int launch_left_outer_dd(float2 *W3, const int *tri, int bj, int ns, int nslot, 
   return cudaGetLastError() == cudaSuccess ? CC3_OK
                                            : CC3_FAIL(CC3_ERR_CUDA, "left outer products launch");
 }
-int launch_slot_exponent(const unsigned int *maxbits, int *ex, int nslot, cudaStream_t st) {
-  slot_exponent_kernel<<<(nslot + 127) / 128, 128, 0, st>>>(maxbits, ex, nslot);
-  return cudaGetLastError() == cudaSuccess ? CC3_OK : CC3_FAIL(CC3_ERR_CUDA, "split element-wise kernel launch");
-}
-// maxbits[u] = max |hi| (as float bits) over slot u's n elements of x
-__global__ void slot_maxabs_dd_kernel(const float2 *__restrict__ x, long long n,
-                                      unsigned int *__restrict__ maxbits) {
-  const float2 *xs = x + (long long)blockIdx.y * n;
-  float m = 0.f;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n;
-       e += (long long)gridDim.x * blockDim.x)
-    m = fmaxf(m, fabsf(xs[e].x));
-  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0) atomicMax(maxbits + blockIdx.y, __float_as_uint(m));
-}
 __global__ void add_int_kernel(const int *__restrict__ a, const int *__restrict__ b,
                                int *__restrict__ c, int n) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) c[i] = a[i] + b[i];
-}
-int launch_slot_maxabs_dd(const float2 *x, long long n, int nslot, unsigned int *maxbits,
-                          cudaStream_t st) {
-  if (nslot <= 0) return CC3_OK;
-  if (nslot > 65535) return CC3_FAIL(CC3_ERR_ARG, "slot_maxabs: slots");
-  const int blocks = (int)std::min<long long>((n + 255) / 256, 1024);
-  slot_maxabs_dd_kernel<<<dim3(blocks, nslot), 256, 0, st>>>(x, n, maxbits);
-  return cudaGetLastError() == cudaSuccess ? CC3_OK : CC3_FAIL(CC3_ERR_CUDA, "slot_maxabs launch");
 }
 int launch_add_int(const int *a, const int *b, int *c, int n, cudaStream_t st) {
   if (n <= 0) return CC3_OK;
@@ -649,7 +626,7 @@ int launch_common_exponent(const unsigned int *maxbits, int *ex, int nslot, int 
   return cudaGetLastError() == cudaSuccess ? CC3_OK : CC3_FAIL(CC3_ERR_CUDA, "split element-wise kernel launch");
 }
 int launch_slice_tt(const float2 *tt, __nv_bfloat16 *const *v, int nv, int vp, int s,
-                    const int *ex, int nslot, int nslot_alloc, cudaStream_t st) {
+                    int *ex, const unsigned int *maxbits, int nslot, cudaStream_t st) {
   if (vp / 16 != (nv + 15) / 16 || s < 1 || s > S_MAX_SLICES_K)
     return CC3_FAIL(CC3_ERR_ARG, "slice_tt layout");
   const int nx = (nv + 15) / 16;
@@ -669,7 +646,7 @@ int launch_slice_tt(const float2 *tt, __nv_bfloat16 *const *v, int nv, int vp, i
     }
   }
   dim3 grid(nx * nx * nx, nslot);
-  slice_tt_kernel<<<grid, 256, smem, st>>>(tt, v, nv, vp, s, ex, nslot_alloc);
+  slice_tt_kernel<<<grid, 256, smem, st>>>(tt, v, nv, vp, s, ex, maxbits);
   return cudaGetLastError() == cudaSuccess ? CC3_OK : CC3_FAIL(CC3_ERR_CUDA, "slice_tt launch");
 }
 

@@ -30,15 +30,13 @@ int launch_maxabs(const double *x, long long n, unsigned long long *out, cudaStr
 // tau from the W build's three partial sums W1 + W2 + W3 (dd, W2 and W3 [slot][c][a][b], W1 [slot][c][b][a])
 // over (w - eps), and tau~ (dd, [slot][a][b][c]) into tt, which may be W2;
 // ev: dd virtual orbital energies, eo: dd e_i + e_j + e_k of each slot
-// tau_out (optional): tau itself, [slot][a][b][c] (dd), written as well
+// tau_out (optional): tau itself, [slot][a][b][c] (dd), written as well, with
+// maxtau[slot] = max |tau.hi| (atomic max; zero it first)
 int launch_tau_contravariant_dd(const float2 *W1, const float2 *W2, const float2 *W3,
                                 float2 *tt, const float2 *ev, const float2 *eo, float w_hi,
                                 float w_lo, int nv, int nslot, unsigned int *maxbits,
-                                cudaStream_t st, float2 *tau_out = nullptr);
-int launch_slot_exponent(const unsigned int *maxbits, int *ex, int nslot, cudaStream_t st);
-// maxbits[u] = max |x.hi| over the n elements of slot u (atomic max; zero it first)
-int launch_slot_maxabs_dd(const float2 *x, long long n, int nslot, unsigned int *maxbits,
-                          cudaStream_t st);
+                                cudaStream_t st, float2 *tau_out = nullptr,
+                                unsigned int *maxtau = nullptr);
 // c[i] = a[i] + b[i]
 int launch_add_int(const int *a, const int *b, int *c, int n, cudaStream_t st);
 // one exponent (that of the largest maximum) for every active slot u (u % bj < ns)
@@ -53,8 +51,9 @@ int launch_to_dd(const double *x, float2 *y, long long n, cudaStream_t st);
 int launch_left_outer_dd(float2 *W3, const int *tri, int bj, int ns, int nslot, const float2 *L1,
                          const float2 *Lt, const float2 *ovov, const float2 *F, int no, int nv,
                          cudaStream_t st);
-// v: device array of 3 pointers (one per cyclic layout)
+// v: device array of 3 pointers (one per cyclic layout); the exponent of a slot
+// comes from maxbits[slot] and is recorded in ex[slot], or from ex (maxbits null)
 int launch_slice_tt(const float2 *tt, __nv_bfloat16 *const *v, int nv, int vp, int s,
-                    const int *ex, int nslot, int nslot_alloc, cudaStream_t st);
+                    int *ex, const unsigned int *maxbits, int nslot, cudaStream_t st);
 
 }  // namespace cc3
