@@ -197,6 +197,17 @@ __device__ __forceinline__ void umma_commit(uint64_t *bar) {
       : "memory");
 }
 
+// The same from the lane whose `lead` is 1 of a converged warp, without a branch.
+__device__ __forceinline__ void umma_commit_a(uint32_t lead, uint64_t *bar) {
+  asm volatile(
+      "{\n\t.reg .pred l;\n\t"
+      "setp.ne.b32 l, %1, 0;\n\t"
+      "@l tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(
+          smem_u32(bar)),
+      "r"(lead)
+      : "memory");
+}
+
 // 32 lanes x 4 columns of 32 bit
 __device__ __forceinline__ void tmem_ld4(uint32_t taddr, float *v) {
   uint32_t r[4];
