@@ -117,6 +117,82 @@ __global__ void slice_gather_kernel(const double *__restrict__ src, __nv_bfloat1
   }
 }
 
+// The same for arrays whose slabs are single (r2, r1) pairs (rps = n0) and whose
+// K blocks lie in one k1: a block takes 8 rows x 16 k of a run of 16 slabs, reads
+// them with the thread index fastest along the dimension of the smallest source
+// stride (js, ks, rs: the bits of an element's number that hold its place in the
+// run, its k and its row), and writes each slab's digits as one contiguous piece
+// (1536 bytes at s = 6).  Bound by HBM: 8 bytes read and 2 s written per element.
+// Staging the no=22 nv=250 integrals element by element, four layouts of 344 M
+// elements read 8 bytes per 32-byte sector, took 41 ms; this takes 10.5.
+struct SlabRun {
+  int mode;      // the run goes over 0: all slabs, r2 fastest; 1: r2; 2: r1
+  int len;       // its length; slabs outside it: blockIdx.x / ceil(len / 16)
+  int nr2;       // extent of r2
+  int js, ks, rs;
+};
+constexpr int SB_RUN = 16, SB_ROW = 17, SB_SLAB = 8 * SB_ROW + 1;  // padded strides (doubles)
+__global__ void __launch_bounds__(256)
+slice_block_kernel(const double *__restrict__ src, __nv_bfloat16 *__restrict__ dst, int s, int e,
+                   Gather g, SlabRun run, int KB) {
+  __shared__ double val[SB_RUN * SB_SLAB];
+  const int nrun = (run.len + SB_RUN - 1) / SB_RUN;
+  const int outer = blockIdx.x / nrun, f0 = blockIdx.x % nrun * SB_RUN;
+  const int row0 = blockIdx.y * 8, kb = blockIdx.z;
+  const int k1 = g.zblk ? kb % g.kin : 16 * kb / g.kin,
+            kbase = g.zblk ? 16 * (kb / g.kin) : 16 * kb % g.kin;
+  auto slab_of = [&](int j, int *r2, int *r1) {  // slab j of the run, false: none
+    const int f = f0 + j;
+    *r2 = run.mode == 0 ? f % run.nr2 : (run.mode == 1 ? f : outer);
+    *r1 = run.mode == 0 ? f / run.nr2 : (run.mode == 1 ? outer : f);
+    return f < run.len;
+  };
+  const double *base = src + g.off + k1 * g.sk1;
+#pragma unroll
+  for (int u = 0; u < SB_RUN * 128 / 256; ++u) {
+    const int x = threadIdx.x + 256 * u;
+    const int j = (x >> run.js) & 15, k = (x >> run.ks) & 15, r = (x >> run.rs) & 7;
+    int r2, r1;
+    double v = 0.0;
+    if (slab_of(j, &r2, &r1) && row0 + r < g.n0 && kbase + k < g.k0v && k1 < g.k1v)
+      v = base[r2 * g.s2 + r1 * g.s1 + (row0 + r) * g.s0 + (kbase + k) * g.sk0];
+    val[j * SB_SLAB + r * SB_ROW + k] = v;
+  }
+  __syncthreads();
+  // one thread: 8 k of one row of one slab, one 16-byte piece per slice
+  const int row = threadIdx.x & 7, kh = (threadIdx.x >> 3) & 1, j = threadIdx.x >> 4;
+  int r2, r1;
+  if (!slab_of(j, &r2, &r1)) return;
+  const int sh = 7 + 8 * (s - 1) - e;
+  long long T[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+    T[i] = fixed_from_double(val[j * SB_SLAB + row * SB_ROW + kh * 8 + i], sh);
+  const long long slab = (long long)r2 * g.n1 + r1;
+  uint4 *out = reinterpret_cast<uint4 *>(
+      dst + ((slab * KB + kb) * gridDim.y + blockIdx.y) * 128LL * s + kh * 64 + row * 8);
+#pragma unroll
+  for (int p = S_MAX_SLICES_K - 1; p >= 0; --p) {
+    if (p >= s) continue;
+    const float scale = slice_scale(p);
+    unsigned int w[4];
+#pragma unroll
+    for (int i = 0; i < 8; i += 2) {
+      float d[2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        // the balanced digit as a float by its place in 1.5 2^23's pattern
+        // (|d_0| <= 128 by the bound on T)
+        const int r = p > 0 ? (((int)T[i + h] + 128) & 255) - 128 : (int)T[i + h];
+        T[i + h] = (T[i + h] - r) >> 8;
+        d[h] = (__int_as_float(0x4B400000 + r) - 12582912.f) * scale;  // an exact BF16
+      }
+      w[i / 2] = __byte_perm(__float_as_uint(d[0]), __float_as_uint(d[1]), 0x7632);
+    }
+    out[p * 16] = make_uint4(w[0], w[1], w[2], w[3]);
+  }
+}
+
 __global__ void maxabs_kernel(const double *__restrict__ x, long long n,
                               unsigned long long *__restrict__ out) {
   unsigned long long m = 0;
@@ -574,6 +650,41 @@ int launch_slice_gather(const double *src, __nv_bfloat16 *dst, int s, int e, con
                         long long nrows, int Kp, int rps, cudaStream_t st) {
   if (Kp % 16 != 0 || rps < 1 || nrows % rps != 0)
     return CC3_FAIL(CC3_ERR_ARG, "slice layout");
+  const long long per = (long long)g.n0 * g.n1;
+  // (slabs of a few rows would spend the block kernel on padding rows)
+  if (rps == g.n0 && 5LL * g.n0 >= 3 * ((g.n0 + 7LL) / 8 * 8) && nrows % per == 0 && g.kin % 16 == (g.zblk ? g.kin % 16 : 0) &&
+      nrows / per < (1 << 30) && g.n1 < (1 << 30) && Kp / 16 <= 65535 && (g.n0 + 7) / 8 <= 65535) {
+    // the run along the faster of the two slab dimensions, or both where the
+    // second continues the first
+    SlabRun run;
+    run.nr2 = (int)(nrows / per);
+    const bool by2 = run.nr2 > 1 && (g.n1 == 1 || g.s2 <= g.s1);
+    const long long sj = by2 ? g.s2 : g.s1;
+    run.mode = by2 ? (g.n1 > 1 && g.s1 == run.nr2 * g.s2 ? 0 : 1) : 2;
+    run.len = run.mode == 0 ? run.nr2 * g.n1 : (run.mode == 1 ? run.nr2 : g.n1);
+    // bits of the element number, the smallest stride lowest
+    if (sj <= g.sk0 && sj <= g.s0) {
+      run.js = 0;
+      run.ks = g.sk0 <= g.s0 ? 4 : 7;
+      run.rs = g.sk0 <= g.s0 ? 8 : 4;
+    } else if (g.sk0 <= g.s0) {
+      run.ks = 0;
+      run.rs = 4;
+      run.js = 7;
+    } else {
+      run.rs = 0;
+      run.ks = 3;
+      run.js = 7;
+    }
+    const long long nrun = (run.len + SB_RUN - 1) / SB_RUN,
+                    gx = nrun * (run.mode == 0 ? 1 : (run.mode == 1 ? g.n1 : run.nr2));
+    if (gx <= 0x7fffffffLL) {
+      slice_block_kernel<<<dim3((unsigned)gx, (g.n0 + 7) / 8, Kp / 16), 256, 0, st>>>(
+          src, dst, s, e, g, run, Kp / 16);
+      return cudaGetLastError() == cudaSuccess ? CC3_OK
+                                               : CC3_FAIL(CC3_ERR_CUDA, "slice kernel launch");
+    }
+  }
   slice_gather_kernel<<<grid_for(nrows * Kp), 256, 0, st>>>(src, dst, s, e, g, nrows, Kp, rps);
   return cudaGetLastError() == cudaSuccess ? CC3_OK : CC3_FAIL(CC3_ERR_CUDA, "split element-wise kernel launch");
 }
