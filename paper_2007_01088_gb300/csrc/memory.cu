@@ -9,11 +9,12 @@
 // device worked 26 ms).  From the pool both cost 1-2 us and order themselves on
 // the calling stream.
 //
-// The pool keeps at most 1/16 of the device's memory while a context exists and
-// at most KEEP bytes after the last one is gone; cc3_serve_stop gives back the
-// rest as well when no context is left.  A failed allocation first returns all
-// that is unused and tries again.  dev_mem_free counts what the pool holds
-// unused as free.
+// The pool keeps at most 1/16 of the device's memory unused while a context
+// exists (trimmed at the end of each entry point that allocated or freed) and at most
+// KEEP bytes after the last one is gone; cc3_serve_stop gives back the rest as
+// well when no context is left.  A failed allocation first returns all that is
+// unused and tries again.  dev_mem_free counts what the pool holds unused as
+// free.
 #include <cuda_runtime.h>
 
 #include <atomic>
@@ -31,8 +32,11 @@ constexpr int MAX_DEV = 64;
 std::mutex g_mu;
 cudaMemPool_t g_pool[MAX_DEV] = {nullptr};
 bool g_tried[MAX_DEV] = {false};
+unsigned long long g_cap[MAX_DEV] = {0};  // unused bytes the pool may keep
 std::atomic<int> g_live{0};
 thread_local cudaStream_t t_stream = nullptr;
+thread_local int t_depth = 0;         // StreamScopes of this thread
+thread_local bool t_touched = false;  // allocated or freed in the outermost one
 
 // The device's pool; null where pools are not supported (then cudaMalloc serves).
 cudaMemPool_t pool_of(int dev) {
@@ -52,7 +56,9 @@ cudaMemPool_t pool_of(int dev) {
     size_t fr = 0, tot = 0;
     if (ok && cudaMemPoolCreate(&pool, &p) == cudaSuccess) {
       cudaMemGetInfo(&fr, &tot);
-      unsigned long long keep = tot / 16;
+      // (a release threshold would count the memory in use as well)
+      unsigned long long keep = ~0ull;
+      g_cap[dev] = tot / 16;
       if (cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) == cudaSuccess)
         g_pool[dev] = pool;
       else
@@ -108,11 +114,34 @@ bool host_take(HostBuf *out, int dev) {
 }
 }  // namespace
 
-StreamScope::StreamScope(cudaStream_t s) : prev(t_stream) { t_stream = s; }
-StreamScope::~StreamScope() { t_stream = prev; }
+// Bytes the pool has reserved and those in use; false: not known.
+static bool pool_state(cudaMemPool_t pool, unsigned long long *held, unsigned long long *used) {
+  if (cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, held) == cudaSuccess &&
+      cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, used) == cudaSuccess)
+    return true;
+  cudaGetLastError();
+  return false;
+}
+
+StreamScope::StreamScope(cudaStream_t s) : prev(t_stream) {
+  t_stream = s;
+  if (t_depth++ == 0) t_touched = false;
+}
+StreamScope::~StreamScope() {
+  t_stream = prev;
+  if (--t_depth > 0 || !t_touched) return;
+  const int dev = device();
+  cudaMemPool_t pool = pool_of(dev);
+  unsigned long long held = 0, used = 0;
+  if (pool && pool_state(pool, &held, &used) && held > used + g_cap[dev]) {
+    cudaMemPoolTrimTo(pool, used + g_cap[dev]);
+    cudaGetLastError();
+  }
+}
 
 cudaError_t dev_malloc_bytes(void **p, size_t n) {
   *p = nullptr;
+  t_touched = true;
   cudaMemPool_t pool = pool_of(device());
   if (!pool) return cudaMalloc(p, n);
   // no allocation becomes part of a caller's graph
@@ -133,6 +162,7 @@ cudaError_t dev_malloc_bytes(void **p, size_t n) {
 
 void dev_free(void *p) {
   if (!p) return;
+  t_touched = true;
   if (!pool_of(device())) {
     cudaFree(p);
   } else if (cudaFreeAsync(p, t_stream) != cudaSuccess) {
@@ -149,10 +179,7 @@ size_t dev_mem_free() {
   }
   if (cudaMemPool_t pool = pool_of(device())) {
     unsigned long long held = 0, used = 0;
-    if (cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &held) == cudaSuccess &&
-        cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess &&
-        held > used)
-      fr += (size_t)(held - used);
+    if (pool_state(pool, &held, &used) && held > used) fr += (size_t)(held - used);
   }
   return fr;
 }

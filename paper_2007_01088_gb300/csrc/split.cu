@@ -1315,7 +1315,8 @@ int split_jacobian(cc3_ctx *c, int nvec, const double *w, const double *R1d, con
   for (Kind &k : kinds) {
     const size_t per = arr_elems(k.K, k.rps, k.slabs, s);
     TRY(B.get(&k.base, per * nvec));
-    CU(cudaMemsetAsync(k.base, 0, per * nvec * sizeof(__nv_bfloat16), st));
+    if (k.rps % 8)  // padding rows (the gather writes everything else)
+      CU(cudaMemsetAsync(k.base, 0, per * nvec * sizeof(__nv_bfloat16), st));
     jr.a[k.map] = make_arr(k.base, k.K, k.rps, k.slabs * nvec, s);
   }
   for (int v = 0; v < nvec; ++v) {
@@ -1370,7 +1371,8 @@ int split_jacobian(cc3_ctx *c, int nvec, const double *w, const double *R1d, con
   for (int L = 0; L < 3; ++L) {
     const size_t n4 = arr_elems((long long)nv * vp, nv, nslot, s);
     TRY(B.get(&Vj[L], n4));
-    CU(cudaMemsetAsync(Vj[L], 0, n4 * sizeof(__nv_bfloat16), st));
+    if (nv % 16)  // padding in K and rows (slice_tt writes everything else)
+      CU(cudaMemsetAsync(Vj[L], 0, n4 * sizeof(__nv_bfloat16), st));
     jr.a[MA_V0 + L] = make_arr(Vj[L], (long long)nv * vp, nv, nslot, s);
     jr.a[MA_V0K + L] = make_arr(Vj[L], vp, (long long)nv * nv8, nslot, s);
   }
@@ -1727,7 +1729,8 @@ int split_left_jacobian(cc3_ctx *c, int nvec, const double *w, const double *L1d
   for (Kind &k : kinds) {
     const size_t per = arr_elems(k.K, k.rps, k.slabs, s);
     TRY(B.get(&k.base, per * nvec));
-    CU(cudaMemsetAsync(k.base, 0, per * nvec * sizeof(__nv_bfloat16), st));
+    if (k.rps % 8)  // padding rows (the gather writes everything else)
+      CU(cudaMemsetAsync(k.base, 0, per * nvec * sizeof(__nv_bfloat16), st));
     jr.a[k.map] = make_arr(k.base, k.K, k.rps, k.slabs * nvec, s);
   }
   for (int v = 0; v < nvec; ++v) {
@@ -1749,7 +1752,9 @@ int split_left_jacobian(cc3_ctx *c, int nvec, const double *w, const double *L1d
   const double per_slot = (double)nv2 * nv * 24.0 + 3.0 * s * nv2 * vp * 2.0;
   const size_t free_b = dev_mem_free();
   const double slot_budget = std::min(120.0e9, 0.4 * (double)free_b);
-  const int bj = std::max(1, std::min(S->batch, (int)(slot_budget / (per_slot * nvec))));
+  // (at most 16 triples: the slots of a batch share one slice exponent)
+  const int bj =
+      std::max(1, std::min(std::min(S->batch, 16), (int)(slot_budget / (per_slot * nvec))));
   const int nslot = nvec * bj;
   float2 *Wj = nullptr, *TTj = nullptr, *W3j = nullptr;
   __nv_bfloat16 *Vj[3] = {nullptr, nullptr, nullptr};
@@ -1769,7 +1774,8 @@ int split_left_jacobian(cc3_ctx *c, int nvec, const double *w, const double *L1d
   for (int L = 0; L < 3; ++L) {
     const size_t n4 = arr_elems((long long)nv * vp, nv, nslot, s);
     TRY(B.get(&Vj[L], n4));
-    CU(cudaMemsetAsync(Vj[L], 0, n4 * sizeof(__nv_bfloat16), st));
+    if (nv % 16)  // padding in K and rows (slice_tt writes everything else)
+      CU(cudaMemsetAsync(Vj[L], 0, n4 * sizeof(__nv_bfloat16), st));
     jr.a[MA_V0 + L] = make_arr(Vj[L], (long long)nv * vp, nv, nslot, s);
     jr.a[MA_V0K + L] = make_arr(Vj[L], vp, (long long)nv * nv8, nslot, s);
   }
@@ -2152,8 +2158,9 @@ int split_density(cc3_ctx *c, double w, const double *L1d, const double *L2d, do
       jr.a[kinds[i].map] = make_arr(a, kinds[i].K, kinds[i].rps, kinds[i].slabs, s);
     }
   }
-  // per batch: L3 slots (the residual's batch size), the slices of L~ and of tau
-  const int bj = S->batch;
+  // per batch: L3 slots (at most 16: they share one slice exponent), the slices
+  // of L~ and of tau
+  const int bj = std::min(S->batch, 16);
   float2 *Wj = nullptr, *TTj = nullptr, *W3j = nullptr, *eol = nullptr;
   __nv_bfloat16 *Vj[3] = {nullptr, nullptr, nullptr}, *Vt[3] = {nullptr, nullptr, nullptr};
   __nv_bfloat16 **vptrj = nullptr, **vptrt = nullptr;
@@ -2178,7 +2185,8 @@ int split_density(cc3_ctx *c, double w, const double *L1d, const double *L2d, do
     const size_t n4 = arr_elems((long long)nv * vp, nv, bj, s);
     TRY(B.get(&Vj[L], n4));
     TRY(B.get(&Vt[L], n4));
-    CU(cudaMemsetAsync(Vj[L], 0, n4 * sizeof(__nv_bfloat16), st));
+    if (nv % 16)  // padding in K and rows (slice_tt writes everything else)
+      CU(cudaMemsetAsync(Vj[L], 0, n4 * sizeof(__nv_bfloat16), st));
     CU(cudaMemsetAsync(Vt[L], 0, n4 * sizeof(__nv_bfloat16), st));
     jr.a[MA_V0 + L] = make_arr(Vj[L], (long long)nv * vp, nv, bj, s);
     jr.a[MA_V0K + L] = make_arr(Vj[L], vp, (long long)nv * nv8, bj, s);
