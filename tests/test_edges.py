@@ -1,0 +1,125 @@
+"""Edges of the kernels' ranges, on the GPU through the C ABI: K ranges around the
+engine's drain points and its split over K with every digit at its largest, column
+tiles that are trimmed, the register blocks of the densities' pair kernel beyond one
+group, and contexts of several threads and streams sharing the memory pool."""
+import threading
+from fractions import Fraction
+
+import numpy as np
+import pytest
+
+import oracle
+from cc3_inputs import make_inputs, make_trial_vectors
+from split_tol import split_close, split_err
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def g():
+    import paper_2007_01088_gb300 as g
+    return g
+
+
+# 16 K per step: a tile of 1, 2, 3 steps; level 3 due (12), its limit (16, 17),
+# level 2's (20, 21), level 1's (24, 28, 29), level 0's (48, 56, 57), the W build of
+# nv = 250 (36); one and two parts of a tile split over K (1600, 1601)
+@pytest.mark.parametrize("steps", [1, 2, 3, 12, 16, 17, 20, 21, 24, 28, 29, 36, 48, 56, 57, 130,
+                                   1600, 1601])
+@pytest.mark.parametrize("slices", [6, 3])
+def test_engine_sums_at_drain_points(g, steps, slices):
+    """Every slice digit 127: each accumulator takes the largest sums it can, so a
+    drain that comes too late loses low bits of all elements at once."""
+    K = 16 * steps
+    T = sum(127 * 256**p for p in range(slices))
+    x = float(T) * 2.0 ** -(7 + 8 * (slices - 1))  # exact for 6 slices: 47 bits
+    A = np.full((130, K), x)
+    B = np.full((24, K), x)
+    B[1::2] *= -1.0
+    B[2::3, ::2] *= -1.0
+    sums = B.sum(axis=1) / x  # small integers
+    ref = np.array([float(Fraction(x) * Fraction(x) * int(s)) for s in sums])
+    C = g.cc3_debug_split_gemm(A, B, slices)
+    # In units of the largest digit product (2^14): products below the last level are
+    # 5 (2) pairs of digits of 2^-8s per k; the shared accumulator (6 slices) holds
+    # 5 2^-32 per k so far and each of the 11 products a step adds to it drops at most
+    # 2^-23 of that: 11 2^-23 5 2^-32 16 (1 + 2 + ... + steps) <= 11 5 16 2^-55 steps^2 / 2
+    # (+ steps).
+    left_out = (slices - 1) * 2.0 ** (-8 * slices) * 1.01 * K
+    rounded = 11 * 5 * 16 * 2.0**-56 * steps * (steps + 1) if slices > 4 else 0.0
+    assert np.abs(C - ref[None, :]).max() <= left_out + rounded + 2.0**-52 * K
+
+
+@pytest.mark.parametrize("N", [16, 81, 97, 112, 177, 200, 250])
+def test_engine_trimmed_column_tiles(g, N):
+    rng = np.random.default_rng(N)
+    A, B = rng.normal(size=(129, 80)), rng.normal(size=(N, 80))
+    C = g.cc3_debug_split_gemm(A, B, 6)
+    scale = np.abs(A).max() * np.abs(B).max() * 80
+    assert np.abs(C - A @ B.T).max() <= 1e-13 * scale
+
+
+# rows and K blocks of the slicing kernels that end inside a block, and batches of
+# unequal size (no = 9: 156 triples)
+@pytest.mark.parametrize("no,nv", [(9, 7), (8, 24), (7, 25), (2, 100)])
+def test_residual_at_slicing_edges(g, no, nv):
+    inp = make_inputs(no, nv, seed=3 * no + nv)
+    ref = oracle.omega_inputs(inp)
+    o1, o2, _ = g.Context(inp).omega(g.CC3_SPLIT_BF16)
+    assert split_close(o1, ref["omega1"]), split_err(o1, ref["omega1"])
+    assert split_close(o2, ref["omega2"]), split_err(o2, ref["omega2"])
+
+
+def test_densities_beyond_one_group_of_blocks(g):
+    # 66 occupied orbitals: 17 x 17 blocks of 4 x 4 products, two groups of 256
+    no, nv = 66, 3
+    inp = make_inputs(no, nv, seed=5)
+    L1, L2 = make_trial_vectors(no, nv, 1, seed=6)
+    ref = oracle.density_inputs(inp, 0.2, L1[0], L2[0])
+    d = g.Context(inp).density(L1[0], L2[0], 0.2, prec=g.CC3_SPLIT_BF16)
+    for x, y in zip(d, (ref["Doo"], ref["Dov"], ref["Dvv"])):
+        assert split_close(x, y), split_err(x, y)
+
+
+# FP64 tiles whose row and column groups end one past, on and one before a multiple
+# of 16, short sums (K = no) and launches split over K (left: 3 tiles, K = 3 n nv)
+@pytest.mark.parametrize("no,nv", [(3, 15), (3, 16), (2, 17), (2, 65)])
+def test_fp64_left_at_tile_edges(g, no, nv):
+    inp = make_inputs(no, nv, seed=no + nv)
+    L1, L2 = make_trial_vectors(no, nv, 2, seed=7)
+    ref = oracle.left_jacobian(inp, L1, L2, [0.2, -0.1])
+    s1, s2 = g.Context(inp).left_jacobian(L1, L2, [0.2, -0.1], g.CC3_FP64)
+    for x, y in ((s1, ref["sigma1"]), (s2, ref["sigma2"])):
+        assert np.abs(x - y).max() <= 1e-11 * np.abs(y).max()
+
+
+def test_contexts_of_several_threads_share_the_pool(g):
+    """Contexts made, used and destroyed by four threads on streams of their own give
+    the results they give alone: no block of the pool serves two of them at a time."""
+    import torch
+    probs = [make_inputs(4, 20 + 7 * t, seed=t) for t in range(4)]
+    alone = []
+    for p in probs:
+        c = g.Context(p)
+        alone.append(c.omega(g.CC3_SPLIT_BF16))
+        c.close()
+    bad = []
+
+    def work(t):
+        st = torch.cuda.Stream()
+        for _ in range(6):
+            c = g.Context(probs[t], stream=st)
+            for _ in range(2):
+                got = c.omega(g.CC3_SPLIT_BF16)
+                for x, y in zip(got, alone[t]):
+                    # atomics add in another order
+                    if not np.abs(x - y).max() <= 1e-13 * np.abs(y).max():
+                        bad.append(t)
+            c.close()
+
+    threads = [threading.Thread(target=work, args=(t,)) for t in range(4)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not bad, bad
