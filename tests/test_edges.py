@@ -42,11 +42,11 @@ def test_engine_sums_at_drain_points(g, steps, slices):
     C = g.cc3_debug_split_gemm(A, B, slices)
     # In units of the largest digit product (2^14): products below the last level are
     # 5 (2) pairs of digits of 2^-8s per k; the shared accumulator (6 slices) holds
-    # 5 2^-32 per k so far and each of the 11 products a step adds to it drops at most
-    # 2^-23 of that: 11 2^-23 5 2^-32 16 (1 + 2 + ... + steps) <= 11 5 16 2^-55 steps^2 / 2
-    # (+ steps).
+    # 5 2^-32 per k so far, and each of the 11 products of a step adds to it in up to two
+    # parts (8 of its 16 k each), each of which drops at most 2^-23 of that:
+    # 22 2^-23 5 2^-32 16 (1 + 2 + ... + steps).
     left_out = (slices - 1) * 2.0 ** (-8 * slices) * 1.01 * K
-    rounded = 11 * 5 * 16 * 2.0**-56 * steps * (steps + 1) if slices > 4 else 0.0
+    rounded = 22 * 5 * 16 * 2.0**-56 * steps * (steps + 1) if slices > 4 else 0.0
     assert np.abs(C - ref[None, :]).max() <= left_out + rounded + 2.0**-52 * K
 
 
