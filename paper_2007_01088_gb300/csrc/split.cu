@@ -11,12 +11,12 @@
 //   XS[(r,z)][y][d]   = (yd|zr)              YS[(r,y)][z][d]  = (yd|zr)
 //   Zg[r][d][(u,w)]   = (ud|wr)              Zh[r][d][(u,w)]  = (wd|ur)
 //   OO[(q,r)][l'][z]  = (ql'|rz) for l' < no, -F_rz for l' = no
-//   OV[(q,r)][0][(u,w)] = (qu|rw)
+//   OVA[r][q][(u,w)]  = (qu|rw)              OVB[r][q][(u,w)] = (ru|qw)
 // and per triple in flight (slot) the contravariant amplitudes in three cyclic
 // layouts V_L (slot L outermost = x, L+1 = y, L+2 = z innermost) with K blocks
 // ordered (z block, y): read as rows x, K = (zb, y, zz) by the vvov and
 // singles contractions, and as rows (y, x), K = z by the ooov and F ones.
-// Zg, Zh and OV use the same (zb, u, zz) K order.
+// Zg, Zh, OVA and OVB use the same (zb, u, zz) K order.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -81,10 +81,10 @@ int ntile_for(int N) {
 
 enum MapId {
   MA_T2S = 0, MA_T2C, MA_T2R, MA_XS, MA_YS, MA_OS, MA_V0, MA_V1, MA_V2, MA_V0K, MA_V1K, MA_V2K,
-  MB_T2S, MB_T2C, MB_T2R, MB_XS, MB_YS, MB_OS, MB_ZG, MB_ZH, MB_OO, MB_OV,
+  MB_T2S, MB_T2C, MB_T2R, MB_XS, MB_YS, MB_OS, MB_ZG, MB_ZH, MB_OO, MB_OVA, MB_OVB,
   // Jacobian: per trial vector (R2 in the t2 layouts, g^ in the integral
   // layouts), F^ of all vectors, and ovov in the layouts of Algorithm 2
-  MJ_R2S, MJ_R2C, MJ_R2R, MJ_XH, MJ_YH, MJ_OH, MJ_FH, MJ_OVD, MJ_OVZA, MJ_OVZB,
+  MJ_R2S, MJ_R2C, MJ_R2R, MJ_XH, MJ_YH, MJ_OH, MJ_FH, MJ_OVD, MJ_OVZB,
   // left transformation: t2 as [(p,q)][d][x] (G), as [p][l][(u,w)] in both K
   // orders (H), and Lt2 of every vector as [(p,q)][v][(u,w)] in both orders (Q)
   ML_T2T, ML_T2ZA, ML_T2ZB, ML_LQA, ML_LQB,
@@ -102,16 +102,16 @@ struct SplitState {
   int s = 0, vp = 0, op = 0, Et = 0, Eg = 0;
   int Nab = 0, N3 = 0, N1 = 16;
   __nv_bfloat16 *T2S = nullptr, *T2C = nullptr, *T2R = nullptr, *XS = nullptr, *YS = nullptr,
-                *OS = nullptr, *Zg = nullptr, *Zh = nullptr, *OO = nullptr, *OV = nullptr;
+                *OS = nullptr, *Zg = nullptr, *Zh = nullptr, *OO = nullptr, *OVA = nullptr,
+                *OVB = nullptr;
   // Jacobian (Algorithm 2 layouts of ovov), staged on first use
-  __nv_bfloat16 *OVD = nullptr, *OVZA = nullptr, *OVZB = nullptr;
+  __nv_bfloat16 *OVD = nullptr, *OVZB = nullptr;
   // Jacobian: the vv block of the Cholesky vectors, rows (b,d), K = J
   __nv_bfloat16 *LVV = nullptr;
   int EL = 0;
   int ks4 = 1;  // K split of the rows-x contractions
   // tunables (autotuner): K steps per vvov tile, N tile of the W build (0: default)
   int ks_target = 400, nt_w = 0;
-  bool stack_vvov = true;  // stack permutations along M in the vvov contraction
   bool pair_ooov = true;   // one ooov job for the two permutations of a z slot
   // the residual's launch sequence as a CUDA graph (captured on the second
   // untraced call on a non-default stream, replayed afterwards)
@@ -155,8 +155,8 @@ void drop_graph(SplitState *S) {
 
 void free_state_buffers(SplitState *S) {
   drop_graph(S);
-  void *bufs[] = {S->T2S, S->T2C, S->T2R, S->XS, S->YS, S->OS, S->Zg, S->Zh, S->OO, S->OV,
-                  S->OVD, S->OVZA, S->OVZB, S->LVV, S->evdd, S->Wdd, S->TTdd, S->W3dd, S->eo_tri, S->V[0], S->V[1], S->V[2], S->vptr, S->maxbits,
+  void *bufs[] = {S->T2S, S->T2C, S->T2R, S->XS, S->YS, S->OS, S->Zg, S->Zh, S->OO, S->OVA, S->OVB,
+                  S->OVD, S->OVZB, S->LVV, S->evdd, S->Wdd, S->TTdd, S->W3dd, S->eo_tri, S->V[0], S->V[1], S->V[2], S->vptr, S->maxbits,
                   S->slot_ex, S->status};
   for (void *p : bufs)
     if (p) dev_free(p);
@@ -277,9 +277,12 @@ int stage(cc3_ctx *c, SplitState *S, cudaStream_t st) {
     CU(cudaStreamSynchronize(st));
     dev_free(oo);
   }
-  // OV[(q,r)][0][(u,w)] = ovov[q][u][r][w]
-  g = {0, 0, (long long)nv * no * nv, nv, (long long)no * nv, 1, no, no, nv, nv, nv, 1};
-  TRY(slab(&S->OV, c->ovov, (long long)no * no, nv * vp, S->Eg, g, 1));
+  // OVA[r][q][(u,w)] = ovov[q][u][r][w], OVB[r][q][(u,w)] = ovov[r][u][q][w]
+  const long long nvo = (long long)no * nv, ovl = nvo * nv;
+  g = {0, 0, nv, ovl, nvo, 1, no, no, nv, nv, nv, 1};
+  TRY(slab(&S->OVA, c->ovov, (long long)no * no, nv * vp, S->Eg, g, no));
+  g = {0, 0, ovl, nv, nvo, 1, no, no, nv, nv, nv, 1};
+  TRY(slab(&S->OVB, c->ovov, (long long)no * no, nv * vp, S->Eg, g, no));
   // dd orbital energies
   {
     std::vector<double> ev(nv);
@@ -335,10 +338,16 @@ int stage(cc3_ctx *c, SplitState *S, cudaStream_t st) {
   M[MB_ZG] = make_arr(S->Zg, n_v * vp, n_v, n_o, s);
   M[MB_ZH] = make_arr(S->Zh, n_v * vp, n_v, n_o, s);
   M[MB_OO] = make_arr(S->OO, vp, n_o + 1, n_o * n_o, s);
-  M[MB_OV] = make_arr(S->OV, n_v * vp, 1, n_o * n_o, s);
+  M[MB_OVA] = make_arr(S->OVA, n_v * vp, n_o, n_o, s);
+  M[MB_OVB] = make_arr(S->OVB, n_v * vp, n_o, n_o, s);
   CU(cudaStreamSynchronize(st));
   S->staged = true;
   return CC3_OK;
+}
+
+// Parts of about `target` K steps each.
+int k_parts(int steps, int target) {
+  return std::max(1, (steps + target - 1) / std::max(16, target));
 }
 
 // ---- plans --------------------------------------------------------------------
@@ -380,6 +389,7 @@ int new_sjob(SPlan &P, int M, int N, int Ntile, int batch, int ksplit, int mode,
   j.expo = expo;
   j.expo_slot = -1;
   j.expo_slot2 = -1;
+  j.tcol = j.tcol2 = -1;
   j.tiles_m = (M + S_BM - 1) / S_BM;
   j.tiles_n = (N + Ntile - 1) / Ntile;
   j.term0 = (int)P.terms.size();
@@ -406,10 +416,12 @@ void add_sterm(SPlan &P, int job, SOpnd A, SOpnd B, int K, int negA, double &exe
   j.nterm++;
   executed += 2.0 * j.tiles_m * S_BM * (double)j.tiles_n * j.Ntile * K * j.batch *
               (slices * (slices + 1) / 2);
-  const double mrows = j.m_pad > 0 ? (double)(j.M / j.m_pad) * j.m_valid +
-                                        std::min(j.M % j.m_pad, j.m_valid)
-                                  : (double)j.M;
-  const double ncols = j.route == 1 ? 2.0 * (j.Nm + j.tw) : (double)(j.n_valid + (j.N - j.Nm));
+  auto upto = [&](int m) {  // rows below m that are not padding
+    return (double)(m / j.m_pad) * j.m_valid + std::min(m % j.m_pad, j.m_valid);
+  };
+  const double mrows = j.m_pad > 0 ? upto(j.m_off + j.M) - upto(j.m_off) : (double)j.M;
+  const double ncols =
+      j.route == 1 ? 2.0 * (j.Nm + j.tw) : (double)(j.n_valid + (j.Nm < j.N ? 1 : 0));
   const double useful = 2.0 * mrows * ncols * K * j.batch;
   P.flop += useful;
   P.slice_flop += useful * (slices * (slices + 1) / 2);
@@ -526,12 +538,10 @@ void append_plan(SPlan &dst, const SPlan &src) {
   dst.slice_flop += src.slice_flop;
 }
 
-// residual contractions of one triple (every distinct permutation); which:
-// bit 0 the vvov + singles jobs (long K), bit 1 the ooov + F jobs (short K),
-// bit 3 leave out the singles and F columns (the left transformation's sigma2
-// contractions)
-void plan_omega_split(SPlan &P, SplitState *S, int no, int nv, const int ijk[3], int slot,
-                      int ksplit4, double &ex, int which = 3) {
+// ooov and F contractions of one triple (every distinct permutation);
+// nof: without the F columns (the left transformation's sigma2 contractions)
+void plan_ooov(SPlan &P, SplitState *S, int no, int nv, const int ijk[3], int slot, double &ex,
+               bool nof = false) {
   static const int PERM6[6][3] = {{0, 1, 2}, {1, 0, 2}, {2, 1, 0},
                                   {0, 2, 1}, {1, 2, 0}, {2, 0, 1}};
   const int s = S->s, vp = S->vp;
@@ -551,36 +561,12 @@ void plan_omega_split(SPlan &P, SplitState *S, int no, int nv, const int ijk[3],
     seen[nseen][1] = q;
     seen[nseen][2] = r;
     ++nseen;
-    // layout with x slot outermost: K order (slot m0+1, slot m0+2)
-    const int L = m[0];
-    const bool yz = (m[1] == (L + 1) % 3);
-    if ((which & 1) && (which & 8)) {  // the vvov contraction alone
-      int jb = new_sjob(P, nv, nv, ntile_for(nv), 1, ksplit4, SEPI_F64_ATOMIC, E, ex, s);
-      P.jobs[jb].expo_slot = slot;
-      P.jobs[jb].C = outd(B_OMT, ((long long)p * no + q) * nv2, nv, 1);
-      P.jobs[jb].Ct = P.jobs[jb].C;
-      add_sterm(P, jb, opd(MA_V0 + L, slot), opd(yz ? MB_ZG : MB_ZH, r), nv * vp, 0, ex, s);
-    } else if (which & 1) {  // Omega~^{ad}_{pq} += sum_{yz} V[x][y][z] (dy|rz)   columns d < nv
-       // Omega1^x_p       += sum_{yz} V[x][y][z] (qy|rz)   tail column nv8
-      const int nv8 = (nv + 7) / 8 * 8;
-      int jb = new_sjob(P, nv, nv8 + 1, ntile_for(nv8 + 1), 1, ksplit4, SEPI_F64_ATOMIC, E, ex, s);
-      P.jobs[jb].expo_slot = slot;
-      P.jobs[jb].Nm = nv8;
-      P.jobs[jb].n_valid = nv;
-      P.jobs[jb].C = outd(B_OMT, ((long long)p * no + q) * nv2, nv, 1);
-      P.jobs[jb].Ct = outd(B_OM1, (long long)p * nv, 1, 0);
-      const SOpnd tail = opd(MB_OV, yz ? q * no + r : r * no + q);
-      add_sterm(P, jb, opd(MA_V0 + L, slot), opd(yz ? MB_ZG : MB_ZH, r), nv * vp, 0, ex, s,
-                &tail, nv8);
-    }
-    if (which & 2) {  // the ooov / F job, formed below
-      ooov[nooov][0] = p;
-      ooov[nooov][1] = q;
-      ooov[nooov][2] = r;
-      ooov[nooov][3] = (m[2] + 1) % 3;  // Lz
-      ooov[nooov][4] = m[0] == (m[2] + 1) % 3 ? 1 : 0;  // xouter
-      ++nooov;
-    }
+    ooov[nooov][0] = p;
+    ooov[nooov][1] = q;
+    ooov[nooov][2] = r;
+    ooov[nooov][3] = (m[2] + 1) % 3;  // Lz
+    ooov[nooov][4] = m[0] == (m[2] + 1) % 3 ? 1 : 0;  // xouter
+    ++nooov;
   }
   // Omega~^{xy}_{pl} -= sum_z V (ql|rz);  Omega~^{xy}_{pq} += sum_z V F_rz.
   // Layout Lz has z innermost; its rows (y_L, x_L) are the perm's (y, x) when
@@ -610,14 +596,14 @@ void plan_omega_split(SPlan &P, SplitState *S, int no, int nv, const int ijk[3],
         break;
       }
     const int Lz = ooov[a][3];
-    const bool notail = (which & 8) != 0;
     if (b < 0) {
       // without the F column the job stops at the last ooov row of OO
-      int jb = new_sjob(P, nv * nv8, notail ? no : no + 1, S->N3, 1, 1, SEPI_F64_ATOMIC, E, ex,
+      int jb = new_sjob(P, nv * nv8, nof ? no : no + 1, S->N3, 1, 1, SEPI_F64_ATOMIC, E, ex,
                         s);
       SJob &J = P.jobs[jb];
       J.expo_slot = slot;
       J.Nm = no;
+      J.tcol = nof ? -1 : no;
       J.m_pad = nv8;
       J.m_valid = nv;
       ooov_out(ooov[a][0], ooov[a][4], ooov[a][1], &J.C, &J.Ct);
@@ -634,7 +620,7 @@ void plan_omega_split(SPlan &P, SplitState *S, int no, int nv, const int ijk[3],
     J.n_valid = N;
     J.route = 1;  // columns [0, cs): first permutation, [cs, N): second
     J.Nm2 = cs;
-    J.tw = notail ? 0 : 1;  // tw = 0: the F columns are computed and dropped
+    J.tw = nof ? 0 : 1;  // tw = 0: the F columns are computed and dropped
     J.m_pad = nv8;
     J.m_valid = nv;
     ooov_out(ooov[a][0], ooov[a][4], ooov[a][1], &J.C, &J.Ct);
@@ -650,10 +636,11 @@ void plan_omega_split(SPlan &P, SplitState *S, int no, int nv, const int ijk[3],
 // output / integral indices.
 struct VvovPerm {
   int slot, L, yz, p, q, r;
-  long long omt_off = 0, om1_off = 0;  // output base of this permutation's vector
+  long long omt_off, om1_off;  // output base of this permutation's vector
 };
 
-void collect_vvov_perms(std::vector<VvovPerm> &out, const int ijk[3], int slot) {
+void collect_vvov_perms(std::vector<VvovPerm> &out, const int ijk[3], int slot,
+                        long long omt_off = 0, long long om1_off = 0) {
   static const int PERM6[6][3] = {{0, 1, 2}, {1, 0, 2}, {2, 1, 0},
                                   {0, 2, 1}, {1, 2, 0}, {2, 0, 1}};
   int seen[6][3], nseen = 0;
@@ -677,64 +664,107 @@ void collect_vvov_perms(std::vector<VvovPerm> &out, const int ijk[3], int slot) 
     v.p = p;
     v.q = q;
     v.r = r;
+    v.omt_off = omt_off;
+    v.om1_off = om1_off;
     out.push_back(v);
   }
 }
 
-// The vvov + singles contraction of a batch with the permutations that share
-// the integral operand (same r and K order) stacked along M: their x rows
-// (nv each) are laid end to end and cut into 128-row tiles, so a tile may hold
-// the last rows of one permutation and the first rows of the next (two A
-// segments, two output row ranges, one singles tail column each).  Without
-// stacking nv = 160 costs two 128-row tiles per permutation, 96 rows of
-// padding in the second; with it, 1.25.  Needs nv a multiple of 8 and >= 128
-// (a tile then spans at most two permutations).
-void plan_vvov_stacked(SPlan &P, SplitState *S, int no, int nv, std::vector<VvovPerm> perms,
-                       int ksplit4, double &ex) {
-  const int s = S->s, vp = S->vp;
+// The vvov + singles contraction of a batch,
+//   Omega~^{xd}_{pq} += sum_{yz} V[x][y][z] (dy|rz)   columns d < nv
+//   Omega1^x_p       += sum_{yz} V[x][y][z] (qy|rz)   one tail column,
+// with the permutations that share the integral operand (same r and K order)
+// stacked along M: their x rows (nv8 = nv up to a multiple of 8) are laid end
+// to end and cut into tiles of up to 128 rows, so a tile may hold the last rows
+// of one permutation and the first rows of the next (two A segments, two output
+// row ranges).  One permutation per tile computes 128 rows for 66 (or 256 for
+// 160).  The tail rows come eight q at a time from OVA / OVB, the row group the
+// operand layout has in any case: a tile whose two permutations have q in the
+// same group of eight (the order they are taken in) needs one group, else two.
+// Against one permutation per tile (which from nv = 128 on was stacked already):
+// no=8 nv=72 3.30 -> 3.01 ms, no=6 nv=45 Jacobian 3.26 -> 2.83 ms, of it 1.31 ->
+// 0.91 in the engine; no change at nv = 250 (two full tiles either way).
+// notail: no singles column.
+void plan_vvov(SPlan &P, SplitState *S, int no, int nv, std::vector<VvovPerm> perms, double &ex,
+               bool notail = false) {
+  const int s = S->s, vp = S->vp, nv8 = (nv + 7) / 8 * 8;
   const long long nv2 = (long long)nv * nv;
-  std::stable_sort(perms.begin(), perms.end(), [](const VvovPerm &a, const VvovPerm &b) {
-    return a.r != b.r ? a.r < b.r : a.yz < b.yz;
+  const bool byq = nv8 % 16 != 0;  // else 8 and 16 tail rows are as many columns
+  std::stable_sort(perms.begin(), perms.end(), [&](const VvovPerm &a, const VvovPerm &b) {
+    if (a.r != b.r) return a.r < b.r;
+    if (a.yz != b.yz) return a.yz < b.yz;
+    return byq && a.q / 8 < b.q / 8;
   });
+  const size_t first = P.jobs.size();
   size_t g0 = 0;
   while (g0 < perms.size()) {
     size_t g1 = g0;
     while (g1 < perms.size() && perms[g1].r == perms[g0].r && perms[g1].yz == perms[g0].yz) ++g1;
-    const long long total = (long long)(g1 - g0) * nv;
-    for (long long R = 0; R < total; R += S_BM) {
-      const size_t k = g0 + (size_t)(R / nv);
-      const int x0 = (int)(R % nv);
-      const int rows0 = (int)std::min<long long>(std::min<long long>(nv - x0, S_BM), total - R);
-      const int rows1 = (rows0 < S_BM && k + 1 < g1) ? std::min(S_BM - rows0, nv) : 0;
-      const VvovPerm &u = perms[k];
-      const int N = rows1 > 0 ? nv + 9 : nv + 1;
-      int jb = new_sjob(P, rows0 + rows1, N, ntile_for(N), 1, ksplit4, SEPI_F64_ATOMIC,
-                        S->Eg - 14, ex, s);
+    const long long total = (long long)(g1 - g0) * nv8;
+    int rows = 0;
+    for (long long R = 0; R < total; R += rows) {
+      const size_t k = g0 + (size_t)(R / nv8);
+      const int x0 = (int)(R % nv8), rows0 = std::min<int>(nv8 - x0, S_BM);
+      const int rows1 = k + 1 < g1 ? std::min<int>(S_BM - rows0, nv8) : 0;
+      rows = rows0 + rows1;
+      const VvovPerm &u = perms[k], &w = perms[rows1 > 0 ? k + 1 : k];
+      const bool two = u.q / 8 != w.q / 8;  // two groups of tail rows
+      const int tc = nv8 + u.q % 8, tc2 = nv8 + (two ? 8 : 0) + w.q % 8;
+      const int N = notail ? nv : std::max(tc, tc2) + 1;
+      int jb = new_sjob(P, rows, N, ntile_for(N), 1, 1, SEPI_F64_ATOMIC, S->Eg - 14, ex, s);
       SJob &J = P.jobs[jb];
       J.expo_slot = u.slot;
-      J.Nm = nv;
+      J.Nm = notail ? nv : nv8;
       J.n_valid = nv;
+      if (nv < nv8) {
+        J.m_pad = nv8;
+        J.m_valid = nv;
+        J.m_off = x0;
+      }
       J.C = outd(B_OMT, u.omt_off + (((long long)u.p * no + u.q) * nv + x0) * nv, nv, 1);
-      J.Ct = outd(B_OM1, u.om1_off + (long long)u.p * nv + x0, 1, 0);
-      const SOpnd tail = opd(MB_OV, u.yz ? u.q * no + u.r : u.r * no + u.q);
-      add_sterm(P, jb, opd(MA_V0 + u.L, u.slot, 0, x0, 0), opd(u.yz ? MB_ZG : MB_ZH, u.r), nv * vp,
-                0, ex, s, &tail, nv);
+      J.Ct = notail ? J.C : outd(B_OM1, u.om1_off + (long long)u.p * nv + x0, 1, 0);
+      J.tcol = notail ? -1 : tc;
+      const int ov = u.yz ? MB_OVA : MB_OVB;
+      const SOpnd tail = opd(ov, u.r, 0, u.q / 8 * 8);
+      add_sterm(P, jb, opd(MA_V0 + u.L, u.slot, 0, x0), opd(u.yz ? MB_ZG : MB_ZH, u.r), nv * vp, 0,
+                ex, s, notail ? nullptr : &tail, nv8);
+      STerm &T = P.terms.back();
+      if (!notail) {  // second group of tail rows; none: past the slab's end
+        T.Bt2 = opd(ov, u.r, 0, (no + 7) / 8 * 8);
+        T.nbm2 = nv8 + 8;
+      }
       if (rows1 > 0) {
-        const VvovPerm &w = perms[k + 1];
         J.msplit = rows0;
-        J.Nm2 = nv + 8;
         J.expo_slot2 = w.slot;
         J.C2 = outd(B_OMT, w.omt_off + ((long long)w.p * no + w.q) * nv2, nv, 1);
-        J.Ct2 = outd(B_OM1, w.om1_off + (long long)w.p * nv, 1, 0);
-        STerm &T = P.terms.back();
+        J.Ct2 = notail ? J.C2 : outd(B_OM1, w.om1_off + (long long)w.p * nv, 1, 0);
+        J.tcol2 = notail ? -1 : tc2;
         T.A2 = opd(MA_V0 + w.L, w.slot);
         T.asplit = rows0;
-        T.Bt2 = opd(MB_OV, w.yz ? w.q * no + w.r : w.r * no + w.q);
-        T.nbm2 = nv + 8;
+        if (!notail && two) T.Bt2.row0 = w.q / 8 * 8;
       }
     }
     g0 = g1;
   }
+  // K split: tiles of at most ks_target steps (the persistent engine balances
+  // them over the SMs; partial sums add in FP64), or one part more where that
+  // shortens the rounds in which the SMs take them by over a tenth.  At
+  // no=11 nv=87 91 tiles a batch in 2 parts leave 31 for the second round:
+  // 3 parts take 12.0 -> 11.7 ms.  More parts alone are slower (partial sums of
+  // one output row meet in its atomics): no=16 nv=160 192.1 -> 193.3 ms in the engine
+  // with 8 parts for 4, no=8 nv=72 2.14 -> 2.21 ms with 2 for 1.
+  long long n = 0;
+  for (size_t j = first; j < P.jobs.size(); ++j) n += P.jobs[j].tiles_m * P.jobs[j].tiles_n;
+  if (n == 0) return;
+  const int kst = nv * vp / S_BK, ks0 = k_parts(kst, S->ks_target);
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  sms = std::max(1, sms);
+  auto rounds = [&](int k) { return (double)((n * k + sms - 1) / sms) / k; };
+  const int ks = kst >= 100 * (ks0 + 1) && rounds(ks0 + 1) < 0.9 * rounds(ks0) ? ks0 + 1 : ks0;
+  for (size_t j = first; j < P.jobs.size(); ++j) P.jobs[j].ksplit = ks;
+  P.tiles += n * (ks - 1);
 }
 
 int build_plans(cc3_ctx *c, SplitState *S, cudaStream_t st) {
@@ -763,14 +793,13 @@ int build_plans(cc3_ctx *c, SplitState *S, cudaStream_t st) {
     CU(cudaStreamSynchronize(st));
   }
   double ex = 0.0;
-  // K split of the vvov contraction: tiles of about 400 K steps, so that the
-  // persistent engine balances them over the SMs (partial sums add in FP64)
+  // K split of the other rows-x contractions: no short tiles fill the end of
+  // their launches, and 200 K steps a tile balance better than 400 (no=12
+  // nv=120 density: 60.8 -> 59.0 ms in the engine; no=9 nv=81 left, with the rule
+  // of plan_vvov: 17.5 -> 17.2 ms); 130 measured the same, 60 slower.
   const int kst = nv * S->vp / S_BK;
-  int ks4 = std::max(1, (kst + S->ks_target - 1) / std::max(16, S->ks_target));
-  S->ks4 = ks4;
+  S->ks4 = k_parts(kst, std::min(200, S->ks_target));
   S->Nab = S->nt_w > 0 ? S->nt_w : ntile_for(nv);
-  // stacked vvov tiles (see plan_vvov_stacked) where they save padding rows
-  const bool stack = S->stack_vvov && nv >= S_BM && nv % 8 == 0 && nv % S_BM != 0;
   for (int t0 = 0; t0 < c->ntri; t0 += S->batch) {
     const int t1 = std::min(c->ntri, t0 + S->batch);
     SPlan pab, pom, pom3;
@@ -778,15 +807,11 @@ int build_plans(cc3_ctx *c, SplitState *S, cudaStream_t st) {
     for (int t = t0; t < t1; ++t) {
       const int *ijk = &c->tri_host[3 * t];
       plan_w_split(pab, S, no, nv, ijk, t - t0, ex);
-      // the long-K tiles first: the persistent engine hands tiles out in order
-      if (stack) {
-        collect_vvov_perms(vperms, ijk, t - t0);
-      } else {
-        plan_omega_split(pom, S, no, nv, ijk, t - t0, ks4, ex, 1);
-      }
-      plan_omega_split(pom3, S, no, nv, ijk, t - t0, ks4, ex, 2);
+      collect_vvov_perms(vperms, ijk, t - t0);
+      plan_ooov(pom3, S, no, nv, ijk, t - t0, ex);
     }
-    if (stack) plan_vvov_stacked(pom, S, no, nv, vperms, ks4, ex);
+    // the long-K tiles first: the persistent engine hands tiles out in order
+    plan_vvov(pom, S, no, nv, vperms, ex);
     append_plan(pom, pom3);
     S->ab.emplace_back();
     S->om.emplace_back();
@@ -1041,7 +1066,7 @@ size_t split_footprint(int no, int nv, int s, int ntri) {
   b += 2 * sl((long long)no * nv, (long long)nv * vp, nv);  // Zg, Zh
   b += sl((long long)no * no * (no + 1), vp, no + 1);  // OO
   b += (size_t)no * no * (no + 1) * nv * sizeof(double);  // its FP64 staging copy
-  b += sl((long long)no * no, (long long)nv * vp, 1);  // OV
+  b += 2 * sl((long long)no * no, (long long)nv * vp, no);  // OVA, OVB
   const int batch = slots_of(nv, s, ntri, true);
   b += 3 * (size_t)batch * nv2 * nv * sizeof(float2);  // Wdd, TTdd, W3dd
   b += (size_t)std::max(1, ntri) * (sizeof(float2) + sizeof(int));  // eo_tri, maxbits
@@ -1082,7 +1107,7 @@ int slice_array(SplitState *S, __nv_bfloat16 **dst, const double *src, long long
 
 // ovov in the layouts of Algorithm 2 (once per context):
 //   OVD[(q,r)][d][z] = (qd|rz)                  (Z~v: rows d, K = z)
-//   OVZA[r][l][(u,w)] = (lu|rw), OVZB[r][l][(u,w)] = (lw|ru)   (Z~o: rows l, K = (zb, u, zz))
+//   OVZB[r][l][(u,w)] = (lw|ru)  (Z~o, with OVA: rows l, K = (zb, u, zz))
 int stage_jac_static(cc3_ctx *c, SplitState *S, cudaStream_t st) {
   if (S->OVD) return CC3_OK;
   const int no = c->no, nv = c->nv, vp = S->vp;
@@ -1090,13 +1115,10 @@ int stage_jac_static(cc3_ctx *c, SplitState *S, cudaStream_t st) {
   Gather g;
   g = {0, ovl, nv, nvo, 0, 1, no, nv, vp, nv, 1};
   TRY(slice_array(S, &S->OVD, c->ovov, (long long)no * no * nv, vp, S->Eg, g, nv, st));
-  g = {0, 0, nv, ovl, nvo, 1, no, no, nv, nv, nv, 1};
-  TRY(slice_array(S, &S->OVZA, c->ovov, (long long)no * no, nv * vp, S->Eg, g, no, st));
   g = {0, 0, nv, ovl, 1, nvo, no, no, nv, nv, nv, 1};
   TRY(slice_array(S, &S->OVZB, c->ovov, (long long)no * no, nv * vp, S->Eg, g, no, st));
   SArr *M = S->arrs.a;
   M[MJ_OVD] = make_arr(S->OVD, vp, nv, (long long)no * no, S->s);
-  M[MJ_OVZA] = make_arr(S->OVZA, (long long)nv * vp, no, no, S->s);
   M[MJ_OVZB] = make_arr(S->OVZB, (long long)nv * vp, no, no, S->s);
   return CC3_OK;
 }
@@ -1125,7 +1147,7 @@ void plan_jac_tau(SPlan *pf, SPlan *pz, SplitState *S, int no, int nv, int nvec,
     seen[nseen][1] = q;
     seen[nseen][2] = r;
     ++nseen;
-    // rows (y_L, x_L) of the z-innermost layout Lz (see plan_omega_split)
+    // rows (y_L, x_L) of the z-innermost layout Lz (see plan_ooov)
     const int Lz = (m[2] + 1) % 3;
     const bool xouter = (m[0] == Lz);
     if (pf) {
@@ -1163,7 +1185,7 @@ void plan_jac_tau(SPlan *pf, SPlan *pz, SplitState *S, int no, int nv, int nvec,
       K.expo_slot = slot;
       K.C = outd(B_ZO, ((long long)q * no + p) * no, (long long)no * no * no, 1);
       K.Ct = K.C;
-      add_sterm(*pz, jb, opd(MA_V0 + L, slot), opd(yz ? MJ_OVZA : MJ_OVZB, r), nv * vp, 0, ex,
+      add_sterm(*pz, jb, opd(MA_V0 + L, slot), opd(yz ? MB_OVA : MJ_OVZB, r), nv * vp, 0, ex,
                 s);
     }
   }
@@ -1384,8 +1406,6 @@ int split_jacobian(cc3_ctx *c, int nvec, const double *w, const double *R1d, con
   double *Zv = nullptr, *Zo = nullptr;
   TRY(jac_z_buffers(c, &Zv, &Zo, prep, st));
   const int rows = (nv + 7) / 8 * 8;
-  const int ks4 = S->ks4;
-  const bool stack = S->stack_vvov && nv >= S_BM && nv % 8 == 0 && nv % S_BM != 0;
   JacPlans pT, pAB, pF, pZ, pO;
   pT.v.resize(nb);
   pAB.v.resize(nb);
@@ -1428,17 +1448,8 @@ int split_jacobian(cc3_ctx *c, int nvec, const double *w, const double *R1d, con
         w_terms_3(ab, j3, set2, no, nv, rows, vp, op, ijk, ex, s);
         // the contractions of R~3 into vector v's rho~ and rho1
         const size_t first = om3.jobs.size();
-        if (stack) {
-          const size_t f0 = vperms.size();
-          collect_vvov_perms(vperms, ijk, u);
-          for (size_t k = f0; k < vperms.size(); ++k) {
-            vperms[k].omt_off = (long long)v * nt2;
-            vperms[k].om1_off = (long long)v * n1;
-          }
-        } else {
-          plan_omega_split(om3, S, no, nv, ijk, u, ks4, ex, 1);
-        }
-        plan_omega_split(om3, S, no, nv, ijk, u, ks4, ex, 2);
+        collect_vvov_perms(vperms, ijk, u, (long long)v * nt2, (long long)v * n1);
+        plan_ooov(om3, S, no, nv, ijk, u, ex);
         for (size_t jx = first; jx < om3.jobs.size(); ++jx) {
           SJob &J = om3.jobs[jx];
           for (OutD *o : {&J.C, &J.Ct, &J.C2, &J.Ct2}) {
@@ -1448,7 +1459,7 @@ int split_jacobian(cc3_ctx *c, int nvec, const double *w, const double *R1d, con
         }
       }
     }
-    if (stack) plan_vvov_stacked(om, S, no, nv, vperms, ks4, ex);
+    plan_vvov(om, S, no, nv, vperms, ex);
     append_plan(om, om3);  // the long-K vvov tiles first
     TRY(s_upload_plan(tb, &pT.v[b], st));
     TRY(s_upload_plan(ab, &pAB.v[b], st));
@@ -1784,7 +1795,6 @@ int split_left_jacobian(cc3_ctx *c, int nvec, const double *w, const double *L1d
   double *Zv = nullptr, *Zo = nullptr;
   TRY(jac_z_buffers(c, &Zv, &Zo, prep, st));
   const int rows = (nv + 7) / 8 * 8;
-  const int ks4 = S->ks4;
   const int Ec = ELt + S->Eg;
   JacPlans pT, pZ, pQ, pAB, pO;
   pT.v.resize(nb);
@@ -1796,7 +1806,8 @@ int split_left_jacobian(cc3_ctx *c, int nvec, const double *w, const double *L1d
   double ex = 0.0, ex_tau = 0.0;
   for (int b = 0; b < nb; ++b) {
     const int t0 = b * bj, t1 = std::min(c->ntri, t0 + bj);
-    SPlan tb, z, qp, ab, om;
+    SPlan tb, z, qp, ab, om, rest;
+    std::vector<VvovPerm> vperms;
     std::vector<GTerm> gterms;
     for (int t = t0; t < t1; ++t) {
       const int *ijk = &c->tri_host[3 * t];
@@ -1820,19 +1831,21 @@ int split_left_jacobian(cc3_ctx *c, int nvec, const double *w, const double *L1d
         w_terms_3(ab, j3, set1, no, nv, rows, vp, op, ijk, ex, s);
         // sigma2 (the residual's vvov and ooov contractions, no singles or F
         // columns), G and H of vector v
-        const size_t first = om.jobs.size();
-        plan_omega_split(om, S, no, nv, ijk, u, ks4, ex, 1 | 8);
-        plan_omega_split(om, S, no, nv, ijk, u, ks4, ex, 2 | 8);
-        for (size_t jx = first; jx < om.jobs.size(); ++jx) {
-          SJob &J = om.jobs[jx];
+        const size_t first = rest.jobs.size();
+        collect_vvov_perms(vperms, ijk, u, (long long)v * nt2);
+        plan_ooov(rest, S, no, nv, ijk, u, ex, true);
+        for (size_t jx = first; jx < rest.jobs.size(); ++jx) {
+          SJob &J = rest.jobs[jx];
           for (OutD *o : {&J.C, &J.Ct, &J.C2, &J.Ct2})
             if (o->buf == B_OMT) o->off += (long long)v * nt2;
         }
-        plan_left_split(&om, nullptr, &gterms, S, no, nv, ELt, nvec, ijk, u, v,
+        plan_left_split(&rest, nullptr, &gterms, S, no, nv, ELt, nvec, ijk, u, v,
                         (long long)v * nh, ex);
       }
     }
-    plan_left_g(om, S, no, nv, gterms, ng, ex);
+    plan_vvov(om, S, no, nv, vperms, ex, true);  // the long-K tiles first
+    plan_left_g(rest, S, no, nv, gterms, ng, ex);
+    append_plan(om, rest);
     TRY(s_upload_plan(tb, &pT.v[b], st));
     if (prep) TRY(s_upload_plan(z, &pZ.v[b], st));
     TRY(s_upload_plan(qp, &pQ.v[b], st));
@@ -2305,7 +2318,7 @@ size_t split_jacobian_footprint(int no, int nv, int s, int nvec) {
   auto sl = [&](long long rows, long long Kp, long long rps) {
     return arr_elems(Kp, rps, rows / rps, s) * sizeof(__nv_bfloat16);
   };
-  size_t b = sl((long long)no * no * nv, vp, nv) + 2 * sl((long long)no * no, (long long)nv * vp, no);
+  size_t b = sl((long long)no * no * nv, vp, nv) + sl((long long)no * no, (long long)nv * vp, no);
   size_t per = sl((long long)no * no * nv, vp, nv) + 2 * sl((long long)no * nv * nv, op, nv) +
                2 * sl((long long)no * nv * nv, vp, nv) + sl((long long)no * no * nv, op, nv);
   b += (size_t)nvec * per + sl((long long)no * nvec, vp, nvec);

@@ -828,10 +828,10 @@ split_engine_kernel(const SJob *__restrict__ jobs, int njobs, const STerm *__res
       const int es = seg2 ? J.expo_slot2 : J.expo_slot;
       const int e2 = J.expo + (es >= 0 ? slot_ex[es] : 0) - S_ACC_FRAC;
       const int mo = seg2 ? m - J.msplit : m;  // row within its output
-      const bool row_ok = m < J.M && !(J.m_pad > 0 && (m % J.m_pad) >= J.m_valid);
+      const bool row_ok = m < J.M && !(J.m_pad > 0 && (m + J.m_off) % J.m_pad >= J.m_valid);
       // the thread's row is fixed for the tile: its output row offsets once.
       // Main columns n < Nm go to C (C2 for second-segment rows), tail
-      // columns n in [tlo, thi) to Ct (Ct2); columns map linearly (n_in >= N,
+      // column tcol (tcol2) to Ct (Ct2); columns map linearly (n_in >= N,
       // checked when the plan is uploaded)
       const OutD &Cm = seg2 ? J.C2 : J.C;
       const long long rowM =
@@ -874,11 +874,8 @@ split_engine_kernel(const SJob *__restrict__ jobs, int njobs, const STerm *__res
             buf = Cm.buf;
           } else {  // tail columns are few: their offsets on the fly
             const OutD &Ctl = seg2 ? J.Ct2 : J.Ct;
-            const int tlo = seg2 ? (J.Nm2 > 0 ? J.Nm2 : J.N) : J.Nm;
-            const int thi = seg2 ? J.N : (J.Nm2 > 0 ? J.Nm2 : J.N);
-            if (n < tlo || n >= thi) continue;
-            off = Ctl.off + (long long)bi * Ctl.sb + s_rowoff(mo, Ctl.m_in, Ctl.sm1, Ctl.sm0) +
-                  (long long)(n - tlo) * Ctl.sn0;
+            if (n != (seg2 ? J.tcol2 : J.tcol)) continue;
+            off = Ctl.off + (long long)bi * Ctl.sb + s_rowoff(mo, Ctl.m_in, Ctl.sm1, Ctl.sm0);
             buf = Ctl.buf;
           }
           const double x = fixed_to_double(acc[0][k], e2);

@@ -76,21 +76,22 @@ struct SJob {
   int mode;
   int expo;       // result = 2^expo * (integer-scaled accumulators)
   int expo_slot;  // >= 0: add the per-triple exponent ex[expo_slot]
-  int m_pad, m_valid;  // m_pad > 0: rows with m % m_pad >= m_valid are padding
+  // m_pad > 0: rows with (m + m_off) % m_pad >= m_valid are padding
+  int m_pad, m_valid, m_off;
   int n_valid;         // columns n in [n_valid, Nm) are padding
   OutD C, Ct;  // output element (b, m, n) for n < Nm, resp. (b, m, n - Nm);
                // buffer of float2 (dd) or double
   // rows m >= msplit (msplit > 0) belong to a second output: main columns to
-  // C2 (row m - msplit), tail columns n >= Nm2 to Ct2 (column n - Nm2), with
-  // the per-triple exponent ex[expo_slot2]; rows below msplit take the tail
-  // columns [Nm, Nm2) only
-  int msplit, Nm2, expo_slot2;
+  // C2 (row m - msplit), with the per-triple exponent ex[expo_slot2].  Of the
+  // tail columns n >= Nm a row takes one: tcol to column 0 of Ct (tcol2 to
+  // that of Ct2 in the second segment); the others are padding
+  int msplit, expo_slot2, tcol, tcol2;
   OutD C2, Ct2;
   // route 1 (column pairs): columns [0, Nm2) and [Nm2, N) are two segments;
   // column j of a segment goes to C / C2 (j < Nm) or Ct / Ct2 (column j - Nm,
   // Nm <= j < Nm + tw); other columns are padding.  All four outputs share
   // m_in.  route 0: the row segments above.
-  int route, tw;
+  int route, tw, Nm2;
   int nv;
   long long tile_base;
 };

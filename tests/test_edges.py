@@ -70,6 +70,31 @@ def test_residual_at_slicing_edges(g, no, nv):
     assert split_close(o2, ref["omega2"]), split_err(o2, ref["omega2"])
 
 
+# permutations stacked along M in the vvov contraction: rows of 8, 64 and one past,
+# 128 and both sides; singles columns of q in one and in two groups of eight (no > 8),
+# the second of which ends on (nv = 80) and past (88) a column tile
+@pytest.mark.parametrize("no,nv", [(17, 5), (9, 31), (9, 64), (3, 65), (9, 80), (9, 88), (2, 127),
+                                   (2, 128), (3, 129)])
+def test_contractions_of_stacked_permutations(g, no, nv):
+    inp = make_inputs(no, nv, seed=no + 2 * nv)
+    ref = oracle.omega_inputs(inp)
+    ctx = g.Context(inp)
+    o1, o2, _ = ctx.omega(g.CC3_SPLIT_BF16)
+    assert split_close(o1, ref["omega1"]), split_err(o1, ref["omega1"])
+    assert split_close(o2, ref["omega2"]), split_err(o2, ref["omega2"])
+    if no * nv > 500:
+        return
+    R1, R2 = make_trial_vectors(no, nv, 2, seed=9)
+    ref = oracle.jacobian(inp, R1, R2, [0.2, -0.1])
+    got = ctx.jacobian(R1, R2, [0.2, -0.1], g.CC3_SPLIT_BF16)
+    for x, k in zip(got, ("rho1", "rho2")):
+        assert split_close(x, ref[k]), split_err(x, ref[k])
+    ref = oracle.left_jacobian(inp, R1, R2, [0.2, -0.1])
+    got = ctx.left_jacobian(R1, R2, [0.2, -0.1], g.CC3_SPLIT_BF16)
+    for x, k in zip(got, ("sigma1", "sigma2")):
+        assert split_close(x, ref[k]), split_err(x, ref[k])
+
+
 def test_densities_beyond_one_group_of_blocks(g):
     # 66 occupied orbitals: 17 x 17 blocks of 4 x 4 products, two groups of 256
     no, nv = 66, 3
