@@ -221,21 +221,24 @@ __global__ void maxabs_kernel(const double *__restrict__ x, long long n,
 // O = tau^{acb} + tau^{cba} + tau^{bac},
 //   tau~ at an even permutation (abc, bca, cab) = 3 tau^{itself} + E - 2 O,
 //   tau~ at an odd one (acb, cba, bac)           = 3 tau^{itself} + O - 2 E.
-// A block takes one triple of 8-cube indices A >= B >= C, forms tau for the
-// (up to six distinct) cubes whose index triples permute it and stages them
-// in shared memory (coalesced row reads), forms all six outputs of each of
-// its points from the six staged values, and writes the output cubes back
-// row by row: every partial sum is read once and every tau~ element written
+// A block takes one triple of 8-cube indices A >= B >= C, sums the partial sums
+// of the (up to six distinct) cubes whose index triples permute it into shared
+// memory (coalesced row reads), forms all six outputs of each of its points
+// from the six staged sums, which share one denominator, and writes the output
+// cubes back row by row: every partial sum is read once and every tau~ element written
 // once.  The locations a block reads are exactly those it writes (the cubes
 // of one permutation orbit, in either layout), so TT may alias W_2: each
 // block reads all of its locations before it writes any.  When cube indices
 // coincide, only points with a >= b (A = B) and b >= c (B = C) are formed,
 // so that each output is produced by one thread.
-// Bound by instruction issue (252 instructions per element before, 74 % of the
-// issue slots, DRAM 46 %): the element offsets within a slot are 32-bit and a
-// thread's two elements of a cube differ by 4 planes only, and the padded
-// strides keep the six permuted reads of a warp nearly free of bank conflicts
-// (3.8 per read with strides 8 and 65).
+// Bound by the L1 pipe (78 % of its peak; the cubes' rows are 64 bytes, four to
+// a request) and instruction issue (65 %), DRAM at 52 %.  The element offsets
+// within a slot are 32-bit and a thread's two elements of a cube differ by 4
+// planes only; the padded strides keep the six permuted reads of a warp nearly
+// free of bank conflicts (3.8 per read with strides 8 and 65); a point's
+// reciprocal stays in the registers of the thread that forms its orbit (staging
+// tau through a shared table of reciprocals: 24.7 ms for the batches of no=16
+// nv=160, so 23.4); packed dd additions, 25.1 -> 24.7.
 constexpr int CV_SX = 9, CV_SZ = 74, CV_SLOT = 8 * CV_SZ;  // padded cube strides (float2)
 __global__ void __launch_bounds__(256, 4)
 tau_contravariant_dd_kernel(const float2 *__restrict__ W1, const float2 *W2,
@@ -301,31 +304,26 @@ tau_contravariant_dd_kernel(const float2 *__restrict__ W1, const float2 *W2,
     }
   };
   issue(0);
-  // 1 / (w + e_ijk - e_a - e_b - e_c) at every point (a, b, c) of cube (A, B, C):
-  // the six permuted points of the orbit share it, so each is formed once
-  // (one dd division per orbit point instead of one per staged element)
-  __shared__ float2 rcp[512];
-  for (int u = t; u < 512; u += 256) {
-    const int a = u >> 6, b = (u >> 3) & 7, c = u & 7;
-    const int ga = A * 8 + a, gb = B * 8 + b, gc = C * 8 + c;
+  // 1 / (w + e_ijk - e_a - e_b - e_c) at this thread's two points (a, b, c) of
+  // cube (A, B, C): the six permuted points of an orbit share it
+  dd::df rcp[2];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int ga = A * 8 + u0 + 4 * h, gb = B * 8 + u1, gc = C * 8 + u2;
+    rcp[h] = dd::df{0.f, 0.f};
     if (ga >= nv || gb >= nv || gc >= nv) continue;
     const float2 ea = ev[ga], eb = ev[gb], ec = ev[gc];
     const dd::df d = dd::add(dd::add(dd::add(wo, dd::df{-ea.x, -ea.y}), dd::df{-eb.x, -eb.y}),
                              dd::df{-ec.x, -ec.y});
-    const dd::df r = dd::div(dd::df{1.f, 0.f}, d);
-    rcp[u] = make_float2(r.hi, r.lo);
+    rcp[h] = dd::div(dd::df{1.f, 0.f}, d);
   }
-  __syncthreads();
-  // stage tau^{xyz} of cube (X, Y, Z) at [z][x][y] (y contiguous in memory);
-  // its point (x, y, z) is the point (a, b, c) of cube (A, B, C) with each
-  // index moved to the slot of its cube index
+  // stage W_1 + W_2 + W_3 of cube (X, Y, Z) at [z][x][y] (y contiguous in memory)
   auto stage = [&](int q0) {
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
       const int q = q0 + k;
       if (slot[q] != q) continue;
-      const int x = u1, y = u2;
-      const bool in = cx[q] * 8 + x < nv && cy[q] * 8 + y < nv;
+      const bool in = cx[q] * 8 + u1 < nv && cy[q] * 8 + u2 < nv;
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const int z = u0 + 4 * h;
@@ -334,14 +332,9 @@ tau_contravariant_dd_kernel(const float2 *__restrict__ W1, const float2 *W2,
           const float2 a1 = la[k][h][0], a2 = la[k][h][1], a3 = la[k][h][2];
           const dd::df sum =
               dd::add(dd::add(dd::df{a1.x, a1.y}, dd::df{a2.x, a2.y}), dd::df{a3.x, a3.y});
-          // (a, b, c) of this point: abc, acb, cba, bac, bca, cab orders of q
-          const int pa[6] = {x, x, z, y, z, y}, pb[6] = {y, z, y, x, x, z},
-                    pc[6] = {z, y, x, z, y, x};
-          const float2 r = rcp[pa[q] * 64 + pb[q] * 8 + pc[q]];
-          const dd::df tau = dd::mul(sum, dd::df{r.x, r.y});
-          v = make_float2(tau.hi, tau.lo);
+          v = make_float2(sum.hi, sum.lo);
         }
-        sm[q][z * CV_SZ + x * CV_SX + y] = v;
+        sm[q][z * CV_SZ + u1 * CV_SX + u2] = v;
       }
     }
   };
@@ -351,8 +344,39 @@ tau_contravariant_dd_kernel(const float2 *__restrict__ W1, const float2 *W2,
   issue(4);
   stage(4);
   __syncthreads();
+  dd::df v[2][6];
+  bool own[2];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int p = t + 256 * h, a = p >> 6, b = (p >> 3) & 7, c = p & 7;
+    const int ga = A * 8 + a, gb = B * 8 + b, gc = C * 8 + c;
+    own[h] = ga < nv && gb < nv && gc < nv && !(A == B && ga < gb) && !(B == C && gb < gc);
+    // term q's element sits at its cube's [z][x][y] with (x, y, z) the
+    // permuted (a, b, c)
+    const int off[6] = {c * CV_SZ + a * CV_SX + b, b * CV_SZ + a * CV_SX + c,
+                        a * CV_SZ + c * CV_SX + b, c * CV_SZ + b * CV_SX + a,
+                        a * CV_SZ + b * CV_SX + c, b * CV_SZ + c * CV_SX + a};
+#pragma unroll
+    for (int q = 0; q < 6; ++q) {
+      const float2 w = sm[slot[q]][off[q]];
+      v[h][q] = dd::mul(dd::df{w.x, w.y}, rcp[h]);  // tau
+    }
+  }
+  __syncthreads();  // every staged value read: the cubes now take the outputs
   if (tau_out) {  // tau itself, [slot][a][b][c] like tau~ (the densities' D_vv and D_oo)
     float mt = 0.f;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      if (!own[h]) continue;
+      const int a = u0 + 4 * h, b = u1, c = u2;
+      const int off[6] = {c * CV_SZ + a * CV_SX + b, b * CV_SZ + a * CV_SX + c,
+                          a * CV_SZ + c * CV_SX + b, c * CV_SZ + b * CV_SX + a,
+                          a * CV_SZ + b * CV_SX + c, b * CV_SZ + c * CV_SX + a};
+#pragma unroll
+      for (int q = 0; q < 6; ++q)
+        sm[slot[q]][off[q]] = make_float2(v[h][q].hi, v[h][q].lo);
+    }
+    __syncthreads();
 #pragma unroll
     for (int q = 0; q < 6; ++q) {
       if (slot[q] != q) continue;
@@ -369,26 +393,8 @@ tau_contravariant_dd_kernel(const float2 *__restrict__ W1, const float2 *W2,
     }
     for (int o = 16; o > 0; o >>= 1) mt = fmaxf(mt, __shfl_xor_sync(0xffffffffu, mt, o));
     if ((t & 31) == 0) atomicMax(maxtau + blockIdx.y, __float_as_uint(mt));
+    __syncthreads();
   }
-  dd::df v[2][6];
-  bool own[2];
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    const int p = t + 256 * h, a = p >> 6, b = (p >> 3) & 7, c = p & 7;
-    const int ga = A * 8 + a, gb = B * 8 + b, gc = C * 8 + c;
-    own[h] = ga < nv && gb < nv && gc < nv && !(A == B && ga < gb) && !(B == C && gb < gc);
-    // term q's element sits at its cube's [z][x][y] with (x, y, z) the
-    // permuted (a, b, c)
-    const int off[6] = {c * CV_SZ + a * CV_SX + b, b * CV_SZ + a * CV_SX + c,
-                        a * CV_SZ + c * CV_SX + b, c * CV_SZ + b * CV_SX + a,
-                        a * CV_SZ + b * CV_SX + c, b * CV_SZ + c * CV_SX + a};
-#pragma unroll
-    for (int q = 0; q < 6; ++q) {
-      const float2 w = sm[slot[q]][off[q]];
-      v[h][q] = dd::df{w.x, w.y};
-    }
-  }
-  __syncthreads();  // every staged value read: the cubes now take the outputs
   float mx = 0.f;
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
@@ -610,7 +616,8 @@ __global__ void to_dd_kernel(const double *__restrict__ x, float2 *__restrict__ 
 // per element): a warp takes a row (c, a), so that no element divides its
 // index, with b along the lanes, and every factor that varies along b is read
 // contiguously.  At no=12 nv=120 the six terms of each element, with their
-// 64-bit index divisions, took 11.0 ms per density.
+// 64-bit index divisions, took 11.0 ms per density;
+// this form takes 5.7 (6.8 before the additions were packed).
 __global__ void __launch_bounds__(256)
 left_outer_dd_kernel(float2 *__restrict__ W3, const int *__restrict__ tri, int bj, int ns,
                      const float2 *__restrict__ L1, const float2 *__restrict__ Lt,
