@@ -468,15 +468,19 @@ __global__ void common_exponent_kernel(const unsigned int *__restrict__ maxbits,
 // ooov and F contractions.  One CTA converts a 16^3 cube of tau~ (read along
 // its innermost index) into digits once, keeps them in shared memory, and
 // writes the cube into all three layouts as whole 16-byte core rows.
-// Digit cube in shared memory: element (a, b, c) of slice p at
-// p * TT_PLANE + a * TT_APLANE + b * TT_PAD + c (bf16).  The a-plane stride is
-// an odd number of 4-byte words, so that the 16 lanes of a layout-0 read
-// (consecutive a) fall in distinct banks.
-constexpr int TT_PAD = 18, TT_APLANE = 16 * TT_PAD + 2, TT_PLANE = 16 * TT_APLANE;
+// Digit cube in shared memory: slices 2 q and 2 q + 1 of element (a, b, c) are the
+// halves of word q * TT_PLANE + a * TT_APLANE + b * TT_PAD + c.  With these
+// strides a warp's writes and its reads in the three layouts take 2, 1, 2 and 2
+// wavefronts (no strides that fit four blocks to an SM take fewer in sum).
+// Staged as single bf16 digits (24 two-byte accesses an element), the kernel was
+// limited by the shared-memory pipe and issue (58 % each) at 5.6 TB/s; in pairs it
+// moves 6.3 TB/s: no=16 nv=160 residual 25.4 -> 22.7 ms, no=12 nv=120 density 17.7 ->
+// 15.8 ms.
+constexpr int TT_PAD = 17, TT_APLANE = 16 * TT_PAD + 2, TT_PLANE = 16 * TT_APLANE;
 __global__ void __launch_bounds__(256)
 slice_tt_kernel(const float2 *__restrict__ tt, __nv_bfloat16 *const *__restrict__ v, int nv,
                 int vp, int s, int *__restrict__ ex, const unsigned int *__restrict__ maxbits) {
-  extern __shared__ __nv_bfloat16 dig[];  // [p][a][b][c] (c padded to TT_PAD)
+  extern __shared__ uint32_t dig[];  // [slice pair][a][b][c] (c padded to TT_PAD)
   const int nx = (nv + 15) / 16, nzb = vp / 16;
   int blk = blockIdx.x;
   const int cb = blk % nx;
@@ -490,7 +494,6 @@ slice_tt_kernel(const float2 *__restrict__ tt, __nv_bfloat16 *const *__restrict_
   const int e = maxbits ? exponent_of_max(maxbits[slot]) : ex[slot];
   if (maxbits && blockIdx.x == 0 && threadIdx.x == 0) ex[slot] = e;
   const int sh = 7 + 8 * (s - 1) - e;
-  const int plane = TT_PLANE;
   // 2^sh and 2^(sh-24) as floats (the 32-bit digit path of s = 6)
   const float s0 = ldexpf(1.f, sh), s24 = ldexpf(1.f, sh - 24);
   // 16 elements per thread, loaded 8 at a time before any is converted (the
@@ -555,8 +558,12 @@ slice_tt_kernel(const float2 *__restrict__ tt, __nv_bfloat16 *const *__restrict_
       }
       const int o = a * TT_APLANE + b * TT_PAD + c;
 #pragma unroll
-      for (int p = 0; p < S_MAX_SLICES_K; ++p)
-        if (p < s) dig[p * plane + o] = __float2bfloat16_rn(d[p] * slice_scale(p));
+      for (int p = 0; p < S_MAX_SLICES_K; p += 2)
+        if (p < s) {
+          const float d1 = p + 1 < s ? d[p + 1] * slice_scale(p + 1) : 0.f;
+          const __nv_bfloat162 w = __floats2bfloat162_rn(d[p] * slice_scale(p), d1);
+          dig[p / 2 * TT_PLANE + o] = *reinterpret_cast<const uint32_t *>(&w);
+        }
     }
   }
   __syncthreads();
@@ -577,9 +584,9 @@ slice_tt_kernel(const float2 *__restrict__ tt, __nv_bfloat16 *const *__restrict_
     for (int h = 0; h < 2; ++h) {
       const long long o = blk0 + cm_off(gx, h * 8, s);
 #pragma unroll 1
-      for (int p = 0; p < s; ++p) {
-        const __nv_bfloat16 *D = dig + p * plane;
-        __align__(16) __nv_bfloat16 out[8];
+      for (int p = 0; p < s; p += 2) {
+        const uint32_t *D = dig + p / 2 * TT_PLANE;
+        uint32_t w[8];
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
           const int z = h * 8 + e;
@@ -587,9 +594,14 @@ slice_tt_kernel(const float2 *__restrict__ tt, __nv_bfloat16 *const *__restrict_
           const int a = L == 0 ? x : (L == 1 ? z : y);
           const int b = L == 0 ? y : (L == 1 ? x : z);
           const int c = L == 0 ? z : (L == 1 ? y : x);
-          out[e] = D[a * TT_APLANE + b * TT_PAD + c];
+          w[e] = D[a * TT_APLANE + b * TT_PAD + c];
         }
-        *reinterpret_cast<uint4 *>(dst + p * 128 + o) = *reinterpret_cast<const uint4 *>(out);
+        uint4 *to = reinterpret_cast<uint4 *>(dst + p * 128 + o);
+        to[0] = make_uint4(__byte_perm(w[0], w[1], 0x5410), __byte_perm(w[2], w[3], 0x5410),
+                           __byte_perm(w[4], w[5], 0x5410), __byte_perm(w[6], w[7], 0x5410));
+        if (p + 1 < s)
+          to[16] = make_uint4(__byte_perm(w[0], w[1], 0x7632), __byte_perm(w[2], w[3], 0x7632),
+                              __byte_perm(w[4], w[5], 0x7632), __byte_perm(w[6], w[7], 0x7632));
       }
     }
   }
@@ -760,7 +772,7 @@ int launch_slice_tt(const float2 *tt, __nv_bfloat16 *const *v, int nv, int vp, i
   if (vp / 16 != (nv + 15) / 16 || s < 1 || s > S_MAX_SLICES_K)
     return CC3_FAIL(CC3_ERR_ARG, "slice_tt layout");
   const int nx = (nv + 15) / 16;
-  const size_t smem = (size_t)s * TT_PLANE * sizeof(__nv_bfloat16);
+  const size_t smem = (size_t)((s + 1) / 2) * TT_PLANE * sizeof(uint32_t);
   {
     static std::mutex mu;
     static bool set[64] = {false};
@@ -768,7 +780,7 @@ int launch_slice_tt(const float2 *tt, __nv_bfloat16 *const *v, int nv, int vp, i
     cudaGetDevice(&dev);
     std::lock_guard<std::mutex> lk(mu);
     if (dev >= 0 && dev < 64 && !set[dev]) {
-      const size_t mx = (size_t)S_MAX_SLICES_K * TT_PLANE * sizeof(__nv_bfloat16);
+      const size_t mx = (size_t)((S_MAX_SLICES_K + 1) / 2) * TT_PLANE * sizeof(uint32_t);
       if (cudaFuncSetAttribute(slice_tt_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)mx) != cudaSuccess)
         return CC3_FAIL(CC3_ERR_CUDA, "slice_tt shared memory");

@@ -70,6 +70,21 @@ def test_residual_at_slicing_edges(g, no, nv):
     assert split_close(o2, ref["omega2"]), split_err(o2, ref["omega2"])
 
 
+@pytest.mark.parametrize("slices", [3, 4, 5, 7])
+def test_residual_with_other_slice_counts(g, slices):
+    # odd counts leave the last pair of slices half filled; each slice less costs 8 bits
+    # of the 1e-10 that six are held to
+    inp = make_inputs(4, 19, seed=11)
+    ref = oracle.omega_inputs(inp)
+    ctx = g.Context(inp)
+    g.cc3_ctx_set_slices(ctx.ctx, slices)
+    got = ctx.omega(g.CC3_SPLIT_BF16)
+    tol = 1e-10 * max(1.0, 256.0 ** (6 - slices))
+    for x, k in zip(got, ("omega1", "omega2")):
+        err, scale = split_err(x, ref[k])
+        assert err <= tol * scale, (err, scale)
+
+
 # permutations stacked along M in the vvov contraction: rows of 8, 64 and one past,
 # 128 and both sides; singles columns of q in one and in two groups of eight (no > 8),
 # the second of which ends on (nv = 80) and past (88) a column tile
