@@ -403,7 +403,7 @@ int density_fp64(cc3_ctx *c, double w, const double *L1d, const double *L2d, dou
 // the low sum; the pair is renormalised after every chunk.  The terms keep
 // ~2^-44 of their size, well inside the FP64 path's agreement.  At no=12 nv=120
 // one thread per product, half of them idle, with rows read element by element
-// took 28.6 ms; this one 18.5 ms.
+// took 28.6 ms; this one 18.5 ms, 14.8 with the grid chosen as below.
 constexpr int DOO_E = 128, DOO_T = 4, DOO_PF = 12;
 __host__ __device__ constexpr int doo_rows(int no) { return (no + DOO_T - 1) / DOO_T * DOO_T; }
 __global__ void __launch_bounds__(256)
@@ -610,8 +610,18 @@ int density_doo_resident(cc3_ctx *c, const float2 *tau_all, const float2 *lt_all
   CU(cudaGetDevice(&dev));
   CU(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
   const int gz = (doo_rows(no) / DOO_T * (doo_rows(no) / DOO_T) + 255) / 256;
-  const long long gx = std::max<long long>(
-      1, std::min<long long>(nunit, (4LL * nsm + (long long)npair * gz - 1) / ((long long)npair * gz)));
+  // blocks per pair: of up to 32 blocks per SM in all, the number whose rounds
+  // over the SMs take the fewest units (one more per block for its start and
+  // reduction).  At no=12 nv=120 about four blocks per SM, 8 per pair, were 2.05
+  // rounds of two per SM: 18.4 ms; this rule takes 35 per pair, 8.98 rounds, 14.8 ms.
+  int per_sm = 0;
+  CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, doo_pairs_kernel, 256, smem));
+  const long long slots = (long long)std::max(1, per_sm) * nsm, per_gx = (long long)npair * gz;
+  long long gx = 1, least = -1;
+  for (long long x = 1; x <= nunit && (x == 1 || x * per_gx <= 32LL * nsm); ++x) {
+    const long long units = (x * per_gx + slots - 1) / slots * ((nunit + x - 1) / x + 1);
+    if (least < 0 || units < least) least = units, gx = x;
+  }
   trace_begin(c, TR_FP64_ELEM, s);
   doo_pairs_kernel<<<dim3((unsigned)gx, npair, gz), 256, smem, s>>>(lt_all, tau_all, dtab, dw, no,
                                                                      nv, ld, C);
