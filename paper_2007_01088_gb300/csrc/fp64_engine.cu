@@ -171,20 +171,17 @@ fp64_engine_kernel(const Job *__restrict__ jobs, int njobs,
 static long long split_small_launch(std::vector<Job> &jobs, const std::vector<Term> &terms) {
   constexpr double FILL = 608.0;
   double work = 0.0;
-  auto longest = [&](const Job &j) {
-    int k = 0;
-    for (int t = 0; t < j.nterm; ++t) k = std::max(k, terms[j.term0 + t].K);
+  auto length = [&](const Job &j) {  // K of a tile: of all its terms
+    long long k = 0;
+    for (int t = 0; t < j.nterm; ++t) k += terms[j.term0 + t].K;
     return k;
   };
-  for (const Job &j : jobs) {
-    double k = 0.0;
-    for (int t = 0; t < j.nterm; ++t) k += terms[j.term0 + t].K;
-    work += k * j.tiles_m * j.tiles_n * j.batch;
-  }
+  for (const Job &j : jobs) work += (double)length(j) * j.tiles_m * j.tiles_n * j.batch;
   const int chunk = (int)std::min(1e9, std::max(64.0, work / FILL));
   long long tiles = 0;
   for (Job &j : jobs) {
-    if (j.mode == EPI_ATOMIC) j.ksplit = std::max(j.ksplit, (longest(j) + chunk - 1) / chunk);
+    if (j.mode == EPI_ATOMIC)
+      j.ksplit = (int)std::max<long long>(j.ksplit, (length(j) + chunk - 1) / chunk);
     j.tile_base = tiles;
     tiles += (long long)j.batch * j.tiles_m * j.tiles_n * j.ksplit;
   }
