@@ -30,6 +30,35 @@ __device__ __forceinline__ long long rowoff(int m, int m_in, long long s1,
   return (long long)(m / m_in) * s1 + (long long)(m % m_in) * s0;
 }
 
+// acc += the products of the first im of a thread's TM rows and jn of its TN
+// columns over kn values of K.  One body per (im, jn), found by descent from
+// (IM, JN): a multiply-add under a predicate takes its turn in the FP64 pipe
+// even where it is off, so that a tile of one column group in four took as long
+// as a full one.  no=6 nv=48 FP64 residual 8.54 -> 7.31 ms; dressing of the integrals
+// at no=16 nv=128: columns of 16 0.82 -> 0.23 ms, K = 16 2.85 -> 1.89 ms per vector.
+template <int BM, int BN, int TM, int TN, int IM, int JN>
+__device__ __forceinline__ void products(int im, int jn, int kn, const double *a0, const double *b0,
+                                         double (&acc)[TM][TN]) {
+  if constexpr (IM > 1) {
+    if (im < IM) return products<BM, BN, TM, TN, IM - 1, JN>(im, jn, kn, a0, b0, acc);
+  }
+  if constexpr (JN > 1) {
+    if (jn < JN) return products<BM, BN, TM, TN, IM, JN - 1>(im, jn, kn, a0, b0, acc);
+  }
+#pragma unroll 4
+  for (int kk = 0; kk < kn; ++kk) {
+    double a[IM], b[JN];
+#pragma unroll
+    for (int i = 0; i < IM; ++i) a[i] = a0[kk * (BM + 1) + i * (BM / TM)];
+#pragma unroll
+    for (int j = 0; j < JN; ++j) b[j] = b0[kk * (BN + 1) + j * (BN / TN)];
+#pragma unroll
+    for (int i = 0; i < IM; ++i)
+#pragma unroll
+      for (int j = 0; j < JN; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+  }
+}
+
 template <int BM, int BN, int TM, int TN, int BK>
 __global__ void __launch_bounds__(256)
 fp64_engine_kernel(const Job *__restrict__ jobs, int njobs,
@@ -110,22 +139,7 @@ fp64_engine_kernel(const Job *__restrict__ jobs, int njobs,
       }
       __syncthreads();
       const int kn = min(BK, kend - k0);  // the occupied sums are short
-#pragma unroll
-      for (int kk = 0; kk < BK; ++kk) {
-        if (kk >= kn) break;
-        double a[TM], b[TN];
-#pragma unroll
-        for (int i = 0; i < TM; ++i) a[i] = i < im ? sA[kk][ty + i * GM] : 0.0;
-#pragma unroll
-        for (int j = 0; j < TN; ++j) b[j] = j < jn ? sB[kk][tx + j * GN] : 0.0;
-#pragma unroll
-        for (int i = 0; i < TM; ++i) {
-          if (i >= im) break;
-#pragma unroll
-          for (int j = 0; j < TN; ++j)
-            if (j < jn) acc[i][j] = fma(a[i], b[j], acc[i][j]);
-        }
-      }
+      products<BM, BN, TM, TN, TM, TN>(im, jn, kn, &sA[0][ty], &sB[0][tx], acc);
       __syncthreads();
     }
   }

@@ -121,9 +121,9 @@ def test_densities_beyond_one_group_of_blocks(g):
         assert split_close(x, y), split_err(x, y)
 
 
-# FP64 tiles whose row and column groups end one past, on and one before a multiple
+# FP64 tiles of one to four row and column groups, ending one past, on and one before a multiple
 # of 16, short sums (K = no) and launches split over K (left: 3 tiles, K = 3 n nv)
-@pytest.mark.parametrize("no,nv", [(3, 15), (3, 16), (2, 17), (2, 65)])
+@pytest.mark.parametrize("no,nv", [(3, 15), (3, 16), (2, 17), (2, 40), (2, 65)])
 def test_fp64_left_at_tile_edges(g, no, nv):
     inp = make_inputs(no, nv, seed=no + nv)
     L1, L2 = make_trial_vectors(no, nv, 2, seed=7)
