@@ -178,12 +178,14 @@ fp64_engine_kernel(const Job *__restrict__ jobs, int njobs,
 }
 
 // Splits the accumulating jobs of a launch over K so that its work spreads
-// over FILL tiles (four per SM): a chunk of K is the launch's total K x tiles
+// over FILL tiles (eight per SM): a chunk of K is the launch's total K x tiles
 // over FILL, at least 64.  Launches of many tiles keep their jobs whole.
 // sigma1's Cholesky contraction at no=9 nv=81 (an 81 x 9 output over K =
-// 21,870: 3 tiles) took 9 ms on 3 SMs.
+// 21,870: 3 tiles) took 9 ms on 3 SMs.  Four tiles per SM, many of them of five
+// on some: no=6 nv=48 FP64 residual 7.29 ms for 6.97, the left transformation's
+// thin launches at no=9 nv=81 2.12 ms for 1.71; 16 per SM take as long as 8.
 static long long split_small_launch(std::vector<Job> &jobs, const std::vector<Term> &terms) {
-  constexpr double FILL = 608.0;
+  constexpr double FILL = 1216.0;
   double work = 0.0;
   auto length = [&](const Job &j) {  // K of a tile: of all its terms
     long long k = 0;
