@@ -124,10 +124,10 @@ int build_omega_plans(cc3_ctx *c, cudaStream_t s) {
       // vvov: its own block for general integrals, else a view of vvvo
       plan_omega_contractions(pom, no, nv, ijk, slot, B_WS_TT, B_OVOV, B_FOV,
                               B_OOOV, !c->general, c->general ? B_VVOV : B_VVVO, B_OMT,
-                              B_OM1, 2, 1);
+                              B_OM1, 2, 1 | 16);
       plan_omega_contractions(pth, no, nv, ijk, slot, B_WS_TT, B_OVOV, B_FOV,
                               B_OOOV, !c->general, c->general ? B_VVOV : B_VVVO, B_OMT,
-                              B_OM1, 1, 2);
+                              B_OM1, 1, 2 | 16);
     }
     executed += plan_flops(pab) + plan_flops(pc) + plan_flops(pom) + plan_flops(pth);
     DevPlan d;

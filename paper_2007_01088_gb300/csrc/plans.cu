@@ -173,7 +173,8 @@ void plan_w_build(Plan &P, int no, int nv, const int ijk[3], int slot,
 // which: bit 0 = vvov + singles job (64x64 tiles), bit 1 = ooov + F job (thin),
 //        bit 2 = F-only job (thin; Jacobian tau~ . F^ term), bit 3 = leave out
 //        the singles and F tail columns of the first two (the left
-//        transformation's sigma2 contractions).
+//        transformation's sigma2 contractions), bit 4 lets the singles columns
+//        move to the jobs of bit 1 (set in both calls or in neither).
 void plan_omega_contractions(Plan &P, int no, int nv, const int ijk[3],
                              int slot, int buf_tt, int buf_ovov, int buf_fov,
                              int buf_ooov, bool vvov_from_vvvo, int buf_vvov,
@@ -182,6 +183,10 @@ void plan_omega_contractions(Plan &P, int no, int nv, const int ijk[3],
                                   {0, 2, 1}, {1, 2, 0}, {2, 0, 1}};
   const long long nv2 = (long long)nv * nv, nv3 = nv2 * nv;
   const long long st[3] = {nv2, nv, 1};  // tau~[a][b][c] slot strides
+  // a multiple of 16 leaves the singles column a group of 16 columns of its own
+  // (64 x 64 tiles); in the thin tiles' 4 columns it costs a third of that: no=6
+  // nv=48 residual 6.97 -> 6.72 ms.  At other nv it rides in the last group.
+  const bool own_tail = (which & 16) && nv % 16 == 0;
   int seen[6][3];
   int nseen = 0;
   if (ijk[0] == ijk[1] && ijk[1] == ijk[2]) return;
@@ -200,7 +205,8 @@ void plan_omega_contractions(Plan &P, int no, int nv, const int ijk[3],
     if (which & 1) {
       // Omega~^{ad}_{pq} += sum_{yz} V[x][y][z] vvov[d][y][r][z]   (N = nv)
       // Omega1^x_p       += sum_{yz} V[x][y][z] ovov[q][y][r][z]   (tail col)
-      int jb = new_job(P, 0, nv, (which & 8) ? nv : nv + 1, nv, 1, ksplit, EPI_ATOMIC);
+      int jb = new_job(P, 0, nv, (which & 8) || own_tail ? nv : nv + 1, nv, 1, ksplit,
+                       EPI_ATOMIC);
       Opnd A = with_k2(op(buf_tt, tt0, st[m[0]], st[m[2]]), nv, st[m[1]]);
       Opnd B;
       if (vvov_from_vvvo)  // vvov[d][y][r][z] = vvvo[y][d][z][r]
@@ -213,6 +219,14 @@ void plan_omega_contractions(Plan &P, int no, int nv, const int ijk[3],
       add_term(P, jb, A, B, (int)nv2, &Bt);
       P.jobs[jb].C = out(buf_omt, ((long long)p * no + q) * nv2, nv, 1);
       P.jobs[jb].Ct = out(buf_om1, (long long)p * nv, 1, 0);
+    }
+    if ((which & 2) && own_tail) {  // the tail column of the job above
+      int jb = new_job(P, 1, nv, 1, 0, 1, 1, EPI_ATOMIC);
+      const Opnd A = with_k2(op(buf_tt, tt0, st[m[0]], st[m[2]]), nv, st[m[1]]);
+      const Opnd Bt = with_k2(
+          op(buf_ovov, (long long)q * nv * no * nv + (long long)r * nv, 0, 1), nv, (long long)no * nv);
+      add_term(P, jb, A, Bt, (int)nv2, &Bt);
+      P.jobs[jb].C = P.jobs[jb].Ct = out(buf_om1, (long long)p * nv, 1, 0);
     }
     if (which & 2) {
       // Omega~^{xy}_{pl} -= sum_z V[x][y][z] ooov[q][l][r][z]     (N = no)
