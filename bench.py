@@ -61,13 +61,13 @@ WORKLOADS = {
 
 
 # DRAM traffic per launch (dram__bytes_read.sum + dram__bytes_write.sum) of
-# the dominant kernel, averaged over the 668 engine launches of one residual
+# the dominant kernel, averaged over 300 engine launches of one residual
 # evaluation of the benchmark workload (one-pass capture of the full
 # workload); None where no capture of the current kernel exists.
-TRAFFIC = {("split_engine_kernel", 22, 250): 15.562e9}
+TRAFFIC = {("split_engine_kernel", 22, 250): 18.521e9}
 TRAFFIC_NOTE = {("split_engine_kernel", 22, 250):
-                "mean of 334 W-build launches (8.00 GB read, 2.23 GB written) and 334 "
-                "contraction launches (20.56 GB read, 0.34 GB written), 6 triples per batch"}
+                "mean of 150 W-build launches (7.99 GB read, 2.23 GB written) and 150 "
+                "contraction launches (26.47 GB read, 0.35 GB written), 6 triples per batch"}
 
 
 def peaks():
