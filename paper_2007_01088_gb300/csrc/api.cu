@@ -336,9 +336,10 @@ const char *cc3_strerror(int status) {
 
 void cc3_ctx_destroy(cc3_ctx *c) {
   if (!c) return;
-  cudaDeviceSynchronize();  // the context's last call may still run, on any stream
-  cudaGetLastError();
-  ctx_release(c, nullptr);
+  // the context's last call may still run, on any stream
+  DeviceScope dev(c->device);
+  cudaStream_t s = ctx_free_stream(c);
+  if (ctx_order(c, s)) ctx_release(c, s);
 }
 
 }  // extern "C"
@@ -366,6 +367,7 @@ void ctx_release(cc3_ctx *c, cudaStream_t s) {
   if (c->status) dev_free(c->status);
   if (c->omt_fx) dev_free(c->omt_fx);
   if (c->om1_fx) dev_free(c->om1_fx);
+  if (c->done) cudaEventDestroy(c->done);
   delete c;
   dev_ctx_gone();
 }
@@ -492,26 +494,29 @@ int cc3_ctx_create_general(cc3_ctx **out, int no, int nv, const double *eps_o,
 int cc3_ctx_set_triples(cc3_ctx *c, int ntri, const int *ijk) {
   if (!c || ntri < 0) return CC3_ERR_ARG;
   std::lock_guard<std::mutex> lk(c->mu);
-  if (ntri == 0 || !ijk) {
-    default_triples(c);
-  } else {
-    std::vector<int> v(ijk, ijk + 3 * (size_t)ntri);
+  std::vector<int> v;
+  if (ntri > 0 && ijk) {
+    v.assign(ijk, ijk + 3 * (size_t)ntri);
     for (int t = 0; t < ntri; ++t) {
       const int i = v[3 * t], j = v[3 * t + 1], k = v[3 * t + 2];
       if (!(i < c->no && i >= j && j >= k && k >= 0)) return CC3_ERR_ARG;
     }
+  }
+  // the buffers freed below may be in use by an earlier call, on any stream
+  DeviceScope dev(c->device);
+  cudaStream_t side = dev_side_stream();
+  if (!ctx_order(c, side)) return CC3_FAIL(CC3_ERR_CUDA, "the context's work cannot be waited for");
+  CallScope scope(c, side);
+  if (v.empty()) {
+    default_triples(c);
+  } else {
     c->tri_host = v;
     c->ntri = ntri;
   }
-  // the buffers freed below may be in use by an earlier call, on any stream
-  cudaDeviceSynchronize();
-  cudaGetLastError();
-  StreamScope scope(nullptr);
   const int nb = choose_batch(c);
   if (nb != c->batch) {
     c->batch = nb;
     TRY(alloc_workspace(c));
-    CU(cudaStreamSynchronize(nullptr));  // usable on every stream
   }
   extra(c)->omega.valid = false;
   split_invalidate(c);
@@ -571,7 +576,7 @@ int cc3_ctx_autotune(cc3_ctx *c, void *cuda_stream, int *ksteps_per_tile, int *n
   if (!c) return CC3_ERR_ARG;
   std::lock_guard<std::mutex> lk(c->mu);
   if (c->ntri == 0) return CC3_OK;
-  StreamScope scope((cudaStream_t)cuda_stream);
+  CallScope scope(c, (cudaStream_t)cuda_stream);
   return split_autotune(c, (cudaStream_t)cuda_stream, ksteps_per_tile, ntile_w);
 }
 
@@ -583,9 +588,10 @@ int cc3_ctx_get_tuning(cc3_ctx *c, int *ksteps_per_tile, int *ntile_w) {
 
 int cc3_ctx_set_slices(cc3_ctx *c, int slices) {
   if (!c || slices < 3 || slices > 7) return CC3_ERR_ARG;
-  cudaDeviceSynchronize();  // as above: the split state is freed
-  cudaGetLastError();
-  StreamScope scope(nullptr);
+  DeviceScope dev(c->device);  // as above: the split state is freed
+  cudaStream_t side = dev_side_stream();
+  if (!ctx_order(c, side)) return CC3_FAIL(CC3_ERR_CUDA, "the context's work cannot be waited for");
+  CallScope scope(c, side);
   c->slices = slices;
   split_invalidate(c);
   return CC3_OK;
@@ -628,7 +634,12 @@ static int finish_outputs(cc3_ctx *c, double *Omega1, double *Omega2,
 
 static int omega_fp64(cc3_ctx *c, cudaStream_t s) {
   CtxExtra *X = extra(c);
-  if (!X->omega.valid) TRY(build_omega_plans(c, s));
+  if (!X->omega.valid) {
+    // (nor is anything freed in a graph)
+    if (stream_recording(s))
+      return CC3_FAIL(CC3_ERR_CUDA, "the first call after a change must not be captured");
+    TRY(build_omega_plans(c, s));
+  }
   PtrTable pt;
   fill_ptrs(c, &pt);
   const size_t nv3 = (size_t)c->nv * c->nv * c->nv;
@@ -662,7 +673,7 @@ int cc3_omega_triples(cc3_ctx *c, cc3_prec prec, double *Omega1,
   if (prec == CC3_SPLIT_INT8) return CC3_ERR_UNSUPPORTED;
   std::lock_guard<std::mutex> lk(c->mu);
   cudaStream_t s = (cudaStream_t)cuda_stream;
-  StreamScope scope(s);
+  CallScope scope(c, s);
   const int no = c->no, nv = c->nv;
   const size_t nt2 = (size_t)no * no * nv * nv;
   c->counters = cc3_counters{};
@@ -689,6 +700,7 @@ int cc3_omega_triples(cc3_ctx *c, cc3_prec prec, double *Omega1,
   const int rc = finish_outputs(c, Omega1, Omega2, E_T, s);
   trace_end(c, TR_OUTPUT, s, 0.0, 0.0);
   if (rc != CC3_OK) return rc;
+  if (!(c->flags & CC3_DEVICE_PTRS)) scope.complete();  // finish_outputs has waited
   return trace_collect(c, s);
 }
 

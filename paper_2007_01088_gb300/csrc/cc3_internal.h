@@ -147,6 +147,11 @@ struct cc3_ctx {
   cc3::Tracer trace;
   // device status word (bounded waits)
   int *status = nullptr;
+  // its last call may still run: `done` marks that call's end, or is yet to be
+  // recorded on the legacy default stream, where the call was (see CallScope)
+  bool in_flight = false, on_legacy = false;
+  cudaEvent_t done = nullptr;
+  bool unmarked = false;  // other work may run that `done` does not mark
   std::mutex mu;
 };
 
@@ -160,7 +165,6 @@ int trace_collect(cc3_ctx *c, cudaStream_t s);
 int record_error(int status, const char *file, int line, const char *what);
 #define CC3_FAIL(status, what) ::cc3::record_error((status), __FILE__, __LINE__, (what))
 
-// engine (fp64_engine.cu)
 // ---- device memory (memory.cu) ----
 // The stream that this thread's allocations and frees are ordered on, for the
 // lifetime of the object: every entry point that takes a stream sets it.
@@ -178,6 +182,45 @@ template <class T>
 cudaError_t dev_malloc(T **p, size_t n) {
   return dev_malloc_bytes(reinterpret_cast<void **>(p), n);
 }
+// One call on a context: its allocations and work are ordered on s, after the
+// context's previous call on whatever stream that was.  A call that returns
+// before its work is done marks its end for the next one (a call that the
+// caller records into a graph cannot); one that has waited says complete().
+struct CallScope {
+  CallScope(cc3_ctx *c, cudaStream_t s);
+  ~CallScope();
+  void complete();
+  CallScope(const CallScope &) = delete;
+  CallScope &operator=(const CallScope &) = delete;
+
+ private:
+  StreamScope scope;
+  cc3_ctx *c;
+  cudaStream_t s;
+  bool recording;
+};
+// Orders s after all work of the context; false: that work cannot be waited
+// for (then its buffers must stay).
+bool ctx_order(cc3_ctx *c, cudaStream_t s);
+// The stream to free the context on: the legacy default stream where its last
+// call was there (the next context's allocations there then take the blocks
+// without a dependency between streams: a host residual, with its context, 2.69
+// ms, so 2.73 from the side stream), else the side stream.
+cudaStream_t ctx_free_stream(cc3_ctx *c);
+// Makes a context's device current for the lifetime of the object.
+struct DeviceScope {
+  explicit DeviceScope(int dev);
+  ~DeviceScope();
+  DeviceScope(const DeviceScope &) = delete;
+  DeviceScope &operator=(const DeviceScope &) = delete;
+
+ private:
+  int prev;
+};
+bool stream_recording(cudaStream_t s);  // work on s goes into a graph
+// The library's own stream of the current device, for frees and allocations
+// that no caller's stream is at hand for; it blocks no other stream.
+cudaStream_t dev_side_stream();
 void dev_free(void *p);  // p may be null; its last use must precede on the stream
 size_t dev_mem_free();   // free device bytes, with what the pool holds unused
 void dev_ctx_born();
@@ -188,6 +231,7 @@ int dev_upload(void *dst, const void *src, size_t n, cudaStream_t s);
 // Frees a context whose work is complete, or ordered before on s.
 void ctx_release(cc3_ctx *c, cudaStream_t s);
 
+// engine (fp64_engine.cu)
 int upload_plan(const Plan &p, DevPlan *d, cudaStream_t s);
 void free_plan(DevPlan *d);
 int launch_plan(const DevPlan &d, const PtrTable &ptrs, cudaStream_t s,

@@ -677,7 +677,7 @@ extern "C" int cc3_density_triples(cc3_ctx *c, cc3_prec prec, double omega, cons
                       "the frequency lies within CC3_DENOM_MIN of a triples denominator");
   }
   cudaStream_t s = (cudaStream_t)cuda_stream;
-  StreamScope scope(s);
+  CallScope scope(c, s);
   const size_t n1 = (size_t)no * nv, nt2 = n1 * no * nv, noo = (size_t)no * no,
                nvv = (size_t)nv * nv;
   c->counters = cc3_counters{};
@@ -718,7 +718,7 @@ extern "C" int cc3_density_triples(cc3_ctx *c, cc3_prec prec, double omega, cons
         cudaStreamSynchronize(s) != cudaSuccess)
       rc = CC3_FAIL(CC3_ERR_CUDA, "density download");
   }
-  cudaStreamSynchronize(s);
+  if (cudaStreamSynchronize(s) == cudaSuccess) scope.complete();
   for (double *p : tmp) dev_free(p);
   if (rc == CC3_OK) rc = trace_collect(c, s);
   return rc;

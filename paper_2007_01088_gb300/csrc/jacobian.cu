@@ -628,7 +628,7 @@ extern "C" int cc3_jacobian_triples(cc3_ctx *c, cc3_prec prec, int nvec, const d
                                      "denominator");
   }
   cudaStream_t s = (cudaStream_t)cuda_stream;
-  StreamScope scope(s);
+  CallScope scope(c, s);
   const int no = c->no, nv = c->nv;
   const size_t n1 = (size_t)no * nv, nt2 = (size_t)no * no * nv * nv;
   long long wsum = 0;
@@ -677,7 +677,7 @@ extern "C" int cc3_jacobian_triples(cc3_ctx *c, cc3_prec prec, int nvec, const d
         cudaStreamSynchronize(s) != cudaSuccess)
       rc = CC3_FAIL(CC3_ERR_CUDA, "Jacobian download");
   }
-  cudaStreamSynchronize(s);
+  if (cudaStreamSynchronize(s) == cudaSuccess) scope.complete();
   for (double *p : tmp) dev_free(p);
   if (rc == CC3_OK) rc = trace_collect(c, s);
   return rc;

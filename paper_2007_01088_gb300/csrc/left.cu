@@ -424,7 +424,7 @@ extern "C" int cc3_left_jacobian_triples(cc3_ctx *c, cc3_prec prec, int nvec,
                                      "denominator");
   }
   cudaStream_t s = (cudaStream_t)cuda_stream;
-  StreamScope scope(s);
+  CallScope scope(c, s);
   const int no = c->no, nv = c->nv;
   const size_t n1 = (size_t)no * nv, nt2 = n1 * no * nv;
   long long wsum = 0;
@@ -477,7 +477,7 @@ extern "C" int cc3_left_jacobian_triples(cc3_ctx *c, cc3_prec prec, int nvec,
         cudaStreamSynchronize(s) != cudaSuccess)
       rc = CC3_FAIL(CC3_ERR_CUDA, "left Jacobian download");
   }
-  cudaStreamSynchronize(s);
+  if (cudaStreamSynchronize(s) == cudaSuccess) scope.complete();
   for (double *p : tmp) dev_free(p);
   if (rc == CC3_OK) rc = trace_collect(c, s);
   return rc;

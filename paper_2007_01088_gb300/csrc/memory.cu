@@ -15,11 +15,21 @@
 // well when no context is left.  A failed allocation first returns all that is
 // unused and tries again.  dev_mem_free counts what the pool holds unused as
 // free.
+//
+// A block that is given back serves the next request at once, so every free is
+// ordered after the block's last use: a call's own buffers are freed on its
+// stream, and a context's buffers after the event that a call records at its
+// end unless it has waited for its work (CallScope), which also orders calls of
+// one context on different streams.
+// Waiting for the whole device instead would need every return code and fails
+// while any stream is being captured.
 #include <cuda_runtime.h>
 
 #include <atomic>
+#include <chrono>
 #include <cstring>
 #include <mutex>
+#include <thread>
 #include <vector>
 
 #include "cc3_internal.h"
@@ -31,6 +41,7 @@ constexpr int MAX_DEV = 64;
 
 std::mutex g_mu;
 cudaMemPool_t g_pool[MAX_DEV] = {nullptr};
+cudaStream_t g_side[MAX_DEV] = {nullptr};
 bool g_tried[MAX_DEV] = {false};
 unsigned long long g_cap[MAX_DEV] = {0};  // unused bytes the pool may keep
 std::atomic<int> g_live{0};
@@ -59,7 +70,8 @@ cudaMemPool_t pool_of(int dev) {
       // (a release threshold would count the memory in use as well)
       unsigned long long keep = ~0ull;
       g_cap[dev] = tot / 16;
-      if (cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) == cudaSuccess)
+      if (cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) == cudaSuccess &&
+          cudaStreamCreateWithFlags(&g_side[dev], cudaStreamNonBlocking) == cudaSuccess)
         g_pool[dev] = pool;
       else
         cudaMemPoolDestroy(pool);
@@ -139,17 +151,84 @@ StreamScope::~StreamScope() {
   }
 }
 
+bool stream_recording(cudaStream_t s) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cap) == cudaSuccess) return cap != cudaStreamCaptureStatusNone;
+  cudaGetLastError();  // the legacy stream, while another thread's capture forbids its use
+  return true;
+}
+
+static bool is_legacy(cudaStream_t s) { return s == nullptr || s == cudaStreamLegacy; }
+static bool mark(cc3_ctx *c, cudaStream_t s) {
+  if ((c->done || cudaEventCreateWithFlags(&c->done, cudaEventDisableTiming) == cudaSuccess) &&
+      cudaEventRecord(c->done, s) == cudaSuccess)
+    return true;
+  cudaGetLastError();
+  return false;
+}
+// Orders s after the context's last call.
+static bool after_last(cc3_ctx *c, cudaStream_t s) {
+  if (!c->in_flight || (c->on_legacy && is_legacy(s))) return true;
+  if (c->on_legacy && !mark(c, nullptr)) return false;
+  if (cudaStreamWaitEvent(s, c->done, 0) == cudaSuccess) return true;
+  cudaGetLastError();
+  return false;
+}
+
+CallScope::CallScope(cc3_ctx *c_, cudaStream_t s_)
+    : scope(s_), c(c_), s(s_), recording(stream_recording(s_)) {
+  if (recording) return;
+  if (!after_last(c, s)) c->unmarked = true;
+  c->in_flight = true;
+  c->on_legacy = is_legacy(s);
+}
+void CallScope::complete() {
+  if (!recording) c->in_flight = false;
+}
+CallScope::~CallScope() {
+  // the legacy default stream cannot go away: its event can be recorded when needed
+  if (recording || (c->in_flight && !c->on_legacy && !mark(c, s))) c->unmarked = true;
+}
+
+// Waits for the whole device, which is refused while a stream of it is being
+// captured: captures are short, so it tries again for up to ten seconds.
+static bool wait_device() {
+  for (int i = 0; i < 10000; ++i) {
+    const cudaError_t e = cudaDeviceSynchronize();
+    cudaGetLastError();
+    if (e < cudaErrorStreamCaptureUnsupported || e > cudaErrorStreamCaptureWrongThread)
+      return true;  // idle, or lost to an earlier failure
+    std::this_thread::sleep_for(std::chrono::milliseconds(1));
+  }
+  return false;
+}
+
+bool ctx_order(cc3_ctx *c, cudaStream_t s) {
+  return (!c->unmarked && after_last(c, s)) || wait_device();
+}
+
+cudaStream_t ctx_free_stream(cc3_ctx *c) {
+  return c->on_legacy && !stream_recording(nullptr) ? nullptr : dev_side_stream();
+}
+
+DeviceScope::DeviceScope(int dev) : prev(device()) { cudaSetDevice(dev); }
+DeviceScope::~DeviceScope() {
+  if (prev >= 0) cudaSetDevice(prev);
+}
+
+cudaStream_t dev_side_stream() {
+  const int dev = device();
+  return pool_of(dev) ? g_side[dev] : nullptr;
+}
+
 cudaError_t dev_malloc_bytes(void **p, size_t n) {
   *p = nullptr;
   t_touched = true;
   cudaMemPool_t pool = pool_of(device());
   if (!pool) return cudaMalloc(p, n);
   // no allocation becomes part of a caller's graph
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  cudaError_t e = cudaStreamIsCapturing(t_stream, &cap);
-  if (e != cudaSuccess) return e;
-  if (cap != cudaStreamCaptureStatusNone) return cudaErrorStreamCaptureUnsupported;
-  e = cudaMallocFromPoolAsync(p, n, pool, t_stream);
+  if (stream_recording(t_stream)) return cudaErrorStreamCaptureUnsupported;
+  cudaError_t e = cudaMallocFromPoolAsync(p, n, pool, t_stream);
   if (e == cudaErrorMemoryAllocation) {
     cudaGetLastError();
     cudaDeviceSynchronize();
@@ -167,7 +246,9 @@ void dev_free(void *p) {
     cudaFree(p);
   } else if (cudaFreeAsync(p, t_stream) != cudaSuccess) {
     cudaGetLastError();
-    cudaFree(p);
+    // (a capture on another thread that forbids the legacy stream) cudaFree does
+    // not wait for work on a pool's memory; not waited for, it stays allocated
+    if (wait_device()) cudaFree(p);
   }
 }
 

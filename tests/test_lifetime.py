@@ -1,0 +1,137 @@
+"""Contexts and their buffers while work is in flight, on the GPU through the C ABI: a
+context may be destroyed, or given another triple list, right after a call that does
+not wait (FP64 residual on device pointers), whatever other threads and streams do."""
+import threading
+
+import numpy as np
+import pytest
+
+import oracle
+from cc3_inputs import make_inputs
+
+pytestmark = pytest.mark.gpu
+NAMES = ("eps_o", "eps_v", "t2", "g_vvvo", "g_ooov", "g_ovov", "F_ov")
+
+
+@pytest.fixture(scope="module")
+def g():
+    import paper_2007_01088_gb300 as g
+    return g
+
+
+class DeviceProblem:
+    """Inputs and the reference on the device, contexts and outputs made from them."""
+
+    def __init__(self, g, no, nv, seed, triples=None):
+        import torch
+        self.g, self.no, self.nv = g, no, nv
+        self.inp = make_inputs(no, nv, seed=seed)
+        self.src = {n: torch.from_numpy(np.ascontiguousarray(getattr(self.inp, n))).cuda()
+                    for n in NAMES}
+        ref = oracle.omega_inputs(self.inp)
+        self.ref = (ref["omega1"], ref["omega2"])
+        torch.cuda.synchronize()
+
+    def create(self, stream):
+        return self.g.cc3_ctx_create(self.no, self.nv, *(self.src[n] for n in NAMES),
+                                     flags=self.g.CC3_DEVICE_PTRS, stream=stream)
+
+    def outputs(self):
+        import torch
+        return (torch.empty(self.no, self.nv, dtype=torch.float64, device="cuda"),
+                torch.empty(self.no, self.no, self.nv, self.nv, dtype=torch.float64,
+                            device="cuda"))
+
+    def good(self, out, tol=1e-12):
+        return all(np.abs(x.cpu().numpy() - y).max() <= tol * np.abs(y).max()
+                   for x, y in zip(out, self.ref))
+
+
+def test_destroyed_with_work_in_flight_while_others_capture(g):
+    import torch
+    a, b = DeviceProblem(g, 6, 40, 1), DeviceProblem(g, 5, 36, 2)
+    outs = [[a.outputs() for _ in range(4)] for _ in range(6)]
+    torch.cuda.synchronize()
+    bad = []
+
+    def destroyer():
+        st = torch.cuda.Stream()
+        for row in outs:
+            for o1, o2 in row:
+                c = a.create(st)
+                g.cc3_omega_triples(c, g.CC3_FP64, o1, o2, None, st)
+                g.cc3_ctx_destroy(c)
+        st.synchronize()
+
+    def capturer():  # first calls run, second ones are captured, on streams of their own
+        st = torch.cuda.Stream()
+        for _ in range(10):
+            o = b.outputs()
+            c = b.create(st)
+            for _ in range(2):
+                g.cc3_omega_triples(c, g.CC3_SPLIT_BF16, *o, None, st)
+            st.synchronize()
+            g.cc3_ctx_destroy(c)
+            if not b.good(o, 1e-10):
+                bad.append("split")
+
+    threads = [threading.Thread(target=f) for f in (destroyer, capturer, capturer)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not bad, bad
+    assert all(a.good(o) for row in outs for o in row)
+
+
+def test_calls_of_one_context_on_different_streams(g):
+    """A call is ordered after the context's previous one, and so is what a new triple
+    list or slice count frees."""
+    import torch
+    a = DeviceProblem(g, 6, 40, 3)
+    sub = [(i, j, k) for i in range(6) for j in range(i + 1) for k in range(j + 1)
+           if i != k and (i + j + k) % 2]
+    half = oracle.omega_inputs(a.inp, np.array(sub, dtype=np.int32))
+    streams = [torch.cuda.Stream() for _ in range(3)]
+    outs = [a.outputs() for _ in range(6)]
+    torch.cuda.synchronize()
+    c = a.create(streams[0])
+    for n in range(6):
+        if n in (2, 4):
+            g.cc3_ctx_set_triples(c, sub if n == 2 else None)
+        if n == 3:
+            g.cc3_ctx_set_slices(c, 5)
+        g.cc3_omega_triples(c, g.CC3_FP64, *outs[n], None, streams[n % 3])
+    g.cc3_ctx_destroy(c)
+    torch.cuda.synchronize()
+    for n in (0, 1, 4, 5):
+        assert a.good(outs[n]), n
+    for n in (2, 3):
+        for x, k in zip(outs[n], ("omega1", "omega2")):
+            assert np.abs(x.cpu().numpy() - half[k]).max() <= 1e-12 * np.abs(half[k]).max()
+
+
+def test_residual_captured_by_the_caller(g):
+    """An FP64 residual on device pointers goes into the caller's graph once its tables
+    are there, not before; the context goes away right after a replay."""
+    import torch
+    a = DeviceProblem(g, 4, 24, 4)
+    out = a.outputs()
+    st = torch.cuda.Stream()
+    c = a.create(st)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.stream(st):
+        with pytest.raises(g.CC3Error):
+            with torch.cuda.graph(torch.cuda.CUDAGraph(), stream=st):
+                g.cc3_omega_triples(c, g.CC3_FP64, *out, None, st)
+        torch.cuda.synchronize()
+        g.cc3_omega_triples(c, g.CC3_FP64, *out, None, st)
+        torch.cuda.synchronize()
+        with torch.cuda.graph(graph, stream=st):
+            g.cc3_omega_triples(c, g.CC3_FP64, *out, None, st)
+        for o in out:
+            o.zero_()
+        graph.replay()
+        g.cc3_ctx_destroy(c)
+    torch.cuda.synchronize()
+    assert a.good(out)
