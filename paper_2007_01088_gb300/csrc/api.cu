@@ -369,7 +369,7 @@ void ctx_release(cc3_ctx *c, cudaStream_t s) {
   if (c->om1_fx) dev_free(c->om1_fx);
   if (c->done) cudaEventDestroy(c->done);
   delete c;
-  dev_ctx_gone();
+  dev_ctx_gone(s);
 }
 }  // namespace cc3
 

@@ -223,8 +223,8 @@ bool stream_recording(cudaStream_t s);  // work on s goes into a graph
 cudaStream_t dev_side_stream();
 void dev_free(void *p);  // p may be null; its last use must precede on the stream
 size_t dev_mem_free();   // free device bytes, with what the pool holds unused
-void dev_ctx_born();
-void dev_ctx_gone();
+void dev_ctx_born();  // (a server counts as a context)
+void dev_ctx_gone(cudaStream_t s);  // s: where the context was freed
 void dev_give_back();  // returns the pool's unused memory if no context is left
 // Copies a host table to the device, ordered on s; src may be reused on return.
 int dev_upload(void *dst, const void *src, size_t n, cudaStream_t s);

@@ -9,12 +9,13 @@
 // device worked 26 ms).  From the pool both cost 1-2 us and order themselves on
 // the calling stream.
 //
-// The pool keeps at most 1/16 of the device's memory unused while a context
-// exists (trimmed at the end of each entry point that allocated or freed) and at most
-// KEEP bytes after the last one is gone; cc3_serve_stop gives back the rest as
-// well when no context is left.  A failed allocation first returns all that is
-// unused and tries again.  dev_mem_free counts what the pool holds unused as
-// free.
+// The pool keeps at most 1/16 of the device's memory unused while a context or
+// a server exists (trimmed at the end of each entry point that freed something)
+// and at most KEEP bytes after the last one is gone; cc3_serve_stop gives back
+// the rest as well when nothing is left.  Only memory whose free the host has seen
+// complete can be trimmed, so the stream of the frees is waited for before.  A
+// failed allocation first returns all that is unused and tries again.
+// dev_mem_free counts what the pool holds unused as free.
 //
 // A block that is given back serves the next request at once, so every free is
 // ordered after the block's last use: a call's own buffers are freed on its
@@ -44,10 +45,10 @@ cudaMemPool_t g_pool[MAX_DEV] = {nullptr};
 cudaStream_t g_side[MAX_DEV] = {nullptr};
 bool g_tried[MAX_DEV] = {false};
 unsigned long long g_cap[MAX_DEV] = {0};  // unused bytes the pool may keep
-std::atomic<int> g_live{0};
+std::atomic<int> g_live{0};  // contexts and servers
 thread_local cudaStream_t t_stream = nullptr;
 thread_local int t_depth = 0;         // StreamScopes of this thread
-thread_local bool t_touched = false;  // allocated or freed in the outermost one
+thread_local bool t_freed = false;    // something was freed in the outermost one
 
 // The device's pool; null where pools are not supported (then cudaMalloc serves).
 cudaMemPool_t pool_of(int dev) {
@@ -137,18 +138,20 @@ static bool pool_state(cudaMemPool_t pool, unsigned long long *held, unsigned lo
 
 StreamScope::StreamScope(cudaStream_t s) : prev(t_stream) {
   t_stream = s;
-  if (t_depth++ == 0) t_touched = false;
+  if (t_depth++ == 0) t_freed = false;
 }
 StreamScope::~StreamScope() {
+  const cudaStream_t s = t_stream;
   t_stream = prev;
-  if (--t_depth > 0 || !t_touched) return;
+  if (--t_depth > 0 || !t_freed) return;
   const int dev = device();
   cudaMemPool_t pool = pool_of(dev);
   unsigned long long held = 0, used = 0;
-  if (pool && pool_state(pool, &held, &used) && held > used + g_cap[dev]) {
+  if (!pool || !pool_state(pool, &held, &used) || held <= g_cap[dev]) return;
+  cudaStreamSynchronize(s);  // frees under way count as used
+  if (pool_state(pool, &held, &used) && held > used + g_cap[dev])
     cudaMemPoolTrimTo(pool, used + g_cap[dev]);
-    cudaGetLastError();
-  }
+  cudaGetLastError();
 }
 
 bool stream_recording(cudaStream_t s) {
@@ -223,7 +226,6 @@ cudaStream_t dev_side_stream() {
 
 cudaError_t dev_malloc_bytes(void **p, size_t n) {
   *p = nullptr;
-  t_touched = true;
   cudaMemPool_t pool = pool_of(device());
   if (!pool) return cudaMalloc(p, n);
   // no allocation becomes part of a caller's graph
@@ -241,7 +243,7 @@ cudaError_t dev_malloc_bytes(void **p, size_t n) {
 
 void dev_free(void *p) {
   if (!p) return;
-  t_touched = true;
+  t_freed = true;
   if (!pool_of(device())) {
     cudaFree(p);
   } else if (cudaFreeAsync(p, t_stream) != cudaSuccess) {
@@ -266,8 +268,9 @@ size_t dev_mem_free() {
 }
 
 void dev_ctx_born() { ++g_live; }
-void dev_ctx_gone() {
+void dev_ctx_gone(cudaStream_t s) {
   if (--g_live > 0) return;
+  cudaStreamSynchronize(s);
   if (cudaMemPool_t pool = pool_of(device())) cudaMemPoolTrimTo(pool, KEEP);
   cudaGetLastError();
 }

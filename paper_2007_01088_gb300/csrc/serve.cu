@@ -205,7 +205,10 @@ void worker_main(cc3_server *S) {
     S->cv_work.notify_all();
     S->cv_done.notify_all();
   }
-  if (st) cudaStreamDestroy(st);
+  if (st) {
+    cudaStreamSynchronize(st);  // what it freed can be given back
+    cudaStreamDestroy(st);
+  }
 }
 
 double percentile(std::vector<double> v, double p) {
@@ -246,6 +249,7 @@ int cc3_serve_start(cc3_server **out, size_t hbm_budget_bytes, int max_slots) {
   S->budget = hbm_budget_bytes;
   S->max_slots = max_slots;
   S->t0 = Clock::now();
+  cc3::dev_ctx_born();  // its requests' contexts share the pool's unused memory
   try {
     for (int i = 0; i < max_slots; ++i) S->workers.emplace_back(worker_main, S);
   } catch (...) {
@@ -255,6 +259,7 @@ int cc3_serve_start(cc3_server **out, size_t hbm_budget_bytes, int max_slots) {
     }
     S->cv_work.notify_all();
     for (auto &t : S->workers) t.join();
+    cc3::dev_ctx_gone(cc3::dev_side_stream());
     delete S;
     return CC3_ERR_OOM;
   }
@@ -409,6 +414,8 @@ int cc3_serve_stop(cc3_server *S) {
   S->cv_work.notify_all();
   S->cv_done.notify_all();
   for (auto &t : S->workers) t.join();
+  cc3::DeviceScope dev(S->device);
+  cc3::dev_ctx_gone(cc3::dev_side_stream());
   delete S;
   cc3::dev_give_back();
   return CC3_OK;

@@ -135,3 +135,43 @@ def test_residual_captured_by_the_caller(g):
         g.cc3_ctx_destroy(c)
     torch.cuda.synchronize()
     assert a.good(out)
+
+
+def test_memory_kept_after_the_last_context():
+    """At most 1 GiB stays in the pool once no context is left, and nothing after a
+    server has stopped.  In a process of its own, so that no other context lives."""
+    import subprocess
+    import sys
+    code = """
+import torch
+import paper_2007_01088_gb300 as g
+from cc3_inputs import make_inputs
+
+def free():
+    torch.cuda.synchronize()
+    return torch.cuda.mem_get_info()[0]
+
+def run(inp):
+    c = g.Context(inp)
+    c.set_triples([(2, 1, 0)])
+    c.omega(g.CC3_SPLIT_BF16)
+    c.omega(g.CC3_FP64)
+    return c
+
+run(make_inputs(3, 8, seed=1)).close()  # the kernels are loaded
+f0 = free()
+big = make_inputs(10, 128, seed=1)
+slack = 64 << 20
+for _ in range(2):
+    c = run(big)
+    assert f0 - free() > 5 << 28, f0 - free()
+    c.close()
+    assert f0 - free() <= (1 << 30) + slack, f0 - free()
+srv = g.Server(max_slots=2)
+tickets = [srv.submit_omega(make_inputs(6, 60, seed=n)) for n in range(4)]
+assert all(srv.wait(t)[0] == g.CC3_OK for t in tickets)
+srv.stop()
+assert f0 - free() <= slack, f0 - free()
+"""
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
