@@ -112,6 +112,7 @@ struct SplitState {
   int ks4 = 1;  // K split of the rows-x contractions
   // tunables (autotuner): K steps per vvov tile, N tile of the W build (0: default)
   int ks_target = 400, nt_w = 0;
+  bool fixed_parts = false;  // reproducible sums: the K split knows nothing of the batch
   bool pair_ooov = true;   // one ooov job for the two permutations of a z slot
   // the residual's launch sequence as a CUDA graph (captured on the second
   // untraced call on a non-default stream, replayed afterwards)
@@ -753,6 +754,9 @@ void plan_vvov(SPlan &P, SplitState *S, int no, int nv, std::vector<VvovPerm> pe
   // 3 parts take 12.0 -> 11.7 ms.  More parts alone are slower (partial sums of
   // one output row meet in its atomics): no=16 nv=160 192.1 -> 193.3 ms in the engine
   // with 8 parts for 4, no=8 nv=72 2.14 -> 2.21 ms with 2 for 1.
+  // Each part is rounded before it adds to a reproducible sum, and a batch holds
+  // fewer triples in the serving loop than outside it: those sums keep the parts
+  // that nv and the target give.
   long long n = 0;
   for (size_t j = first; j < P.jobs.size(); ++j) n += P.jobs[j].tiles_m * P.jobs[j].tiles_n;
   if (n == 0) return;
@@ -762,7 +766,8 @@ void plan_vvov(SPlan &P, SplitState *S, int no, int nv, std::vector<VvovPerm> pe
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   sms = std::max(1, sms);
   auto rounds = [&](int k) { return (double)((n * k + sms - 1) / sms) / k; };
-  const int ks = kst >= 100 * (ks0 + 1) && rounds(ks0 + 1) < 0.9 * rounds(ks0) ? ks0 + 1 : ks0;
+  const bool more = !S->fixed_parts && kst >= 100 * (ks0 + 1) && rounds(ks0 + 1) < 0.9 * rounds(ks0);
+  const int ks = more ? ks0 + 1 : ks0;
   for (size_t j = first; j < P.jobs.size(); ++j) P.jobs[j].ksplit = ks;
   P.tiles += n * (ks - 1);
 }
@@ -862,6 +867,7 @@ int split_ready(cc3_ctx *c, SplitState **out, cudaStream_t st) {
     S = new (std::nothrow) SplitState();
     if (!S) return CC3_ERR_OOM;
     S->s = s;
+    S->fixed_parts = c->omt_fx != nullptr;
     c->split = S;
     std::lock_guard<std::mutex> lk(g_tune_mu);
     auto it = g_tuned.find(TuneKey{c->no, c->nv, s});

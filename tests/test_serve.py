@@ -166,6 +166,8 @@ def test_footprint_bounds_device_memory(g):
 def test_deterministic_requests_are_bitwise_equal_alone_and_in_the_mix(g):
     probs = [(make_inputs(4 + n, 20 + 6 * n, seed=80 + n),
               g.CC3_SPLIT_BF16 if n % 2 else g.CC3_FP64) for n in range(5)]
+    # a served context has 16 of these in a batch, one outside the server 38 and 39
+    probs += [(make_inputs(no, nv, seed=90 + no), g.CC3_SPLIT_BF16) for no, nv in ((8, 64), (9, 66))]
     alone = []
     for inp, prec in probs:
         ctx = g.Context(inp, flags=g.CC3_DETERMINISTIC)
