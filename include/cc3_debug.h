@@ -29,6 +29,17 @@ int cc3_debug_split_gemm(int M, int N, int K, const double *A, const double *B, 
  * of range.  Synchronous, on the legacy default stream of the current device.
  * Exists to test the failure path without a GPU fault. */
 int cc3_debug_wait_timeout(double limit_s);
+
+/* The split densities' D_oo kernel alone: D_oo[l][k] (row-major, no x no) of
+ * given double-float tensors tau and L3~, host arrays [T][a][b][c][2] (high part,
+ * low part) over the triples i >= j >= k in loop order, i = j = k included:
+ *   D_oo[l][k] = -1/2 sum_{i >= j} (2 - delta_ij) sum_{abc} L3~^{abc}_{ijk} tau^{abc}_{ijl},
+ * L3~ taken as zero at i = j = k; each tensor read in the order of (i, j, k) that
+ * its triple stores.  blocks_per_pair: thread blocks that share a pair's sum (0:
+ * as in cc3_density_triples); fewer give each thread longer sums.  Exists to
+ * measure the sums' rounding.  Synchronous, on the legacy default stream. */
+int cc3_debug_doo_pairs(int no, int nv, const float *tau, const float *lt, double *D_oo,
+                        int blocks_per_pair);
 #ifdef __cplusplus
 }
 #endif

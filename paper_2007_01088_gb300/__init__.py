@@ -41,7 +41,7 @@ EXPORTED = ["cc3_ctx_create", "cc3_ctx_destroy", "cc3_ctx_set_triples",
             "cc3_ctx_trace", "cc3_omega_triples_noalloc", "cc3_serve_footprint",
             "cc3_ctx_autotune", "cc3_ctx_get_tuning", "cc3_cvs_triples",
             "cc3_denominator_gap", "cc3_debug_wait_timeout", "cc3_ctx_create_general",
-            "cc3_left_jacobian_triples", "cc3_density_triples"]
+            "cc3_left_jacobian_triples", "cc3_density_triples", "cc3_debug_doo_pairs"]
 
 
 class CC3Error(RuntimeError):
@@ -118,6 +118,8 @@ def _load():
     L.cc3_ctx_set_slices.restype = I
     L.cc3_debug_split_gemm.argtypes = [I, I, I, P, P, P, I]
     L.cc3_debug_split_gemm.restype = I
+    L.cc3_debug_doo_pairs.argtypes = [I, I, P, P, P, I]
+    L.cc3_debug_doo_pairs.restype = I
     L.cc3_debug_wait_timeout.argtypes = [D]
     L.cc3_debug_wait_timeout.restype = I
     L.cc3_ctx_set_tracing.argtypes = [P, I]
@@ -353,6 +355,21 @@ def cc3_debug_split_gemm(A, B, slices=6):
     _check(lib.cc3_debug_split_gemm(M, N, K, _ptr(A), _ptr(B), _ptr(C), int(slices)),
            "cc3_debug_split_gemm")
     return C
+
+
+def cc3_debug_doo_pairs(tau, lt, blocks_per_pair=0):
+    """D_oo of the split densities from tau and L3~ of every triple i >= j >= k, float32
+    arrays [T][a][b][c][2] of double-float pairs (diagnostic)."""
+    tau, lt = (np.ascontiguousarray(x, dtype=np.float32) for x in (tau, lt))
+    no = 1
+    while no * (no + 1) * (no + 2) // 6 < tau.shape[0]:
+        no += 1
+    if tau.shape != lt.shape or tau.shape[0] != no * (no + 1) * (no + 2) // 6 or tau.shape[-1] != 2:
+        raise ValueError("arrays [T][a][b][c][2]")
+    out = np.zeros((no, no))
+    _check(lib.cc3_debug_doo_pairs(no, tau.shape[1], _ptr(tau), _ptr(lt), _ptr(out),
+                                   int(blocks_per_pair)), "cc3_debug_doo_pairs")
+    return out
 
 
 # ---- convenience wrapper -----------------------------------------------------

@@ -297,7 +297,8 @@ int left_finish(cc3_ctx *c, const PtrTable &pt, const double *s2raw, double *s2d
 // every triple of tri (3 ints each, sorted i >= j >= k) held resident
 int density_tail(cc3_ctx *c, const PtrTable &pt, double *Dvv, cudaStream_t s);
 int density_doo_resident(cc3_ctx *c, const float2 *tau_all, const float2 *lt_all,
-                         const std::vector<int> &tri, double *Doo, cudaStream_t s);
+                         const std::vector<int> &tri, double *Doo, cudaStream_t s,
+                         int blocks_per_pair = 0);  // 0: as many as the rule gives
 
 // smallest |w - eps^{abc}_{ijk}| over every (a, b, c) and the ntri triples
 // ijk (host arrays; ntri = 0: the full loop); api.cu

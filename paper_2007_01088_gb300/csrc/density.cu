@@ -39,6 +39,7 @@
 #include <vector>
 
 #include "cc3_internal.h"
+#include "dd.cuh"
 #include "split.h"
 
 namespace cc3 {
@@ -400,10 +401,11 @@ int density_fp64(cc3_ctx *c, double w, const double *L1d, const double *L2d, dou
 //   of 256 blocks when no > 64).
 // Each product is its rounded high part plus its error and cross terms (FMA);
 // the high parts are summed with their rounding errors (two-sum), which join
-// the low sum; the pair is renormalised after every chunk.  The terms keep
-// ~2^-44 of their size, well inside the FP64 path's agreement.  At no=12 nv=120
-// one thread per product, half of them idle, with rows read element by element
-// took 28.6 ms; this one 18.5 ms, 14.8 with the grid chosen as below.
+// the low sum.  A pair takes at most DOO_E terms and then joins the thread's
+// total, three FP32 values summed with their rounding errors (72 bits; an FP64
+// addition takes 16 clocks of this part's FP64 pipe per warp, and the totals of
+// a block of products would not fit the registers: they are in local memory).
+// The terms keep ~2^-44 of their size, well inside the FP64 path's agreement.
 constexpr int DOO_E = 128, DOO_T = 4, DOO_PF = 12;
 __host__ __device__ constexpr int doo_rows(int no) { return (no + DOO_T - 1) / DOO_T * DOO_T; }
 __global__ void __launch_bounds__(256)
@@ -431,6 +433,36 @@ __global__ void __launch_bounds__(256)
   for (int i = 0; i < DOO_T; ++i)
 #pragma unroll
     for (int j = 0; j < DOO_T; ++j) hi[i][j] = lo[i][j] = 0.f;
+  // the totals, one row of the block at a time (the loop stays rolled: rows of
+  // pairs move up, so that the totals keep out of the registers)
+  float tot[DOO_T][3 * DOO_T];
+#pragma unroll 1
+  for (int i = 0; i < DOO_T; ++i)
+#pragma unroll
+    for (int j = 0; j < 3 * DOO_T; ++j) tot[i][j] = 0.f;
+  const int per = (DOO_E + G - 1) / G, most = DOO_E / per;  // terms a chunk, chunks a pair takes
+  int chunks = 0;
+  auto join = [&]() {
+#pragma unroll 1
+    for (int i = 0; i < DOO_T; ++i) {
+      float *t = tot[i];
+#pragma unroll
+      for (int j = 0; j < DOO_T; ++j) {
+        const dd::df s = dd::two_sum(t[3 * j], hi[0][j]), u = dd::two_sum(t[3 * j + 1], lo[0][j]),
+                     v = dd::two_sum(u.hi, s.lo);
+        t[3 * j] = s.hi;
+        t[3 * j + 1] = v.hi;
+        t[3 * j + 2] = __fadd_rn(t[3 * j + 2], __fadd_rn(u.lo, v.lo));
+      }
+#pragma unroll
+      for (int k = 0; k < DOO_T; ++k)
+#pragma unroll
+        for (int j = 0; j < DOO_T; ++j) {
+          hi[k][j] = k + 1 < DOO_T ? hi[k + 1 < DOO_T ? k + 1 : k][j] : 0.f;
+          lo[k][j] = k + 1 < DOO_T ? lo[k + 1 < DOO_T ? k + 1 : k][j] : 0.f;
+        }
+    }
+  };
   // chunks (a4, b4, c8), c8 innermost; a block takes every gridDim.x-th (a4, b4)
   const int n4 = (nv + 3) / 4, n8 = (nv + 7) / 8;
   const int4 *view = tab + ((long long)blockIdx.y * 2 + h) * no;
@@ -489,28 +521,30 @@ __global__ void __launch_bounds__(256)
             lo[i][j] = __fadd_rn(lo[i][j], __fadd_rn(er, pl));
           }
       }
+      if (++chunks == most) {
+        join();
+        chunks = 0;
+      } else {  // the low parts back below the high ones' last place
 #pragma unroll
-      for (int i = 0; i < DOO_T; ++i)
+        for (int i = 0; i < DOO_T; ++i)
 #pragma unroll
-        for (int j = 0; j < DOO_T; ++j) {
-          const float sn = __fadd_rn(hi[i][j], lo[i][j]);
-          lo[i][j] = __fsub_rn(lo[i][j], __fsub_rn(sn, hi[i][j]));
-          hi[i][j] = sn;
-        }
+          for (int j = 0; j < DOO_T; ++j) {
+            const dd::df s = dd::fast_two_sum(hi[i][j], lo[i][j]);
+            hi[i][j] = s.hi;
+            lo[i][j] = s.lo;
+          }
+      }
     }
   }
+  join();
   // the block's sums over its e groups, then one atomic per product
   __syncthreads();
   double *red = reinterpret_cast<double *>(sm2);  // [256 / ...][16] one thread's products
   const double w = wgt[blockIdx.y];
+#pragma unroll 1
   for (int q = 0; q < DOO_T * DOO_T; ++q) {
-    float vh = 0.f, vl = 0.f;
-#pragma unroll
-    for (int i = 0; i < DOO_T; ++i)
-#pragma unroll
-      for (int j = 0; j < DOO_T; ++j)
-        if (q == i * DOO_T + j) vh = hi[i][j], vl = lo[i][j];
-    red[t] = (double)vh + (double)vl;
+    const float *v = tot[q / DOO_T] + 3 * (q % DOO_T);
+    red[t] = (double)v[0] + ((double)v[1] + (double)v[2]);
     __syncthreads();
     const int k = blk / nb * DOO_T + q / DOO_T, l = blk % nb * DOO_T + q % DOO_T;
     if (g == 0 && k < no && l < no) {
@@ -552,7 +586,8 @@ int density_tail(cc3_ctx *c, const PtrTable &pt, double *Dvv, cudaStream_t s) {
 // the pair (j, i) gives the same sum over (a,b,c) as (i, j): the pairs i > j count
 // twice, i = j once, and one launch covers them all.
 int density_doo_resident(cc3_ctx *c, const float2 *tau_all, const float2 *lt_all,
-                         const std::vector<int> &tri, double *Doo, cudaStream_t s) {
+                         const std::vector<int> &tri, double *Doo, cudaStream_t s,
+                         int blocks_per_pair) {
   const int no = c->no, nv = c->nv;
   const long long nv2 = (long long)nv * nv;
   const int nt = (int)tri.size() / 3;
@@ -617,8 +652,9 @@ int density_doo_resident(cc3_ctx *c, const float2 *tau_all, const float2 *lt_all
   int per_sm = 0;
   CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, doo_pairs_kernel, 256, smem));
   const long long slots = (long long)std::max(1, per_sm) * nsm, per_gx = (long long)npair * gz;
-  long long gx = 1, least = -1;
-  for (long long x = 1; x <= nunit && (x == 1 || x * per_gx <= 32LL * nsm); ++x) {
+  long long gx = std::max(1, blocks_per_pair), least = -1;
+  for (long long x = 1; blocks_per_pair == 0 && x <= nunit && (x == 1 || x * per_gx <= 32LL * nsm);
+       ++x) {
     const long long units = (x * per_gx + slots - 1) / slots * ((nunit + x - 1) / x + 1);
     if (least < 0 || units < least) least = units, gx = x;
   }
@@ -722,4 +758,33 @@ extern "C" int cc3_density_triples(cc3_ctx *c, cc3_prec prec, double omega, cons
   for (double *p : tmp) dev_free(p);
   if (rc == CC3_OK) rc = trace_collect(c, s);
   return rc;
+}
+
+extern "C" int cc3_debug_doo_pairs(int no, int nv, const float *tau, const float *lt, double *D_oo,
+                                   int blocks_per_pair) {
+  using namespace cc3;
+  if (no < 1 || no > 112 || nv < 1 || nv > 1024 || !tau || !lt || !D_oo || blocks_per_pair < 0 ||
+      blocks_per_pair > 65535)
+    return CC3_ERR_ARG;
+  StreamScope scope(nullptr);
+  cc3_ctx c;
+  c.no = no;
+  c.nv = nv;
+  std::vector<int> tri;
+  for (int i = 0; i < no; ++i)
+    for (int j = 0; j <= i; ++j)
+      for (int k = 0; k <= j; ++k) tri.insert(tri.end(), {i, j, k});
+  const size_t n = tri.size() / 3 * (size_t)nv * nv * nv;
+  Bufs B;
+  float2 *dt = nullptr, *dl = nullptr;
+  double *doo = nullptr;
+  TRY(B.get(&dt, n));
+  TRY(B.get(&dl, n));
+  TRY(B.get(&doo, (size_t)no * no));
+  CU(cudaMemcpyAsync(dt, tau, sizeof(float2) * n, cudaMemcpyHostToDevice, nullptr));
+  CU(cudaMemcpyAsync(dl, lt, sizeof(float2) * n, cudaMemcpyHostToDevice, nullptr));
+  TRY(density_doo_resident(&c, dt, dl, tri, doo, nullptr, blocks_per_pair));
+  CU(cudaMemcpyAsync(D_oo, doo, sizeof(double) * no * no, cudaMemcpyDeviceToHost, nullptr));
+  CU(cudaStreamSynchronize(nullptr));
+  return CC3_OK;
 }

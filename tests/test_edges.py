@@ -121,6 +121,44 @@ def test_densities_beyond_one_group_of_blocks(g):
         assert split_close(x, y), split_err(x, y)
 
 
+def test_doo_sums_of_many_terms(g):
+    """2286 products of one sign in each thread's sums (one block per pair): their pairs
+    of FP32 values take 128 terms at most before they join the total."""
+    no, nv = 9, 40
+    trip = [(i, j, k) for i in range(no) for j in range(i + 1) for k in range(j + 1)]
+    idx = {t: n for n, t in enumerate(trip)}
+    rng = np.random.default_rng(3)
+    orders = ((0, 1, 2), (1, 0, 2), (2, 1, 0), (0, 2, 1), (1, 2, 0), (2, 0, 1))
+
+    def pairs():
+        x = np.abs(rng.normal(size=(len(trip), nv, nv, nv)))
+        hi = x.astype(np.float32)
+        return np.stack([hi, (x - hi).astype(np.float32)], -1)
+
+    def view(x, *pqr):
+        s = tuple(sorted(pqr, reverse=True))
+        m = next(m for m in orders if tuple(s[u] for u in m) == pqr)
+        y = x[idx[s]].astype(np.float64).sum(-1)  # 48 bits: exact
+        return y.transpose(m).reshape(-1)
+
+    tau, lt = pairs(), pairs()
+    ref = np.zeros((no, no))
+    for i in range(no):
+        for j in range(i + 1):
+            T = [view(tau, i, j, k) for k in range(no)]
+            for k in range(no):
+                if not i == j == k:
+                    L = view(lt, i, j, k) * (1.0 if i == j else 2.0)
+                    for l in range(no):
+                        ref[l, k] -= 0.5 * float(np.sum(L * T[l], dtype=np.longdouble))
+    got = g.cc3_debug_doo_pairs(tau, lt, blocks_per_pair=1)
+    # A pair's low part, some 2^-24 of its sum S, is rounded to 2^-24 of itself in each of
+    # 128 additions: about 2^-48 0.3 sqrt(128 / 3) S at random, over the root of the 500
+    # pairs of an element 3e-16 of it; the same again for the products' own cross terms.
+    # Pairs that take all 2286 terms are off by 3.3e-15.
+    assert (np.abs(got - ref) / np.abs(ref)).max() <= 1.2e-15
+
+
 # FP64 tiles of one to four row and column groups, ending one past, on and one before a multiple
 # of 16, short sums (K = no) and launches split over K (left: 3 tiles, K = 3 n nv)
 @pytest.mark.parametrize("no,nv", [(3, 15), (3, 16), (2, 17), (2, 40), (2, 65)])
