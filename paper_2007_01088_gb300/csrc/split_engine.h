@@ -8,10 +8,11 @@ namespace cc3 {
 
 enum { SMAX_MAPS = 48, S_BM = 128, S_BK = 16, S_STAGES_MAX = 6, S_MAX_SLICES = 7,
        S_NT_MAX = 96, S_EPI_WARPS = 16, S_THREADS = 96 + 32 * S_EPI_WARPS,
-       // fraction bits of the epilogue's fixed-point sums, and the K steps of a
-       // tile that keep them in 64 bits (and the shared accumulator's terms in 32:
-       // 5 2^14 (1 + 2^-6) 16 S_MAX_TILE_STEPS < 2^31)
-       S_ACC_FRAC = 32, S_MAX_TILE_STEPS = 1600,
+       // fraction bits of the epilogue's fixed-point sums (their rounding is then
+       // a quarter or less of what the products left out by 6 slices cost), and the
+       // K steps of a tile that keep them in 64 bits and the shared accumulator's
+       // terms in 32: 5 2^14 (1 + 2^-6) 16 S_MAX_TILE_STEPS 2 < 2^31
+       S_ACC_FRAC = 33, S_MAX_TILE_STEPS = 800,
        S_TERM_CHUNK = 8 };  // terms the decoder reads at a time
 
 // A BF16 slice array in the tensor cores' canonical no-swizzle K-major order

@@ -23,31 +23,53 @@ def g():
 
 # 16 K per step: a tile of 1, 2, 3 steps; level 3 due (12), its limit (16, 17),
 # level 2's (20, 21), level 1's (24, 28, 29), level 0's (48, 56, 57), the W build of
-# nv = 250 (36); one and two parts of a tile split over K (1600, 1601)
+# nv = 250 (36); one and two parts of a tile split over K (800, 801)
 @pytest.mark.parametrize("steps", [1, 2, 3, 12, 16, 17, 20, 21, 24, 28, 29, 36, 48, 56, 57, 130,
-                                   1600, 1601])
-@pytest.mark.parametrize("slices", [6, 3])
+                                   800, 801])
+@pytest.mark.parametrize("slices", [6, 7, 5, 4, 3])
 def test_engine_sums_at_drain_points(g, steps, slices):
     """Every slice digit 127: each accumulator takes the largest sums it can, so a
     drain that comes too late loses low bits of all elements at once."""
     K = 16 * steps
     T = sum(127 * 256**p for p in range(slices))
-    x = float(T) * 2.0 ** -(7 + 8 * (slices - 1))  # exact for 6 slices: 47 bits
+    T -= 3 if slices == 7 else 0  # 53 of 55 bits: the last digit is 124
+    x = float(T) * 2.0 ** -(7 + 8 * (slices - 1))
     A = np.full((130, K), x)
     B = np.full((24, K), x)
     B[1::2] *= -1.0
     B[2::3, ::2] *= -1.0
     sums = B.sum(axis=1) / x  # small integers
-    ref = np.array([float(Fraction(x) * Fraction(x) * int(s)) for s in sums])
+    ref = np.array([float(Fraction(x) * Fraction(x) * round(s)) for s in sums])
     C = g.cc3_debug_split_gemm(A, B, slices)
     # In units of the largest digit product (2^14): products below the last level are
-    # 5 (2) pairs of digits of 2^-8s per k; the shared accumulator (6 slices) holds
-    # 5 2^-32 per k so far, and each of the 11 products of a step adds to it in up to two
-    # parts (8 of its 16 k each), each of which drops at most 2^-23 of that:
-    # 22 2^-23 5 2^-32 16 (1 + 2 + ... + steps).
+    # slices - 1 pairs of digits of 2^-8s per k; the shared accumulator (levels from 4
+    # on) holds 5 2^-32 per k so far, and each of its products of a step (5, 11 or 18)
+    # adds to it in up to two parts (8 of its 16 k each), each of which drops at most
+    # 2^-23 of that: 22 2^-23 5 2^-32 16 (1 + 2 + ... + steps) for 6 slices.
     left_out = (slices - 1) * 2.0 ** (-8 * slices) * 1.01 * K
-    rounded = 22 * 5 * 16 * 2.0**-56 * steps * (steps + 1) if slices > 4 else 0.0
+    shared = sum(L + 1 for L in range(4, slices))
+    rounded = 2 * shared * 5 * 16 * 2.0**-56 * steps * (steps + 1)
     assert np.abs(C - ref[None, :]).max() <= left_out + rounded + 2.0**-52 * K
+
+
+@pytest.mark.parametrize("slices,left_out", [(6, 2.0**-44), (7, 0.0)])
+def test_engine_keeps_the_last_levels_of_small_elements(g, slices, left_out):
+    """Elements of digits -1, 0, 1 in the second to fourth slice, next to a large one
+    that sets the scale: products of the levels 2 to 6, whose sums the accumulators hold
+    exactly, down to 2^-48 of a digit product's unit (2^-14 here)."""
+    rng = np.random.default_rng(slices)
+
+    def operand(rows):
+        d = rng.integers(-1, 2, size=(rows, 16, 3))
+        x = (d * 2.0 ** (-8.0 * np.arange(1, 4))).sum(-1)
+        x[0, 0] = 127.0
+        return x / 128
+
+    A, B = operand(130), operand(40)
+    C = g.cc3_debug_split_gemm(A, B, slices)
+    err = np.abs(C - A @ B.T)[1:, 1:].max() * 2.0**14
+    # 6 slices leave out the 16 products of level 6; the sums are read to 2^-47
+    assert err <= left_out + (2.0**-34 if slices == 6 else 2.0**-48), err
 
 
 @pytest.mark.parametrize("N", [16, 81, 97, 112, 177, 200, 250])
@@ -73,13 +95,14 @@ def test_residual_at_slicing_edges(g, no, nv):
 @pytest.mark.parametrize("slices", [3, 4, 5, 7])
 def test_residual_with_other_slice_counts(g, slices):
     # odd counts leave the last pair of slices half filled; each slice less costs 8 bits
-    # of the 1e-10 that six are held to
+    # of the 1e-10 that six are held to; the seventh takes these sums to the floor of the
+    # double-float steps (1.4e-13 of Omega1; 5e-13 with six slices)
     inp = make_inputs(4, 19, seed=11)
     ref = oracle.omega_inputs(inp)
     ctx = g.Context(inp)
     g.cc3_ctx_set_slices(ctx.ctx, slices)
     got = ctx.omega(g.CC3_SPLIT_BF16)
-    tol = 1e-10 * max(1.0, 256.0 ** (6 - slices))
+    tol = 2.5e-13 if slices == 7 else 1e-10 * 256.0 ** (6 - slices)
     for x, k in zip(got, ("omega1", "omega2")):
         err, scale = split_err(x, ref[k])
         assert err <= tol * scale, (err, scale)
