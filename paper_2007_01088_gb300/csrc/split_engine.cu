@@ -265,10 +265,12 @@ __device__ __forceinline__ double fixed_to_double(long long a, int e2) {
   if (u == 0ull || e < 0) return 0.0;
   const unsigned long long m = u << lz;
   const unsigned long long r = (m >> 11) + ((m >> 10) & 1ull);
-  const unsigned long long b = ((unsigned long long)min(e, 2045) << 52) + r;
+  // (beyond the largest double: infinite)
+  const unsigned long long b = e > 2045 ? 0x7FF0000000000000ull : ((unsigned long long)e << 52) + r;
   return __longlong_as_double((long long)(b | sign));
 }
-// a 2^e2 as a double-float pair: the leading 24 bits, rounded, and 24 more.
+// a 2^e2 as a double-float pair: the leading 24 bits, rounded, and 24 more
+// (infinite from 2^127 on).
 __device__ __forceinline__ float2 fixed_to_dd(long long a, int e2) {
   const unsigned int sign = a < 0 ? 0x80000000u : 0u;
   const unsigned long long u = a < 0 ? 0ull - (unsigned long long)a : (unsigned long long)a;
@@ -278,7 +280,7 @@ __device__ __forceinline__ float2 fixed_to_dd(long long a, int e2) {
   const unsigned long long m = u << lz;
   const unsigned int h = (unsigned int)(m >> 40) + ((unsigned int)(m >> 39) & 1u);
   const int rest = (int)((long long)(m - ((unsigned long long)h << 40)) >> 9);  // |.| <= 2^30
-  const float f = __int_as_float((int)(((unsigned int)min(e, 254) << 23) | sign));
+  const float f = __int_as_float((int)(((unsigned int)min(e, 255) << 23) | sign));
   return make_float2(__uint2float_rn(h) * 0x1p-24f * f, __int2float_rn(rest) * 0x1p-55f * f);
 }
 

@@ -72,6 +72,13 @@ def test_engine_keeps_the_last_levels_of_small_elements(g, slices, left_out):
     assert err <= left_out + (2.0**-34 if slices == 6 else 2.0**-48), err
 
 
+def test_engine_overflow_is_infinite(g):
+    A = np.full((3, 16), 1e200)
+    assert np.all(g.cc3_debug_split_gemm(A, np.full((2, 16), -1e200), 6) == -np.inf)
+    C = g.cc3_debug_split_gemm(A, np.full((2, 16), 1e100), 6)
+    assert np.abs(C / 1.6e301 - 1.0).max() <= 1e-13
+
+
 @pytest.mark.parametrize("N", [16, 81, 97, 112, 177, 200, 250])
 def test_engine_trimmed_column_tiles(g, N):
     rng = np.random.default_rng(N)
