@@ -347,6 +347,7 @@ void cc3_ctx_destroy(cc3_ctx *c) {
 namespace cc3 {
 void ctx_release(cc3_ctx *c, cudaStream_t s) {
   StreamScope scope(s);
+  GoneScope gone(c->space != dev_space());
   CtxExtra *X = extra(c);
   if (X) {
     free_omega_plans(X->omega);
@@ -367,9 +368,10 @@ void ctx_release(cc3_ctx *c, cudaStream_t s) {
   if (c->status) dev_free(c->status);
   if (c->omt_fx) dev_free(c->omt_fx);
   if (c->om1_fx) dev_free(c->om1_fx);
-  if (c->done) cudaEventDestroy(c->done);
+  if (c->done && !dev_gone()) cudaEventDestroy(c->done);
+  const unsigned long long space = c->space;
   delete c;
-  dev_ctx_gone(s);
+  dev_ctx_gone(space, s);
 }
 }  // namespace cc3
 
@@ -395,7 +397,7 @@ static int ctx_create_impl(cc3_ctx **out, int no, int nv, const double *eps_o,
   c->ext = new (std::nothrow) CtxExtra();
   if (!c->ext) { delete c; return CC3_ERR_OOM; }
   StreamScope scope(s);
-  dev_ctx_born();
+  c->space = dev_ctx_born();
   c->no = no;
   c->nv = nv;
   c->naux = chol_L ? naux : 0;

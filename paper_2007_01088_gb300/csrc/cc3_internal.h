@@ -152,6 +152,7 @@ struct cc3_ctx {
   bool in_flight = false, on_legacy = false;
   cudaEvent_t done = nullptr;
   bool unmarked = false;  // other work may run that `done` does not mark
+  unsigned long long space = 0;  // the device context that it lives in (dev_space)
   std::mutex mu;
 };
 
@@ -223,8 +224,25 @@ bool stream_recording(cudaStream_t s);  // work on s goes into a graph
 cudaStream_t dev_side_stream();
 void dev_free(void *p);  // p may be null; its last use must precede on the stream
 size_t dev_mem_free();   // free device bytes, with what the pool holds unused
-void dev_ctx_born();  // (a server counts as a context)
-void dev_ctx_gone(cudaStream_t s);  // s: where the context was freed
+// The device context the library works in, as an id that no other has had:
+// after a cudaDeviceReset another one.
+unsigned long long dev_space();
+// A context of the library begins (a server counts as one), in the device
+// context returned; it is gone, and was freed on s.
+unsigned long long dev_ctx_born();
+void dev_ctx_gone(unsigned long long space, cudaStream_t s);
+// While a GoneScope(true) lives, this thread's frees are of things that went
+// with a reset device context: nothing is left to free.
+struct GoneScope {
+  explicit GoneScope(bool gone);
+  ~GoneScope();
+  GoneScope(const GoneScope &) = delete;
+  GoneScope &operator=(const GoneScope &) = delete;
+
+ private:
+  bool prev;
+};
+bool dev_gone();
 void dev_give_back();  // returns the pool's unused memory if no context is left
 // Copies a host table to the device, ordered on s; src may be reused on return.
 int dev_upload(void *dst, const void *src, size_t n, cudaStream_t s);

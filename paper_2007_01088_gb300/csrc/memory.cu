@@ -24,6 +24,7 @@
 // one context on different streams.
 // Waiting for the whole device instead would need every return code and fails
 // while any stream is being captured.
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <atomic>
@@ -38,49 +39,36 @@
 namespace cc3 {
 namespace {
 constexpr size_t KEEP = 1ull << 30;
-constexpr int MAX_DEV = 64;
+
+// Pinned buffers for table uploads: taken when the copy out of them is done.
+struct HostBuf {
+  char *p;
+  cudaEvent_t done;
+};
+constexpr size_t HOST_BYTES = 256 << 10;
+constexpr int HOST_MAX = 64;
+
+// What the library keeps in one device context.  A context that cudaDeviceReset
+// destroys takes all of it along: the next one, on the same device, has another
+// id and gets a Space of its own.
+struct Space {
+  unsigned long long id = 0;
+  cudaMemPool_t pool = nullptr;  // null where pools are not supported (then cudaMalloc serves)
+  cudaStream_t side = nullptr;
+  unsigned long long cap = 0;  // unused bytes the pool may keep
+  std::atomic<int> live{0};    // contexts and servers
+  std::mutex host_mu;
+  std::vector<HostBuf> host;  // idle or with a copy in flight (see done)
+  int host_made = 0;
+};
 
 std::mutex g_mu;
-cudaMemPool_t g_pool[MAX_DEV] = {nullptr};
-cudaStream_t g_side[MAX_DEV] = {nullptr};
-bool g_tried[MAX_DEV] = {false};
-unsigned long long g_cap[MAX_DEV] = {0};  // unused bytes the pool may keep
-std::atomic<int> g_live{0};  // contexts and servers
+std::vector<Space *> g_spaces;  // few: one per device and reset; they stay
 thread_local cudaStream_t t_stream = nullptr;
-thread_local int t_depth = 0;         // StreamScopes of this thread
-thread_local bool t_freed = false;    // something was freed in the outermost one
-
-// The device's pool; null where pools are not supported (then cudaMalloc serves).
-cudaMemPool_t pool_of(int dev) {
-  if (dev < 0 || dev >= MAX_DEV) return nullptr;
-  std::lock_guard<std::mutex> lk(g_mu);
-  if (!g_tried[dev]) {
-    g_tried[dev] = true;
-    int ok = 0;
-    cudaDeviceGetAttribute(&ok, cudaDevAttrMemoryPoolsSupported, dev);
-    cudaMemPoolProps p;
-    std::memset(&p, 0, sizeof(p));
-    p.allocType = cudaMemAllocationTypePinned;
-    p.handleTypes = cudaMemHandleTypeNone;
-    p.location.type = cudaMemLocationTypeDevice;
-    p.location.id = dev;
-    cudaMemPool_t pool = nullptr;
-    size_t fr = 0, tot = 0;
-    if (ok && cudaMemPoolCreate(&pool, &p) == cudaSuccess) {
-      cudaMemGetInfo(&fr, &tot);
-      // (a release threshold would count the memory in use as well)
-      unsigned long long keep = ~0ull;
-      g_cap[dev] = tot / 16;
-      if (cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) == cudaSuccess &&
-          cudaStreamCreateWithFlags(&g_side[dev], cudaStreamNonBlocking) == cudaSuccess)
-        g_pool[dev] = pool;
-      else
-        cudaMemPoolDestroy(pool);
-    }
-    cudaGetLastError();
-  }
-  return g_pool[dev];
-}
+thread_local int t_depth = 0;           // StreamScopes of this thread
+thread_local Space *t_space = nullptr;  // that of the outermost one
+thread_local bool t_freed = false;      // something was freed in the outermost one
+thread_local bool t_gone = false;       // frees are of memory that went with a reset
 
 int device() {
   int dev = -1;
@@ -88,30 +76,89 @@ int device() {
   return dev;
 }
 
-// Pinned buffers for table uploads: taken when the copy out of them is done.
-struct HostBuf {
-  char *p;
-  cudaEvent_t done;
-  int dev;
-};
-constexpr size_t HOST_BYTES = 256 << 10;
-constexpr int HOST_MAX = 64;
-std::mutex g_host_mu;
-std::vector<HostBuf> g_host;  // idle or with a copy in flight (see done)
-int g_host_made = 0;
+// The id of the device context that the runtime works in (through its driver
+// entry points, so that the library does not link the driver library): it
+// outlives no reset, while the context's address may return.  0: not known.
+unsigned long long context_id() {
+  using GetCurrent = CUresult (*)(CUcontext *);
+  using GetId = CUresult (*)(CUcontext, unsigned long long *);
+  static GetCurrent current = nullptr;
+  static GetId id_of = nullptr;
+  static std::once_flag once;
+  std::call_once(once, [] {
+    auto find = [](const char *name) -> void * {
+      void *f = nullptr;
+      cudaDriverEntryPointQueryResult q;
+      if (cudaGetDriverEntryPointByVersion(name, &f, 12000, cudaEnableDefault, &q) !=
+              cudaSuccess ||
+          q != cudaDriverEntryPointSuccess) {
+        cudaGetLastError();
+        return nullptr;
+      }
+      return f;
+    };
+    current = reinterpret_cast<GetCurrent>(find("cuCtxGetCurrent"));
+    id_of = reinterpret_cast<GetId>(find("cuCtxGetId"));
+  });
+  if (!current || !id_of) return 0;
+  for (int tries = 0; tries < 2; ++tries) {
+    CUcontext c = nullptr;
+    unsigned long long id = 0;
+    if (current(&c) == CUDA_SUCCESS && c && id_of(c, &id) == CUDA_SUCCESS) return id;
+    // none is current in this thread yet, or it was reset: the runtime makes one
+    if (cudaFree(nullptr) != cudaSuccess) cudaGetLastError();
+  }
+  return 0;
+}
 
-bool host_take(HostBuf *out, int dev) {
-  std::lock_guard<std::mutex> lk(g_host_mu);
-  for (size_t i = 0; i < g_host.size(); ++i)
-    if (g_host[i].dev == dev && cudaEventQuery(g_host[i].done) == cudaSuccess) {
-      *out = g_host[i];
-      g_host[i] = g_host.back();
-      g_host.pop_back();
+Space *find_space() {
+  unsigned long long id = context_id();
+  const int dev = device();
+  if (id == 0) id = ~0ull - (unsigned long long)dev;  // by device alone
+  std::lock_guard<std::mutex> lk(g_mu);
+  for (Space *s : g_spaces)
+    if (s->id == id) return s;
+  Space *s = new Space();
+  s->id = id;
+  int ok = 0;
+  cudaDeviceGetAttribute(&ok, cudaDevAttrMemoryPoolsSupported, dev);
+  cudaMemPoolProps p;
+  std::memset(&p, 0, sizeof(p));
+  p.allocType = cudaMemAllocationTypePinned;
+  p.handleTypes = cudaMemHandleTypeNone;
+  p.location.type = cudaMemLocationTypeDevice;
+  p.location.id = dev;
+  cudaMemPool_t pool = nullptr;
+  size_t fr = 0, tot = 0;
+  if (ok && cudaMemPoolCreate(&pool, &p) == cudaSuccess) {
+    cudaMemGetInfo(&fr, &tot);
+    // (a release threshold would count the memory in use as well)
+    unsigned long long keep = ~0ull;
+    s->cap = tot / 16;
+    if (cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) == cudaSuccess &&
+        cudaStreamCreateWithFlags(&s->side, cudaStreamNonBlocking) == cudaSuccess)
+      s->pool = pool;
+    else
+      cudaMemPoolDestroy(pool);
+  }
+  cudaGetLastError();
+  g_spaces.push_back(s);
+  return s;
+}
+Space *space() { return t_depth > 0 && t_space ? t_space : find_space(); }
+
+bool host_take(Space *S, HostBuf *out) {
+  std::lock_guard<std::mutex> lk(S->host_mu);
+  for (size_t i = 0; i < S->host.size(); ++i)
+    if (cudaEventQuery(S->host[i].done) == cudaSuccess) {
+      *out = S->host[i];
+      S->host[i] = S->host.back();
+      S->host.pop_back();
       return true;
     }
   cudaGetLastError();  // cudaErrorNotReady of the queries
-  if (g_host_made >= HOST_MAX) return false;
-  HostBuf b{nullptr, nullptr, dev};
+  if (S->host_made >= HOST_MAX) return false;
+  HostBuf b{nullptr, nullptr};
   if (cudaMallocHost(&b.p, HOST_BYTES) != cudaSuccess) {
     cudaGetLastError();
     return false;
@@ -121,7 +168,7 @@ bool host_take(HostBuf *out, int dev) {
     cudaFreeHost(b.p);
     return false;
   }
-  ++g_host_made;
+  ++S->host_made;
   *out = b;
   return true;
 }
@@ -138,19 +185,22 @@ static bool pool_state(cudaMemPool_t pool, unsigned long long *held, unsigned lo
 
 StreamScope::StreamScope(cudaStream_t s) : prev(t_stream) {
   t_stream = s;
-  if (t_depth++ == 0) t_freed = false;
+  if (t_depth == 0) {
+    t_space = find_space();
+    t_freed = false;
+  }
+  ++t_depth;
 }
 StreamScope::~StreamScope() {
   const cudaStream_t s = t_stream;
   t_stream = prev;
   if (--t_depth > 0 || !t_freed) return;
-  const int dev = device();
-  cudaMemPool_t pool = pool_of(dev);
+  const Space *S = t_space;
   unsigned long long held = 0, used = 0;
-  if (!pool || !pool_state(pool, &held, &used) || held <= g_cap[dev]) return;
+  if (!S->pool || !pool_state(S->pool, &held, &used) || held <= S->cap) return;
   cudaStreamSynchronize(s);  // frees under way count as used
-  if (pool_state(pool, &held, &used) && held > used + g_cap[dev])
-    cudaMemPoolTrimTo(pool, used + g_cap[dev]);
+  if (pool_state(S->pool, &held, &used) && held > used + S->cap)
+    cudaMemPoolTrimTo(S->pool, used + S->cap);
   cudaGetLastError();
 }
 
@@ -207,6 +257,7 @@ static bool wait_device() {
 }
 
 bool ctx_order(cc3_ctx *c, cudaStream_t s) {
+  if (c->space != dev_space()) return true;  // its memory and its work went with a reset
   return (!c->unmarked && after_last(c, s)) || wait_device();
 }
 
@@ -219,14 +270,12 @@ DeviceScope::~DeviceScope() {
   if (prev >= 0) cudaSetDevice(prev);
 }
 
-cudaStream_t dev_side_stream() {
-  const int dev = device();
-  return pool_of(dev) ? g_side[dev] : nullptr;
-}
+unsigned long long dev_space() { return space()->id; }
+cudaStream_t dev_side_stream() { return space()->side; }
 
 cudaError_t dev_malloc_bytes(void **p, size_t n) {
   *p = nullptr;
-  cudaMemPool_t pool = pool_of(device());
+  cudaMemPool_t pool = space()->pool;
   if (!pool) return cudaMalloc(p, n);
   // no allocation becomes part of a caller's graph
   if (stream_recording(t_stream)) return cudaErrorStreamCaptureUnsupported;
@@ -242,9 +291,9 @@ cudaError_t dev_malloc_bytes(void **p, size_t n) {
 }
 
 void dev_free(void *p) {
-  if (!p) return;
+  if (!p || t_gone) return;
   t_freed = true;
-  if (!pool_of(device())) {
+  if (!space()->pool) {
     cudaFree(p);
   } else if (cudaFreeAsync(p, t_stream) != cudaSuccess) {
     cudaGetLastError();
@@ -260,37 +309,48 @@ size_t dev_mem_free() {
     cudaGetLastError();
     return 0;
   }
-  if (cudaMemPool_t pool = pool_of(device())) {
+  if (cudaMemPool_t pool = space()->pool) {
     unsigned long long held = 0, used = 0;
     if (pool_state(pool, &held, &used) && held > used) fr += (size_t)(held - used);
   }
   return fr;
 }
 
-void dev_ctx_born() { ++g_live; }
-void dev_ctx_gone(cudaStream_t s) {
-  if (--g_live > 0) return;
+unsigned long long dev_ctx_born() {
+  Space *S = space();
+  ++S->live;
+  return S->id;
+}
+void dev_ctx_gone(unsigned long long id, cudaStream_t s) {
+  Space *S = space();
+  if (id != S->id || --S->live > 0) return;
   cudaStreamSynchronize(s);
-  if (cudaMemPool_t pool = pool_of(device())) cudaMemPoolTrimTo(pool, KEEP);
+  if (S->pool) cudaMemPoolTrimTo(S->pool, KEEP);
   cudaGetLastError();
 }
 void dev_give_back() {
-  if (g_live > 0) return;
-  if (cudaMemPool_t pool = pool_of(device())) cudaMemPoolTrimTo(pool, 0);
+  Space *S = space();
+  if (S->live > 0 || !S->pool) return;
+  cudaMemPoolTrimTo(S->pool, 0);
   cudaGetLastError();
 }
+
+GoneScope::GoneScope(bool gone) : prev(t_gone) { t_gone = gone; }
+GoneScope::~GoneScope() { t_gone = prev; }
+bool dev_gone() { return t_gone; }
 
 int dev_upload(void *dst, const void *src, size_t n, cudaStream_t s) {
   if (n == 0) return CC3_OK;
   HostBuf b;
-  if (n <= HOST_BYTES && host_take(&b, device())) {
+  Space *S = space();
+  if (n <= HOST_BYTES && host_take(S, &b)) {
     std::memcpy(b.p, src, n);
     cudaError_t e = cudaMemcpyAsync(dst, b.p, n, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaEventRecord(b.done, s);
     if (e != cudaSuccess) cudaStreamSynchronize(s);  // no copy out of the buffer is left
     {
-      std::lock_guard<std::mutex> lk(g_host_mu);
-      g_host.push_back(b);
+      std::lock_guard<std::mutex> lk(S->host_mu);
+      S->host.push_back(b);
     }
     return e == cudaSuccess ? CC3_OK : CC3_FAIL(CC3_ERR_CUDA, cudaGetErrorString(e));
   }

@@ -93,6 +93,7 @@ void copy_in(std::vector<T> &dst, const T *src, size_t n) {
 
 struct cc3_server {
   int device = 0;
+  unsigned long long space = 0;  // see dev_ctx_born
   size_t budget = 0, in_use = 0, peak = 0;
   int max_slots = 1;
   std::mutex mu;
@@ -249,7 +250,8 @@ int cc3_serve_start(cc3_server **out, size_t hbm_budget_bytes, int max_slots) {
   S->budget = hbm_budget_bytes;
   S->max_slots = max_slots;
   S->t0 = Clock::now();
-  cc3::dev_ctx_born();  // its requests' contexts share the pool's unused memory
+  // its requests' contexts share the pool's unused memory
+  S->space = cc3::dev_ctx_born();
   try {
     for (int i = 0; i < max_slots; ++i) S->workers.emplace_back(worker_main, S);
   } catch (...) {
@@ -259,7 +261,7 @@ int cc3_serve_start(cc3_server **out, size_t hbm_budget_bytes, int max_slots) {
     }
     S->cv_work.notify_all();
     for (auto &t : S->workers) t.join();
-    cc3::dev_ctx_gone(cc3::dev_side_stream());
+    cc3::dev_ctx_gone(S->space, cc3::dev_side_stream());
     delete S;
     return CC3_ERR_OOM;
   }
@@ -415,7 +417,7 @@ int cc3_serve_stop(cc3_server *S) {
   S->cv_done.notify_all();
   for (auto &t : S->workers) t.join();
   cc3::DeviceScope dev(S->device);
-  cc3::dev_ctx_gone(cc3::dev_side_stream());
+  cc3::dev_ctx_gone(S->space, cc3::dev_side_stream());
   delete S;
   cc3::dev_give_back();
   return CC3_OK;

@@ -149,7 +149,7 @@ int alloc(T **p, size_t n) {
 }
 
 void drop_graph(SplitState *S) {
-  if (S->gexec) cudaGraphExecDestroy(S->gexec);
+  if (S->gexec && !dev_gone()) cudaGraphExecDestroy(S->gexec);
   S->gexec = nullptr;
   S->g_calls = 0;
 }

@@ -175,3 +175,36 @@ assert f0 - free() <= slack, f0 - free()
 """
     r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, r.stderr[-2000:]
+
+
+def test_device_reset_between_contexts():
+    """After a cudaDeviceReset new contexts work, and a context from before it can still
+    be destroyed.  In a process of its own."""
+    import subprocess
+    import sys
+    code = """
+import ctypes
+import numpy as np
+import paper_2007_01088_gb300 as g
+from cc3_inputs import make_inputs
+
+rt = ctypes.CDLL("libcudart.so.13")
+inp = make_inputs(4, 16, seed=1)
+
+def run():
+    old = g.Context(inp)
+    res = [old.omega(p)[1] for p in (g.CC3_FP64, g.CC3_SPLIT_BF16)]
+    g.Context(inp).close()
+    return old, res
+
+old, ref = run()
+for _ in range(2):
+    assert rt.cudaDeviceReset() == 0
+    new, got = run()
+    old.close()
+    old = new
+    for x, y in zip(got, ref):
+        assert np.abs(x - y).max() <= 1e-13 * np.abs(y).max()
+"""
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
