@@ -17,7 +17,6 @@
 // stale).  All calls share the array, so calls that overlap on the GPU race;
 // the contents left by the previous call are not relied on (the accumulators
 // are cleared at the start of each call).
-#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -36,30 +35,10 @@ static __device__ __align__(256) double g_noalloc_scratch[kScratchDoubles];
 
 std::mutex g_mu;
 struct ScratchSlot {
-  CUcontext ctx = nullptr;  // the device context the address belongs to
+  unsigned long long space = 0;  // the device context the address belongs to
   double *ptr = nullptr;
 };
 ScratchSlot g_slot[64];
-
-// The calling thread's current driver context (the runtime's primary context
-// of the current device once it is initialised), through the runtime's
-// driver entry point so that the library does not link the driver library.
-CUcontext current_context() {
-  using GetCurrent = CUresult (*)(CUcontext *);
-  static GetCurrent fn = nullptr;
-  static std::once_flag once;
-  std::call_once(once, [] {
-    void *f = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &f, 12000, cudaEnableDefault, &q) ==
-            cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<GetCurrent>(f);
-  });
-  CUcontext c = nullptr;
-  if (!fn || fn(&c) != CUDA_SUCCESS) return nullptr;
-  return c;
-}
 
 // Device address of the scratch array for the current device: set up on the
 // first call per device, and again when the device's context changed.
@@ -69,13 +48,13 @@ int scratch_for_current_device(double **out) {
     return CC3_FAIL(CC3_ERR_CUDA, "no current device");
   std::lock_guard<std::mutex> lk(g_mu);
   ScratchSlot &S = g_slot[dev];
-  CUcontext now = current_context();
-  if (!S.ptr || !now || now != S.ctx) {
+  const unsigned long long now = cc3::dev_space();
+  if (!S.ptr || now != S.space) {
     void *p = nullptr;
     const cudaError_t e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
     if (e != cudaSuccess || !p) return CC3_FAIL(CC3_ERR_CUDA, cudaGetErrorString(e));
     S.ptr = static_cast<double *>(p);
-    S.ctx = current_context();  // the lookup made the device's context current
+    S.space = now;
   }
   *out = S.ptr;
   return CC3_OK;

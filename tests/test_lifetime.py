@@ -178,8 +178,8 @@ assert f0 - free() <= slack, f0 - free()
 
 
 def test_device_reset_between_contexts():
-    """After a cudaDeviceReset new contexts work, and a context from before it can still
-    be destroyed.  In a process of its own."""
+    """After a cudaDeviceReset new contexts work, the residual without allocation too,
+    and a context from before it can still be destroyed.  In a process of its own."""
     import subprocess
     import sys
     code = """
@@ -191,11 +191,30 @@ from cc3_inputs import make_inputs
 rt = ctypes.CDLL("libcudart.so.13")
 inp = make_inputs(4, 16, seed=1)
 
+def noalloc():
+    bufs = []
+    def dev(n, x=None):
+        p = ctypes.c_void_p()
+        assert rt.cudaMalloc(ctypes.byref(p), ctypes.c_size_t(8 * n)) == 0
+        if x is not None:
+            x = np.ascontiguousarray(x)
+            assert rt.cudaMemcpy(p, x.ctypes.data_as(ctypes.c_void_p),
+                                 ctypes.c_size_t(8 * n), 1) == 0
+        return p
+    src = [dev(getattr(inp, k).size, getattr(inp, k))
+           for k in ("eps_o", "eps_v", "t2", "g_vvvo", "g_ooov", "g_ovov", "F_ov")]
+    o1, o2, e = dev(64), dev(16 * 256), dev(1)
+    assert g.lib.cc3_omega_triples_noalloc(4, 16, *src, o1, o2, e, None) == 0
+    out = np.zeros((4, 4, 16, 16))
+    assert rt.cudaMemcpy(out.ctypes.data_as(ctypes.c_void_p), o2,
+                         ctypes.c_size_t(out.nbytes), 2) == 0
+    return out
+
 def run():
     old = g.Context(inp)
     res = [old.omega(p)[1] for p in (g.CC3_FP64, g.CC3_SPLIT_BF16)]
     g.Context(inp).close()
-    return old, res
+    return old, res + [noalloc()]
 
 old, ref = run()
 for _ in range(2):
