@@ -28,6 +28,14 @@
  * on that context (inputs and outputs) is a device pointer; otherwise all are
  * host pointers and the call copies and synchronises.
  *
+ * Device memory: all of it comes from a pool of the library's own.  What
+ * contexts and calls give back stays in the pool for the next ones, up to 1/16
+ * of the device's memory while a context or a server exists and up to 1 GiB
+ * after the last is gone; other allocators of the process do not see it.
+ * cc3_serve_stop returns it when no context is left, cc3_memory_release at any
+ * time.  A context may be destroyed, or given other triples, while a call on it
+ * is still running; calls on one context from different streams run in order.
+ *
  * Threading: calls on one context are serialised by the caller; distinct
  * contexts may be used from different threads.  cuda_stream may be NULL (the
  * legacy default stream) or a cudaStream_t.
@@ -318,6 +326,12 @@ int cc3_ctx_autotune(cc3_ctx *ctx, void *cuda_stream, int *ksteps_per_tile, int 
 /* The split path's current tiling (tuned or default). */
 int cc3_ctx_get_tuning(cc3_ctx *ctx, int *ksteps_per_tile, int *ntile_w);
 
+/* Returns to the device what the library holds unused on the current device
+ * (see "Device memory" above), and its idle host buffers.  Waits for the
+ * device, so it must not be called while a stream is being captured
+ * (CC3_ERR_CUDA). */
+int cc3_memory_release(void);
+
 const char *cc3_strerror(int status);
 
 /* Detail of the most recent failure on the calling thread (the library call
@@ -356,7 +370,8 @@ typedef struct {
 /* Starts a server on the current device with max_slots (1..64) worker
  * threads, each with its own CUDA stream; at most max_slots requests run at
  * once.  hbm_budget_bytes bounds the summed device footprint of the running
- * requests (0: 90 % of the free device memory at start). */
+ * requests (0: 90 % of the free device memory at start); what the pool holds
+ * unused between them (see "Device memory") is not counted. */
 int cc3_serve_start(cc3_server **out, size_t hbm_budget_bytes, int max_slots);
 /* Device bytes a request needs while it runs (inputs, workspace, the
  * Jacobian's intermediates and per-vector buffers); the admission test. */

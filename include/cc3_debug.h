@@ -14,6 +14,7 @@
  */
 #ifndef CC3_DEBUG_H
 #define CC3_DEBUG_H
+#include <stddef.h>
 #ifdef __cplusplus
 extern "C" {
 #endif
@@ -40,6 +41,11 @@ int cc3_debug_wait_timeout(double limit_s);
  * measure the sums' rounding.  Synchronous, on the legacy default stream. */
 int cc3_debug_doo_pairs(int no, int nv, const float *tau, const float *lt, double *D_oo,
                         int blocks_per_pair);
+
+/* Bytes that the library's pool on the current device holds, those in use, and
+ * the most in use since the last call (which starts that count anew).  Waits for
+ * the device.  CC3_ERR_UNSUPPORTED where the device has no pools. */
+int cc3_debug_memory(size_t *held, size_t *used, size_t *peak);
 #ifdef __cplusplus
 }
 #endif

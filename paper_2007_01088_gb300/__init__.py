@@ -41,7 +41,8 @@ EXPORTED = ["cc3_ctx_create", "cc3_ctx_destroy", "cc3_ctx_set_triples",
             "cc3_ctx_trace", "cc3_omega_triples_noalloc", "cc3_serve_footprint",
             "cc3_ctx_autotune", "cc3_ctx_get_tuning", "cc3_cvs_triples",
             "cc3_denominator_gap", "cc3_debug_wait_timeout", "cc3_ctx_create_general",
-            "cc3_left_jacobian_triples", "cc3_density_triples", "cc3_debug_doo_pairs"]
+            "cc3_left_jacobian_triples", "cc3_density_triples", "cc3_debug_doo_pairs",
+            "cc3_memory_release", "cc3_debug_memory"]
 
 
 class CC3Error(RuntimeError):
@@ -120,6 +121,11 @@ def _load():
     L.cc3_debug_split_gemm.restype = I
     L.cc3_debug_doo_pairs.argtypes = [I, I, P, P, P, I]
     L.cc3_debug_doo_pairs.restype = I
+    SP = ctypes.POINTER(ctypes.c_size_t)
+    L.cc3_memory_release.argtypes = []
+    L.cc3_memory_release.restype = I
+    L.cc3_debug_memory.argtypes = [SP, SP, SP]
+    L.cc3_debug_memory.restype = I
     L.cc3_debug_wait_timeout.argtypes = [D]
     L.cc3_debug_wait_timeout.restype = I
     L.cc3_ctx_set_tracing.argtypes = [P, I]
@@ -337,6 +343,19 @@ def cc3_ctx_get_tuning(ctx):
 
 def cc3_ctx_set_slices(ctx, slices):
     _check(lib.cc3_ctx_set_slices(ctx, int(slices)), "cc3_ctx_set_slices")
+
+
+def cc3_memory_release():
+    """Returns to the device what the library holds unused on the current device."""
+    _check(lib.cc3_memory_release(), "cc3_memory_release")
+
+
+def cc3_debug_memory():
+    """Bytes the library's pool holds, those in use, and the most in use since the last
+    call (diagnostic)."""
+    v = [ctypes.c_size_t(0) for _ in range(3)]
+    _check(lib.cc3_debug_memory(*(ctypes.byref(x) for x in v)), "cc3_debug_memory")
+    return tuple(x.value for x in v)
 
 
 def cc3_debug_wait_timeout(limit_s=1e-3):

@@ -12,7 +12,7 @@
 // The pool keeps at most 1/16 of the device's memory unused while a context or
 // a server exists (trimmed at the end of each entry point that freed something)
 // and at most KEEP bytes after the last one is gone; cc3_serve_stop gives back
-// the rest as well when nothing is left.  Only memory whose free the host has seen
+// the rest as well when nothing is left, cc3_memory_release at any time.  Only memory whose free the host has seen
 // complete can be trimmed, so the stream of the frees is waited for before.  A
 // failed allocation first returns all that is unused and tries again.
 // dev_mem_free counts what the pool holds unused as free.
@@ -361,3 +361,36 @@ int dev_upload(void *dst, const void *src, size_t n, cudaStream_t s) {
 }
 
 }  // namespace cc3
+
+extern "C" int cc3_memory_release(void) {
+  using namespace cc3;
+  Space *S = space();
+  if (cudaDeviceSynchronize() != cudaSuccess)  // what is being freed can be given back too
+    return CC3_FAIL(CC3_ERR_CUDA, cudaGetErrorString(cudaGetLastError()));
+  if (S->pool && cudaMemPoolTrimTo(S->pool, 0) != cudaSuccess)
+    return CC3_FAIL(CC3_ERR_CUDA, cudaGetErrorString(cudaGetLastError()));
+  std::lock_guard<std::mutex> lk(S->host_mu);
+  for (HostBuf &b : S->host) {  // (no copy out of them is left)
+    cudaEventDestroy(b.done);
+    cudaFreeHost(b.p);
+  }
+  S->host_made -= (int)S->host.size();
+  S->host.clear();
+  return CC3_OK;
+}
+
+extern "C" int cc3_debug_memory(size_t *held, size_t *used, size_t *peak) {
+  using namespace cc3;
+  if (!held || !used || !peak) return CC3_ERR_ARG;
+  cudaMemPool_t pool = space()->pool;
+  if (!pool) return CC3_ERR_UNSUPPORTED;
+  unsigned long long h = 0, u = 0, p = 0, zero = 0;
+  if (cudaDeviceSynchronize() != cudaSuccess || !pool_state(pool, &h, &u) ||
+      cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemHigh, &p) != cudaSuccess ||
+      cudaMemPoolSetAttribute(pool, cudaMemPoolAttrUsedMemHigh, &zero) != cudaSuccess)
+    return CC3_FAIL(CC3_ERR_CUDA, cudaGetErrorString(cudaGetLastError()));
+  *held = h;
+  *used = u;
+  *peak = p;
+  return CC3_OK;
+}

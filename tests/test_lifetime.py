@@ -167,6 +167,12 @@ for _ in range(2):
     assert f0 - free() > 5 << 28, f0 - free()
     c.close()
     assert f0 - free() <= (1 << 30) + slack, f0 - free()
+live = run(make_inputs(3, 8, seed=1))
+run(big).close()
+assert f0 - free() > 5 << 28, f0 - free()
+g.cc3_memory_release()
+assert f0 - free() <= slack, f0 - free()
+live.close()
 srv = g.Server(max_slots=2)
 tickets = [srv.submit_omega(make_inputs(6, 60, seed=n)) for n in range(4)]
 assert all(srv.wait(t)[0] == g.CC3_OK for t in tickets)
