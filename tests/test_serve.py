@@ -144,21 +144,24 @@ def test_cancel_queued_and_wait_timeout(g):
 
 
 def test_footprint_bounds_device_memory(g):
-    import torch
-    torch.cuda.init()
+    """The most device memory in use at a time while a request is served, alone."""
     srv = g.Server(max_slots=1)
     try:
         for prec, no, nv in [(g.CC3_FP64, 6, 60), (g.CC3_SPLIT_BF16, 6, 60),
-                             (g.CC3_FP64, 10, 48)]:
+                             (g.CC3_FP64, 10, 48), (g.CC3_SPLIT_BF16, 9, 33)]:
             inp = make_inputs(no, nv, seed=9)
-            fp = srv.footprint(0, prec, inp)
-            torch.cuda.synchronize()
-            free0 = torch.cuda.mem_get_info()[0]
-            ctx = g.Context(inp)
-            ctx.omega(prec)
-            used = free0 - torch.cuda.mem_get_info()[0]
-            ctx.close()
-            assert used <= fp, (prec, no, nv, used, fp)
+            R1, R2 = make_trial_vectors(no, nv, 2, seed=9)
+            for kind in (0, 1):
+                w = np.array([0.2, -0.1])
+                fp = srv.footprint(kind, prec, inp, *((2, w, R1, R2) if kind else ()))
+                before = g.cc3_debug_memory()[1]
+                t = (srv.submit_jacobian(inp, R1, R2, w, prec) if kind
+                     else srv.submit_omega(inp, prec))
+                assert srv.wait(t)[0] == g.CC3_OK
+                used = g.cc3_debug_memory()[2] - before
+                assert used <= fp, (prec, no, nv, kind, used, fp)
+                # and not far above: the budget is there to be used
+                assert fp <= 3 * used + (64 << 20), (prec, no, nv, kind, used, fp)
     finally:
         srv.stop()
 
