@@ -48,7 +48,7 @@ __device__ __forceinline__ unsigned long long sub2(unsigned long long a, unsigne
 // The two-sums of the high and of the low parts run as one packed two-sum: 14
 // issue slots for 20 at the same FP32 lanes (a packed addition takes as long as
 // two, 123 lane operations a clock and SM for 126), so it pays where issue is
-// the limit: left_outer_dd 2.06 -> 1.73 ms at no=9 nv=81.
+// the limit: left_outer_dd 1.73 ms at no=9 nv=81, 2.06 with single operations.
 __device__ __forceinline__ df add(df a, df b) {
   const unsigned long long x = pack2(a.hi, a.lo), y = pack2(b.hi, b.lo);
   const unsigned long long s2 = add2(x, y), bb = sub2(s2, x);

@@ -406,6 +406,10 @@ int density_fp64(cc3_ctx *c, double w, const double *L1d, const double *L2d, dou
 // addition takes 16 clocks of this part's FP64 pipe per warp, and the totals of
 // a block of products would not fit the registers: they are in local memory).
 // The terms keep ~2^-44 of their size, well inside the FP64 path's agreement.
+// no=12 nv=120: 15.5 ms (one thread per product, rows read element by element,
+// 28.6; 14.8 with one pair for all of a thread's terms).  DOO_PF rows in flight:
+// 12 of 6, 12, 16 and 20 take least at no = 8 and 12, within 5 % of the least at no
+// = 16, 20 and 26 (no=16 nv=64 7.4, 6.7, 6.4 and 6.7 ms).
 constexpr int DOO_E = 128, DOO_T = 4, DOO_PF = 12;
 __host__ __device__ constexpr int doo_rows(int no) { return (no + DOO_T - 1) / DOO_T * DOO_T; }
 __global__ void __launch_bounds__(256)
@@ -647,8 +651,9 @@ int density_doo_resident(cc3_ctx *c, const float2 *tau_all, const float2 *lt_all
   const int gz = (doo_rows(no) / DOO_T * (doo_rows(no) / DOO_T) + 255) / 256;
   // blocks per pair: of up to 32 blocks per SM in all, the number whose rounds
   // over the SMs take the fewest units (one more per block for its start and
-  // reduction).  At no=12 nv=120 about four blocks per SM, 8 per pair, were 2.05
-  // rounds of two per SM: 18.4 ms; this rule takes 35 per pair, 8.98 rounds, 14.8 ms.
+  // reduction).  At no=12 nv=120 about four blocks per SM, 8 per pair, would be 2.05
+  // rounds of two per SM and take a quarter longer than the rule's 35 per pair, 8.98
+  // rounds.
   int per_sm = 0;
   CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, doo_pairs_kernel, 256, smem));
   const long long slots = (long long)std::max(1, per_sm) * nsm, per_gx = (long long)npair * gz;

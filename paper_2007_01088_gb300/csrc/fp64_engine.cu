@@ -183,7 +183,9 @@ fp64_engine_kernel(const Job *__restrict__ jobs, int njobs,
 // sigma1's Cholesky contraction at no=9 nv=81 (an 81 x 9 output over K =
 // 21,870: 3 tiles) took 9 ms on 3 SMs.  Four tiles per SM, many of them of five
 // on some: no=6 nv=48 FP64 residual 7.29 ms for 6.97, the left transformation's
-// thin launches at no=9 nv=81 2.12 ms for 1.71; 16 per SM take as long as 8.
+// thin launches at no=9 nv=81 2.12 ms for 1.71; 16 per SM take as long as 8.  FILL
+// is a constant (152 SMs), not the device's count: with reproducible sums the
+// parts decide the bits.
 static long long split_small_launch(std::vector<Job> &jobs, const std::vector<Term> &terms) {
   constexpr double FILL = 1216.0;
   double work = 0.0;

@@ -184,8 +184,10 @@ void plan_omega_contractions(Plan &P, int no, int nv, const int ijk[3],
   const long long nv2 = (long long)nv * nv, nv3 = nv2 * nv;
   const long long st[3] = {nv2, nv, 1};  // tau~[a][b][c] slot strides
   // a multiple of 16 leaves the singles column a group of 16 columns of its own
-  // (64 x 64 tiles); in the thin tiles' 4 columns it costs a third of that: no=6
-  // nv=48 residual 6.97 -> 6.72 ms.  At other nv it rides in the last group.
+  // (64 x 64 tiles); in the thin tiles' 4 columns it costs a third of that.
+  // Residual with it there and here: nv=32 1.64 and 1.71 ms, 48 6.62 and 6.92, 64
+  // 18.6 and 21.0, 96 54.5 and 55.4, 128 79.4 and 84.6.  At other nv it rides in the
+  // last group.
   const bool own_tail = (which & 16) && nv % 16 == 0;
   int seen[6][3];
   int nseen = 0;

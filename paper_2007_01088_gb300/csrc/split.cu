@@ -168,10 +168,11 @@ void free_state_buffers(SplitState *S) {
 // Triples in flight: up to 16 within 6 GB of workspace and, where they are
 // small, up to 48 within 1 GB, in batches of about equal size: a batch costs
 // four launches and two tails of the engine's tiles, which at nv = 30 is most
-// of its time.  Contexts of the serving loop keep to 16, the figure its
-// footprints are computed with.  Measured (with the launches per batch going
-// from nine to four): no=5 nv=30 307 -> 240 us, no=8 nv=72 4.20 -> 3.47 ms, no=11
-// nv=87 14.1 -> 12.9 ms; at nv = 160 the rule keeps 16.
+// of its time.  With at most 16, 32, 48 and 64: no=5 nv=30 215, 150, 149 and 152
+// us, no=8 nv=40 1.18, 0.85, 0.73 and 0.67 ms, no=12 nv=48 4.48, 3.13, 2.87 and
+// 2.81, no=10 nv=60 3.65, 3.15, 2.94 and 2.91; at nv = 87 1 GB holds 23 and 11.4
+// for 11.7 ms is all of it, at nv = 160 the rule keeps 16.  Contexts of the serving
+// loop keep to 16, the figure its footprints are computed with.
 int slots_of(int nv, int s, int ntri, bool small) {
   const double nv2 = (double)nv * nv, per_slot = nv2 * nv * 24.0 + 6.0 * s * nv2 * rup(nv, 16);
   double most = std::min(16.0, 6.0e9 / per_slot);

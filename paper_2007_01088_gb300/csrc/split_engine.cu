@@ -10,8 +10,11 @@
 // each level L = p + q <= 3 gets its own tensor-memory accumulator, whose
 // values stay exactly representable (multiples of 2^-8L below 2^(24-8L))
 // because it is drained into 64-bit fixed-point registers every 256 to 900 K;
-// the levels >= 4 share a fifth, rounded accumulator (its error stays below
-// 2^-50 of the result).
+// the levels >= 4 share a fifth, rounded accumulator that a tile keeps to its
+// end.  What that rounds off grows with the tile's K steps n: at most
+// 22 2^-23 5 2^-32 16 n (n + 1) / 2 of the largest digit product at 6 slices; on
+// random operands 6e-14 of it at n = 100, 4.8e-13 at 400 and 1.4e-12 at 800, next to
+// 1.1e-13, 2.1e-13 and 3.0e-13 that the products left out cost.
 //
 // Warp roles (608 threads): warp 18 decodes tiles and their terms ahead of the
 // others; warp 0 issues one bulk copy per operand tile (all
@@ -31,18 +34,15 @@
 // with levels 0..3 while that one is read.
 //
 // What bounds it: a 128 x 96 x 16 product takes 53 clocks here (48 at the
-// nominal rate; 21 of them per K step, 1118 clocks, next to 43 KB of operands
-// arriving), so the issuer must add little to that.  Measured in the engine on
-// 96 triples of the no=22 nv=250 residual, clocks per K step: 1902 with the
-// sums in double-float arithmetic (a tile's read-back 7600 clocks, its outputs
-// 23,700: FP64 conversions, one 8-byte store per 32-byte sector in the W
-// build's first phase); 1570 with fixed-point sums and overlapped tile ends;
-// 1525 with the decoder warp; 1361 with the issuer's operands known to be
-// uniform (4 instructions per product instead of 11; the kernel's code
-// 178 -> 88 KB, it had outgrown the instruction cache), one level drained at a
-// time and the last column tile trimmed.  Pairs of steps in sequence instead of
-// with interleaved A runs (a stage is then free 1000 clocks earlier) and the
-// next pair's signs read ahead: 166.9 -> 158.8 ms for those triples.  Every wait is
+// nominal rate), the 21 of a K step 1118 next to 43 KB of operands arriving, so
+// the issuer must add little to that.  It takes 1271 on 96 triples of the no=22
+// nv=250 residual (1902 with one divergent thread issuing, double-float sums and
+// the tile's ends one after the other): its operands are known to be uniform (4
+// instructions per product, not 11), one level is drained at a time, the last
+// column tile is trimmed, steps run in sequence (pairs with interleaved A runs
+// hold a stage 1000 clocks longer: 158.8 ms for those triples, so 166.9) and the
+// next pair's signs are read ahead.  The kernel's code is kept at 88 KB: at 178 KB
+// it had outgrown the instruction cache.  Every wait is
 // bounded: on timeout the CTA sets an error word that the host turns into
 // CC3_ERR_TIMEOUT; before it exits, the CTA waits (bounded again) for its own
 // bulk copies and tensor-core products in flight, then frees its tensor
