@@ -642,8 +642,9 @@ int density_doo_resident(cc3_ctx *c, const float2 *tau_all, const float2 *lt_all
   if (bytes() > 227 * 1024) ld = DOO_E;
   const size_t smem = bytes();
   if (smem > 227 * 1024) return CC3_FAIL(CC3_ERR_UNSUPPORTED, "too many occupied orbitals");
+  // the limit, not this call's size: another thread may set it before the launch
   CU(cudaFuncSetAttribute(doo_pairs_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                          (int)smem));
+                          227 * 1024));
   const long long nunit = (long long)((nv + 3) / 4) * ((nv + 3) / 4);
   int dev = 0, nsm = 0;
   CU(cudaGetDevice(&dev));

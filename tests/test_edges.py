@@ -201,6 +201,35 @@ def test_fp64_left_at_tile_edges(g, no, nv):
         assert np.abs(x - y).max() <= 1e-11 * np.abs(y).max()
 
 
+def test_densities_of_several_sizes_at_once(g):
+    """The D_oo kernel takes 8 KB of shared memory for 4 occupied orbitals, 57 KB for 28."""
+    probs = []
+    for no, nv in ((4, 8), (28, 3)):
+        inp = make_inputs(no, nv, seed=no)
+        L1, L2 = make_trial_vectors(no, nv, 1, seed=no)
+        ref = oracle.density_inputs(inp, 0.2, L1[0], L2[0])
+        probs.append((inp, L1[0], L2[0], [ref[k] for k in ("Doo", "Dov", "Dvv")]))
+    bad = []
+
+    def work(p):
+        inp, L1, L2, ref = probs[p]
+        c = g.Context(inp)
+        for _ in range(40):
+            try:
+                d = c.density(L1, L2, 0.2, prec=g.CC3_SPLIT_BF16)
+                if not all(split_close(x, y) for x, y in zip(d, ref)):
+                    bad.append(p)
+            except g.CC3Error as e:
+                bad.append(str(e))
+
+    threads = [threading.Thread(target=work, args=(p,)) for p in (0, 0, 1, 1)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not bad, bad
+
+
 def test_contexts_of_several_threads_share_the_pool(g):
     """Contexts made, used and destroyed by four threads on streams of their own give
     the results they give alone: no block of the pool serves two of them at a time."""
